@@ -105,8 +105,10 @@ struct amph_ctx {
   size_t fork_used = 0;
   cudaEvent_t join_ev = nullptr;
   bool side_dirty = false;                // helpers were launched since the last join
-  cudaGraphExec_t graph_exec = nullptr;   // captured draft -> verify -> accept schedule of amph_step
-  long long graph_key = -1; // attention split counts the captured grids were sized for
+  // captured draft -> verify -> accept schedules of amph_step, by the attention grids they were sized for
+  struct StepGraph { long long key; cudaGraphExec_t exec; unsigned long long used; };
+  std::vector<StepGraph> graphs;          // at most kMaxGraphs
+  unsigned long long graph_tick = 0;
   bool graph_off = false;   // capture is not possible (legacy stream, flag) or failed once
   bool prof_on = false;     // bracket projection launches with events (amph_profile_begin / end)
   std::vector<cudaEvent_t> prof_ev;
@@ -121,6 +123,7 @@ struct amph_ctx {
   DevState* state(int b) const { return grp<DevState>(lay.state, lay.state_s, b); }
   RowMeta* meta_v(int g) const { return grp<RowMeta>(lay.meta_v, lay.meta_s_, g); }
   RowMeta* meta_s(int g) const { return grp<RowMeta>(lay.meta_s, lay.meta_s_, g); }
+  void drop_graphs() { for (auto& g : graphs) cudaGraphExecDestroy(g.exec); graphs.clear(); }
   int max_ctx_hi() const { int m = 0; for (int b = 0; b < B; ++b) m = ctx_hi[b] > m ? ctx_hi[b] : m; return m; }
 };
 
@@ -827,9 +830,20 @@ amph_status check_capacity(amph_ctx* ctx) {
   return AMPH_OK;
 }
 
-// The captured schedule depends on the host's bounds only through the attention launches of every sequence.
+// Captured schedules kept per context.  A text grows through one split count per 128 tokens and starts over with the next
+// prompt (or with amph_set_state), so the grids recur.  Capturing and instantiating the 300 launches of a 7B step anew costs
+// the stream about 0.4 ms per change: 12 steps from C = 512, which cross two of them, 45.99 -> 45.12 ms; a batch, whose key
+// used to hold every sequence's count, 166.2 -> 164.4 ms (4 sequences, 16 steps).  Seven split counts in two passes (the
+// drafting one runs at most one split behind) are 13 combinations.
+constexpr size_t kMaxGraphs = 16;
+
+// The captured schedule depends on the host's bounds only through the attention launches: one per sequence, or, where the
+// sequences of a batch share a launch (layer_forward), one sized for the longest of them.
 long long graph_key_of(const amph_ctx* ctx) {
   long long key = 0;
+  if (ctx->attn_tc && ctx->B > 1 && !(ctx->cfg.flags & AMPH_FLAG_SEPARATE_MERGE))
+    return attn_splits_for(ctx, ctx->max_ctx_hi(), ctx->rows_small) * 128 +
+           attn_splits_for(ctx, ctx->max_ctx_hi() + ctx->tree_host.n_nodes, ctx->Mver);
   for (int b = 0; b < ctx->B; ++b)
     key = key * 4099 + attn_splits_for(ctx, ctx->ctx_hi[b], ctx->rows_small) * 128 +
           attn_splits_for(ctx, ctx->ctx_hi[b] + ctx->tree_host.n_nodes, ctx->Mver);
@@ -945,11 +959,7 @@ amph_status amph_load_weights(amph_ctx* ctx, const amph_tensor* tensors, int32_t
     ctx->tensors[t.name] = r;
   }
   ctx->resolved = false;
-  if (ctx->graph_exec) {                       // the captured schedule holds the old pointers
-    cudaGraphExecDestroy(ctx->graph_exec);
-    ctx->graph_exec = nullptr;
-    ctx->graph_key = -1;
-  }
+  ctx->drop_graphs();                          // the captured schedules hold the old pointers
   return AMPH_OK;
 }
 
@@ -1091,23 +1101,31 @@ amph_status amph_step(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n) {
   if (rc != AMPH_OK) return rc;
   const amph_config& c = ctx->cfg;
   const bool use_graph = !ctx->graph_off && !ctx->prof_on && !(c.flags & AMPH_FLAG_NO_GRAPH) && ctx->stream != nullptr;
+  cudaGraphExec_t exec = nullptr;
   if (use_graph) {
     // The kernels read every length from device state; only the attention grids depend on the host's
-    // bound of the context length, so the captured schedule is reused until that grid size changes.
+    // bound of the context length, so a captured schedule serves every step with the same grids.
     const long long key = graph_key_of(ctx);
-    if (!ctx->graph_exec || key != ctx->graph_key) {
-      if (ctx->graph_exec) { cudaGraphExecDestroy(ctx->graph_exec); ctx->graph_exec = nullptr; }
+    for (auto& g : ctx->graphs)
+      if (g.key == key) { exec = g.exec; g.used = ++ctx->graph_tick; }
+    if (!exec) {
       cudaGraph_t graph = nullptr;
       if (cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
         rc = do_draft(ctx, nullptr, nullptr);
         if (rc == AMPH_OK) rc = do_verify(ctx, nullptr, nullptr);
         if (rc == AMPH_OK) rc = do_accept(ctx, nullptr, nullptr, nullptr, nullptr);
         const cudaError_t e = cudaStreamEndCapture(ctx->stream, &graph);
-        if (rc == AMPH_OK && e == cudaSuccess && graph &&
-            cudaGraphInstantiate(&ctx->graph_exec, graph, 0) == cudaSuccess) {
-          ctx->graph_key = key;
+        if (rc == AMPH_OK && e == cudaSuccess && graph && cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess) {
+          if (ctx->graphs.size() == kMaxGraphs) {          // the least recently used one makes room (its replays may still run:
+            size_t old = 0;                                // CUDA keeps a launched executable until it has finished)
+            for (size_t i = 1; i < ctx->graphs.size(); ++i)
+              if (ctx->graphs[i].used < ctx->graphs[old].used) old = i;
+            cudaGraphExecDestroy(ctx->graphs[old].exec);
+            ctx->graphs.erase(ctx->graphs.begin() + old);
+          }
+          ctx->graphs.push_back({key, exec, ++ctx->graph_tick});
         } else {
-          ctx->graph_exec = nullptr;
+          exec = nullptr;
           ctx->graph_off = true;
         }
         if (graph) cudaGraphDestroy(graph);
@@ -1117,8 +1135,8 @@ amph_status amph_step(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n) {
       cudaGetLastError();
     }
   }
-  if (use_graph && ctx->graph_exec) {
-    rc = cuda_check(ctx, cudaGraphLaunch(ctx->graph_exec, ctx->stream), "graph launch");
+  if (exec) {
+    rc = cuda_check(ctx, cudaGraphLaunch(exec, ctx->stream), "graph launch");
   } else {
     rc = do_draft(ctx, nullptr, nullptr);
     if (rc == AMPH_OK) rc = do_verify(ctx, nullptr, nullptr);
@@ -1396,7 +1414,7 @@ void amph_destroy(amph_ctx* ctx) {
   if (!ctx) return;
   if (ctx->tc) tc_gemm_destroy(ctx->tc);
   if (ctx->attn_tc) attn_tc_destroy(ctx->attn_tc);
-  if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
+  ctx->drop_graphs();
   for (auto& e : ctx->fork_ev) cudaEventDestroy(e);
   if (ctx->join_ev) cudaEventDestroy(ctx->join_ev);
   if (ctx->side) cudaStreamDestroy(ctx->side);

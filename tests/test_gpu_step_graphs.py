@@ -1,0 +1,39 @@
+"""amph_step keeps a bounded set of captured schedules, one per combination of attention grids.  Lengths that come back must
+find the right one, more combinations than are kept must still be right, and so must every sequence length a kept schedule is
+replayed at: the emitted tokens equal those of a context that launches its kernels one by one (bit for bit the same kernels)."""
+import pytest
+import torch
+
+import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _decode(model, prompts, steps):
+    tok = torch.zeros(model.B, model.shape.K + 1, dtype=torch.int32, device="cuda:0")
+    n = torch.zeros(model.B, dtype=torch.int32, device="cuda:0")
+    out = [model.prefill(p, seq=b) for b, p in enumerate(prompts)]
+    for _ in range(steps):
+        model.step(tok, n)
+        torch.cuda.synchronize()
+        out += tok.flatten().tolist() + n.tolist()
+    return out
+
+
+# fp32 caches: every sequence's own split count is part of the combination, 25 of them for two sequences (more than are kept);
+# bf16 caches: one launch sized for the longest sequence
+@pytest.mark.parametrize("name,lengths", [("tiny", (20, 150, 280, 410, 540)), ("small_bf16", (60, 300, 700))])
+def test_lengths_that_come_back(name, lengths):
+    from paper_2406_13170_b200 import Amphista
+    shape = inputs.get_shape(name)
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    texts = {n: inputs.make_prompt(shape.with_(prompt_len=n), seed=n).tolist() for n in lengths}
+    graphs = Amphista(shape, topo, w, max_batch=2, max_ctx=1024)
+    plain = Amphista(shape, topo, w, max_batch=2, max_ctx=1024, flags=2)
+    pairs = [(a, b) for a in lengths for b in lengths]
+    for a, b in pairs + pairs[:3] + pairs[-2:]:
+        prompts = [texts[a], texts[b]]
+        assert _decode(graphs, prompts, 2) == _decode(plain, prompts, 2), (a, b)
+    graphs.close()
+    plain.close()
