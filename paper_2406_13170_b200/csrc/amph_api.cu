@@ -638,6 +638,14 @@ amph_status copy_out(amph_ctx* ctx, void* dst, const void* src, size_t bytes) {
   return cuda_check(ctx, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, ctx->stream), "copy of a result");
 }
 
+// `n` ints of every sequence's state (src: the field in sequence 0's) to dst [B][n]: one strided copy for the whole batch.
+amph_status copy_out_seq(amph_ctx* ctx, int32_t* dst, const int* src, int n) {
+  if (!dst) return AMPH_OK;
+  if (ctx->B == 1) return copy_out(ctx, dst, src, sizeof(int) * n);
+  return cuda_check(ctx, cudaMemcpy2DAsync(dst, sizeof(int) * n, src, ctx->lay.state_s, sizeof(int) * n, ctx->B, cudaMemcpyDefault,
+                                           ctx->stream), "copy of a result");
+}
+
 amph_status finish(amph_ctx* ctx, const char* what) { return cuda_check(ctx, cudaGetLastError(), what); }
 
 amph_status refresh_ctx_hi(amph_ctx* ctx) {
@@ -790,22 +798,26 @@ amph_status do_accept(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n, int32_
   const Layout& l = ctx->lay;
   cudaStream_t st = ctx->stream;
   join_side(ctx);
-  amph_status rc = AMPH_OK;
-  for (int b = 0; b < ctx->B && rc == AMPH_OK; ++b) {
-    DevState* ds = ctx->state(b);
-    { ProfScope p(ctx, AMPH_PROF_ACCEPT);
-    launch_accept(ctx->at<TreeDev>(l.tree), ds, ctx->at<int>(l.tok) + b * ctx->Mver, ctx->at<int>(l.amax) + b * ctx->Mver, st);
-    }
-    { ProfScope p(ctx, AMPH_PROF_ACCEPT);
-    launch_compact(ds, ctx->grp<KvView>(l.kv_tab, l.kv_tab_s, b), c.n_layers, ctx->dtype, c.n_heads, c.head_dim, c.max_ctx,
-                   ctx->at<float>(l.hidden) + (size_t)b * ctx->Mver * c.d_model,
-                   ctx->at<float>(l.pend_h) + (size_t)b * kSmallRows * c.d_model, c.d_model, st);
-    }
-    if (out_tokens) rc = copy_out(ctx, out_tokens + b * (c.K + 1), ds->out_tok, sizeof(int) * (c.K + 1));
-    if (rc == AMPH_OK && out_n) rc = copy_out(ctx, out_n + b, &ds->L, sizeof(int));
-    if (rc == AMPH_OK && out_path) rc = copy_out(ctx, out_path + b * (c.K + 1), ds->path, sizeof(int) * (c.K + 1));
-    if (rc == AMPH_OK && out_next_root) rc = copy_out(ctx, out_next_root + b, &ds->next_root, sizeof(int));
+  { ProfScope p(ctx, AMPH_PROF_ACCEPT);
+  AcceptArgs a;
+  a.tree = ctx->at<TreeDev>(l.tree);
+  a.state = ctx->ws + l.state;    a.state_stride = l.state_s;
+  a.meta = ctx->ws + l.meta_v;    a.meta_stride = l.meta_s_;
+  a.kv_tab = ctx->ws + l.kv_tab;  a.kv_tab_stride = l.kv_tab_s;
+  a.tok = ctx->at<int>(l.tok);
+  a.amax = ctx->at<int>(l.amax);
+  a.rows = ctx->Mver;
+  a.n_layers = c.n_layers; a.n_heads = c.n_heads; a.dh = c.head_dim; a.max_ctx = c.max_ctx; a.d = c.d_model;
+  a.hidden = ctx->at<float>(l.hidden);
+  a.pend_h = ctx->at<float>(l.pend_h);
+  a.pend_rows = kSmallRows;
+  launch_accept_compact(a, ctx->B, ctx->dtype, st);
   }
+  const DevState* ds = ctx->state(0);
+  amph_status rc = copy_out_seq(ctx, out_tokens, ds->out_tok, c.K + 1);
+  if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_n, &ds->L, 1);
+  if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_path, ds->path, c.K + 1);
+  if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_next_root, &ds->next_root, 1);
   return rc;
 }
 
@@ -1142,11 +1154,9 @@ amph_status amph_step(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n) {
     if (rc == AMPH_OK) rc = do_verify(ctx, nullptr, nullptr);
     if (rc == AMPH_OK) rc = do_accept(ctx, nullptr, nullptr, nullptr, nullptr);
   }
-  for (int b = 0; b < ctx->B && rc == AMPH_OK; ++b) {
-    DevState* ds = ctx->state(b);
-    if (out_tokens) rc = copy_out(ctx, out_tokens + b * (c.K + 1), ds->out_tok, sizeof(int) * (c.K + 1));
-    if (rc == AMPH_OK && out_n) rc = copy_out(ctx, out_n + b, &ds->L, sizeof(int));
-  }
+  const DevState* ds = ctx->state(0);
+  if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_tokens, ds->out_tok, c.K + 1);
+  if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_n, &ds->L, 1);
   if (rc == AMPH_OK) rc = finish(ctx, "step");
   if (rc == AMPH_OK)
     for (int b = 0; b < ctx->B; ++b) ctx->ctx_hi[b] += c.K + 1;

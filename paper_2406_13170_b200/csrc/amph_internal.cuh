@@ -225,7 +225,21 @@ void launch_meta_chain(RowMeta* meta, int base, int n_rows, cudaStream_t st);   
 void launch_meta_pending(RowMeta* meta, const DevState* s, cudaStream_t st);              // adaptation rows
 void launch_tree_build(const TreeDev* tree, DevState* s, const int* topk_ids, const int* override_tok,
                        int* tok, RowMeta* meta, cudaStream_t st);
-void launch_accept(const TreeDev* tree, DevState* s, const int* tok, const int* amax, cudaStream_t st);
+// Acceptance and KV compaction of every sequence of a batch.
+struct AcceptArgs {
+  const TreeDev* tree;
+  char* state; size_t state_stride;            // DevState of sequence b at state + b * state_stride
+  const char* meta; size_t meta_stride;        // RowMeta of the verification pass
+  const char* kv_tab; size_t kv_tab_stride;    // KvView[n_layers]
+  const int* tok;                              // [B][rows]: tree tokens
+  const int* amax;                             // [B][rows]: choices
+  int rows;
+  int n_layers, n_heads, dh, max_ctx, d;
+  const float* hidden;                         // [B][rows][d]
+  float* pend_h;                               // [B][pend_rows][d]
+  int pend_rows;
+};
+void launch_accept_compact(const AcceptArgs& a, int batch, int dtype, cudaStream_t st);
 // Sampling at temperature T > 0 (Table 2): choice[r] for rows row0 .. row0 + n_rows - 1 = the token the target draws after
 // that row from softmax(logits / T) with the row's own uniform (Philox4x32-10 keyed by seed; counter = row - row0, the
 // sequence's step count, seq, stream).  With a tree (tok != NULL) the vocabulary is walked in the order (tokens of the
@@ -234,8 +248,6 @@ void launch_accept(const TreeDev* tree, DevState* s, const int* tok, const int* 
 void launch_sample_rows(const float* logits, int vocab, int row0, int n_rows, const TreeDev* tree, const int* tok,
                         const DevState* s, int seq, int stream_id, float temperature, unsigned long long seed, int* choice,
                         float* uniforms_out, cudaStream_t st);
-void launch_compact(const DevState* s, const KvView* kv_layers, int n_layers, int dtype, int n_heads,
-                    int head_dim, int max_ctx, const float* hidden, float* pend_h, int d, cudaStream_t st);
 void launch_reduce_partials(PartialView P, float* y, int rows, int cols, cudaStream_t st);
 void launch_kv_export(KvView kv, int which, int dtype, int row0, int rows, int n_heads, int head_dim, int max_ctx,
                       float* dst, cudaStream_t st);

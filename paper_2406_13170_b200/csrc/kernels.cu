@@ -1039,41 +1039,85 @@ void launch_tree_build(const TreeDev* tree, DevState* s, const int* topk_ids, co
 
 // Greedy acceptance: node n matches if its token equals the target's choice at its parent; it is
 // accepted if every node on its root path matches; the deepest accepted node wins (lowest index
-// among equals).  One block; the match set is a 128-bit mask tested against the ancestor masks.
-__global__ void accept_kernel(const TreeDev* __restrict__ tree, DevState* s, const int* __restrict__ tok,
-                              const int* __restrict__ amax) {
+// among equals).  The match set is a 128-bit mask tested against the ancestor masks.
+// Compaction: slot C + j <- slot C + path[j] in every layer's cache, accepted hidden rows to the next draft's queue.
+//
+// One launch for all sequences (blockIdx.y).  Every block finds the accepted path for itself (tokens, choices and tree are a
+// few KB of L2; C is the row table's base, since one block moves the state on), then moves its own piece: one block per layer
+// and K / V half, one per queued hidden row.  Bound: latency (two dependent L2 round trips and the copy's own).
+// 16-byte copies with all of a thread's loads issued before its first store.  A launch for the acceptance and, per sequence,
+// one of a block per layer that copied 2-byte elements in path order cost a step 12 us more at 7B (31 us of them on the
+// chain, part of them hidden behind the next graph launch) and 345 us more with eight sequences.
+template <typename T>
+__global__ void __launch_bounds__(256)
+accept_compact_kernel(const AcceptArgs a) {
   pdl_wait();
   pdl_launch_dependents();
   __shared__ u64 match[2];
-  __shared__ int best_key;
-  const int n = threadIdx.x;
-  const int N = tree->n_nodes;
+  __shared__ int best_key, L_s;
+  __shared__ int path_s[kPendMax];
+  const TreeDev* tree = a.tree;
+  const int b = blockIdx.y, n = threadIdx.x, N = tree->n_nodes;
+  const int* tok = a.tok + (size_t)b * a.rows;
+  const int* amax = a.amax + (size_t)b * a.rows;
+  const int C = reinterpret_cast<const RowMeta*>(a.meta + a.meta_stride * b)->base;
   if (n < 2) match[n] = 0ull;
   if (n == 0) best_key = 0;
-  __syncthreads();
+  u64 anc0 = 0, anc1 = 0;
+  bool m = false;
   if (n < N) {
-    const bool m = n == 0 || tok[n] == amax[tree->parent[n]];
-    if (m) atomicOr(&match[n >> 6], 1ull << (n & 63));
+    anc0 = tree->anc[n][0];
+    anc1 = tree->anc[n][1];
+    m = n == 0 || tok[n] == amax[tree->parent[n]];
   }
   __syncthreads();
-  if (n < N) {
-    const bool ok = ((tree->anc[n][0] & ~match[0]) | (tree->anc[n][1] & ~match[1])) == 0ull;
-    if (ok) atomicMax(&best_key, tree->depth[n] * 256 + (255 - n));
-  }
+  const unsigned votes = __ballot_sync(0xffffffffu, m);
+  if ((n & 31) == 0 && n < kMaxRows) atomicOr(&match[n >> 6], (u64)votes << (n & 32));
   __syncthreads();
-  if (n == 0) {
-    const int best = 255 - (best_key & 255);
-    const int C = s->C;
-    u64 a0 = tree->anc[best][0], a1 = tree->anc[best][1];
+  if (n < N && ((anc0 & ~match[0]) | (anc1 & ~match[1])) == 0ull) atomicMax(&best_key, tree->depth[n] * 256 + (255 - n));
+  __syncthreads();
+  const int best = 255 - (best_key & 255);
+  if (n == best) {                                     // the ancestors of the deepest accepted node, in node order
     int L = 0;
-    while (a0 && L < kPendMax) { s->path[L++] = __ffsll((long long)a0) - 1; a0 &= a0 - 1; }
-    while (a1 && L < kPendMax) { s->path[L++] = 64 + __ffsll((long long)a1) - 1; a1 &= a1 - 1; }
-    const int nr = amax[best];
-    for (int j = 0; j < L; ++j) {
-      s->out_tok[j] = tok[s->path[j]];
-      s->pend_tok[j] = j + 1 < L ? tok[s->path[j + 1]] : nr;
+    while (anc0 && L < kPendMax) { path_s[L++] = __ffsll((long long)anc0) - 1; anc0 &= anc0 - 1; }
+    while (anc1 && L < kPendMax) { path_s[L++] = 64 + __ffsll((long long)anc1) - 1; anc1 &= anc1 - 1; }
+    L_s = L;
+  }
+  __syncthreads();
+  const int L = L_s;
+  if ((int)blockIdx.x < 2 * a.n_layers) {
+    // path is strictly increasing with path[j] >= j, so no source slot is the destination of an earlier move
+    const KvView kv = reinterpret_cast<const KvView*>(a.kv_tab + a.kv_tab_stride * b)[blockIdx.x >> 1];
+    T* cache = (T*)((blockIdx.x & 1) ? kv.v : kv.k);
+    constexpr int E = 16 / sizeof(T);
+    const int per_head = a.dh / E, items = a.n_heads * per_head;
+    for (int i = n; i < items; i += blockDim.x) {
+      const int h = i / per_head;
+      uint4* base = reinterpret_cast<uint4*>(cache + ((size_t)h * a.max_ctx + C) * a.dh + (i - h * per_head) * E);
+      uint4 v[kPendMax];
+#pragma unroll
+      for (int j = 1; j < kPendMax; ++j)
+        if (j < L && path_s[j] != j && C + path_s[j] < a.max_ctx) v[j] = base[(size_t)path_s[j] * per_head];
+#pragma unroll
+      for (int j = 1; j < kPendMax; ++j)
+        if (j < L && path_s[j] != j && C + path_s[j] < a.max_ctx) base[(size_t)j * per_head] = v[j];
     }
-    for (int j = L; j < kPendMax; ++j) { s->path[j] = -1; s->out_tok[j] = -1; }
+    return;
+  }
+  const int j = blockIdx.x - 2 * a.n_layers;           // queued hidden row
+  if (j < L) {
+    const float* src = a.hidden + ((size_t)b * a.rows + path_s[j]) * a.d;
+    float* dst = a.pend_h + ((size_t)b * a.pend_rows + j) * a.d;
+    for (int c = n * 4; c < a.d; c += blockDim.x * 4) store4(dst + c, load4(src + c));
+  }
+  if (j == 0 && n == 0) {
+    DevState* s = reinterpret_cast<DevState*>(a.state + a.state_stride * b);
+    const int nr = amax[best];
+    for (int i = 0; i < kPendMax; ++i) {
+      s->path[i] = i < L ? path_s[i] : -1;
+      s->out_tok[i] = i < L ? tok[path_s[i]] : -1;
+      if (i < L) s->pend_tok[i] = i + 1 < L ? tok[path_s[i + 1]] : nr;
+    }
     s->L = L;
     s->C_old = C;
     s->best = best;
@@ -1085,8 +1129,8 @@ __global__ void accept_kernel(const TreeDev* __restrict__ tree, DevState* s, con
   }
 }
 
-void launch_accept(const TreeDev* tree, DevState* s, const int* tok, const int* amax, cudaStream_t st) {
-  launch_pdl(accept_kernel, dim3(1), dim3(kMaxRows), 0, st, tree, s, tok, amax);
+void launch_accept_compact(const AcceptArgs& a, int batch, int dtype, cudaStream_t st) {
+  AMPH_DISPATCH(dtype, launch_pdl(accept_compact_kernel<T>, dim3(2 * a.n_layers + kPendMax, batch), dim3(256), 0, st, a));
 }
 
 // --------------------------------------------------------------------------------------------
@@ -1224,41 +1268,6 @@ void launch_sample_rows(const float* logits, int vocab, int row0, int n_rows, co
                         float* uniforms_out, cudaStream_t st) {
   launch_pdl(sample_rows_kernel, dim3(n_rows), dim3(kSampleThreads), 0, st, logits, vocab, row0, tree, tok, s, seq, stream_id,
              1.0f / temperature, (uint32_t)(seed & 0xffffffffull), (uint32_t)(seed >> 32), choice, uniforms_out);
-}
-
-// Block l < n_layers moves layer l's accepted key / value rows: slot C_old + j <- C_old + path[j].
-// path is strictly increasing with path[j] >= j, so no source is overwritten before it is read and
-// the moves are independent.  The extra last block queues the accepted hidden rows for the next draft.
-template <typename T>
-__global__ void compact_kernel(const DevState* __restrict__ s, const KvView* __restrict__ kv, int n_layers,
-                               int n_heads, int dh, int max_ctx, const float* __restrict__ hidden,
-                               float* __restrict__ pend_h, int d) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int L = s->L, C0 = s->C_old;
-  if ((int)blockIdx.x == n_layers) {
-    for (int j = 0; j < L; ++j)
-      for (int c = threadIdx.x; c < d; c += blockDim.x) pend_h[(size_t)j * d + c] = hidden[(size_t)s->path[j] * d + c];
-    return;
-  }
-  T* kc = (T*)kv[blockIdx.x].k;
-  T* vc = (T*)kv[blockIdx.x].v;
-  for (int j = 1; j < L; ++j) {
-    const int src = C0 + s->path[j], dst = C0 + j;
-    if (src == dst || src >= max_ctx) continue;
-    for (int i = threadIdx.x; i < n_heads * dh; i += blockDim.x) {
-      const int h = i / dh, c = i - h * dh;
-      const size_t so = ((size_t)h * max_ctx + src) * dh + c, dd = ((size_t)h * max_ctx + dst) * dh + c;
-      kc[dd] = kc[so];
-      vc[dd] = vc[so];
-    }
-  }
-}
-
-void launch_compact(const DevState* s, const KvView* kv_layers, int n_layers, int dtype, int n_heads,
-                    int head_dim, int max_ctx, const float* hidden, float* pend_h, int d, cudaStream_t st) {
-  AMPH_DISPATCH(dtype, launch_pdl(compact_kernel<T>, dim3(n_layers + 1), dim3(256), 0, st, s, kv_layers, n_layers, n_heads, head_dim,
-                                                                       max_ctx, hidden, pend_h, d));
 }
 
 __global__ void reduce_partials_kernel(PartialView P, float* __restrict__ y, int rows, int cols) {
