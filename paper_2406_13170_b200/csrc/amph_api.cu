@@ -661,6 +661,21 @@ amph_status refresh_ctx_hi(amph_ctx* ctx) {
   return AMPH_OK;
 }
 
+TopkTreeArgs topk_tree_args(const amph_ctx* ctx) {
+  const Layout& l = ctx->lay;
+  TopkTreeArgs a;
+  a.ids = ctx->ws + l.topk_ids;       a.ids_stride = l.topk_ids_s;
+  a.vals = ctx->ws + l.topk_vals;     a.vals_stride = l.topk_vals_s;
+  a.d_logits = ctx->ws + l.d_logits;  a.d_logits_stride = l.d_logits_s;
+  a.cand = ctx->ws + l.topk_cand;     a.cand_stride = l.topk_cand_s;
+  a.state = ctx->ws + l.state;        a.state_stride = l.state_s;
+  a.meta = ctx->ws + l.meta_v;        a.meta_stride = l.meta_s_;
+  a.tree = ctx->at<TreeDev>(l.tree);
+  a.tok = ctx->at<int>(l.tok);
+  a.rows = ctx->Mver;
+  return a;
+}
+
 // out_ids / out_vals: [B][K][AMPH_TOPK_STRIDE]
 amph_status do_draft(amph_ctx* ctx, int32_t* out_ids, float* out_vals) {
   const amph_config& c = ctx->cfg;
@@ -721,16 +736,8 @@ amph_status do_draft(amph_ctx* ctx, int32_t* out_ids, float* out_vals) {
   } else {
     P = project(ctx, XB_AO, ctx->draft_lm, K, c.vocab, c.d_model, B * K);                             // Eq. 6
   }
-  for (int b = 0; b < B; ++b) {
-    { ProfScope p(ctx, AMPH_PROF_SELECT);
-    launch_topk_heads(rows_from(P, b * K), c.vocab, K, c.topk, ctx->grp<int>(l.topk_ids, l.topk_ids_s, b),
-                      ctx->grp<float>(l.topk_vals, l.topk_vals_s, b), ctx->grp<float>(l.d_logits, l.d_logits_s, b),
-                      ctx->grp<float>(l.topk_cand, l.topk_cand_s, b), st);
-    }
-    { ProfScope p(ctx, AMPH_PROF_OTHER);
-    launch_tree_build(ctx->at<TreeDev>(l.tree), ctx->state(b), ctx->grp<int>(l.topk_ids, l.topk_ids_s, b), nullptr,
-                      ctx->at<int>(l.tok) + b * ctx->Mver, ctx->meta_v(b), st);
-    }
+  { ProfScope p(ctx, AMPH_PROF_SELECT);
+  launch_topk_tree(P, c.vocab, K, c.topk, topk_tree_args(ctx), B, st);
   }
   amph_status rc = AMPH_OK;
   for (int b = 0; b < B && rc == AMPH_OK; ++b) {
@@ -767,13 +774,14 @@ amph_status do_verify(amph_ctx* ctx, const int32_t* tree_tokens, int32_t* out_ar
     ps.rope[b] = ctx->grp<float2>(l.rope_v, l.rope_s_, b);
     ps.seq[b] = b;
     ps.keys[b] = ctx->ctx_hi[b] + N;
-    if (tree_tokens) {
-      int* ov = ctx->at<int>(l.override_tok) + b * ctx->Mver;
-      amph_status rc = cuda_check(ctx, cudaMemcpyAsync(ov, tree_tokens + (size_t)b * N, sizeof(int) * N, cudaMemcpyDefault, st), "copy of tree tokens");
-      if (rc != AMPH_OK) return rc;
-      ProfScope p(ctx, AMPH_PROF_OTHER);
-      launch_tree_build(ctx->at<TreeDev>(l.tree), ctx->state(b), nullptr, ov, ctx->at<int>(l.tok) + b * ctx->Mver, ctx->meta_v(b), st);
-    }
+  }
+  if (tree_tokens) {
+    int* ov = ctx->at<int>(l.override_tok);
+    amph_status rc = cuda_check(ctx, cudaMemcpy2DAsync(ov, sizeof(int) * ctx->Mver, tree_tokens, sizeof(int) * N, sizeof(int) * N, B,
+                                                       cudaMemcpyDefault, st), "copy of tree tokens");
+    if (rc != AMPH_OK) return rc;
+    ProfScope p(ctx, AMPH_PROF_OTHER);
+    launch_tree_override(topk_tree_args(ctx), ov, B, st);
   }
   target_forward(ctx, ps);
   target_head(ctx, ps.rows());

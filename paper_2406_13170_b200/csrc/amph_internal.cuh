@@ -212,19 +212,29 @@ void launch_aeb_attention(PartialView P, void* out_act, int dtype, int K, int n_
                           cudaStream_t st);
 // out_act[k][j] = P(row k, column k * r + j): row k of the k-th low-rank projection, as the next projection's input
 void launch_gather_diag(PartialView P, void* out_act, int dtype, int K, int r, cudaStream_t st);
-// per head k: top-c_k of row k of segment k; also stores the row into d_logits[k]
-// cand: scratch for the slices' candidates, kMaxK * kTopkCandChunks * kTopkStride (value, id) pairs
+// Per sequence b and head k: top-c_k of row b * K + k of segment k (also stored into d_logits), then the candidate tree built
+// from them (Appendix A.1).  cand: scratch for the slices' candidates, kMaxK * kTopkCandChunks * kTopkStride (value, id) pairs.
+// Pointers with a stride are sequence 0's copy of a per-sequence buffer, the next sequence's `stride` bytes further on.
 constexpr int kTopkCandChunks = 32;
-void launch_topk_heads(PartialView P, int vocab, int K, const int* ck, int* ids, float* vals,
-                       float* d_logits, float* cand, cudaStream_t st);
+struct TopkTreeArgs {
+  char* ids;       size_t ids_stride;        // int   [K][kTopkStride]
+  char* vals;      size_t vals_stride;       // float [K][kTopkStride]
+  char* d_logits;  size_t d_logits_stride;   // float [K][vocab]
+  char* cand;      size_t cand_stride;
+  const char* state; size_t state_stride;    // DevState
+  char* meta;      size_t meta_stride;       // RowMeta of the verification pass
+  const TreeDev* tree;
+  int* tok;                                  // [B][rows]
+  int rows;
+};
+void launch_topk_tree(PartialView P, int vocab, int K, const int* ck, const TopkTreeArgs& a, int batch, cudaStream_t st);
+void launch_tree_override(const TopkTreeArgs& a, const int* override_tok, int batch, cudaStream_t st);   // override_tok [B][rows]
 // cand: scratch for the slices' candidates, kMaxRows * 8 (value, id) pairs
 void launch_argmax_rows(PartialView P, int vocab, int rows, int* amax, float* logits_out, float* cand, cudaStream_t st);
 
 // ---- control kernels
 void launch_meta_chain(RowMeta* meta, int base, int n_rows, cudaStream_t st);             // prefill chunk
 void launch_meta_pending(RowMeta* meta, const DevState* s, cudaStream_t st);              // adaptation rows
-void launch_tree_build(const TreeDev* tree, DevState* s, const int* topk_ids, const int* override_tok,
-                       int* tok, RowMeta* meta, cudaStream_t st);
 // Acceptance and KV compaction of every sequence of a batch.
 struct AcceptArgs {
   const TreeDev* tree;

@@ -815,84 +815,154 @@ __device__ void block_best(float& v, int& i, float* sv, int* si) {
 
 struct TopkCounts { int c[kMaxK]; };
 
-// Stage 1: block (head k, chunk j) reduces the split-K partials of its slice of the head's logits, stores
-// them (debug tap) and selects the slice's own top-c_k in the order above.  Stage 2: one block per head
-// merges the slices' candidates.  The global top-c_k are each among their slice's top-c_k, so the result is
-// the exact top-c_k of the row, in order.
+// Selection keys: a larger key is a better candidate in the order above.  The high word orders the values (-0 counts as +0),
+// 0 is below every value and marks "nothing left".
+__device__ __forceinline__ uint32_t order_key(float v) {
+  const uint32_t u = __float_as_uint(v == 0.f ? 0.f : v);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+// Stage 1: block (head k, chunk j, sequence b) reduces the split-K partials of its slice of the head's logits, stores them
+// (debug tap) and selects the slice's own top-c_k; stage 2 (topk_tree_kernel) merges the slices' candidates.  The global
+// top-c_k are each among their slice's top-c_k, so the result is the exact top-c_k of the row, in order.
+// Every warp selects from an eighth of the slice (one warp-wide maximum and one minimum of ids per pick, no block barrier),
+// then the first warp merges the eight sorted lists.  Bound: latency: picks made by the whole block, with two barriers each,
+// and three launches per sequence cost a step 18 us more at 7B (32000 ids, 10 candidates) and 100 us more with eight sequences.
 constexpr int kTopkChunks = kTopkCandChunks;
 constexpr int kTopkThreads = 256;
+constexpr int kTopkWarps = kTopkThreads / 32;
+
+// One pick over the lanes of a warp: the best (key, lowest id) and the lane that holds it (-1: nothing left).
+__device__ __forceinline__ int warp_pick(uint32_t key, int id, uint32_t& best_key, int& best_id) {
+  best_key = __reduce_max_sync(0xffffffffu, key);
+  best_id = (int)__reduce_min_sync(0xffffffffu, key == best_key ? (uint32_t)id : 0xffffffffu);
+  const unsigned own = __ballot_sync(0xffffffffu, key == best_key && id == best_id);
+  return best_key == 0u ? -1 : __ffs(own) - 1;
+}
 
 __global__ void __launch_bounds__(kTopkThreads)
-topk_slice_kernel(PartialView P, int vocab, int chunk, TopkCounts ck, float2* __restrict__ cand,
-                  float* __restrict__ d_logits, int vec) {
+topk_slice_kernel(PartialView P, int vocab, int chunk, int K, TopkCounts ck, char* __restrict__ cand, size_t cand_stride,
+                  char* __restrict__ d_logits, size_t d_logits_stride, int vec) {
   pdl_wait();
   pdl_launch_dependents();
   extern __shared__ __align__(16) float slice[];
-  __shared__ float sv[32];
-  __shared__ int si[32];
-  const int k = blockIdx.x, j = blockIdx.y;
+  __shared__ float2 lists[kTopkWarps][kTopkStride];
+  const int k = blockIdx.x, j = blockIdx.y, b = blockIdx.z, row = b * K + k;
   const int lo = j * chunk, hi = lo + chunk < vocab ? lo + chunk : vocab;
-  float* grow = d_logits + (size_t)k * vocab;
+  float* grow = reinterpret_cast<float*>(d_logits + d_logits_stride * b) + (size_t)k * vocab;
   for (int c = lo + threadIdx.x * 4; c < hi; c += blockDim.x * 4) {
     if (vec && c + 3 < hi) {
-      const float4 v = sum_partials4(P, k, k * vocab + c);
+      const float4 v = sum_partials4(P, row, k * vocab + c);
       store4(grow + c, v);
       store4(slice + (c - lo), v);
     } else {
       for (int e = c; e < hi && e < c + 4; ++e) {
-        const float v = sum_partials(P, k, k * vocab + e);
+        const float v = sum_partials(P, row, k * vocab + e);
         grow[e] = v;
         slice[e - lo] = v;
       }
     }
   }
   __syncthreads();
-  float pv = INFINITY;
-  int pi = -1;
-  for (int t = 0; t < ck.c[k]; ++t) {
-    float bv = -INFINITY;
-    int bi = 0x7fffffff;
-    for (int c = lo + threadIdx.x; c < hi; c += blockDim.x) {
-      const float v = slice[c - lo];
-      const bool after_prev = v < pv || (v == pv && c > pi);       // strictly after the previous pick
-      if (after_prev && better(v, c, bv, bi)) { bv = v; bi = c; }
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, want = ck.c[k], n = hi - lo;
+  const int part = (n + kTopkWarps - 1) / kTopkWarps, p0 = w * part, p1 = p0 + part < n ? p0 + part : n;
+  // this lane's best entry strictly after the last pick it lost (its entries are p0 + lane, p0 + lane + 32, ...: ascending ids)
+  uint32_t key = 0u, prev = 0xffffffffu;
+  int id = 0x7fffffff, prev_id = -1;
+  bool rescan = true;
+  for (int t = 0; t < want; ++t) {
+    if (rescan) {
+      key = 0u;
+      id = 0x7fffffff;
+      for (int i = p0 + lane; i < p1; i += 32) {
+        const uint32_t o = order_key(slice[i]);
+        if (o > key && (o < prev || (o == prev && i > prev_id))) { key = o; id = i; }
+      }
     }
-    block_best(bv, bi, sv, si);
-    if (threadIdx.x == 0) cand[((size_t)k * gridDim.y + j) * kTopkStride + t] = make_float2(bv, __int_as_float(bi));
-    pv = bv; pi = bi;
-    __syncthreads();
+    uint32_t bk;
+    int bi;
+    const int owner = warp_pick(key, id, bk, bi);
+    if (lane == 0) lists[w][t] = owner < 0 ? make_float2(-INFINITY, __int_as_float(0x7fffffff)) : make_float2(slice[bi], __int_as_float(bi));
+    rescan = lane == owner;
+    if (rescan) { prev = bk; prev_id = bi; }
+  }
+  __syncthreads();
+  if (w != 0) return;
+  float2* out = reinterpret_cast<float2*>(cand + cand_stride * b) + ((size_t)k * gridDim.y + j) * kTopkStride;
+  int at = 0;                                            // lane l < 8: next entry of warp l's sorted list
+  for (int t = 0; t < want; ++t) {
+    float2 e = make_float2(0.f, __int_as_float(0x7fffffff));
+    if (lane < kTopkWarps && at < want) e = lists[lane][at];
+    const int eid = __float_as_int(e.y);
+    uint32_t bk;
+    int bi;
+    const int owner = warp_pick(eid == 0x7fffffff ? 0u : order_key(e.x), eid, bk, bi);
+    if (owner < 0) { if (lane == 0) out[t] = make_float2(-INFINITY, __int_as_float(0x7fffffff)); continue; }
+    if (lane == owner) { out[t] = make_float2(e.x, __int_as_float(lo + eid)); ++at; }
   }
 }
 
+// Node n of the verification pass of one sequence (Appendix A.1): tok[0] = root; tok[n] = head depth[n]'s candidate of
+// rank rank[n]; optional overrides; row table: position C + depth, slot C + n, mask = ancestors (Fig. 5).
+__device__ __forceinline__ void tree_row(const TreeDev* __restrict__ tree, const DevState* s, const int* topk_ids,
+                                         const int* __restrict__ override_tok, int* __restrict__ tok, RowMeta* meta, int n) {
+  const int N = tree->n_nodes, C = s->C;
+  if (n == 0) { meta->base = C; meta->n_rows = N; }
+  if (n < N) {
+    if (n == 0) {
+      tok[0] = s->root;
+    } else {
+      if (topk_ids) tok[n] = topk_ids[(tree->depth[n] - 1) * kTopkStride + tree->rank[n]];
+      if (override_tok && override_tok[n] >= 0) tok[n] = override_tok[n];
+    }
+    meta->pos[n] = C + tree->depth[n];
+    meta->slot[n] = C + n;
+    meta->mask[n][0] = tree->anc[n][0];
+    meta->mask[n][1] = tree->anc[n][1];
+  } else {
+    meta->pos[n] = C;
+    meta->slot[n] = -1;
+    meta->mask[n][0] = meta->mask[n][1] = 0ull;
+  }
+}
+
+// Stage 2 and the candidate tree, one block per sequence: warp k merges head k's slice lists (lane j walks the sorted list of
+// slice j), then the block lays the tree out from the merged candidates.
 __global__ void __launch_bounds__(kTopkThreads)
-topk_merge_kernel(const float2* __restrict__ cand, int n_chunks, TopkCounts ck, int* __restrict__ ids,
-                  float* __restrict__ vals) {
+topk_tree_kernel(const TopkTreeArgs a, int n_chunks, int K, TopkCounts ck) {
   pdl_wait();
   pdl_launch_dependents();
-  __shared__ float sv[32];
-  __shared__ int si[32];
-  const int k = blockIdx.x, ckk = ck.c[k];
-  const int n = n_chunks * ckk;                                    // candidates of this head
-  float pv = INFINITY;
-  int pi = -1;
-  for (int t = 0; t < ckk; ++t) {
-    float bv = -INFINITY;
-    int bi = 0x7fffffff;
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-      const float2 e = cand[((size_t)k * n_chunks + c / ckk) * kTopkStride + c % ckk];
-      const int id = __float_as_int(e.y);
-      const bool after_prev = e.x < pv || (e.x == pv && id > pi);
-      if (id != 0x7fffffff && after_prev && better(e.x, id, bv, bi)) { bv = e.x; bi = id; }
+  __shared__ int ids_s[kMaxK * kTopkStride];
+  const int b = blockIdx.x, k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (k < K) {
+    const int want = ck.c[k];
+    const float2* list = reinterpret_cast<const float2*>(a.cand + a.cand_stride * b) + ((size_t)k * n_chunks + lane) * kTopkStride;
+    int* oid = reinterpret_cast<int*>(a.ids + a.ids_stride * b) + k * kTopkStride;
+    float* oval = reinterpret_cast<float*>(a.vals + a.vals_stride * b) + k * kTopkStride;
+    const float2 none = make_float2(0.f, __int_as_float(0x7fffffff));
+    int at = 0;
+    float2 e = lane < n_chunks ? list[0] : none, nx = lane < n_chunks && want > 1 ? list[1] : none;
+    for (int t = 0; t < want; ++t) {
+      const int eid = __float_as_int(e.y);
+      uint32_t bk;
+      int bi;
+      const int owner = warp_pick(eid == 0x7fffffff ? 0u : order_key(e.x), eid, bk, bi);
+      if (lane == (owner < 0 ? 0 : owner)) { oid[t] = bi; oval[t] = owner < 0 ? -INFINITY : e.x; ids_s[k * kTopkStride + t] = bi; }
+      if (lane == owner) {                               // the entry after the next is fetched while the next one competes
+        ++at;
+        e = nx;
+        nx = at + 1 < want ? list[at + 1] : none;
+      }
     }
-    block_best(bv, bi, sv, si);
-    if (threadIdx.x == 0) { ids[k * kTopkStride + t] = bi; vals[k * kTopkStride + t] = bv; }
-    pv = bv; pi = bi;
-    __syncthreads();
   }
+  __syncthreads();
+  if (threadIdx.x < kMaxRows)
+    tree_row(a.tree, reinterpret_cast<const DevState*>(a.state + a.state_stride * b), ids_s, nullptr, a.tok + (size_t)b * a.rows,
+             reinterpret_cast<RowMeta*>(a.meta + a.meta_stride * b), threadIdx.x);
 }
+static_assert(kTopkWarps >= kMaxK && kTopkChunks <= 32 && kTopkThreads >= kMaxRows, "a warp per head, a lane per slice, a thread per node");
 
-void launch_topk_heads(PartialView P, int vocab, int K, const int* ck, int* ids, float* vals, float* d_logits,
-                       float* cand, cudaStream_t st) {
+void launch_topk_tree(PartialView P, int vocab, int K, const int* ck, const TopkTreeArgs& a, int batch, cudaStream_t st) {
   TopkCounts c;
   for (int k = 0; k < kMaxK; ++k) c.c[k] = k < K ? ck[k] : 0;
   const int vec = vocab % 4 == 0 && P.ld % 4 == 0;
@@ -900,10 +970,10 @@ void launch_topk_heads(PartialView P, int vocab, int K, const int* ck, int* ids,
   chunk = (chunk + 3) / 4 * 4;
   const int n_chunks = (vocab + chunk - 1) / chunk;
   const size_t bytes = (size_t)chunk * sizeof(float);
-  if (bytes > 48 * 1024) cudaFuncSetAttribute(topk_slice_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  launch_pdl(topk_slice_kernel, dim3(K, n_chunks), dim3(kTopkThreads), bytes, st, P, vocab, chunk, c,
-             reinterpret_cast<float2*>(cand), d_logits, vec);
-  launch_pdl(topk_merge_kernel, dim3(K), dim3(kTopkThreads), 0, st, reinterpret_cast<const float2*>(cand), n_chunks, c, ids, vals);
+  if (bytes > 46 * 1024) cudaFuncSetAttribute(topk_slice_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  launch_pdl(topk_slice_kernel, dim3(K, n_chunks, batch), dim3(kTopkThreads), bytes, st, P, vocab, chunk, K, c, a.cand, a.cand_stride,
+             a.d_logits, a.d_logits_stride, vec);
+  launch_pdl(topk_tree_kernel, dim3(batch), dim3(kTopkThreads), 0, st, a, n_chunks, K, c);
 }
 
 // Greedy choice per verified row in two stages, like the top-k above: block (row, slice) reduces the partials of
@@ -1004,37 +1074,17 @@ void launch_meta_pending(RowMeta* meta, const DevState* s, cudaStream_t st) {
   launch_pdl(meta_pending_kernel, dim3(1), dim3(kMaxRows), 0, st, meta, s);
 }
 
-// tok[0] = root; tok[n] = head depth[n]'s candidate of rank rank[n] (Appendix A.1); optional overrides;
-// row table of the verification pass: position C + depth, slot C + n, mask = ancestors (Fig. 5).
-__global__ void tree_build_kernel(const TreeDev* __restrict__ tree, DevState* s, const int* __restrict__ topk_ids,
-                                  const int* __restrict__ override_tok, int* __restrict__ tok, RowMeta* meta) {
+// The tree of every sequence laid out again with the caller's tokens (entries < 0 keep the drafted ones).
+__global__ void tree_override_kernel(const TopkTreeArgs a, const int* __restrict__ override_tok) {
   pdl_wait();
   pdl_launch_dependents();
-  const int n = threadIdx.x;
-  const int N = tree->n_nodes;
-  const int C = s->C;
-  if (n == 0) { meta->base = C; meta->n_rows = N; }
-  if (n < N) {
-    if (n == 0) {
-      tok[0] = s->root;
-    } else {
-      if (topk_ids) tok[n] = topk_ids[(tree->depth[n] - 1) * kTopkStride + tree->rank[n]];
-      if (override_tok && override_tok[n] >= 0) tok[n] = override_tok[n];
-    }
-    meta->pos[n] = C + tree->depth[n];
-    meta->slot[n] = C + n;
-    meta->mask[n][0] = tree->anc[n][0];
-    meta->mask[n][1] = tree->anc[n][1];
-  } else {
-    meta->pos[n] = C;
-    meta->slot[n] = -1;
-    meta->mask[n][0] = meta->mask[n][1] = 0ull;
-  }
+  const int b = blockIdx.x;
+  tree_row(a.tree, reinterpret_cast<const DevState*>(a.state + a.state_stride * b), nullptr, override_tok + (size_t)b * a.rows,
+           a.tok + (size_t)b * a.rows, reinterpret_cast<RowMeta*>(a.meta + a.meta_stride * b), threadIdx.x);
 }
 
-void launch_tree_build(const TreeDev* tree, DevState* s, const int* topk_ids, const int* override_tok, int* tok,
-                       RowMeta* meta, cudaStream_t st) {
-  launch_pdl(tree_build_kernel, dim3(1), dim3(kMaxRows), 0, st, tree, s, topk_ids, override_tok, tok, meta);
+void launch_tree_override(const TopkTreeArgs& a, const int* override_tok, int batch, cudaStream_t st) {
+  launch_pdl(tree_override_kernel, dim3(batch), dim3(kMaxRows), 0, st, a, override_tok);
 }
 
 // Greedy acceptance: node n matches if its token equals the target's choice at its parent; it is
