@@ -414,12 +414,34 @@ RowScale row_scale_of(const amph_ctx* ctx, size_t off) {
 struct Pass {
   int G = 1;
   int rpg = 0;
+  PassRows src;
   const RowMeta* meta[kMaxSeq];
   float2* rope[kMaxSeq];
   int seq[kMaxSeq];
   int keys[kMaxSeq];
   int rows() const { return G * rpg; }
 };
+
+// Points the pass's tables at the verification (or prefill) set, or at the adaptation layers' own.
+void bind_tables(const amph_ctx* ctx, Pass* ps, bool sal, int source) {
+  const Layout& l = ctx->lay;
+  PassRows& p = ps->src;
+  p.source = source;
+  p.rpg = ps->rpg;
+  p.half = ctx->cfg.head_dim / 2;
+  p.meta = ctx->ws + (sal ? l.meta_s : l.meta_v);
+  p.meta_stride = l.meta_s_;
+  p.rope = ctx->ws + (sal ? l.rope_s : l.rope_v);
+  p.rope_stride = l.rope_s_;
+  p.inv_freq = ctx->at<double>(l.inv_freq);
+  p.state = ctx->ws + l.state;
+  p.state_stride = l.state_s;
+  for (int g = 0; g < kMaxSeq; ++g) p.base[g] = p.n[g] = 0;
+  for (int g = 0; g < ps->G; ++g) {
+    ps->meta[g] = reinterpret_cast<const RowMeta*>(p.meta + p.meta_stride * g);
+    ps->rope[g] = reinterpret_cast<float2*>(p.rope + p.rope_stride * g);
+  }
+}
 
 PartialView rows_from(PartialView P, int row0) {
   P.p += (size_t)row0 * P.ld;
@@ -428,13 +450,6 @@ PartialView rows_from(PartialView P, int row0) {
 RowScale rows_from(RowScale rs, int row0) {
   if (rs.ss) rs.ss += (size_t)row0 * rs.chunks;
   return rs;
-}
-
-void pass_rope_tables(amph_ctx* ctx, const Pass& ps) {
-  for (int g = 0; g < ps.G; ++g) {
-    ProfScope p(ctx, AMPH_PROF_OTHER);
-    launch_rope_table(ps.meta[g], ctx->at<double>(ctx->lay.inv_freq), ps.rope[g], ps.rpg, ctx->cfg.head_dim / 2, ctx->stream);
-  }
 }
 
 // While attention, the output projection and the residual kernel of a layer run, HBM is nearly idle (they are latency
@@ -574,16 +589,10 @@ void target_forward(amph_ctx* ctx, const Pass& ps) {
   const amph_config& c = ctx->cfg;
   const Layout& l = ctx->lay;
   cudaStream_t st = ctx->stream;
-  const int rows = ps.rows();
   float* x = ctx->at<float>(l.x);
-  pass_rope_tables(ctx, ps);
   { ProfScope p(ctx, AMPH_PROF_OTHER);
-  launch_embed(ctx->tok_emb, ctx->dtype, ctx->at<int>(l.tok), c.vocab, rows, c.d_model, x, st);
-  }
-  PartialView none = {nullptr, 0, 0, 0};
-  { ProfScope p(ctx, AMPH_PROF_NORM);
-  launch_resid_norm(x, none, 0, 0, ctx->layers[0].attn_norm, ctx->dtype, ctx->ws + l.xn, nullptr, c.rms_eps, rows,
-                    c.d_model, st);
+  launch_target_rows(ps.src, ps.G, ctx->tok_emb, ctx->dtype, ctx->at<int>(l.tok), c.vocab, c.d_model, ctx->layers[0].attn_norm, c.rms_eps, x,
+                     ctx->ws + l.xn, st);
   }
   bool deferred = false;
   for (int i = 0; i < c.n_layers; ++i) {
@@ -604,23 +613,20 @@ void target_head(amph_ctx* ctx, int rows) {
   }
 }
 
-// Eq. 1: both adaptation stages over the rows of the pass.  feat: fp32 rows [rows][d]; next_tok[g]: the ids of the
-// tokens that follow group g's rows (rpg entries).
-void run_sals(amph_ctx* ctx, const float* feat, const int* const* next_tok, const Pass& ps) {
+// Eq. 1: both adaptation stages over the rows of the pass.  feat: fp32 rows [rows][d]; next_tok: the ids of the
+// tokens that follow group 0's rows (rpg entries), group g's next_stride * g bytes further on.
+void run_sals(amph_ctx* ctx, const float* feat, const int* next_tok, size_t next_stride, const Pass& ps) {
   const amph_config& c = ctx->cfg;
   const Layout& l = ctx->lay;
   cudaStream_t st = ctx->stream;
   const int rows = ps.rows();
   const bool with_tok = !(c.flags & AMPH_FLAG_NO_SAMPLED_TOKEN);             // Section 4.5, "w/o Sampled-Token"
-  const size_t cat_pitch = (with_tok ? 2 : 1) * (size_t)c.d_model * ctx->esz;
-  pass_rope_tables(ctx, ps);
   const float* in_feat = feat;
   for (int s = 0; s < c.n_sal; ++s) {
     float* hbuf = ctx->at<float>(s == 0 ? l.h1 : l.h2);
-    for (int g = 0; g < ps.G; ++g) {
-      ProfScope p(ctx, AMPH_PROF_OTHER);
-      launch_concat(in_feat + (size_t)g * ps.rpg * c.d_model, with_tok ? ctx->tok_emb : nullptr, next_tok[g], c.vocab,
-                    ctx->ws + l.cat + cat_pitch * g * ps.rpg, ctx->dtype, ps.rpg, c.d_model, st);
+    { ProfScope p(ctx, AMPH_PROF_OTHER);
+    launch_sal_rows(ps.src, ps.G, s == 0, in_feat, with_tok ? ctx->tok_emb : nullptr, next_tok, next_stride, c.vocab, ctx->ws + l.cat,
+                    ctx->dtype, c.d_model, st);
     }
     const void* w[1] = {ctx->fc[s]};
     PartialView P = project(ctx, XB_CAT, w, 1, c.d_model, (with_tok ? 2 : 1) * c.d_model, rows);
@@ -682,43 +688,33 @@ amph_status do_draft(amph_ctx* ctx, int32_t* out_ids, float* out_vals) {
   const Layout& l = ctx->lay;
   cudaStream_t st = ctx->stream;
   const int B = ctx->B, K = c.K;
-  const size_t d = c.d_model;
   Pass ps;
   ps.G = B;
   ps.rpg = ctx->rows_small;
-  const int* next_tok[kMaxSeq];
+  bind_tables(ctx, &ps, true, PassRows::kPending);
   for (int b = 0; b < B; ++b) {
-    ps.meta[b] = ctx->meta_s(b);
-    ps.rope[b] = ctx->grp<float2>(l.rope_s, l.rope_s_, b);
     ps.seq[b] = b;
     ps.keys[b] = ctx->ctx_hi[b];
-    next_tok[b] = ctx->state(b)->pend_tok;
-    ProfScope p(ctx, AMPH_PROF_OTHER);
-    launch_meta_pending(ctx->meta_s(b), ctx->state(b), st);
   }
   float* pend_h = ctx->at<float>(l.pend_h);            // [B][16][d] = the rows of this pass
-  run_sals(ctx, pend_h, next_tok, ps);
+  run_sals(ctx, pend_h, ctx->state(0)->pend_tok, l.state_s, ps);
   // without adaptation layers (the "w/o Staged-Adaptation" ablation) every head reads the target's hidden state itself
   const float* s1 = c.n_sal == 0 ? pend_h : ctx->at<float>(l.h1);
   const float* s2 = c.n_sal == 0 ? pend_h : ctx->at<float>(c.n_sal == 2 ? l.h2 : l.h1);
-  for (int b = 0; b < B; ++b) {                        // rows 2 b, 2 b + 1 of the head MLPs' input: the last row of each stage
-    ProfScope p(ctx, AMPH_PROF_OTHER);
-    launch_gather_last(s1 + (size_t)b * ps.rpg * d, s2 + (size_t)b * ps.rpg * d, ctx->state(b), ctx->grp<float>(l.last, l.last_s, b),
-                       ctx->ws + l.last_act + ctx->esz * 2 * b * d, ctx->dtype, c.d_model, st);
+  { ProfScope p(ctx, AMPH_PROF_OTHER);                 // rows 2 b, 2 b + 1 of the head MLPs' input: the last row of each stage
+  launch_gather_last(s1, s2, ps.rpg, ctx->state(0), l.state_s, ctx->ws + l.last, l.last_s, ctx->ws + l.last_act, ctx->dtype, c.d_model, B, st);
   }
   PartialView P = project(ctx, XB_LAST, ctx->mlp_w, K, c.d_model, c.d_model, 2 * B);                 // Eq. 2
   float* hp = ctx->at<float>(l.hp);
   float* ao = ctx->at<float>(l.attn_o);
-  for (int b = 0; b < B; ++b) {                                                                       // Eq. 3-4
-    ProfScope p(ctx, AMPH_PROF_OTHER);
-    launch_mlp_heads(rows_from(P, 2 * b), ctx->grp<float>(l.last, l.last_s, b), ctx->mlp_b, ctx->pe, hp + (size_t)b * kMaxK * d,
-                     ao + (size_t)b * K * d, ctx->ws + l.ao_act + ctx->esz * b * K * d, ctx->dtype, K, c.n_sal, c.d_model, st);
+  { ProfScope p(ctx, AMPH_PROF_OTHER);                                                                // Eq. 3-4
+  launch_mlp_heads(P, ctx->ws + l.last, l.last_s, ctx->mlp_b, ctx->pe, hp, kMaxK, ao, ctx->ws + l.ao_act, ctx->dtype, K, c.n_sal, c.d_model,
+                   B, st);
   }
   for (int a = 0; a < c.aeb_layers; ++a) {                                                            // Eq. 5
     P = project(ctx, XB_AO, ctx->aeb_w[a], 3, c.d_model, c.d_model, B * K);
-    for (int b = 0; b < B; ++b) {                       // the K rows of a sequence attend to each other only
-      ProfScope p(ctx, AMPH_PROF_ATTENTION);
-      launch_aeb_attention(rows_from(P, b * K), ctx->ws + l.aeb_act + ctx->esz * b * K * d, ctx->dtype, K, c.n_heads, c.head_dim, st);
+    { ProfScope p(ctx, AMPH_PROF_ATTENTION);
+    launch_aeb_attention(P, ctx->ws + l.aeb_act, ctx->dtype, K, c.n_heads, c.head_dim, B, st);
     }
     const void* wo[1] = {ctx->aeb_w[a][3]};
     P = project(ctx, XB_AEB, wo, 1, c.d_model, c.d_model, B * K);
@@ -728,9 +724,8 @@ amph_status do_draft(amph_ctx* ctx, int32_t* out_ids, float* out_vals) {
   }
   if (c.lm_rank > 0) {                                                                                // Appendix A.2.4
     P = project(ctx, XB_AO, ctx->draft_lm_a, K, c.lm_rank, c.d_model, B * K);
-    for (int b = 0; b < B; ++b) {
-      ProfScope p(ctx, AMPH_PROF_OTHER);
-      launch_gather_diag(rows_from(P, b * K), ctx->ws + l.lr_act + ctx->esz * b * K * (size_t)c.lm_rank, ctx->dtype, K, c.lm_rank, st);
+    { ProfScope p(ctx, AMPH_PROF_OTHER);
+    launch_gather_diag(P, ctx->ws + l.lr_act, ctx->dtype, K, c.lm_rank, B, st);
     }
     P = project(ctx, XB_LR, ctx->draft_lm, K, c.vocab, c.lm_rank, B * K);
   } else {
@@ -769,9 +764,8 @@ amph_status do_verify(amph_ctx* ctx, const int32_t* tree_tokens, int32_t* out_ar
   Pass ps;
   ps.G = B;
   ps.rpg = ctx->Mver;
+  bind_tables(ctx, &ps, false, PassRows::kTree);
   for (int b = 0; b < B; ++b) {
-    ps.meta[b] = ctx->meta_v(b);
-    ps.rope[b] = ctx->grp<float2>(l.rope_v, l.rope_s_, b);
     ps.seq[b] = b;
     ps.keys[b] = ctx->ctx_hi[b] + N;
   }
@@ -1025,11 +1019,11 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
     Pass ps;
     ps.G = G;
     ps.rpg = rpg;
+    bind_tables(ctx, &ps, false, PassRows::kChain);
     for (int g = 0; g < G; ++g) {
       const int nr = cnt - g * M < M ? cnt - g * M : M;
-      launch_meta_chain(ctx->meta_v(g), start + g * M, nr, st);
-      ps.meta[g] = ctx->meta_v(g);
-      ps.rope[g] = ctx->grp<float2>(l.rope_v, l.rope_s_, g);
+      ps.src.base[g] = start + g * M;
+      ps.src.n[g] = nr;
       ps.seq[g] = seq;
       ps.keys[g] = start + g * M + nr;
     }
@@ -1042,17 +1036,15 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
       Pass pss;
       pss.G = (nrs + M - 1) / M;
       pss.rpg = rpg;
-      const int* next_tok[kMaxSeq];
+      bind_tables(ctx, &pss, true, PassRows::kChain);
       for (int g = 0; g < pss.G; ++g) {
         const int nr = nrs - g * M < M ? nrs - g * M : M;
-        launch_meta_chain(ctx->meta_s(g), start + g * M, nr, st);
-        pss.meta[g] = ctx->meta_s(g);
-        pss.rope[g] = ctx->grp<float2>(l.rope_s, l.rope_s_, g);
+        pss.src.base[g] = start + g * M;
+        pss.src.n[g] = nr;
         pss.seq[g] = seq;
         pss.keys[g] = start + g * M + nr;
-        next_tok[g] = ctx->at<int>(l.next_tok) + g * rpg;
       }
-      run_sals(ctx, ctx->at<float>(l.hidden), next_tok, pss);
+      run_sals(ctx, ctx->at<float>(l.hidden), ctx->at<int>(l.next_tok), sizeof(int) * rpg, pss);
     }
     if (last && c.temperature > 0.f)        // the token after the prompt is drawn, not the arg-max (stream 1 of the generator, step 0)
       launch_sample_rows(ctx->at<float>(l.logits), c.vocab, cnt - 1, 1, nullptr, nullptr, ctx->state(seq), seq, 1, c.temperature,

@@ -124,8 +124,22 @@ __device__ __forceinline__ float row_scale(const RowScale& rs, int row) {
 #endif
 
 // ---- launchers (one per kernel family); dtype = AMPH_DTYPE_* of weights / activations / cache
-void launch_embed(const void* tok_emb, int dtype, const int* toks, int vocab, int rows, int d,
-                  float* x, cudaStream_t st);
+// Rows of a pass in G groups of rpg: where their positions come from and where the row / rotary tables go (group 0's copy, the
+// next group's `stride` bytes further on).
+struct PassRows {
+  enum Source { kTree = 0, kChain = 1, kPending = 2 };   // table already written | base[g], n[g] | the state's pending rows
+  int source, rpg, half;
+  char* meta;        size_t meta_stride;     // RowMeta
+  char* rope;        size_t rope_stride;     // float2 [rows][half]
+  const double* inv_freq;
+  const char* state; size_t state_stride;    // DevState (kPending)
+  int base[AMPH_MAX_BATCH], n[AMPH_MAX_BATCH];
+};
+void launch_target_rows(const PassRows& p, int G, const void* tok_emb, int dtype, const int* toks, int vocab, int d, const void* gain,
+                        float eps, float* x, void* xn, cudaStream_t st);
+// next_tok: ids of the tokens that follow group 0's rows, the next group's next_stride bytes further on
+void launch_sal_rows(const PassRows& p, int G, int setup, const float* feat, const void* tok_emb, const void* next_tok, size_t next_stride,
+                     int vocab, void* cat, int dtype, int d, cudaStream_t st);
 
 // x <- (mode 0: x, mode 1: x + sum P, mode 2: sum P); then, if gain != NULL, RMSNorm of the result
 // into xn (storage dtype) and hid (fp32); with gain == NULL xn / hid receive the plain row.
@@ -140,9 +154,6 @@ void launch_resid_norm(float* x, PartialView P, int col_off, int mode, const voi
 // predecessor's grid is fully resident (one wave), so that the early starter cannot take its slots.
 void launch_resid_scale(float* x, PartialView P, int col_off, int mode, const void* gain, int dtype, void* xn,
                         float* ss_part, int rows, int d, cudaStream_t st, int early = 0);
-
-void launch_rope_table(const RowMeta* meta, const double* inv_freq, float2* table, int rows, int half,
-                       cudaStream_t st);
 
 // q <- rope(sum P[:, 0:d]); K cache <- rope(sum P[:, d:2d]); V cache <- sum P[:, 2d:3d]
 void launch_qkv_rope(PartialView P, const RowMeta* meta, const float2* rope, void* q, KvView kv,
@@ -192,26 +203,23 @@ bool launch_tree_attention_tc_groups(AttnTc* a, const void* q, int q_rows_cap, i
 void launch_swiglu(PartialView P, void* act, int dtype, int rows, int f, cudaStream_t st, RowScale rs = RowScale(),
                    int early = 0);
 
-// cat[r] = [feat[r] ; tok_emb[next[r]]]   (Eq. 1's concatenation)
-void launch_concat(const float* feat, const void* tok_emb, const int* next_tok, int vocab, void* cat,
-                   int dtype, int rows, int d, cudaStream_t st);
-
 struct GemmSeg { const void* w; };
 // P[row][seg*out + o] = sum_k X[row][k] * W_seg[o][k]; plain CUDA-core kernel, one split.
 void launch_gemm_generic(const void* x, int ldx, const GemmSeg* segs, int n_seg, int out, int in,
                          float* P, int ldp, int rows, int dtype, cudaStream_t st);
 
 // ---- draft-module specific
-void launch_gather_last(const float* h1, const float* h2, const DevState* st_dev, float* last /*[2][d]*/,
-                        void* last_act /*[>=2][d]*/, int dtype, int d, cudaStream_t st);
-// Hp[k] = src_k + silu(sum P[row_k][k*d + :] + b_k) + PE[k]   (Eq. 2-4)
-void launch_mlp_heads(PartialView P, const float* last, const void* const* bias, const void* pe,
-                      float* hp, float* ao, void* ao_act, int dtype, int K, int n_sal, int d, cudaStream_t st);
+// (one launch per batch; a void* with a stride is sequence 0's copy of a per-sequence buffer, the next `stride` bytes further on)
+void launch_gather_last(const float* h1, const float* h2, int rows_per, const void* state, size_t state_stride, void* last /*[2][d]*/,
+                        size_t last_stride, void* last_act /*[batch * 2][d]*/, int dtype, int d, int batch, cudaStream_t st);
+// Hp[k] = src_k + silu(sum P[2 b + row_k][k*d + :] + b_k) + PE[k]   (Eq. 2-4); hp [batch][hp_rows][d], ao / ao_act [batch * K][d]
+void launch_mlp_heads(PartialView P, const void* last, size_t last_stride, const void* const* bias, const void* pe, float* hp, int hp_rows,
+                      float* ao, void* ao_act, int dtype, int K, int n_sal, int d, int batch, cudaStream_t st);
 // unmasked attention across the K rows, one block per attention head (Eq. 5)
-void launch_aeb_attention(PartialView P, void* out_act, int dtype, int K, int n_heads, int head_dim,
+void launch_aeb_attention(PartialView P, void* out_act, int dtype, int K, int n_heads, int head_dim, int batch,
                           cudaStream_t st);
-// out_act[k][j] = P(row k, column k * r + j): row k of the k-th low-rank projection, as the next projection's input
-void launch_gather_diag(PartialView P, void* out_act, int dtype, int K, int r, cudaStream_t st);
+// out_act[row][j] = P(row, column (row % K) * r + j): the diagonal blocks of the low-rank projection, as the next projection's input
+void launch_gather_diag(PartialView P, void* out_act, int dtype, int K, int r, int batch, cudaStream_t st);
 // Per sequence b and head k: top-c_k of row b * K + k of segment k (also stored into d_logits), then the candidate tree built
 // from them (Appendix A.1).  cand: scratch for the slices' candidates, kMaxK * kTopkCandChunks * kTopkStride (value, id) pairs.
 // Pointers with a stride are sequence 0's copy of a per-sequence buffer, the next sequence's `stride` bytes further on.
@@ -233,8 +241,6 @@ void launch_tree_override(const TopkTreeArgs& a, const int* override_tok, int ba
 void launch_argmax_rows(PartialView P, int vocab, int rows, int* amax, float* logits_out, float* cand, cudaStream_t st);
 
 // ---- control kernels
-void launch_meta_chain(RowMeta* meta, int base, int n_rows, cudaStream_t st);             // prefill chunk
-void launch_meta_pending(RowMeta* meta, const DevState* s, cudaStream_t st);              // adaptation rows
 // Acceptance and KV compaction of every sequence of a batch.
 struct AcceptArgs {
   const TreeDev* tree;

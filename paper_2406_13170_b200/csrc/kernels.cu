@@ -78,28 +78,6 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 }
 
 // --------------------------------------------------------------------------------------------
-// embedding rows
-// --------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void embed_kernel(const T* __restrict__ emb, const int* __restrict__ toks, int vocab, int d,
-                             float* __restrict__ x) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int r = blockIdx.x;
-  int t = toks[r];
-  t = t < 0 ? 0 : (t >= vocab ? vocab - 1 : t);
-  const T* e = emb + (size_t)t * d;
-  for (int c = (blockIdx.y * blockDim.x + threadIdx.x) * 4; c < d; c += gridDim.y * blockDim.x * 4)
-    store4(x + (size_t)r * d + c, load4(e + c));
-}
-
-void launch_embed(const void* tok_emb, int dtype, const int* toks, int vocab, int rows, int d, float* x,
-                  cudaStream_t st) {
-  const int gy = (d / 4 + 255) / 256;
-  AMPH_DISPATCH(dtype, launch_pdl(embed_kernel<T>, dim3(rows, gy), dim3(256), 0, st, (const T*)tok_emb, toks, vocab, d, x));
-}
-
-// --------------------------------------------------------------------------------------------
 // residual update + RMSNorm (one block per row)
 // --------------------------------------------------------------------------------------------
 template <typename T>
@@ -189,24 +167,110 @@ void launch_resid_scale(float* x, PartialView P, int col_off, int mode, const vo
 }
 
 // --------------------------------------------------------------------------------------------
-// rotary table for the rows of one call: table[r][i] = (cos, sin)(pos[r] * theta^(-2i/dh))
+// start of a pass: row tables, rotary tables, and the rows themselves
 // --------------------------------------------------------------------------------------------
-__global__ void rope_table_kernel(const RowMeta* __restrict__ meta, const double* __restrict__ inv_freq,
-                                  float2* __restrict__ table, int half) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int r = blockIdx.x;
-  const double p = (double)meta->pos[r];
-  for (int i = threadIdx.x; i < half; i += blockDim.x) {
-    double s, c;
-    sincos(p * inv_freq[i], &s, &c);
-    table[r * half + i] = make_float2((float)c, (float)s);
+__device__ __forceinline__ void chain_mask(int r, u64* m) {       // bits 0..r
+  m[0] = r >= 63 ? ~0ull : ((1ull << (r + 1)) - 1ull);
+  m[1] = r < 64 ? 0ull : (r >= 127 ? ~0ull : ((1ull << (r - 63)) - 1ull));
+}
+
+// Row `rl` of group g: its rotary table row, and (row 0 of a chain) the group's whole row table.  A chain is a run of tokens
+// at consecutive positions, each seeing the ones before it: prompt chunks, or the rows an adaptation layer has pending.
+__device__ __forceinline__ void setup_row(const PassRows& p, int g, int rl) {
+  RowMeta* meta = reinterpret_cast<RowMeta*>(p.meta + p.meta_stride * g);
+  int pos;
+  if (p.source == PassRows::kTree) {                             // the table was written with the tree
+    pos = meta->pos[rl];
+  } else {
+    int base = p.base[g], n = p.n[g];
+    if (p.source == PassRows::kPending) {
+      const DevState* s = reinterpret_cast<const DevState*>(p.state + p.state_stride * g);
+      n = s->n_pending;
+      n = n < 0 ? 0 : (n > kPendMax ? kPendMax : n);
+      base = s->C - n;
+    }
+    pos = base + rl;
+    if (rl == 0) {
+      if (threadIdx.x == 0) { meta->base = base; meta->n_rows = n; }
+      for (int r = threadIdx.x; r < kMaxRows; r += blockDim.x) {
+        meta->pos[r] = base + r;
+        meta->slot[r] = base + r;
+        chain_mask(r, meta->mask[r]);
+      }
+    }
+  }
+  // table[r][i] = (cos, sin)(pos * theta^(-2i/dh)), in double: positions of thousands leave no room for a float angle
+  float2* table = reinterpret_cast<float2*>(p.rope + p.rope_stride * g) + (size_t)rl * p.half;
+  for (int i = threadIdx.x; i < p.half; i += blockDim.x) {
+    double sn, cs;
+    sincos((double)pos * p.inv_freq[i], &sn, &cs);
+    table[i] = make_float2((float)cs, (float)sn);
   }
 }
 
-void launch_rope_table(const RowMeta* meta, const double* inv_freq, float2* table, int rows, int half,
-                       cudaStream_t st) {
-  launch_pdl(rope_table_kernel, dim3(rows), dim3(64), 0, st, meta, inv_freq, table, half);
+// Start of a target pass, one block per row: row set-up, x = the token's embedding, xn = its RMSNorm with the first layer's
+// gain, in one launch for all groups.  Latency: a launch of its own for each costs 1.2-1.8 us of the chain, per group for the
+// tables (six launches fewer per step: 275 -> 269 us on a three-layer model of width 512).  A chain's row table is read by the attention kernel before its dependency wait, and the projection between lets
+// that kernel start at once: such a pass triggers its successor only by ending.
+template <typename T>
+__global__ void __launch_bounds__(1024)
+target_rows_kernel(const PassRows p, const T* __restrict__ emb, const int* __restrict__ toks, int vocab, int d,
+                   const T* __restrict__ gain, float eps, float* __restrict__ x, T* __restrict__ xn) {
+  pdl_wait();
+  if (p.source == PassRows::kTree) pdl_launch_dependents();
+  extern __shared__ __align__(16) float rowbuf[];
+  __shared__ float red[32];
+  const int r = blockIdx.x, g = r / p.rpg;
+  int t = toks[r];
+  t = t < 0 ? 0 : (t >= vocab ? vocab - 1 : t);
+  const T* e = emb + (size_t)t * d;
+  float ss = 0.f;
+  for (int c = threadIdx.x * 4; c < d; c += blockDim.x * 4) {
+    const float4 v = load4(e + c);
+    store4(x + (size_t)r * d + c, v);
+    store4(rowbuf + c, v);
+    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+  }
+  setup_row(p, g, r - g * p.rpg);
+  const float inv = 1.0f / sqrtf(block_sum(ss, red) / (float)d + eps);
+  for (int c = threadIdx.x * 4; c < d; c += blockDim.x * 4) {
+    const float4 v = load4(rowbuf + c), w = load4(gain + c);
+    store4(xn + (size_t)r * d + c, make_float4(w.x * (v.x * inv), w.y * (v.y * inv), w.z * (v.z * inv), w.w * (v.w * inv)));
+  }
+}
+
+void launch_target_rows(const PassRows& p, int G, const void* tok_emb, int dtype, const int* toks, int vocab, int d, const void* gain,
+                        float eps, float* x, void* xn, cudaStream_t st) {
+  int threads = (d / 4 + 31) / 32 * 32;
+  if (threads > 1024) threads = 1024;
+  AMPH_DISPATCH(dtype, launch_pdl(target_rows_kernel<T>, dim3(G * p.rpg), dim3(threads), d * sizeof(float), st, p, (const T*)tok_emb, toks,
+                                  vocab, d, (const T*)gain, eps, x, (T*)xn));
+}
+
+// Start of an adaptation stage (Eq. 1), all groups: cat[r] = [feature ; embedding of the next token], and for the first stage
+// (setup != 0) the pass's row set-up.  emb == NULL: the ablation without the sampled token; the row is the feature alone.
+template <typename T>
+__global__ void __launch_bounds__(256)
+sal_rows_kernel(const PassRows p, int setup, const float* __restrict__ feat, const T* __restrict__ emb, const char* next_tok,
+                size_t next_stride, int vocab, T* __restrict__ cat, int d) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int r = blockIdx.x, g = r / p.rpg, rl = r - g * p.rpg;
+  const size_t pitch = emb ? 2 * (size_t)d : (size_t)d;
+  int t = reinterpret_cast<const int*>(next_tok + next_stride * g)[rl];
+  t = t < 0 ? 0 : (t >= vocab ? vocab - 1 : t);
+  for (int c = (blockIdx.y * blockDim.x + threadIdx.x) * 4; c < d; c += gridDim.y * blockDim.x * 4) {
+    store4(cat + (size_t)r * pitch + c, load4(feat + (size_t)r * d + c));
+    if (emb) store4(cat + (size_t)r * pitch + d + c, load4(emb + (size_t)t * d + c));
+  }
+  if (setup && blockIdx.y == 0) setup_row(p, g, rl);
+}
+
+void launch_sal_rows(const PassRows& p, int G, int setup, const float* feat, const void* tok_emb, const void* next_tok, size_t next_stride,
+                     int vocab, void* cat, int dtype, int d, cudaStream_t st) {
+  const int gy = (d / 4 + 255) / 256;
+  AMPH_DISPATCH(dtype, launch_pdl(sal_rows_kernel<T>, dim3(G * p.rpg, gy), dim3(256), 0, st, p, setup, feat, (const T*)tok_emb,
+                                  (const char*)next_tok, next_stride, vocab, (T*)cat, d));
 }
 
 // --------------------------------------------------------------------------------------------
@@ -572,31 +636,6 @@ void launch_swiglu(PartialView P, void* act, int dtype, int rows, int f, cudaStr
 }
 
 // --------------------------------------------------------------------------------------------
-// Eq. 1's concatenation [feature ; embedding of the next token]
-// --------------------------------------------------------------------------------------------
-// emb == NULL: the ablation without the sampled token; the row is the feature alone (pitch d)
-template <typename T>
-__global__ void concat_kernel(const float* __restrict__ feat, const T* __restrict__ emb,
-                              const int* __restrict__ next_tok, int vocab, T* __restrict__ cat, int d) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int r = blockIdx.x;
-  const size_t pitch = emb ? 2 * (size_t)d : (size_t)d;
-  int t = next_tok[r];
-  t = t < 0 ? 0 : (t >= vocab ? vocab - 1 : t);
-  for (int c = (blockIdx.y * blockDim.x + threadIdx.x) * 4; c < d; c += gridDim.y * blockDim.x * 4) {
-    store4(cat + (size_t)r * pitch + c, load4(feat + (size_t)r * d + c));
-    if (emb) store4(cat + (size_t)r * pitch + d + c, load4(emb + (size_t)t * d + c));
-  }
-}
-
-void launch_concat(const float* feat, const void* tok_emb, const int* next_tok, int vocab, void* cat, int dtype,
-                   int rows, int d, cudaStream_t st) {
-  const int gy = (d / 4 + 255) / 256;
-  AMPH_DISPATCH(dtype, launch_pdl(concat_kernel<T>, dim3(rows, gy), dim3(256), 0, st, feat, (const T*)tok_emb, next_tok, vocab, (T*)cat, d));
-}
-
-// --------------------------------------------------------------------------------------------
 // Plain projection kernel: one warp per output feature, 128-bit weight loads, fp32 accumulate.
 // Used for fp32 models, for shapes the tensor-core kernel does not cover, and as its A/B check.
 // --------------------------------------------------------------------------------------------
@@ -671,76 +710,83 @@ void launch_gemm_generic(const void* x, int ldx, const GemmSeg* segs, int n_seg,
 // --------------------------------------------------------------------------------------------
 // draft module: last-row gather, head MLP epilogue (Eq. 2-4), fused K x K attention (Eq. 5)
 // --------------------------------------------------------------------------------------------
+// Rows 2 b, 2 b + 1 of `last`: the last pending row of each stage of sequence b (blockIdx.z), whose rows_per rows start at row
+// b * rows_per of h1 / h2.
 template <typename T>
-__global__ void gather_last_kernel(const float* __restrict__ h1, const float* __restrict__ h2,
-                                   const DevState* __restrict__ s, float* __restrict__ last,
+__global__ void gather_last_kernel(const float* __restrict__ h1, const float* __restrict__ h2, int rows_per,
+                                   const char* __restrict__ state, size_t state_stride, char* __restrict__ last, size_t last_stride,
                                    T* __restrict__ last_act, int d) {
   pdl_wait();
   pdl_launch_dependents();
-  int lr = s->n_pending - 1;
+  const int b = blockIdx.z;
+  int lr = reinterpret_cast<const DevState*>(state + state_stride * b)->n_pending - 1;
   lr = lr < 0 ? 0 : (lr >= kPendMax ? kPendMax - 1 : lr);
-  const float* src = blockIdx.x == 0 ? h1 : h2;
+  const float* src = (blockIdx.x == 0 ? h1 : h2) + ((size_t)b * rows_per + lr) * d;
+  float* dst = reinterpret_cast<float*>(last + last_stride * b) + (size_t)blockIdx.x * d;
+  T* act = last_act + ((size_t)b * 2 + blockIdx.x) * d;
   for (int c = (blockIdx.y * blockDim.x + threadIdx.x) * 4; c < d; c += gridDim.y * blockDim.x * 4) {
-    const float4 v = load4(src + (size_t)lr * d + c);
-    store4(last + (size_t)blockIdx.x * d + c, v);
-    store4(last_act + (size_t)blockIdx.x * d + c, v);
+    const float4 v = load4(src + c);
+    store4(dst + c, v);
+    store4(act + c, v);
   }
 }
 
-void launch_gather_last(const float* h1, const float* h2, const DevState* st_dev, float* last, void* last_act,
-                        int dtype, int d, cudaStream_t st) {
+void launch_gather_last(const float* h1, const float* h2, int rows_per, const void* state, size_t state_stride, void* last,
+                        size_t last_stride, void* last_act, int dtype, int d, int batch, cudaStream_t st) {
   const int gy = (d / 4 + 255) / 256;
-  AMPH_DISPATCH(dtype, launch_pdl(gather_last_kernel<T>, dim3(2, gy), dim3(256), 0, st, h1, h2, st_dev, last, (T*)last_act, d));
+  AMPH_DISPATCH(dtype, launch_pdl(gather_last_kernel<T>, dim3(2, gy, batch), dim3(256), 0, st, h1, h2, rows_per, (const char*)state,
+                                  state_stride, (char*)last, last_stride, (T*)last_act, d));
 }
 
 template <typename T>
-__global__ void gather_diag_kernel(PartialView P, T* __restrict__ out, int r) {
+__global__ void gather_diag_kernel(PartialView P, T* __restrict__ out, int K, int r) {
   pdl_wait();
   pdl_launch_dependents();
-  const int k = blockIdx.x;
-  for (int j = threadIdx.x; j < r; j += blockDim.x) out[(size_t)k * r + j] = from_f<T>(sum_partials(P, k, k * r + j));
+  const int row = blockIdx.x, k = row % K;
+  for (int j = threadIdx.x; j < r; j += blockDim.x) out[(size_t)row * r + j] = from_f<T>(sum_partials(P, row, k * r + j));
 }
 
-void launch_gather_diag(PartialView P, void* out_act, int dtype, int K, int r, cudaStream_t st) {
-  AMPH_DISPATCH(dtype, launch_pdl(gather_diag_kernel<T>, dim3(K), dim3(256), 0, st, P, (T*)out_act, r));
+void launch_gather_diag(PartialView P, void* out_act, int dtype, int K, int r, int batch, cudaStream_t st) {
+  AMPH_DISPATCH(dtype, launch_pdl(gather_diag_kernel<T>, dim3(K * batch), dim3(256), 0, st, P, (T*)out_act, K, r));
 }
 
 struct BiasPtrs { const void* b[kMaxK]; };
 
 template <typename T>
-__global__ void mlp_heads_kernel(PartialView P, const float* __restrict__ last, BiasPtrs bias,
-                                 const T* __restrict__ pe, float* __restrict__ hp, float* __restrict__ ao,
+__global__ void mlp_heads_kernel(PartialView P, const char* __restrict__ last, size_t last_stride, BiasPtrs bias,
+                                 const T* __restrict__ pe, float* __restrict__ hp, int hp_rows, float* __restrict__ ao,
                                  T* __restrict__ ao_act, int K, int n_sal, int d) {
   pdl_wait();
   pdl_launch_dependents();
-  const int k = blockIdx.x;
+  const int k = blockIdx.x, s = blockIdx.z;                 // head, sequence
   const int row = (k < K / 2 || n_sal == 1) ? 0 : 1;       // Eq. 2: first half of the heads <- stage 1
   const T* b = (const T*)bias.b[k];
+  const float* src = reinterpret_cast<const float*>(last + last_stride * s) + (size_t)row * d;
   for (int c = (blockIdx.y * blockDim.x + threadIdx.x) * 4; c < d; c += gridDim.y * blockDim.x * 4) {
-    const float4 w = sum_partials4(P, row, k * d + c), bb = load4(b + c), l = load4(last + (size_t)row * d + c),
-                 e = load4(pe + (size_t)k * d + c);
+    const float4 w = sum_partials4(P, 2 * s + row, k * d + c), bb = load4(b + c), l = load4(src + c), e = load4(pe + (size_t)k * d + c);
     float4 v;
     float pre;
     pre = w.x + bb.x; v.x = l.x + pre / (1.0f + expf(-pre)) + e.x;
     pre = w.y + bb.y; v.y = l.y + pre / (1.0f + expf(-pre)) + e.y;
     pre = w.z + bb.z; v.z = l.z + pre / (1.0f + expf(-pre)) + e.z;
     pre = w.w + bb.w; v.w = l.w + pre / (1.0f + expf(-pre)) + e.w;
-    store4(hp + (size_t)k * d + c, v);
-    store4(ao + (size_t)k * d + c, v);          // the attention block updates this copy in place
-    store4(ao_act + (size_t)k * d + c, v);
+    store4(hp + ((size_t)s * hp_rows + k) * d + c, v);
+    store4(ao + ((size_t)s * K + k) * d + c, v);          // the attention block updates this copy in place
+    store4(ao_act + ((size_t)s * K + k) * d + c, v);
   }
 }
 
-void launch_mlp_heads(PartialView P, const float* last, const void* const* bias, const void* pe, float* hp,
-                      float* ao, void* ao_act, int dtype, int K, int n_sal, int d, cudaStream_t st) {
+void launch_mlp_heads(PartialView P, const void* last, size_t last_stride, const void* const* bias, const void* pe, float* hp, int hp_rows,
+                      float* ao, void* ao_act, int dtype, int K, int n_sal, int d, int batch, cudaStream_t st) {
   BiasPtrs bp;
   for (int k = 0; k < kMaxK; ++k) bp.b[k] = k < K ? bias[k] : nullptr;
   const int gy = (d / 4 + 127) / 128;
-  AMPH_DISPATCH(dtype, launch_pdl(mlp_heads_kernel<T>, dim3(K, gy), dim3(128), 0, st, P, last, bp, (const T*)pe, hp, ao, (T*)ao_act,
-                                                              K, n_sal, d));
+  AMPH_DISPATCH(dtype, launch_pdl(mlp_heads_kernel<T>, dim3(K, gy, batch), dim3(128), 0, st, P, (const char*)last, last_stride, bp,
+                                  (const T*)pe, hp, hp_rows, ao, (T*)ao_act, K, n_sal, d));
 }
 
-// One block per attention head: the K x K score matrix, softmax and mixing stay in shared memory.
+// One block per attention head and sequence (blockIdx.y: its K rows attend to each other only): the K x K score matrix,
+// softmax and mixing stay in shared memory.
 template <typename T>
 __global__ void aeb_attention_kernel(PartialView P, T* __restrict__ out, int K, int n_heads, int dh) {
   pdl_wait();
@@ -750,12 +796,12 @@ __global__ void aeb_attention_kernel(PartialView P, T* __restrict__ out, int K, 
   float* ks = qs + K * dh;
   float* vs = ks + K * dh;
   float* pr = vs + K * dh;        // [K][K]
-  const int h = blockIdx.x, d = n_heads * dh;
+  const int h = blockIdx.x, row0 = blockIdx.y * K, d = n_heads * dh;
   const int per = K * dh / 4;                            // float4 items per q / k / v block
   for (int i = threadIdx.x; i < 3 * per; i += blockDim.x) {
     const int which = i / per, j = (i - which * per) * 4;
     const int r = j / dh, c = j - r * dh;
-    store4(sm + which * K * dh + j, sum_partials4(P, r, which * d + h * dh + c));
+    store4(sm + which * K * dh + j, sum_partials4(P, row0 + r, which * d + h * dh + c));
   }
   __syncthreads();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -780,14 +826,14 @@ __global__ void aeb_attention_kernel(PartialView P, T* __restrict__ out, int K, 
     const int i = idx / dh, c = idx - i * dh;
     float acc = 0.f;
     for (int j = 0; j < K; ++j) acc += pr[i * K + j] * vs[j * dh + c];
-    out[(size_t)i * d + h * dh + c] = from_f<T>(acc);
+    out[(size_t)(row0 + i) * d + h * dh + c] = from_f<T>(acc);
   }
 }
 
-void launch_aeb_attention(PartialView P, void* out_act, int dtype, int K, int n_heads, int head_dim,
+void launch_aeb_attention(PartialView P, void* out_act, int dtype, int K, int n_heads, int head_dim, int batch,
                           cudaStream_t st) {
   const size_t smem = sizeof(float) * (3 * K * head_dim + K * K);
-  AMPH_DISPATCH(dtype, launch_pdl(aeb_attention_kernel<T>, dim3(n_heads), dim3(128), smem, st, P, (T*)out_act, K, n_heads, head_dim));
+  AMPH_DISPATCH(dtype, launch_pdl(aeb_attention_kernel<T>, dim3(n_heads, batch), dim3(128), smem, st, P, (T*)out_act, K, n_heads, head_dim));
 }
 
 // --------------------------------------------------------------------------------------------
@@ -1036,44 +1082,8 @@ void launch_argmax_rows(PartialView P, int vocab, int rows, int* amax, float* lo
 }
 
 // --------------------------------------------------------------------------------------------
-// control: row tables, tree tokens, acceptance, compaction
+// control: tree tokens, acceptance, compaction
 // --------------------------------------------------------------------------------------------
-__device__ __forceinline__ void chain_mask(int r, u64* m) {       // bits 0..r
-  m[0] = r >= 63 ? ~0ull : ((1ull << (r + 1)) - 1ull);
-  m[1] = r < 64 ? 0ull : (r >= 127 ? ~0ull : ((1ull << (r - 63)) - 1ull));
-}
-
-__global__ void meta_chain_kernel(RowMeta* meta, int base, int n_rows) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int r = threadIdx.x;
-  if (r == 0) { meta->base = base; meta->n_rows = n_rows; }
-  meta->pos[r] = base + r;
-  meta->slot[r] = base + r;
-  chain_mask(r, meta->mask[r]);
-}
-
-void launch_meta_chain(RowMeta* meta, int base, int n_rows, cudaStream_t st) {
-  launch_pdl(meta_chain_kernel, dim3(1), dim3(kMaxRows), 0, st, meta, base, n_rows);
-}
-
-__global__ void meta_pending_kernel(RowMeta* meta, const DevState* s) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int r = threadIdx.x;
-  int np = s->n_pending;
-  np = np < 0 ? 0 : (np > kPendMax ? kPendMax : np);
-  const int base = s->C - np;
-  if (r == 0) { meta->base = base; meta->n_rows = np; }
-  meta->pos[r] = base + r;
-  meta->slot[r] = base + r;
-  chain_mask(r, meta->mask[r]);
-}
-
-void launch_meta_pending(RowMeta* meta, const DevState* s, cudaStream_t st) {
-  launch_pdl(meta_pending_kernel, dim3(1), dim3(kMaxRows), 0, st, meta, s);
-}
-
 // The tree of every sequence laid out again with the caller's tokens (entries < 0 keep the drafted ones).
 __global__ void tree_override_kernel(const TopkTreeArgs a, const int* __restrict__ override_tok) {
   pdl_wait();
