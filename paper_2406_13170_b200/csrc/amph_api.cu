@@ -748,12 +748,10 @@ void sample_tree_choices(amph_ctx* ctx) {
   const Layout& l = ctx->lay;
   const amph_config& c = ctx->cfg;
   const unsigned long long seed = ((unsigned long long)c.seed_hi << 32) | c.seed_lo;
-  for (int b = 0; b < ctx->B; ++b) {
-    ProfScope p(ctx, AMPH_PROF_SELECT);
-    launch_sample_rows(ctx->at<float>(l.logits), c.vocab, b * ctx->Mver, ctx->tree_host.n_nodes, ctx->at<TreeDev>(l.tree),
-                       ctx->at<int>(l.tok) + b * ctx->Mver, ctx->state(b), b, 0, c.temperature, seed, ctx->at<int>(l.amax),
-                       ctx->at<float>(l.uniforms) + b * ctx->Mver, ctx->stream);
-  }
+  ProfScope p(ctx, AMPH_PROF_SELECT);
+  launch_sample_rows(ctx->at<float>(l.logits), c.vocab, 0, ctx->tree_host.n_nodes, ctx->Mver, ctx->B, ctx->at<TreeDev>(l.tree),
+                     ctx->at<int>(l.tok), ctx->state(0), l.state_s, 0, 0, c.temperature, seed, ctx->at<int>(l.amax),
+                     ctx->at<float>(l.uniforms), ctx->stream);
 }
 
 // tree_tokens / out_argmax: [B][n_nodes]
@@ -1047,7 +1045,7 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
       run_sals(ctx, ctx->at<float>(l.hidden), ctx->at<int>(l.next_tok), sizeof(int) * rpg, pss);
     }
     if (last && c.temperature > 0.f)        // the token after the prompt is drawn, not the arg-max (stream 1 of the generator, step 0)
-      launch_sample_rows(ctx->at<float>(l.logits), c.vocab, cnt - 1, 1, nullptr, nullptr, ctx->state(seq), seq, 1, c.temperature,
+      launch_sample_rows(ctx->at<float>(l.logits), c.vocab, cnt - 1, 1, 1, 1, nullptr, nullptr, ctx->state(seq), l.state_s, seq, 1, c.temperature,
                          ((unsigned long long)c.seed_hi << 32) | c.seed_lo, ctx->at<int>(l.amax), nullptr, st);
     if (last)
       launch_prefill_tail(ctx->state(seq), ctx->at<int>(l.amax), cnt - 1, ctx->at<float>(l.hidden),

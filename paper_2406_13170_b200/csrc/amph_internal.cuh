@@ -256,14 +256,14 @@ struct AcceptArgs {
   int pend_rows;
 };
 void launch_accept_compact(const AcceptArgs& a, int batch, int dtype, cudaStream_t st);
-// Sampling at temperature T > 0 (Table 2): choice[r] for rows row0 .. row0 + n_rows - 1 = the token the target draws after
-// that row from softmax(logits / T) with the row's own uniform (Philox4x32-10 keyed by seed; counter = row - row0, the
-// sequence's step count, seq, stream).  With a tree (tok != NULL) the vocabulary is walked in the order (tokens of the
-// row's children in node order, then every other id ascending), so that a child is accepted iff its token is the choice:
-// the rejection-sampling test of Section 2 for point-mass proposals.  uniforms_out (may be NULL) receives the uniforms.
-void launch_sample_rows(const float* logits, int vocab, int row0, int n_rows, const TreeDev* tree, const int* tok,
-                        const DevState* s, int seq, int stream_id, float temperature, unsigned long long seed, int* choice,
-                        float* uniforms_out, cudaStream_t st);
+// Sampling at temperature T > 0 (Table 2): choice[row] for rows row0 + b * rows_per + r, r < n_rows, of every sequence b = the
+// token the target draws after that row from softmax(logits / T) with the row's own uniform (Philox4x32-10 keyed by seed; counter
+// = r, the sequence's step count, seq0 + b, stream).  With a tree (tok [batch][rows_per]) the vocabulary is walked in the order
+// (tokens of the row's children in node order, then every other id ascending), so that a child is accepted iff its token is the
+// choice: the rejection-sampling test of Section 2 for point-mass proposals.  uniforms_out [batch][rows_per] (may be NULL).
+void launch_sample_rows(const float* logits, int vocab, int row0, int n_rows, int rows_per, int batch, const TreeDev* tree, const int* tok,
+                        const void* state, size_t state_stride, int seq0, int stream_id, float temperature, unsigned long long seed,
+                        int* choice, float* uniforms_out, cudaStream_t st);
 void launch_reduce_partials(PartialView P, float* y, int rows, int cols, cudaStream_t st);
 void launch_kv_export(KvView kv, int which, int dtype, int row0, int rows, int n_heads, int head_dim, int max_ctx,
                       float* dst, cudaStream_t st);

@@ -1211,74 +1211,122 @@ __device__ __forceinline__ uint32_t philox_first_word(uint32_t c0, uint32_t c1, 
 }
 
 constexpr int kSampleThreads = 1024;
+constexpr int kSampleWarps = kSampleThreads / 32;
 constexpr int kSampleMaxChildren = 16;       // candidates a head keeps at most = children a node has at most
 
-// One block per row.  w(v) = exp((l_v - max) / T); the row's uniform scaled by the sum of all weights is compared with
-// running sums of w, so nothing is divided.  Sums are taken in a fixed order (deterministic).
+// One block per row and sequence (blockIdx.y).  w(v) = exp((l_v - max) / T); the row's uniform scaled by the sum of all weights
+// is compared with running sums of w, so nothing is divided.  Every thread owns a contiguous range of ids; sums over threads
+// are block-wide scans in a fixed order (deterministic).  Bound: latency, then the logits' L2 reads: with the children
+// collected and the range sums added one after the other by one thread, and a launch per sequence, a step of eight sequences
+// of 48 rows took 410 us more (32000 ids).
 __global__ void __launch_bounds__(kSampleThreads)
-sample_rows_kernel(const float* __restrict__ logits, int vocab, int row0, const TreeDev* __restrict__ tree,
-                   const int* __restrict__ tok, const DevState* __restrict__ s, int seq, int stream_id, float inv_t,
+sample_rows_kernel(const float* __restrict__ logits, int vocab, int row0, int rows_per, const TreeDev* __restrict__ tree,
+                   const int* __restrict__ tok, const char* __restrict__ state, size_t state_stride, int seq0, int stream_id, float inv_t,
                    uint32_t k0, uint32_t k1, int* __restrict__ choice, float* __restrict__ uniforms_out) {
   pdl_wait();
   pdl_launch_dependents();
-  __shared__ float red[kSampleThreads / 32];
-  __shared__ float part[kSampleThreads];
+  __shared__ float red[kSampleWarps];
+  __shared__ int kids_all[kMaxRows];
   __shared__ int kid_tok[kSampleMaxChildren];
-  __shared__ int n_kids_s, result_s;
+  __shared__ float kid_w[kSampleMaxChildren];
+  __shared__ uint32_t kid_votes[kMaxRows / 32];
+  __shared__ int n_kids_s, result_s, owner_s, last_s;
   __shared__ float target_s, base_s;
-  const int r = blockIdx.x, row = row0 + r, tid = threadIdx.x;
+  const int r = blockIdx.x, b = blockIdx.y, row = row0 + b * rows_per + r, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const float* l = logits + (size_t)row * vocab;
-  // row maximum
+  const bool vec = vocab % 4 == 0;
+  // row maximum; meanwhile the first warps find the row's children
   float m = -INFINITY;
-  for (int v = tid; v < vocab; v += kSampleThreads) m = fmaxf(m, l[v]);
+  if (vec) {
+    for (int v = tid * 4; v < vocab; v += kSampleThreads * 4) {
+      const float4 x = load4(l + v);
+      m = fmaxf(m, fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
+    }
+  } else {
+    for (int v = tid; v < vocab; v += kSampleThreads) m = fmaxf(m, l[v]);
+  }
+  const bool kids_given = tree != nullptr && tok != nullptr;
+  bool is_kid = false;
+  if (tid < kMaxRows) {
+    is_kid = kids_given && tid > r && tid < tree->n_nodes && tree->parent[tid] == r;
+    const uint32_t v = __ballot_sync(0xffffffffu, is_kid);
+    if (lane == 0) kid_votes[warp] = v;
+  }
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((tid & 31) == 0) red[tid >> 5] = m;
+  if (lane == 0) red[warp] = m;
+  if (tid == 0) { result_s = -1; owner_s = kSampleThreads; last_s = -1; }
   __syncthreads();
-  m = red[0];
-  for (int i = 1; i < kSampleThreads / 32; ++i) m = fmaxf(m, red[i]);
+  m = red[lane];
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (is_kid) {                                            // node order = order of the votes
+    int at = __popc(kid_votes[warp] & ((1u << lane) - 1u));
+    for (int w = 0; w < warp; ++w) at += __popc(kid_votes[w]);
+    kids_all[at] = tok[(size_t)b * rows_per + tid];
+  }
   __syncthreads();
-  // the distinct tokens of the row's children, in node order
-  if (tid == 0) {
-    int nk = 0;
-    if (tree != nullptr && tok != nullptr) {
-      const int N = tree->n_nodes;
-      for (int c = r + 1; c < N && nk < kSampleMaxChildren; ++c) {
-        if (tree->parent[c] != r) continue;
-        const int x = tok[c];
-        bool seen = x < 0 || x >= vocab;
-        for (int j = 0; j < nk; ++j) seen = seen || kid_tok[j] == x;
-        if (!seen) kid_tok[nk++] = x;
-      }
+  if (tid == 0) {                                          // the distinct tokens of the row's children, in node order
+    int n = 0, nk = 0;
+    for (int w = 0; w < kMaxRows / 32; ++w) n += __popc(kid_votes[w]);
+    for (int c = 0; c < n && nk < kSampleMaxChildren; ++c) {
+      const int x = kids_all[c];
+      bool seen = x < 0 || x >= vocab;
+      for (int j = 0; j < nk; ++j) seen = seen || kid_tok[j] == x;
+      if (!seen) kid_tok[nk++] = x;
     }
     n_kids_s = nk;
-    result_s = -1;
   }
   __syncthreads();
   const int nk = n_kids_s;
-  // every thread owns a contiguous range of ids; its weight sum leaves the children's tokens out
-  const int chunk = (vocab + kSampleThreads - 1) / kSampleThreads;
+  if (tid < nk) kid_w[tid] = __expf((l[kid_tok[tid]] - m) * inv_t);
+  // this thread's ids (whole groups of four); its weight sum leaves the children's tokens out
+  const int chunk = ((vocab + kSampleThreads - 1) / kSampleThreads + 3) / 4 * 4;
   const int lo = tid * chunk, hi = lo + chunk < vocab ? lo + chunk : vocab;
+  bool kid_here = false;
+  for (int j = 0; j < nk; ++j) kid_here = kid_here || (kid_tok[j] >= lo && kid_tok[j] < hi);
   float mine = 0.f;
-  for (int v = lo; v < hi; ++v) {
-    bool kid = false;
-    for (int j = 0; j < nk; ++j) kid = kid || kid_tok[j] == v;
-    if (!kid) mine += __expf((l[v] - m) * inv_t);
+  if (kid_here || !vec) {
+    for (int v = lo; v < hi; ++v) {
+      bool kid = false;
+      for (int j = 0; j < nk; ++j) kid = kid || kid_tok[j] == v;
+      if (!kid) mine += __expf((l[v] - m) * inv_t);
+    }
+  } else {
+    for (int v = lo; v < hi; v += 4) {                     // vocab % 4 == 0: the last group is whole
+      const float4 x = load4(l + v);
+      mine += __expf((x.x - m) * inv_t);
+      mine += __expf((x.y - m) * inv_t);
+      mine += __expf((x.z - m) * inv_t);
+      mine += __expf((x.w - m) * inv_t);
+    }
   }
-  part[tid] = mine;
+  // inclusive scan of the range sums over the block
+  float run = mine;
+  for (int o = 1; o < 32; o <<= 1) {
+    const float up = __shfl_up_sync(0xffffffffu, run, o);
+    if (lane >= o) run += up;
+  }
+  if (lane == 31) red[warp] = run;                         // every thread has read the maxima before the two barriers above
   __syncthreads();
+  float wsum = red[lane];
+  for (int o = 1; o < 32; o <<= 1) {
+    const float up = __shfl_up_sync(0xffffffffu, wsum, o);
+    if (lane >= o) wsum += up;
+  }
+  const float rest = __shfl_sync(0xffffffffu, wsum, 31);
+  const float below = __shfl_sync(0xffffffffu, wsum, warp == 0 ? 0 : warp - 1);
+  const float before = warp == 0 ? 0.f : below;
   if (tid == 0) {
-    const uint32_t w = philox_first_word((uint32_t)r, (uint32_t)s->step, (uint32_t)seq, (uint32_t)stream_id, k0, k1);
+    const DevState* s = reinterpret_cast<const DevState*>(state + state_stride * b);
+    const uint32_t w = philox_first_word((uint32_t)r, (uint32_t)s->step, (uint32_t)(seq0 + b), (uint32_t)stream_id, k0, k1);
     const float u = (float)(w >> 8) * (1.0f / 16777216.0f);
-    if (uniforms_out) uniforms_out[r] = u;
-    float kids = 0.f, rest = 0.f;
-    float wk[kSampleMaxChildren];
-    for (int j = 0; j < nk; ++j) { wk[j] = __expf((l[kid_tok[j]] - m) * inv_t); kids += wk[j]; }
-    for (int i = 0; i < kSampleThreads; ++i) rest += part[i];
+    if (uniforms_out) uniforms_out[b * rows_per + r] = u;
+    float kids = 0.f;
+    for (int j = 0; j < nk; ++j) kids += kid_w[j];
     const float target = u * (kids + rest);
     float acc = 0.f;
     int res = -1;
     for (int j = 0; j < nk && res < 0; ++j) {            // children first: accepted iff the running sum passes the target
-      acc += wk[j];
+      acc += kid_w[j];
       if (target < acc) res = kid_tok[j];
     }
     result_s = res;
@@ -1291,43 +1339,34 @@ sample_rows_kernel(const float* __restrict__ logits, int vocab, int row0, const 
     return;
   }
   // residual distribution: the first id, ascending, children's tokens left out, whose running sum exceeds the target
-  if (tid == 0) {
-    float acc = base_s;
-    int owner = -1;
-    for (int i = 0; i < kSampleThreads; ++i) {
-      if (acc + part[i] > target_s && part[i] > 0.f) { owner = i; break; }
-      acc += part[i];
-    }
-    if (owner < 0) {                                       // rounding left the target above the total: the last admissible id
-      for (int i = kSampleThreads - 1; i >= 0 && owner < 0; --i)
-        if (part[i] > 0.f) { owner = i; acc = -INFINITY; }   // its walk then ends on its last admissible id
-    }
-    n_kids_s = nk;
-    result_s = -2 - owner;                                 // owner thread, encoded
-    base_s = acc;
+  if (mine > 0.f) {
+    if (base_s + (before + run) > target_s) atomicMin(&owner_s, tid);
+    atomicMax(&last_s, tid);
   }
   __syncthreads();
-  const int owner = -2 - result_s;
-  if (tid == owner) {
-    float acc = base_s;
+  const bool beyond = owner_s == kSampleThreads;           // rounding left the target above the total: the last admissible id
+  if (tid == (beyond ? last_s : owner_s)) {
+    float acc = beyond ? -INFINITY : base_s + (before + (run - mine));
     int res = -1, last = -1;
     for (int v = lo; v < hi; ++v) {
       bool kid = false;
       for (int j = 0; j < nk; ++j) kid = kid || kid_tok[j] == v;
       if (kid) continue;
-      last = v;
-      acc += __expf((l[v] - m) * inv_t);
+      const float w = __expf((l[v] - m) * inv_t);
+      if (w > 0.f) last = v;
+      acc += w;
       if (acc > target_s) { res = v; break; }
     }
     choice[row] = res >= 0 ? res : last;
   }
 }
 
-void launch_sample_rows(const float* logits, int vocab, int row0, int n_rows, const TreeDev* tree, const int* tok,
-                        const DevState* s, int seq, int stream_id, float temperature, unsigned long long seed, int* choice,
-                        float* uniforms_out, cudaStream_t st) {
-  launch_pdl(sample_rows_kernel, dim3(n_rows), dim3(kSampleThreads), 0, st, logits, vocab, row0, tree, tok, s, seq, stream_id,
-             1.0f / temperature, (uint32_t)(seed & 0xffffffffull), (uint32_t)(seed >> 32), choice, uniforms_out);
+void launch_sample_rows(const float* logits, int vocab, int row0, int n_rows, int rows_per, int batch, const TreeDev* tree, const int* tok,
+                        const void* state, size_t state_stride, int seq0, int stream_id, float temperature, unsigned long long seed,
+                        int* choice, float* uniforms_out, cudaStream_t st) {
+  launch_pdl(sample_rows_kernel, dim3(n_rows, batch), dim3(kSampleThreads), 0, st, logits, vocab, row0, rows_per, tree, tok,
+             (const char*)state, state_stride, seq0, stream_id, 1.0f / temperature, (uint32_t)(seed & 0xffffffffull), (uint32_t)(seed >> 32),
+             choice, uniforms_out);
 }
 
 __global__ void reduce_partials_kernel(PartialView P, float* __restrict__ y, int rows, int cols) {
