@@ -56,7 +56,7 @@ struct Layout {
   size_t tok, amax, override_tok, next_tok, amax_cand, uniforms;        // [Rcap] ints / candidates / floats
   size_t x, hidden, h1, h2, pend_h, hp, attn_o;                           // fp32 rows
   size_t xn, q, att, act, cat, last_act, ao_act, aeb_act, lr_act;        // storage-type rows
-  size_t partial, logits, ss_a, ss_b;
+  size_t partial, logits, ss_a, ss_b, wide_flags;
   size_t partial_floats;
   int attn_splits;
 };
@@ -283,6 +283,7 @@ void make_layout(const amph_config& c, int n_nodes, Layout* L, int* Mcap_out, si
   l.logits = l.take(4 * (size_t)Rcap * V);
   l.ss_a = l.take(4 * (size_t)Rcap * 32);
   l.ss_b = l.take(4 * (size_t)Rcap * 32);
+  l.wide_flags = l.take(sizeof(int) * kWideFlags);
   *L = l;
   *Mcap_out = Mcap;
   const size_t per_layer = 2 * (size_t)c.n_heads * c.max_ctx * c.head_dim * esz;
@@ -493,7 +494,21 @@ bool layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, c
   const RowScale rs = entry_deferred ? row_scale_of(ctx, l.ss_a) : RowScale();
   PartialView P = {nullptr, 0, 0, 0};
   bool fused_rope = false;
-  if (ctx->tc && ps.G == 1 && !(c.flags & AMPH_FLAG_SEPARATE_ROPE)) {   // q / k / v projection that rotates and writes the cache itself
+  RopeGroups gr;
+  gr.G = ps.G;
+  gr.rpg = ps.rpg;
+  for (int g = 0; g < ps.G; ++g) {
+    const KvView kv = cache_of(ps.seq[g]);
+    gr.meta[g] = ps.meta[g]; gr.rope[g] = ps.rope[g]; gr.kc[g] = kv.k; gr.vc[g] = kv.v;
+  }
+  if (ctx->tc && rows > kWideFrom && !(c.flags & AMPH_FLAG_SEPARATE_ROPE)) {
+    ProfScope p(ctx, AMPH_PROF_PROJECTION);
+    fused_rope = tc_wide_launch_qkv_rope(ctx->tc, XB_XN, w.wq, w.wk, w.wv, c.n_heads, c.head_dim, c.d_model, rows, ctx->ws + l.q, gr,
+                                         c.max_ctx, rs, st);
+    if (fused_rope && p.rec) ctx->prof_bytes += 3LL * c.d_model * c.d_model * (int64_t)ctx->esz;
+    if (!fused_rope) cudaGetLastError();
+  }
+  if (!fused_rope && ctx->tc && ps.G == 1 && !(c.flags & AMPH_FLAG_SEPARATE_ROPE)) {   // q / k / v projection that rotates and writes the cache itself
     ProfScope p(ctx, AMPH_PROF_PROJECTION);
     fused_rope = tc_gemm_launch_qkv_rope(ctx->tc, XB_XN, w.wq, w.wk, w.wv, c.n_heads, c.head_dim, c.d_model, rows, ctx->ws + l.q,
                                          cache_of(ps.seq[0]), ps.meta[0], ps.rope[0], c.max_ctx, rs, st);
@@ -505,13 +520,6 @@ bool layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, c
   bool grouped_rope = false;
   if (!fused_rope && ps.G > 1) {                      // every group's rotary embedding + cache write in one launch
     ProfScope p(ctx, AMPH_PROF_ROPE_KV);
-    RopeGroups gr;
-    gr.G = ps.G;
-    gr.rpg = ps.rpg;
-    for (int g = 0; g < ps.G; ++g) {
-      const KvView kv = cache_of(ps.seq[g]);
-      gr.meta[g] = ps.meta[g]; gr.rope[g] = ps.rope[g]; gr.kc[g] = kv.k; gr.vc[g] = kv.v;
-    }
     launch_qkv_rope_groups(P, gr, ctx->ws + l.q, ctx->dtype, c.n_heads, c.head_dim, c.max_ctx, st, rs);
     grouped_rope = true;
   }
@@ -561,8 +569,12 @@ bool layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, c
   bool fused_gu = false;
   if (ctx->tc && !(c.flags & AMPH_FLAG_SEPARATE_SWIGLU)) {         // gate / up projection with SwiGLU in its epilogue
     ProfScope p(ctx, AMPH_PROF_PROJECTION);
-    fused_gu = tc_gemm_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act,
-                                     row_scale_of(ctx, l.ss_b), st);
+    if (rows > kWideFrom)
+      fused_gu = tc_wide_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act,
+                                       row_scale_of(ctx, l.ss_b), st);
+    else
+      fused_gu = tc_gemm_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act,
+                                       row_scale_of(ctx, l.ss_b), st);
     if (fused_gu && p.rec) ctx->prof_bytes += 2LL * c.d_ffn * c.d_model * (int64_t)ctx->esz;
     if (fused_gu) ctx->last_proj_one_wave = false;
   }
@@ -995,6 +1007,7 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
                                  c.d_model, c.d_model, c.d_model,
                                  c.lm_rank > 0 ? c.lm_rank : 8};
     ctx->tc = tc_gemm_create(xb, xrows, xcols, XB_COUNT, &ctx->state(0)->err);
+    if (ctx->tc) tc_wide_bind(ctx->tc, ctx->at<float>(ctx->lay.partial), ctx->lay.partial_floats, ctx->at<int>(ctx->lay.wide_flags));
   }
   if (!ctx->attn_tc && c.kv_dtype == AMPH_DTYPE_BF16 && !(c.flags & AMPH_FLAG_MMA_SYNC_ATTENTION))
     ctx->attn_tc = attn_tc_create();

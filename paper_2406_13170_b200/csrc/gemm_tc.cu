@@ -479,6 +479,7 @@ TcGemm* tc_gemm_create(void* const* xbufs, const int* xrows, const int* xcols, i
   cudaFuncSetAttribute(tc_gemm_kernel<EPI_PARTIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, g->max_smem - 2048);
   cudaFuncSetAttribute(tc_gemm_kernel<EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, g->max_smem - 2048);
   cudaFuncSetAttribute(tc_gemm_kernel<EPI_ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, g->max_smem - 2048);
+  tc_wide_init(g);
   return g;
 }
 
@@ -487,6 +488,7 @@ bool tc_gemm_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   if (!g || xb < 0 || xb >= g->n_x) return false;
   if (out % kTileM || in % kTileK || n_seg < 1 || n_seg > kMaxSeg || rows < 1) return false;
   if (g->xcols[xb] != in) return false;
+  if (rows > kWideFrom && g->extra_tx == 0 && tc_wide_launch(g, xb, w, n_seg, out, in, rows, P, p_floats, splits_out, split_stride, st)) return true;
   // up to 128 rows: one MMA of N = rows rounded up to 16; more: 2..4 row blocks of 128 rows that share every weight tile
   // (the tile is streamed from HBM once and multiplied with each block: batched verification, dense prefill)
   const int nt_all = rows <= 16 ? 16 : (rows <= 128 ? (rows + 15) / 16 * 16 : (rows + 127) / 128 * 128);

@@ -36,6 +36,19 @@ bool tc_gemm_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
                              int rows, void* q, KvView kv, const RowMeta* meta, const float2* rope, int max_ctx,
                              const RowScale& rs, cudaStream_t st);
 
+// The pair kernel (gemm_wide.cu) for many activation rows.  tc_wide_bind names the scratch (fp32) and the flags (zeroed,
+// kWideFlags ints) that cut tiles go through; the fused forms need them.  tc_gemm_launch takes the plain form by itself.
+constexpr int kWideFrom = 128;           // rows above this take it
+constexpr int kWideFlags = 256;
+void tc_wide_init(TcGemm* g);
+void tc_wide_bind(TcGemm* g, float* scratch, size_t scratch_floats, int* flags);
+bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out, int in, int rows, float* P, size_t p_floats,
+                    int* splits, size_t* split_stride, cudaStream_t st);
+bool tc_wide_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_up, int f, int in, int rows, void* act, const RowScale& rs,
+                           cudaStream_t st);
+bool tc_wide_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, const void* wv, int n_heads, int dh, int in, int rows, void* q,
+                             const RopeGroups& gr, int max_ctx, const RowScale& rs, cudaStream_t st);
+
 // Asks for the head of every gate / up weight tile (about budget_bytes in all: the first K blocks of all rows of both
 // matrices) to be brought into L2.  A plain launch for a side stream: meant to run while the main stream's kernels leave
 // HBM idle.  Returns false, nothing launched, if the two matrices cannot be described by one tensor map.
