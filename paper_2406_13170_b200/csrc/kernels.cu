@@ -381,32 +381,35 @@ void launch_qkv_rope(PartialView P, const RowMeta* meta, const float2* rope, voi
 }
 
 // --------------------------------------------------------------------------------------------
-// Tree attention, split over the KV axis (flash-decoding form), with the tree as a bitmask.
-// Grid (head, split, row block of 64).  Slots below meta->base are visible to every row;
-// slot base + m is visible to row r iff bit m of mask[r] is set.
+// Tree attention on CUDA cores (fp32 caches), split over the KV axis (flash-decoding form), with the tree as a bitmask.
+// Grid (head, split, row block of 16).  Slots below meta->base are visible to every row; slot base + m is visible to row r iff
+// bit m of mask[r] is set.  Sixteen threads share a row: four keys of a tile each for the scores, a sixteenth of the head
+// dimension each for the output.  Bound: latency (one L2 round trip per 64 keys, all of a tile's loads in flight together).
+// A single split writes the final rows itself.  At 16 rows and 70 keys 5.7 us; 64-row blocks (mostly empty) with 32-key tiles
+// fetched four bytes at a time, and a merge launch always, took 15.
 // --------------------------------------------------------------------------------------------
-constexpr int kAttRows = 64;     // query rows per block
-constexpr int kAttTile = 32;     // keys per inner tile
+constexpr int kAttRows = 16;     // query rows per block
+constexpr int kAttTile = 64;     // keys per inner tile
 constexpr int kAttThreads = 256;
 
 template <typename T, int DH>
 __global__ void __launch_bounds__(kAttThreads)
 tree_attn_kernel(const T* __restrict__ q, const T* __restrict__ kc, const T* __restrict__ vc,
-                 const RowMeta* __restrict__ meta, float* __restrict__ po, float* __restrict__ pml,
+                 const RowMeta* __restrict__ meta, float* __restrict__ po, float* __restrict__ pml, T* __restrict__ out,
                  int rows_cap, int n_heads, int max_ctx) {
   pdl_wait();
   pdl_launch_dependents();
   constexpr int QS = DH + 4;                       // padded row strides (bank-conflict free float4 reads)
-  constexpr int SEG = DH / 4;                      // output dims owned by one thread
+  constexpr int SEG = DH / 16;                     // output dims owned by one thread
+  constexpr int KEYS = kAttTile / 16;              // keys of a tile per thread
   extern __shared__ __align__(16) float sm[];
-  float* Qs = sm;                                  // [64][QS]
-  float* Ks = Qs + kAttRows * QS;                  // [32][QS]
-  float* Vs = Ks + kAttTile * QS;                  // [32][DH]
-  float* Ss = Vs + kAttTile * DH;                  // [64][33]
-  const int h = blockIdx.x, split = blockIdx.y, rb = blockIdx.z;
-  const int tid = threadIdx.x;
-  const int r = tid >> 2, qd = tid & 3;
-  const int rg = rb * kAttRows + r;                // global row
+  float* Qs = sm;                                  // [16][QS]
+  float* Ks = Qs + kAttRows * QS;                  // [64][QS]
+  float* Vs = Ks + kAttTile * QS;                  // [64][DH]
+  float* Ss = Vs + kAttTile * DH;                  // [16][65]
+  const int h = blockIdx.x, split = blockIdx.y, tid = threadIdx.x;
+  const int r = tid >> 4, l16 = tid & 15;
+  const int rg = blockIdx.z * kAttRows + r;        // global row
   const int base = meta->base, n_rows = meta->n_rows;
   const int d = n_heads * DH;
   const int total = base + n_rows;                 // slots that can be visible
@@ -419,10 +422,10 @@ tree_attn_kernel(const T* __restrict__ q, const T* __restrict__ kc, const T* __r
   const bool live = rg < n_rows;
   u64 m0 = 0, m1 = 0;
   if (live) { m0 = meta->mask[rg][0]; m1 = meta->mask[rg][1]; }
-  for (int i = tid; i < kAttRows * DH; i += kAttThreads) {
-    const int rr = i / DH, c = i - rr * DH;
-    const int g = rb * kAttRows + rr;
-    Qs[rr * QS + c] = g < rows_cap ? to_f(q[(size_t)g * d + h * DH + c]) : 0.f;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int i = tid; i < kAttRows * DH / 4; i += kAttThreads) {
+    const int rr = i / (DH / 4), c = (i - rr * (DH / 4)) * 4, g = blockIdx.z * kAttRows + rr;
+    store4(Qs + rr * QS + c, g < rows_cap ? load4(q + (size_t)g * d + h * DH + c) : zero);
   }
   float acc[SEG];
 #pragma unroll
@@ -432,87 +435,89 @@ tree_attn_kernel(const T* __restrict__ q, const T* __restrict__ kc, const T* __r
   const T* kh = kc + (size_t)h * max_ctx * DH;
   const T* vh = vc + (size_t)h * max_ctx * DH;
   for (int t0 = s_lo; t0 < s_hi; t0 += kAttTile) {
-    __syncthreads();
-    for (int i = tid; i < kAttTile * DH; i += kAttThreads) {
-      const int j = i / DH, c = i - j * DH;
-      const int s = t0 + j;
-      float kvv = 0.f, vvv = 0.f;
-      if (s < s_hi) { kvv = to_f(kh[(size_t)s * DH + c]); vvv = to_f(vh[(size_t)s * DH + c]); }
-      Ks[j * QS + c] = kvv;
-      Vs[j * DH + c] = vvv;
+    constexpr int PER = kAttTile * DH / 4 / kAttThreads;
+    float4 kr[PER], vr[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int e = tid + i * kAttThreads, j = e / (DH / 4), c = (e - j * (DH / 4)) * 4;
+      const bool in_range = t0 + j < s_hi;
+      kr[i] = in_range ? load4(kh + (size_t)(t0 + j) * DH + c) : zero;
+      vr[i] = in_range ? load4(vh + (size_t)(t0 + j) * DH + c) : zero;
+    }
+    __syncthreads();                               // the previous tile has been read
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int e = tid + i * kAttThreads, j = e / (DH / 4), c = (e - j * (DH / 4)) * 4;
+      store4(Ks + j * QS + c, kr[i]);
+      store4(Vs + j * DH + c, vr[i]);
     }
     __syncthreads();
-    float sc[kAttTile / 4];
+    float sc[KEYS];
+#pragma unroll
+    for (int jj = 0; jj < KEYS; ++jj) sc[jj] = 0.f;
+    const float4* qa = reinterpret_cast<const float4*>(Qs + r * QS);
+#pragma unroll 4
+    for (int c = 0; c < DH / 4; ++c) {
+      const float4 a = qa[c];
+#pragma unroll
+      for (int jj = 0; jj < KEYS; ++jj) {
+        const float4 b = *reinterpret_cast<const float4*>(Ks + (jj * 16 + l16) * QS + 4 * c);
+        sc[jj] += a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w;
+      }
+    }
     float tmax = -INFINITY;
 #pragma unroll
-    for (int jj = 0; jj < kAttTile / 4; ++jj) {
-      const int j = jj * 4 + qd;
-      const int s = t0 + j;
+    for (int jj = 0; jj < KEYS; ++jj) {
+      const int s = t0 + jj * 16 + l16;
       bool vis = live && s < s_hi;
       if (vis && s >= base) {
         const int m = s - base;
         vis = m < 64 ? ((m0 >> m) & 1ull) : ((m1 >> (m - 64)) & 1ull);
       }
-      float dot = -INFINITY;
-      if (vis) {
-        const float4* qa = reinterpret_cast<const float4*>(Qs + r * QS);
-        const float4* ka = reinterpret_cast<const float4*>(Ks + j * QS);
-        dot = 0.f;
-#pragma unroll 8
-        for (int c = 0; c < DH / 4; ++c) {
-          const float4 a = qa[c], b = ka[c];
-          dot += a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w;
-        }
-        dot *= scale;
-        tmax = fmaxf(tmax, dot);
-      }
-      sc[jj] = dot;
+      sc[jj] = vis ? sc[jj] * scale : -INFINITY;
+      tmax = fmaxf(tmax, sc[jj]);
     }
-    tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 1));
-    tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, 2));
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
     const float mnew = fmaxf(mrun, tmax);
-    float corr = 1.f, psum = 0.f;
-    if (mnew == -INFINITY) {                       // nothing visible yet for this row
+    const bool any = mnew != -INFINITY;            // else nothing is visible yet for this row
+    const float corr = any ? expf(mrun - mnew) : 1.f;      // exp(-inf) = 0 on the first visible tile
+    float psum = 0.f;
 #pragma unroll
-      for (int jj = 0; jj < kAttTile / 4; ++jj) Ss[r * (kAttTile + 1) + jj * 4 + qd] = 0.f;
-    } else {
-      corr = expf(mrun - mnew);                    // exp(-inf) = 0 on the first visible tile
-#pragma unroll
-      for (int jj = 0; jj < kAttTile / 4; ++jj) {
-        const float p = sc[jj] == -INFINITY ? 0.f : expf(sc[jj] - mnew);
-        Ss[r * (kAttTile + 1) + jj * 4 + qd] = p;
-        psum += p;
-      }
+    for (int jj = 0; jj < KEYS; ++jj) {
+      const float p = any && sc[jj] != -INFINITY ? expf(sc[jj] - mnew) : 0.f;
+      Ss[r * (kAttTile + 1) + jj * 16 + l16] = p;
+      psum += p;
     }
-    psum += __shfl_xor_sync(0xffffffffu, psum, 1);
-    psum += __shfl_xor_sync(0xffffffffu, psum, 2);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, o);
     lrun = lrun * corr + psum;
     mrun = mnew;
-    __syncwarp();
+    __syncwarp();                                  // a row's sixteen threads sit in one warp
 #pragma unroll
     for (int i = 0; i < SEG; ++i) acc[i] *= corr;
+#pragma unroll 4
     for (int j = 0; j < kAttTile; ++j) {
       const float p = Ss[r * (kAttTile + 1) + j];
-      if (p != 0.f) {
-        const float4* va = reinterpret_cast<const float4*>(Vs + j * DH + qd * SEG);
 #pragma unroll
-        for (int c = 0; c < SEG / 4; ++c) {
-          const float4 v = va[c];
-          acc[c * 4 + 0] += p * v.x; acc[c * 4 + 1] += p * v.y;
-          acc[c * 4 + 2] += p * v.z; acc[c * 4 + 3] += p * v.w;
-        }
+      for (int c = 0; c < SEG; c += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(Vs + j * DH + l16 * SEG + c);
+        acc[c] += p * v.x; acc[c + 1] += p * v.y; acc[c + 2] += p * v.z; acc[c + 3] += p * v.w;
       }
     }
-    __syncwarp();
   }
-  if (rg < rows_cap) {
-    const size_t o = (((size_t)split * n_heads + h) * rows_cap + rg);
-    float4* dst = reinterpret_cast<float4*>(po + o * DH + qd * SEG);
+  if (rg >= rows_cap) return;
+  if (out != nullptr) {
+    const float inv = lrun > 0.f ? 1.0f / lrun : 0.f;
 #pragma unroll
-    for (int c = 0; c < SEG / 4; ++c)
-      dst[c] = make_float4(acc[c * 4], acc[c * 4 + 1], acc[c * 4 + 2], acc[c * 4 + 3]);
-    if (qd == 0) { pml[o * 2] = mrun; pml[o * 2 + 1] = lrun; }
+    for (int c = 0; c < SEG; c += 4)
+      store4(out + (size_t)rg * d + h * DH + l16 * SEG + c, make_float4(acc[c] * inv, acc[c + 1] * inv, acc[c + 2] * inv, acc[c + 3] * inv));
+    return;
   }
+  const size_t o = (((size_t)split * n_heads + h) * rows_cap + rg);
+#pragma unroll
+  for (int c = 0; c < SEG; c += 4) store4(po + o * DH + l16 * SEG + c, make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]));
+  if (l16 == 0) { pml[o * 2] = mrun; pml[o * 2 + 1] = lrun; }
 }
 
 template <typename T>
@@ -569,14 +574,13 @@ __global__ void attn_combine_kernel(const float* __restrict__ po, const float* _
 template <typename T, int DH>
 static void tree_attention_t(const void* q, KvView kv, const RowMeta* meta, AttnScratch sc, void* out,
                              int rows, int n_heads, int max_ctx, int splits, cudaStream_t st) {
-  const size_t smem = sizeof(float) * (kAttRows * (DH + 4) + kAttTile * (DH + 4) + kAttTile * DH +
-                                       kAttRows * (kAttTile + 1));
+  const size_t smem = sizeof(float) * (kAttRows * (DH + 4) + kAttTile * (DH + 4) + kAttTile * DH + kAttRows * (kAttTile + 1));
   cudaFuncSetAttribute(tree_attn_kernel<T, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  dim3 grid(n_heads, splits, (rows + kAttRows - 1) / kAttRows);
-  launch_pdl(tree_attn_kernel<T, DH>, dim3(grid), dim3(kAttThreads), smem, st, (const T*)q, (const T*)kv.k, (const T*)kv.v, meta,
-                                                          sc.o, sc.ml, rows, n_heads, max_ctx);
-  launch_pdl(attn_combine_kernel<T>, dim3(dim3(rows, n_heads)), dim3(DH < 128 ? 64 : 128), 0, st, sc.o, sc.ml, (T*)out, splits, rows,
-                                                                              n_heads, DH, 0);
+  launch_pdl(tree_attn_kernel<T, DH>, dim3(n_heads, splits, (rows + kAttRows - 1) / kAttRows), dim3(kAttThreads), smem, st, (const T*)q,
+             (const T*)kv.k, (const T*)kv.v, meta, sc.o, sc.ml, splits == 1 ? (T*)out : (T*)nullptr, rows, n_heads, max_ctx);
+  if (splits > 1)
+    launch_pdl(attn_combine_kernel<T>, dim3(rows, n_heads), dim3(DH < 128 ? 64 : 128), 0, st, sc.o, sc.ml, (T*)out, splits, rows,
+               n_heads, DH, 0);
 }
 
 void launch_attn_combine(AttnScratch sc, void* out, int dtype, int splits, int rows, int n_heads, int head_dim,
@@ -636,23 +640,25 @@ void launch_swiglu(PartialView P, void* act, int dtype, int rows, int f, cudaStr
 }
 
 // --------------------------------------------------------------------------------------------
-// Plain projection kernel: one warp per output feature, 128-bit weight loads, fp32 accumulate.
-// Used for fp32 models, for shapes the tensor-core kernel does not cover, and as its A/B check.
+// Plain projection kernel, fp32 accumulate: fp32 models, shapes the tensor-core kernel does not cover, and its A/B check.
+// Grid (8 * O features, weight matrix, R rows).  A warp owns O features and all R rows of its block: weights straight to
+// registers, each lane 32 bytes of 1 KB of the row, fetched before the dependency wait and one chunk ahead after it;
+// activations through shared memory (cp.async, two buffers), so the block's eight warps read them from L2 once.
+// Bound: latency at the sizes fp32 models are run at (16 rows, 256 columns: 2.7 us of the chain; with one launch per weight
+// matrix, activations read by every warp for itself and weights again for every eight rows: 7.3 us a launch).
 // --------------------------------------------------------------------------------------------
 template <typename T> struct Vec16;
 template <> struct Vec16<float> { static constexpr int N = 4; };
 template <> struct Vec16<bf16> { static constexpr int N = 8; };
 
 template <typename T>
-__device__ __forceinline__ void load16(const T* p, float* out);
+__device__ __forceinline__ void unpack16(const uint4& v, float* out);
 template <>
-__device__ __forceinline__ void load16<float>(const float* p, float* out) {
-  const float4 v = *reinterpret_cast<const float4*>(p);
-  out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
+__device__ __forceinline__ void unpack16<float>(const uint4& v, float* out) {
+  out[0] = __uint_as_float(v.x); out[1] = __uint_as_float(v.y); out[2] = __uint_as_float(v.z); out[3] = __uint_as_float(v.w);
 }
 template <>
-__device__ __forceinline__ void load16<bf16>(const bf16* p, float* out) {
-  const uint4 v = *reinterpret_cast<const uint4*>(p);
+__device__ __forceinline__ void unpack16<bf16>(const uint4& v, float* out) {
   const unsigned w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -660,51 +666,117 @@ __device__ __forceinline__ void load16<bf16>(const bf16* p, float* out) {
     out[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
   }
 }
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool live) {      // zeros where !live
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(live ? 16 : 0)
+               : "memory");
+}
 
-template <typename T, int R>
-__global__ void __launch_bounds__(256)
-gemm_generic_kernel(const T* __restrict__ X, int ldx, const T* __restrict__ W, int out, int in,
-                    float* __restrict__ P, int ldp, int col_off, int rows) {
-  pdl_wait();
+struct GemmSegs { GemmSeg s[kMaxK]; };
+constexpr int kPlainThreads = 256;
+constexpr int kPlainChunk = 1024;        // bytes of a row per step: two 16-byte loads per lane
+
+template <typename T, int R, int O>
+__global__ void __launch_bounds__(kPlainThreads)
+gemm_generic_kernel(const T* __restrict__ X, int ldx, const __grid_constant__ GemmSegs segs, int out, int in, float* __restrict__ P, int ldp, int rows) {
   pdl_launch_dependents();
-  constexpr int V = Vec16<T>::N;
-  const int o = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (o >= out) return;
-  const T* w = W + (size_t)o * in;
-  for (int r0 = 0; r0 < rows; r0 += R) {
-    float acc[R];
+  constexpr int V = Vec16<T>::N, KC = kPlainChunk / (int)sizeof(T);
+  __shared__ __align__(16) uint4 xs[2][R][kPlainChunk / 16];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int o0 = (blockIdx.x * (kPlainThreads / 32) + warp) * O, r0 = blockIdx.z * R;
+  const T* W = (const T*)segs.s[blockIdx.y].w;
+  const int chunks = (in + KC - 1) / KC;
+  uint4 w[O][2];
+  auto load_w = [&](int c) {
 #pragma unroll
-    for (int i = 0; i < R; ++i) acc[i] = 0.f;
-    for (int k = lane * V; k < in; k += 32 * V) {
-      float wv[V];
-      load16<T>(w + k, wv);
+    for (int i = 0; i < O; ++i)
 #pragma unroll
-      for (int i = 0; i < R; ++i) {
-        if (r0 + i < rows) {
-          float xv[V];
-          load16<T>(X + (size_t)(r0 + i) * ldx + k, xv);
+      for (int v = 0; v < 2; ++v) {
+        const int k = c * KC + (v * 32 + lane) * V;
+        w[i][v] = make_uint4(0u, 0u, 0u, 0u);
+        if (o0 + i < out && k < in) w[i][v] = *reinterpret_cast<const uint4*>(W + (size_t)(o0 + i) * in + k);
+      }
+  };
+  auto load_x = [&](int c) {
+    for (int i = threadIdx.x; i < R * (kPlainChunk / 16); i += kPlainThreads) {
+      const int r = i / (kPlainChunk / 16), j = i - r * (kPlainChunk / 16), k = c * KC + j * V;
+      const bool live = r0 + r < rows && k < in;
+      cp_async16(&xs[c & 1][r][j], live ? X + (size_t)(r0 + r) * ldx + k : X, live);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  load_w(0);
+  pdl_wait();
+  load_x(0);
+  float acc[O][R];
 #pragma unroll
-          for (int e = 0; e < V; ++e) acc[i] += wv[e] * xv[e];
+  for (int i = 0; i < O; ++i)
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[i][r] = 0.f;
+  for (int c = 0; c < chunks; ++c) {
+    float wv[O][2][V];
+#pragma unroll
+    for (int i = 0; i < O; ++i)
+#pragma unroll
+      for (int v = 0; v < 2; ++v) unpack16<T>(w[i][v], wv[i][v]);
+    if (c + 1 < chunks) {
+      load_x(c + 1);
+      load_w(c + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        float xv[V];
+        unpack16<T>(xs[c & 1][r][v * 32 + lane], xv);
+#pragma unroll
+        for (int i = 0; i < O; ++i)
+#pragma unroll
+          for (int e = 0; e < V; ++e) acc[i][r] += wv[i][v][e] * xv[e];
+      }
+    __syncthreads();
+  }
+  // sums over the lanes: at every step a lane keeps half of its rows and hands the other half to its partner
+#pragma unroll
+  for (int i = 0; i < O; ++i) {
+    int row = 0;
+#pragma unroll
+    for (int h = R / 2, m = 16; m > 0; h >>= 1, m >>= 1) {
+      if (h > 0) {
+        const bool up = (lane & m) != 0;
+        row += up ? h : 0;
+#pragma unroll
+        for (int r = 0; r < h; ++r) {
+          const float give = up ? acc[i][r] : acc[i][r + h], keep = up ? acc[i][r + h] : acc[i][r];
+          acc[i][r] = keep + __shfl_xor_sync(0xffffffffu, give, m);
         }
+      } else {
+        acc[i][0] += __shfl_xor_sync(0xffffffffu, acc[i][0], m);
       }
     }
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-      float v = acc[i];
-      for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-      if (lane == 0 && r0 + i < rows) P[(size_t)(r0 + i) * ldp + col_off + o] = v;
-    }
+    constexpr int same = 32 / R;                       // lanes that end up with the same row
+    if (lane % same == 0 && r0 + row < rows && o0 + i < out) P[(size_t)(r0 + row) * ldp + blockIdx.y * out + o0 + i] = acc[i][0];
   }
 }
 
+// R = 4 for the drafting heads' few rows, else 16; two features a warp (half of the shared-memory reads) once one feature a warp
+// gives more than two blocks per SM.
 void launch_gemm_generic(const void* x, int ldx, const GemmSeg* segs, int n_seg, int out, int in, float* P,
                          int ldp, int rows, int dtype, cudaStream_t st) {
+  GemmSegs gs;
+  for (int s = 0; s < kMaxK; ++s) gs.s[s].w = s < n_seg ? segs[s].w : nullptr;
   const int blocks = (out + 7) / 8;
-  for (int s = 0; s < n_seg; ++s) {
-    AMPH_DISPATCH(dtype, launch_pdl(gemm_generic_kernel<T, 8>, dim3(blocks), dim3(256), 0, st, 
-                             (const T*)x, ldx, (const T*)segs[s].w, out, in, P, ldp, s * out, rows));
-  }
+  auto run = [&](auto kernel, int R, int O, auto* X) {
+    launch_pdl(kernel, dim3((out + 8 * O - 1) / (8 * O), n_seg, (rows + R - 1) / R), dim3(kPlainThreads), 0, st, X, ldx, gs, out, in, P, ldp,
+               rows);
+  };
+  AMPH_DISPATCH(dtype, const T* X = (const T*)x;
+                if (rows <= 4) run(gemm_generic_kernel<T, 4, 1>, 4, 1, X);
+                else if ((long long)blocks * n_seg * ((rows + 15) / 16) <= 296) run(gemm_generic_kernel<T, 16, 1>, 16, 1, X);
+                else run(gemm_generic_kernel<T, 16, 2>, 16, 2, X));
 }
 
 // --------------------------------------------------------------------------------------------
