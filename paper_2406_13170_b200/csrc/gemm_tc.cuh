@@ -38,7 +38,7 @@ bool tc_gemm_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
 
 // The pair kernel (gemm_wide.cu) for many activation rows.  tc_wide_bind names the scratch (fp32) and the flags (zeroed,
 // kWideFlags ints) that cut tiles go through; the fused forms need them.  tc_gemm_launch takes the plain form by itself.
-constexpr int kWideFrom = 128;           // rows above this take it
+constexpr int kWideFrom = 64;            // rows above this take it
 constexpr int kWideFlags = 256;
 void tc_wide_init(TcGemm* g);
 void tc_wide_bind(TcGemm* g, float* scratch, size_t scratch_floats, int* flags);

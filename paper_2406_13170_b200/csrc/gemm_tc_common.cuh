@@ -147,41 +147,24 @@ struct TcGemm {
     return &(rope_cache[key] = m);
   }
 
-  // Forms of the pair kernel (gemm_wide.cu): a box is 128 rows of one K block, 16 rows of one kind and the 16 rows they are
-  // combined with in turn.  Gate / up: (column, 16 rows, matrix, group of 16 rows).
-  const CUtensorMap* get_wide_pair(const void* lo, const void* hi, int rows, int cols) {
-    auto key = std::make_tuple(lo, hi, rows, cols, -1);
+  // The same for the pair kernel (gemm_wide.cu), as (column, row, matrix, K block): per K block, 64 rows of the lower matrix
+  // are followed by 64 of the upper one.
+  const CUtensorMap* get_wide_pair(const void* lo, const void* hi, int rows, int cols, int box_kb) {
+    auto key = std::make_tuple(lo, hi, rows, cols, -box_kb);
     auto it = pair_cache.find(key);
     if (it != pair_cache.end()) return &it->second;
     const uint64_t gap = (uint64_t)((const char*)hi - (const char*)lo);
     if (gap == 0 || (gap & 15) || gap >= (1ull << 40)) return nullptr;
     CUtensorMap m;
-    const cuuint64_t dims[4] = {(cuuint64_t)cols, 16, 2, (cuuint64_t)rows / 16};
-    const cuuint64_t strides[3] = {(cuuint64_t)cols * 2, (cuuint64_t)gap, (cuuint64_t)cols * 32};
-    const cuuint32_t box[4] = {(cuuint32_t)tc::kTileK, 16, 2, 4};
+    const cuuint64_t dims[4] = {(cuuint64_t)tc::kTileK, (cuuint64_t)rows, 2, (cuuint64_t)cols / tc::kTileK};
+    const cuuint64_t strides[3] = {(cuuint64_t)cols * 2, (cuuint64_t)gap, (cuuint64_t)tc::kTileK * 2};
+    const cuuint32_t box[4] = {(cuuint32_t)tc::kTileK, (cuuint32_t)(tc::kTileM / 2), 2, (cuuint32_t)box_kb};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     const CUresult r = encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(lo), dims, strides, box, estr,
                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return nullptr;
     return &(pair_cache[key] = m);
-  }
-  // q / k / v: (column, 16 rows, half of the head, group of 16 pairs, head); a box is one head of 128 rows or two of 64.
-  const CUtensorMap* get_wide_rope(const void* ptr, int heads, int dh, int cols) {
-    auto key = std::make_tuple(ptr, heads, cols, dh, -1);
-    auto it = rope_cache.find(key);
-    if (it != rope_cache.end()) return &it->second;
-    CUtensorMap m;
-    const cuuint64_t pitch = (cuuint64_t)cols * 2;
-    const cuuint64_t dims[5] = {(cuuint64_t)cols, 16, 2, (cuuint64_t)dh / 32, (cuuint64_t)heads};
-    const cuuint64_t strides[4] = {pitch, pitch * (dh / 2), pitch * 16, pitch * dh};
-    const cuuint32_t box[5] = {(cuuint32_t)tc::kTileK, 16, 2, (cuuint32_t)dh / 32, (cuuint32_t)(tc::kTileM / dh)};
-    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    const CUresult r = encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(ptr), dims, strides, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return nullptr;
-    return &(rope_cache[key] = m);
   }
 
   // pair kernel: CTA pairs that run at a time (0: not available), scratch and flags of cut tiles

@@ -3,9 +3,10 @@
 // A cluster of two CTAs owns 256 weight rows and a block of up to 256 activation rows: one tcgen05.mma.cta_group::2 (M = 256,
 // N <= 256) per 16 columns of K.  Each CTA stages its own 128 weight rows and HALF of the activation rows: 32 KB per 64
 // columns of K at N = 256, i.e. 64 bytes of L2 -> SM traffic per clock of MMA, against 80 with one CTA per 128 weight rows and
-// 512 activation rows (which made L2 the bound).  With 257..512 rows two neighbouring pairs take the two row blocks of the
-// same weights at the same time, so weights still cross HBM once.  Tensor memory holds two accumulators: the epilogue of
-// one piece of work runs under the main loop of the next.
+// 512 activation rows (which made L2 the bound).  Stages hold two K blocks, one copy of up to 32 KB per operand: an SM retires
+// about one copy per 400 clocks, so with 16 KB copies the main loop ran at 790 clocks per K block instead of the MMA's 512.
+// With 257..512 rows two neighbouring pairs take the two row blocks of the same weights at the same time, so weights still
+// cross HBM once.  Tensor memory holds two accumulators: the epilogue of one piece of work runs under the next main loop.
 //
 // Balance: a launch is `tiles` x K work.  Cut tile by tile, 48 tiles (q / k / v at d = 4096) keep 65 % of the 74 pairs busy and
 // 86 (gate / up) take two waves of 58 %.  So group g of pairs (a pair per row block) takes the g-th of equal ranges of the
@@ -15,7 +16,7 @@
 // against the launch order, so a pair only ever waits for pairs that became resident before it; the wait is bounded all the
 // same.  Where the consumer adds split-K sums anyway (output and down projections) the K ranges are cut evenly per tile.
 //
-// Warp roles: 0 = TMA producer, 1 = MMA issuer (of the even CTA), 2-9 = epilogue (two warps per TMEM lane quarter).
+// Warp roles: 0 = TMA producer, 1 = MMA issuer (of the even CTA), 2-17 = epilogue.
 #include "gemm_tc_common.cuh"
 
 namespace amph {
@@ -24,9 +25,9 @@ using namespace tc;
 
 namespace {
 
-constexpr int kWideThreads = 320;
-constexpr int kEpiThreads = 256;
-constexpr int kUnitKb = 2;            // K blocks per unit of work: ranges are cut at multiples of 128 columns
+constexpr int kEpiThreads = 512;      // four warps per TMEM lane quarter
+constexpr int kWideThreads = 64 + kEpiThreads;
+constexpr int kUnitKb = 2;            // K blocks per pipeline stage = unit of work: ranges are cut at multiples of 128 columns
 constexpr int kMaxWideRows = 512;
 constexpr int kMaxStages = 8;
 
@@ -48,7 +49,7 @@ struct WideParams {
   float* P;                 // PLAIN: P[split][row][feature]
   size_t split_stride;
   int ld;
-  float* scratch;           // [pair][cta][chunk of 16 rows][row quad][128 features] float4: partial sums of a pair's first segment
+  float* scratch;           // [pair][cta][quad of rows][128 features] float4: partial sums of a pair's first segment
   int* flags;               // [pair][cta]; zero between launches (whoever consumes a flag lowers it)
   __nv_bfloat16* act;       // SWIGLU
   int f, up_first;
@@ -60,20 +61,18 @@ struct WideParams {
   unsigned long long wait_limit_ns;
 };
 
-struct Segment { int tile, kb0, kb1; };
+struct Segment { int tile, u0, u1; };     // units [u0, u1) of a tile's K range
 
 // The segments of one group's range of work units, in order.
 struct SegIter {
-  int u, end, upt, kblocks;
+  int u, end, upt;
   __device__ bool next(Segment& s) {
     if (u >= end) return false;
-    const int t = u / upt, a = u - t * upt;
-    int e = end - t * upt;
-    if (e > upt) e = upt;
+    const int t = u / upt;
     s.tile = t;
-    s.kb0 = a * kUnitKb;
-    s.kb1 = e * kUnitKb < kblocks ? e * kUnitKb : kblocks;
-    u = t * upt + e;
+    s.u0 = u - t * upt;
+    s.u1 = end - t * upt < upt ? end - t * upt : upt;
+    u = t * upt + s.u1;
     return true;
   }
 };
@@ -122,12 +121,6 @@ __device__ __forceinline__ void tma_pair_4d(void* dst, const CUtensorMap* map, i
       ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar), "l"(pol)
       : "memory");
 }
-__device__ __forceinline__ void tma_pair_5d(void* dst, const CUtensorMap* map, int x, int y, int z, int w, int v, uint32_t bar, uint64_t pol) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4, %5, %6}], [%7], %8;"
-      ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(v), "r"(bar), "l"(pol)
-      : "memory");
-}
 __device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
@@ -141,28 +134,24 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
-        "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-
-// Rows of a tile, in both fused forms: 16 rows of one kind, then the 16 rows they are combined with (gate / up, or the two
-// members of 16 rotation pairs), four times over.  Lanes l and l + 16 of an epilogue warp then hold the two operands of one
-// output feature for 16 activation rows; after one exchange lane l < 16 has both for the first eight rows, lane l + 16 for
-// the other eight, and half a warp writes 16 neighbouring features (32 bytes) of a row.
-__device__ __forceinline__ void pair_up(const float* v, int lane, float* first, float* second) {
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\ttcgen05.wait::ld.sync.aligned;"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const float got = __shfl_xor_sync(0xffffffffu, lane < 16 ? v[8 + j] : v[j], 16);
-    first[j] = lane < 16 ? v[j] : got;
-    second[j] = lane < 16 ? got : v[8 + j];
-  }
+  for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(r[e]);
 }
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
+
+// The fused forms combine two features of a tile that sit in different TMEM lanes (gate / up, or the members of a rotation
+// pair), so a batch of rows goes through shared memory in fp32: a warp parks its 32 features x 8 rows, then every thread
+// finishes four neighbouring outputs (pairs) of one row.  Bound: instruction issue; combining them by shuffles between the
+// lanes that hold them took three times the instructions (about 300 per warp and 16 rows; 8-11 us per 256 rows).
+constexpr int kChunk = 8;                               // activation rows a warp takes from tensor memory at a time
+constexpr int kBatch = kEpiThreads / 128 * kChunk;      // rows of a batch
+constexpr int kPark = kBatch * kTileM * 4;              // bytes
 
 template <int EPI>
 __global__ void __launch_bounds__(kWideThreads, 1)
@@ -170,6 +159,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ float inv_s[EPI == WIDE_PLAIN ? 1 : 256];             // 1 / rms of this pair's activation rows
   __shared__ int slot_s[EPI == WIDE_ROPE ? 256 : 1];               // cache slot of a row, -1: not stored
+  __shared__ const float2* table_s[EPI == WIDE_ROPE ? 256 : 1];    // its rotary table row
   __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], accum_full[2], accum_empty[2];
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
@@ -180,11 +170,12 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   const int pair = prm.groups * prm.nrb - 1 - (int)(blockIdx.x >> 1);        // against the launch order (see above)
   const int group = pair / prm.nrb, rb = pair - group * prm.nrb;
   const int stages = prm.stages, n = prm.n;
-  const uint32_t b_tile = (uint32_t)n / 2 * 128, a_tile = kTileM * 128;
-  const uint32_t stage_bytes = a_tile + b_tile;
+  const uint32_t b_tile = (uint32_t)n / 2 * 128, a_tile = kTileM * 128;         // one K block of each operand
+  const uint32_t stage_bytes = kUnitKb * (a_tile + b_tile);
   const unsigned long long limit_ns = prm.wait_limit_ns;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  const SegIter first = {range_begin(prm, group), range_begin(prm, group + 1), prm.units_per_tile, prm.kblocks};
+  float* const park = reinterpret_cast<float*>(smem + (size_t)stages * stage_bytes);       // fused forms: [kBatch][128]
+  const SegIter first = {range_begin(prm, group), range_begin(prm, group + 1), prm.units_per_tile};
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -206,47 +197,46 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     // ---------------- TMA producer of this CTA's half of the operands
     const bool leader = elect_one();
     const uint64_t wpol = l2_evict_first_policy();
-    auto load_w = [&](int st, const Segment& s, int kb) {
+    auto load_w = [&](int st, const Segment& s, int u) {
       const int seg = s.tile / prm.tiles_per_seg, lt = s.tile - seg * prm.tiles_per_seg;
       const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), 0);
       uint8_t* dst = smem + (size_t)st * stage_bytes;
       if (rank == 0) mbar_expect_tx(&full_bar[st], 2 * stage_bytes);
-      if (EPI == WIDE_SWIGLU) tma_pair_4d(dst, &maps.w[0], kb * kTileK, 0, 0, (lt * 2 + (int)rank) * 4, bar, wpol);
-      else if (EPI == WIDE_ROPE) tma_pair_5d(dst, &maps.w[seg], kb * kTileK, 0, 0, 0, (lt * 2 + (int)rank) * kTileM / prm.dh, bar, wpol);
-      else tma_pair_3d(dst, &maps.w[seg], 0, (lt * 2 + (int)rank) * kTileM, kb, bar, wpol);
+      if (EPI == WIDE_SWIGLU) tma_pair_4d(dst, &maps.w[0], 0, (lt * 2 + (int)rank) * (kTileM / 2), 0, u * kUnitKb, bar, wpol);
+      else tma_pair_3d(dst, &maps.w[seg], 0, (lt * 2 + (int)rank) * kTileM, u * kUnitKb, bar, wpol);
     };
-    auto load_x = [&](int st, int kb) {
+    auto load_x = [&](int st, int u) {
       const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), 0);
-      tma_pair_3d(smem + (size_t)st * stage_bytes + a_tile, &maps.x, 0, rb * n + (int)rank * (n / 2), kb, bar);
+      tma_pair_3d(smem + (size_t)st * stage_bytes + kUnitKb * a_tile, &maps.x, 0, rb * n + (int)rank * (n / 2), u * kUnitKb, bar);
     };
     // weights do not depend on the kernel before: fill the ring with them, then wait, then fetch those stages' activations
     SegIter it = first;
     Segment sg;
     bool have = it.next(sg);
-    int kb = have ? sg.kb0 : 0, i = 0;
+    int u = have ? sg.u0 : 0, i = 0;
     for (; i < stages && have; ++i) {
-      if (leader) load_w(i, sg, kb);
-      if (++kb == sg.kb1) { have = it.next(sg); kb = sg.kb0; }
+      if (leader) load_w(i, sg, u);
+      if (++u == sg.u1) { have = it.next(sg); u = sg.u0; }
     }
     __syncwarp();
     pdl_wait();
     {
       SegIter bt = first;
       Segment bs;
-      bool more = bt.next(bs);
-      int bk = more ? bs.kb0 : 0;
+      bt.next(bs);
+      int bu = bs.u0;
       for (int j = 0; j < i; ++j) {
-        if (leader) load_x(j, bk);
-        if (++bk == bs.kb1) { more = bt.next(bs); bk = bs.kb0; }
+        if (leader) load_x(j, bu);
+        if (++bu == bs.u1) { bt.next(bs); bu = bs.u0; }
       }
     }
     __syncwarp();
     for (; have; ++i) {
       const int st = i % stages, round = i / stages;
       if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[st], (round & 1) ^ 1, &abort_flag, limit_ns))) break;
-      if (leader) { load_w(st, sg, kb); load_x(st, kb); }
+      if (leader) { load_w(st, sg, u); load_x(st, u); }
       __syncwarp();
-      if (++kb == sg.kb1) { have = it.next(sg); kb = sg.kb0; }
+      if (++u == sg.u1) { have = it.next(sg); u = sg.u0; }
     }
     if (abort_flag && rank == 0 && lane == 0) {          // drain: both CTAs' copies signal the even CTA's barriers
       const unsigned long long t0 = now_ns();
@@ -267,17 +257,20 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
         if (around > 0) ok = __all_sync(0xffffffffu, mbar_wait(&accum_empty[as], (around & 1) ^ 1, &abort_flag, limit_ns));
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d = tmem_d + (uint32_t)(as * n);
-        for (int kb = sg.kb0; ok && kb < sg.kb1; ++kb, ++i) {
+        for (int u = sg.u0; ok && u < sg.u1; ++u, ++i) {
           const int st = i % stages;
           ok = __all_sync(0xffffffffu, mbar_wait(&full_bar[st], (i / stages) & 1, &abort_flag, limit_ns));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          if (leader) {
+          if (leader) {                                  // K blocks past the end of K have arrived as zeros
             const uint32_t a_addr = smem_u32(smem + (size_t)st * stage_bytes);
-            const uint64_t ad = umma_desc(a_addr), bd = umma_desc(a_addr + a_tile);
 #pragma unroll
-            for (int k = 0; k < kTileK / kUmmaK; ++k)
-              umma_pair(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, kb > sg.kb0 || k > 0 ? 1u : 0u);
+            for (int kk = 0; kk < kUnitKb; ++kk) {
+              const uint64_t ad = umma_desc(a_addr + kk * a_tile), bd = umma_desc(a_addr + kUnitKb * a_tile + kk * b_tile);
+#pragma unroll
+              for (int k = 0; k < kTileK / kUmmaK; ++k)
+                umma_pair(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, u > sg.u0 || kk > 0 || k > 0 ? 1u : 0u);
+            }
             umma_commit_pair(&empty_bar[st]);
           }
           __syncwarp();
@@ -288,8 +281,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     }
   } else {
     // ---------------- epilogue
-    const int quarter = warp & 3, half = (warp - 2) >> 2, et = threadIdx.x - 64;
-    const int chunks = n / 16;                           // chunks of 16 activation rows
+    const int quarter = warp & 3, sub = (warp - 2) >> 2, et = threadIdx.x - 64;
     const int row0 = rb * n, my_rows = prm.rows - row0 < n ? prm.rows - row0 : n;
     pdl_wait();
     if constexpr (EPI != WIDE_PLAIN) {
@@ -301,10 +293,11 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
         const RowMeta* meta = prm.gr.meta[g];
         const int slot = meta->slot[rl];
         slot_s[et] = rl < meta->n_rows && slot >= 0 && slot < prm.max_ctx ? slot : -1;
+        table_s[et] = prm.gr.rope[g] + (size_t)rl * (prm.dh >> 1);
       }
     }
     epi_sync();
-    const size_t slot_quads = (size_t)chunks * 4 * kTileM;           // float4s of one CTA's partial sums
+    const size_t slot_quads = (size_t)(n / 4) * kTileM;  // float4s of one CTA's partial sums
     const int frow = quarter * 32 + lane;                // row of this CTA's tile
     float4* const scratch = reinterpret_cast<float4*>(prm.scratch) + frow;
     SegIter it = first;
@@ -314,28 +307,27 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
       bool ok = __all_sync(0xffffffffu, mbar_wait(&accum_full[as], (j >> 1) & 1, &abort_flag, limit_ns));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t t0 = tmem_d + (uint32_t)(as * n) + ((uint32_t)(quarter * 32) << 16);
-      if (prm.splits == 0 && sg.kb0 > 0) {               // not the tile's first K columns: leave the sums to the pair that has them
-        float4* dst = scratch + ((size_t)pair * 2 + rank) * slot_quads;
-        for (int c = half; c < chunks; c += 2) {
-          uint32_t v[16];
-          tmem_ld16(t0 + (uint32_t)c * 16, v);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            __stcg(dst + (size_t)(c * 4 + e) * kTileM,
-                   ok ? make_float4(__uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1]), __uint_as_float(v[4 * e + 2]), __uint_as_float(v[4 * e + 3]))
-                      : make_float4(0.f, 0.f, 0.f, 0.f));
-        }
+      auto release = [&]() {                             // this warp has read the accumulator
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&accum_empty[as]), 0));
+      };
+      if (prm.splits == 0 && sg.u0 > 0) {                // not the tile's first K columns: leave the sums to the pair that has them
+        float4* dst = scratch + ((size_t)pair * 2 + rank) * slot_quads;
+        for (int r = sub * kChunk; ok && r < my_rows; r += kBatch) {
+          float v[kChunk];
+          tmem_ld8(t0 + (uint32_t)r, v);
+          __stcg(dst + (size_t)(r / 4) * kTileM, make_float4(v[0], v[1], v[2], v[3]));
+          __stcg(dst + (size_t)(r / 4 + 1) * kTileM, make_float4(v[4], v[5], v[6], v[7]));
+        }
+        release();
         __threadfence();
         epi_sync();
         if (et == 0) asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(prm.flags + pair * 2 + rank), "r"(1) : "memory");
         continue;
       }
       int helpers = 0;                                    // groups after this one that hold the rest of the tile
-      if (prm.splits == 0 && sg.kb1 < prm.kblocks) {
+      if (prm.splits == 0 && sg.u1 < prm.units_per_tile) {
         const int tile_end = (sg.tile + 1) * prm.units_per_tile;
         while (group + 1 + helpers < prm.groups && range_begin(prm, group + 1 + helpers) < tile_end) ++helpers;
         if (et < helpers) {
@@ -351,94 +343,94 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
         epi_sync();
         ok = ok && *(volatile int*)&abort_flag == 0;
       }
+      // a wait that gave up (the error flag is raised): this piece is not written.  Uniform over the epilogue warps only behind
+      // a barrier, so the fused forms, which need barriers of their own, run through with whatever the accumulator holds.
       const int seg = sg.tile / prm.tiles_per_seg, lt = sg.tile - seg * prm.tiles_per_seg;
       const float4* src = scratch + ((size_t)(pair + prm.nrb) * 2 + rank) * slot_quads;
       const size_t next_helper = (size_t)prm.nrb * 2 * slot_quads;
-      const int gph = prm.dh >> 5, hdim = prm.dh >> 1;                    // ROPE: groups of 16 pairs per head
-      for (int c = half; c < chunks; c += 2) {
-        const int r0 = c * 16;                            // first activation row of the chunk, within this pair's block
-        if (r0 >= my_rows) break;
-        const int rl8 = r0 + (lane >> 4) * 8;             // first of the eight rows this lane finishes (fused forms)
-        // every load of the chunk is in flight before the first use
-        float4 o[4];
-        if (helpers > 0) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) o[e] = __ldcg(src + (size_t)(c * 4 + e) * kTileM);
-        }
-        float2 cs[8];
-        int g = 0, i0 = 0;
-        if constexpr (EPI == WIDE_ROPE) {
-          g = (row0 + r0) / prm.gr.rpg;                   // a group's height is a multiple of 16
-          i0 = (quarter % gph) * 16 + (lane & 15);
-          if (seg < 2) {
-            const float2* table = prm.gr.rope[g] + (size_t)(row0 + rl8 - g * prm.gr.rpg) * hdim + i0;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) cs[e] = table[e * hdim];
-          } else {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) cs[e] = make_float2(1.f, 0.f);
-          }
-        }
-        uint32_t raw[16];
-        tmem_ld16(t0 + (uint32_t)r0, raw);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        float v[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) v[e] = ok ? __uint_as_float(raw[e]) : 0.f;
+      // Sums of rows r .. r + 7 over all K; every load is in flight before the first use.
+      auto load_rows = [&](int r, float* v) {
+        float4 o0, o1;
+        const float4* p = src + (size_t)(r / 4) * kTileM;
+        if (helpers > 0) { o0 = __ldcg(p); o1 = __ldcg(p + kTileM); }
+        tmem_ld8(t0 + (uint32_t)r, v);
         for (int hp = 0; hp < helpers; ++hp) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) { v[4 * e] += o[e].x; v[4 * e + 1] += o[e].y; v[4 * e + 2] += o[e].z; v[4 * e + 3] += o[e].w; }
+          v[0] += o0.x; v[1] += o0.y; v[2] += o0.z; v[3] += o0.w;
+          v[4] += o1.x; v[5] += o1.y; v[6] += o1.z; v[7] += o1.w;
           if (hp + 1 < helpers) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) o[e] = __ldcg(src + (hp + 1) * next_helper + (size_t)(c * 4 + e) * kTileM);
+            p += next_helper;
+            o0 = __ldcg(p);
+            o1 = __ldcg(p + kTileM);
           }
         }
-        if constexpr (EPI == WIDE_PLAIN) {
-          const int split = prm.splits > 0 ? group % prm.splits : 0;
-          float* out = prm.P + (size_t)split * prm.split_stride + (size_t)(row0 + r0) * prm.ld + (size_t)sg.tile * 256 + rank * kTileM + frow;
+      };
+      if constexpr (EPI == WIDE_PLAIN) {
+        const int split = prm.splits > 0 ? group % prm.splits : 0;
+        float* out = prm.P + (size_t)split * prm.split_stride + (size_t)(row0 + sub * kChunk) * prm.ld + (size_t)sg.tile * 256 + rank * kTileM + frow;
+        for (int r = sub * kChunk; ok && r < my_rows; r += kBatch, out += (size_t)kBatch * prm.ld) {
+          float v[kChunk];
+          load_rows(r, v);
 #pragma unroll
-          for (int e = 0; e < 16; ++e)
-            if (r0 + e < my_rows) out[(size_t)e * prm.ld] = v[e];
-        } else {
-          float x0[8], x1[8];
-          pair_up(v, lane, x0, x1);
-          if constexpr (EPI == WIDE_SWIGLU) {
-            __nv_bfloat16* out = prm.act + (size_t)(row0 + rl8) * prm.f + (lt * 2 + (int)rank) * 64 + quarter * 16 + (lane & 15);
+          for (int e = 0; e < kChunk; ++e)
+            if (r + e < my_rows) out[(size_t)e * prm.ld] = v[e];
+        }
+        release();
+      } else {
+        // this thread's item of a batch: row et / 16, outputs 4 (et % 16) .. + 3 (SwiGLU) or as many rotation pairs
+        const int ir = et >> 4, p4 = (et & 15) * 4;
+        const int hdim = prm.dh >> 1;
+        const int lo_at = EPI == WIDE_ROPE ? p4 / hdim * prm.dh + p4 % hdim : p4;
+        const int hi_at = EPI == WIDE_ROPE ? lo_at + hdim : p4 + kTileM / 2;
+        const int head = EPI == WIDE_ROPE ? (lt * 2 + (int)rank) * kTileM / prm.dh + p4 / hdim : 0;
+        for (int b0 = 0; b0 < my_rows; b0 += kBatch) {
+          const int r = b0 + sub * kChunk, rl = b0 + ir;
+          float4 cs0 = make_float4(1.f, 0.f, 1.f, 0.f), cs1 = cs0;
+          if (EPI == WIDE_ROPE && seg < 2 && rl < my_rows) {
+            const float4* t = reinterpret_cast<const float4*>(table_s[rl] + p4 % hdim);
+            cs0 = t[0];
+            cs1 = t[1];
+          }
+          if (r < my_rows) {
+            float v[kChunk];
+            load_rows(r, v);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              if (rl8 + e < my_rows) {
-                const float sc = inv_s[rl8 + e];
-                const float t = (prm.up_first ? x1[e] : x0[e]) * sc, u = (prm.up_first ? x0[e] : x1[e]) * sc;
-                out[(size_t)e * prm.f] = __float2bfloat16(__fdividef(t, 1.0f + __expf(-t)) * u);
-              }
-            }
-          } else {
-            const int head = (lt * 2 + (int)rank) * kTileM / prm.dh + quarter / gph;
-            __nv_bfloat16* cache = (__nv_bfloat16*)(seg == 1 ? prm.gr.kc[g] : prm.gr.vc[g]) + (size_t)head * prm.max_ctx * prm.dh + i0;
-            __nv_bfloat16* qrow = prm.q + (size_t)(row0 + rl8) * prm.n_heads * prm.dh + head * prm.dh + i0;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              if (rl8 + e >= my_rows) continue;
-              const float sc = inv_s[rl8 + e];
-              const float lo = x0[e] * sc, hi = x1[e] * sc;
-              __nv_bfloat16* dst = qrow + (size_t)e * prm.n_heads * prm.dh;
-              if (seg > 0) {
-                const int slot = slot_s[rl8 + e];
-                dst = slot >= 0 ? cache + (size_t)slot * prm.dh : nullptr;
+            for (int e = 0; e < kChunk; ++e) park[(sub * kChunk + e) * kTileM + frow] = v[e];
+          }
+          if (b0 + kBatch >= my_rows) release();
+          epi_sync();
+          if (rl < my_rows) {
+            const float sc = inv_s[rl];
+            float4 a = *reinterpret_cast<const float4*>(park + ir * kTileM + lo_at), b = *reinterpret_cast<const float4*>(park + ir * kTileM + hi_at);
+            a.x *= sc; a.y *= sc; a.z *= sc; a.w *= sc; b.x *= sc; b.y *= sc; b.z *= sc; b.w *= sc;
+            if constexpr (EPI == WIDE_SWIGLU) {
+              if (prm.up_first) { const float4 t = a; a = b; b = t; }
+              const __nv_bfloat162 y0 = __floats2bfloat162_rn(__fdividef(a.x, 1.0f + __expf(-a.x)) * b.x, __fdividef(a.y, 1.0f + __expf(-a.y)) * b.y);
+              const __nv_bfloat162 y1 = __floats2bfloat162_rn(__fdividef(a.z, 1.0f + __expf(-a.z)) * b.z, __fdividef(a.w, 1.0f + __expf(-a.w)) * b.w);
+              *reinterpret_cast<uint2*>(prm.act + (size_t)(row0 + rl) * prm.f + (lt * 2 + (int)rank) * (kTileM / 2) + p4) =
+                  make_uint2(*reinterpret_cast<const uint32_t*>(&y0), *reinterpret_cast<const uint32_t*>(&y1));
+            } else {
+              __nv_bfloat16* dst = nullptr;
+              if (seg == 0) {
+                dst = prm.q + (size_t)(row0 + rl) * prm.n_heads * prm.dh + head * prm.dh + p4 % hdim;
+              } else if (slot_s[rl] >= 0) {
+                const int g = (row0 + rl) / prm.gr.rpg;
+                dst = (__nv_bfloat16*)(seg == 1 ? prm.gr.kc[g] : prm.gr.vc[g]) + ((size_t)head * prm.max_ctx + slot_s[rl]) * prm.dh + p4 % hdim;
               }
               if (dst != nullptr) {
-                dst[0] = __float2bfloat16(lo * cs[e].x - hi * cs[e].y);
-                dst[hdim] = __float2bfloat16(hi * cs[e].x + lo * cs[e].y);
+                const __nv_bfloat162 l0 = __floats2bfloat162_rn(a.x * cs0.x - b.x * cs0.y, a.y * cs0.z - b.y * cs0.w);
+                const __nv_bfloat162 l1 = __floats2bfloat162_rn(a.z * cs1.x - b.z * cs1.y, a.w * cs1.z - b.w * cs1.w);
+                const __nv_bfloat162 h0 = __floats2bfloat162_rn(b.x * cs0.x + a.x * cs0.y, b.y * cs0.z + a.y * cs0.w);
+                const __nv_bfloat162 h1 = __floats2bfloat162_rn(b.z * cs1.x + a.z * cs1.y, b.w * cs1.z + a.w * cs1.w);
+                *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
+                *reinterpret_cast<uint2*>(dst + hdim) = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
               }
             }
           }
+          epi_sync();                                     // the batch's rows have been read
         }
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&accum_empty[as]), 0));
       if (helpers > 0) {                                  // every thread has read the sums: lower the flags for the next launch
-        epi_sync();
+        if (EPI == WIDE_PLAIN) epi_sync();
         if (et < helpers) prm.flags[(pair + (1 + et) * prm.nrb) * 2 + rank] = 0;
       }
     }
@@ -453,18 +445,20 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   if (threadIdx.x == 0 && abort_flag && prm.err_flag) *prm.err_flag = AMPH_ERR_TIMEOUT;
 }
 
-constexpr size_t kWideSmem = 221 * 1024;                  // ring + alignment; the static part needs up to 3 KB of the 227
+constexpr size_t kWideSmem = 221 * 1024;                  // ring + alignment; the static part needs up to 5 KB of the 227
 
 // Everything of a launch that does not depend on the epilogue; false: the shape is not covered.
+template <int EPI>
 bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int rows, int splits, float* scratch_end, size_t scratch_floats,
                  WideMaps* maps, WideParams* prm) {
+  constexpr size_t out_bytes = EPI == WIDE_PLAIN ? 0 : kPark;
   if (!g || g->wide_pairs < 2 || xb < 0 || xb >= g->n_x || g->xcols[xb] != in) return false;
   if (in % kTileK || rows < 32 || rows > kMaxWideRows || rows > g->xrows[xb] || n_seg < 1 || n_seg > kMaxSeg) return false;
   memset(maps, 0, sizeof *maps);
   memset(prm, 0, sizeof *prm);
   prm->nrb = rows > 256 ? 2 : 1;
   prm->n = ((rows + prm->nrb - 1) / prm->nrb + 31) / 32 * 32;        // an M = 256 pair MMA takes N in steps of 32
-  const CUtensorMap* mx = g->get(g->xptr[xb], g->xrows[xb], in, prm->n / 2, 1);
+  const CUtensorMap* mx = g->get(g->xptr[xb], g->xrows[xb], in, prm->n / 2, kUnitKb);
   if (!mx) return false;
   maps->x = *mx;
   prm->tmem_cols = 64;
@@ -489,8 +483,8 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
     prm->scratch = scratch_end - (size_t)prm->groups * per_group;    // the buffer's end: its beginning may hold the result
   }
   prm->rows = rows;
-  const size_t stage = (size_t)kTileM * 128 + (size_t)prm->n / 2 * 128;
-  prm->stages = (int)((kWideSmem - 1024) / stage);
+  const size_t stage = kUnitKb * ((size_t)kTileM * 128 + (size_t)prm->n / 2 * 128);
+  prm->stages = (int)((kWideSmem - 1024 - out_bytes) / stage);
   if (prm->stages > kMaxStages) prm->stages = kMaxStages;
   prm->flags = g->wide_flags;
   prm->err_flag = g->err_flag;
@@ -521,7 +515,7 @@ bool wide_run(const WideMaps& maps, const WideParams& prm, cudaStream_t st) {
 
 void tc_wide_init(TcGemm* g) {
   g->wide_pairs = 0;
-  if ((size_t)g->max_smem < kWideSmem + 4 * 1024) return;
+  if ((size_t)g->max_smem < kWideSmem + 6 * 1024) return;
   int clusters = 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(g->sm_count / 2 * 2);
@@ -570,10 +564,10 @@ bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   WideParams prm;
   // a cut tile's sums go to the end of the caller's buffer, behind the result
   const size_t end = p_floats / 64 * 64, used = (stride + 63) / 64 * 64;
-  if (!wide_params(g, xb, n_seg, out / 256, in, rows, splits, P + end, end > used ? end - used : 0, &maps, &prm)) return false;
+  if (!wide_params<WIDE_PLAIN>(g, xb, n_seg, out / 256, in, rows, splits, P + end, end > used ? end - used : 0, &maps, &prm)) return false;
   for (int s = 0; s < n_seg; ++s) {
     if ((uintptr_t)w[s] & 15) return false;
-    const CUtensorMap* m = g->get(w[s], out, in, kTileM, 1);
+    const CUtensorMap* m = g->get(w[s], out, in, kTileM, kUnitKb);
     if (!m) return false;
     maps.w[s] = *m;
   }
@@ -591,9 +585,9 @@ bool tc_wide_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_
   if (!g || !g->wide_scratch || !w_gate || !w_up || !act || f % 128 || (((uintptr_t)w_gate | (uintptr_t)w_up) & 15)) return false;
   WideMaps maps;
   WideParams prm;
-  if (!wide_params(g, xb, 1, f / 128, in, rows, 0, g->wide_scratch + g->wide_scratch_floats, g->wide_scratch_floats, &maps, &prm)) return false;
+  if (!wide_params<WIDE_SWIGLU>(g, xb, 1, f / 128, in, rows, 0, g->wide_scratch + g->wide_scratch_floats, g->wide_scratch_floats, &maps, &prm)) return false;
   const bool up_first = (const char*)w_up < (const char*)w_gate;
-  const CUtensorMap* m = g->get_wide_pair(up_first ? w_up : w_gate, up_first ? w_gate : w_up, f, in);
+  const CUtensorMap* m = g->get_wide_pair(up_first ? w_up : w_gate, up_first ? w_gate : w_up, f, in, kUnitKb);
   if (!m) return false;
   maps.w[0] = *m;
   prm.act = (__nv_bfloat16*)act;
@@ -610,10 +604,10 @@ bool tc_wide_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
   if (((uintptr_t)wq | (uintptr_t)wk | (uintptr_t)wv) & 15) return false;
   WideMaps maps;
   WideParams prm;
-  if (!wide_params(g, xb, 3, d / 256, in, rows, 0, g->wide_scratch + g->wide_scratch_floats, g->wide_scratch_floats, &maps, &prm)) return false;
+  if (!wide_params<WIDE_ROPE>(g, xb, 3, d / 256, in, rows, 0, g->wide_scratch + g->wide_scratch_floats, g->wide_scratch_floats, &maps, &prm)) return false;
   const void* w[3] = {wq, wk, wv};
   for (int s = 0; s < 3; ++s) {
-    const CUtensorMap* m = g->get_wide_rope(w[s], n_heads, dh, in);
+    const CUtensorMap* m = g->get(w[s], d, in, kTileM, kUnitKb);
     if (!m) return false;
     maps.w[s] = *m;
   }
