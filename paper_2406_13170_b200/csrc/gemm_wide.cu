@@ -43,6 +43,7 @@ struct WideParams {
   int kblocks, units_per_tile;
   int splits;               // 0: equal ranges of all work (fix-up through scratch); > 0: K ranges per tile, one per group
   int groups, nrb;          // groups of nrb pairs (row blocks)
+  int snap;                 // see range_begin
   int n;                    // activation rows per MMA (a multiple of 32)
   int tmem_cols;
   int rows, stages;
@@ -83,7 +84,13 @@ __device__ __forceinline__ int range_begin(const WideParams& prm, int group) {
     const int t = group / prm.splits, s = group - t * prm.splits;
     return t * prm.units_per_tile + s * prm.units_per_tile / prm.splits;
   }
-  return (int)((long long)group * prm.tiles * prm.units_per_tile / prm.groups);
+  // a cut within prm.snap units of a tile's edge moves to the edge: the piece it would leave costs a whole epilogue (5-10 us
+  // when nothing runs above it) for a few units of 0.6 us
+  int u = (int)((long long)group * prm.tiles * prm.units_per_tile / prm.groups);
+  const int rem = u % prm.units_per_tile;
+  if (rem <= prm.snap) u -= rem;
+  else if (rem >= prm.units_per_tile - prm.snap) u += prm.units_per_tile - rem;
+  return u;
 }
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -146,9 +153,11 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 // The fused forms combine two features of a tile that sit in different TMEM lanes (gate / up, or the members of a rotation
-// pair), so a batch of rows goes through shared memory in fp32: a warp parks its 32 features x 8 rows, then every thread
-// finishes four neighbouring outputs (pairs) of one row.  Bound: instruction issue; combining them by shuffles between the
-// lanes that hold them took three times the instructions (about 300 per warp and 16 rows; 8-11 us per 256 rows).
+// pair), so a batch of rows goes through shared memory in fp32: warps park 32 features x 8 rows at a time, then every thread
+// finishes four neighbouring outputs (pairs) of a row.  Combining them by shuffles between the lanes that hold them took three
+// times the instructions (about 300 per warp and 16 rows).  A batch is 32 rows while the ring is in use; behind the pair's last
+// main loop the ring is free and all rows are one batch, because each batch costs a round trip to the partial sums in L2 and
+// two barriers (about 1 us): 256 rows in batches of 32 kept that last, exposed epilogue at 9-11 us.
 constexpr int kChunk = 8;                               // activation rows a warp takes from tensor memory at a time
 constexpr int kBatch = kEpiThreads / 128 * kChunk;      // rows of a batch
 constexpr int kPark = kBatch * kTileM * 4;              // bytes
@@ -174,7 +183,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   const uint32_t stage_bytes = kUnitKb * (a_tile + b_tile);
   const unsigned long long limit_ns = prm.wait_limit_ns;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  float* const park = reinterpret_cast<float*>(smem + (size_t)stages * stage_bytes);       // fused forms: [kBatch][128]
+  float* const small_park = reinterpret_cast<float*>(smem + (size_t)stages * stage_bytes); // fused forms: [kBatch][128]
   const SegIter first = {range_begin(prm, group), range_begin(prm, group + 1), prm.units_per_tile};
 
   if (threadIdx.x == 0) {
@@ -348,7 +357,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
       const int seg = sg.tile / prm.tiles_per_seg, lt = sg.tile - seg * prm.tiles_per_seg;
       const float4* src = scratch + ((size_t)(pair + prm.nrb) * 2 + rank) * slot_quads;
       const size_t next_helper = (size_t)prm.nrb * 2 * slot_quads;
-      // Sums of rows r .. r + 7 over all K; every load is in flight before the first use.
+      // Sums of rows r .. r + 7 over all K; the partial sums' loads are in flight before the first use.
       auto load_rows = [&](int r, float* v) {
         float4 o0, o1;
         const float4* p = src + (size_t)(r / 4) * kTileM;
@@ -376,31 +385,37 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
         }
         release();
       } else {
-        // this thread's item of a batch: row et / 16, outputs 4 (et % 16) .. + 3 (SwiGLU) or as many rotation pairs
-        const int ir = et >> 4, p4 = (et & 15) * 4;
+        // item i of a batch: row i / 16, outputs 4 (i % 16) .. + 3 (SwiGLU) or as many rotation pairs
+        const int p4 = (et & 15) * 4;
         const int hdim = prm.dh >> 1;
         const int lo_at = EPI == WIDE_ROPE ? p4 / hdim * prm.dh + p4 % hdim : p4;
         const int hi_at = EPI == WIDE_ROPE ? lo_at + hdim : p4 + kTileM / 2;
         const int head = EPI == WIDE_ROPE ? (lt * 2 + (int)rank) * kTileM / prm.dh + p4 / hdim : 0;
-        for (int b0 = 0; b0 < my_rows; b0 += kBatch) {
-          const int r = b0 + sub * kChunk, rl = b0 + ir;
-          float4 cs0 = make_float4(1.f, 0.f, 1.f, 0.f), cs1 = cs0;
-          if (EPI == WIDE_ROPE && seg < 2 && rl < my_rows) {
-            const float4* t = reinterpret_cast<const float4*>(table_s[rl] + p4 % hdim);
-            cs0 = t[0];
-            cs1 = t[1];
-          }
-          if (r < my_rows) {
+        const bool last = it.u >= it.end;                 // the ring is free
+        float* const park = last ? reinterpret_cast<float*>(smem) : small_park;
+        const int batch = last ? my_rows : kBatch;
+        for (int b0 = 0; b0 < my_rows; b0 += batch) {
+          const int b1 = b0 + batch < my_rows ? b0 + batch : my_rows;
+#pragma unroll 2
+          for (int r = b0 + sub * kChunk; r < b1; r += kBatch) {
             float v[kChunk];
             load_rows(r, v);
 #pragma unroll
-            for (int e = 0; e < kChunk; ++e) park[(sub * kChunk + e) * kTileM + frow] = v[e];
+            for (int e = 0; e < kChunk; ++e) park[(r - b0 + e) * kTileM + frow] = v[e];
           }
-          if (b0 + kBatch >= my_rows) release();
+          if (b1 == my_rows && !last) release();          // (nothing waits for the last accumulator)
           epi_sync();
-          if (rl < my_rows) {
+#pragma unroll 2
+          for (int rl = b0 + (et >> 4); rl < b1; rl += kEpiThreads / 16) {
             const float sc = inv_s[rl];
-            float4 a = *reinterpret_cast<const float4*>(park + ir * kTileM + lo_at), b = *reinterpret_cast<const float4*>(park + ir * kTileM + hi_at);
+            float4 cs0 = make_float4(1.f, 0.f, 1.f, 0.f), cs1 = cs0;
+            if (EPI == WIDE_ROPE && seg < 2) {
+              const float4* t = reinterpret_cast<const float4*>(table_s[rl] + p4 % hdim);
+              cs0 = __ldg(t);
+              cs1 = __ldg(t + 1);
+            }
+            const float* row = park + (rl - b0) * kTileM;
+            float4 a = *reinterpret_cast<const float4*>(row + lo_at), b = *reinterpret_cast<const float4*>(row + hi_at);
             a.x *= sc; a.y *= sc; a.z *= sc; a.w *= sc; b.x *= sc; b.y *= sc; b.z *= sc; b.w *= sc;
             if constexpr (EPI == WIDE_SWIGLU) {
               if (prm.up_first) { const float4 t = a; a = b; b = t; }
@@ -426,7 +441,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
               }
             }
           }
-          epi_sync();                                     // the batch's rows have been read
+          if (!last) epi_sync();                          // the batch's rows have been read
         }
       }
       if (helpers > 0) {                                  // every thread has read the sums: lower the flags for the next launch
@@ -480,6 +495,7 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
     const size_t per_group = (size_t)prm->nrb * 2 * prm->n * kTileM;
     if ((size_t)prm->groups > scratch_floats / per_group) prm->groups = (int)(scratch_floats / per_group);
     if (prm->groups < 1 || !scratch_end || !g->wide_flags || 2 * prm->groups * prm->nrb > kWideFlags) return false;
+    prm->snap = units / prm->groups / 4 < prm->units_per_tile / 8 ? units / prm->groups / 4 : prm->units_per_tile / 8;
     prm->scratch = scratch_end - (size_t)prm->groups * per_group;    // the buffer's end: its beginning may hold the result
   }
   prm->rows = rows;
