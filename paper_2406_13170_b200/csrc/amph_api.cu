@@ -534,7 +534,7 @@ bool layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, c
     KvView kvs[kMaxSeq];
     int keys = 0;
     for (int g = 0; g < ps.G; ++g) { kvs[g] = cache_of(ps.seq[g]); keys = ps.keys[g] > keys ? ps.keys[g] : keys; }
-    const int splits = attn_tc_splits(ctx->attn_tc, keys, c.n_heads, ps.rpg, l.attn_splits);
+    const int splits = attn_tc_splits(ctx->attn_tc, keys, c.n_heads, ps.rpg, ps.G, l.attn_splits);
     grouped_attn = launch_tree_attention_tc_groups(ctx->attn_tc, ctx->ws + l.q, ctx->Rcap, ps.G, kvs, ps.meta, ps.rpg, c.n_heads,
                                                    c.head_dim, c.max_ctx, splits, keys, st, ctx->ws + l.att, &ctx->state(0)->err);
     if (!grouped_attn) cudaGetLastError();
@@ -548,7 +548,7 @@ bool layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, c
     const bool last_g = g + 1 == ps.G;
     bool done = false;
     if (ctx->attn_tc) {
-      const int splits = attn_tc_splits(ctx->attn_tc, ps.keys[g], c.n_heads, ps.rpg, l.attn_splits);
+      const int splits = attn_tc_splits(ctx->attn_tc, ps.keys[g], c.n_heads, ps.rpg, 1, l.attn_splits);
       const bool merged = !(c.flags & AMPH_FLAG_SEPARATE_MERGE);
       done = launch_tree_attention_tc(ctx->attn_tc, qg, ctx->Rcap - g * ps.rpg, kv, ps.meta[g], sc, ps.rpg, c.n_heads, c.head_dim,
                                       c.max_ctx, splits, ps.keys[g], st, merged ? og : nullptr, &ctx->state(0)->err);
@@ -833,9 +833,9 @@ amph_status do_accept(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n, int32_
   return rc;
 }
 
-int attn_splits_for(const amph_ctx* ctx, int ctx_hi, int rows) {
+int attn_splits_for(const amph_ctx* ctx, int ctx_hi, int rows, int groups) {
   if (ctx->attn_tc) {         // split count and ring depth both shape the captured launch
-    const int sp = attn_tc_splits(ctx->attn_tc, ctx_hi, ctx->cfg.n_heads, rows, ctx->lay.attn_splits);
+    const int sp = attn_tc_splits(ctx->attn_tc, ctx_hi, ctx->cfg.n_heads, rows, groups, ctx->lay.attn_splits);
     return sp * 8 + attn_tc_stages(ctx_hi, sp, ctx->cfg.head_dim);
   }
   int s = (ctx_hi + 127) / 128;
@@ -866,11 +866,11 @@ constexpr size_t kMaxGraphs = 16;
 long long graph_key_of(const amph_ctx* ctx) {
   long long key = 0;
   if (ctx->attn_tc && ctx->B > 1 && !(ctx->cfg.flags & AMPH_FLAG_SEPARATE_MERGE))
-    return attn_splits_for(ctx, ctx->max_ctx_hi(), ctx->rows_small) * 128 +
-           attn_splits_for(ctx, ctx->max_ctx_hi() + ctx->tree_host.n_nodes, ctx->Mver);
+    return attn_splits_for(ctx, ctx->max_ctx_hi(), ctx->rows_small, ctx->B) * 128 +
+           attn_splits_for(ctx, ctx->max_ctx_hi() + ctx->tree_host.n_nodes, ctx->Mver, ctx->B);
   for (int b = 0; b < ctx->B; ++b)
-    key = key * 4099 + attn_splits_for(ctx, ctx->ctx_hi[b], ctx->rows_small) * 128 +
-          attn_splits_for(ctx, ctx->ctx_hi[b] + ctx->tree_host.n_nodes, ctx->Mver);
+    key = key * 4099 + attn_splits_for(ctx, ctx->ctx_hi[b], ctx->rows_small, 1) * 128 +
+          attn_splits_for(ctx, ctx->ctx_hi[b] + ctx->tree_host.n_nodes, ctx->Mver, 1);
   return key;
 }
 

@@ -190,7 +190,7 @@ void launch_attn_combine(AttnScratch sc, void* out, int dtype, int splits, int r
 struct AttnTc;
 AttnTc* attn_tc_create();
 void attn_tc_destroy(AttnTc* a);
-int attn_tc_splits(const AttnTc* a, int keys_bound, int n_heads, int rows, int max_splits);
+int attn_tc_splits(const AttnTc* a, int keys_bound, int n_heads, int rows, int groups, int max_splits);
 int attn_tc_stages(int keys_bound, int splits, int head_dim);
 bool launch_tree_attention_tc(AttnTc* a, const void* q, int q_rows_cap, KvView kv, const RowMeta* meta, AttnScratch sc, int rows,
                               int n_heads, int head_dim, int max_ctx, int splits, int keys_bound, cudaStream_t st,

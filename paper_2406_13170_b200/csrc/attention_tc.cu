@@ -642,13 +642,18 @@ AttnTc* attn_tc_create() {
 void attn_tc_destroy(AttnTc* a) { delete a; }
 
 // KV splits per head: a split owns at least one chunk of 128 keys; the splits of a head form one cluster.
-int attn_tc_splits(const AttnTc* a, int keys_bound, int n_heads, int rows, int max_splits) {
-  (void)a; (void)n_heads; (void)rows;
+int attn_tc_splits(const AttnTc* a, int keys_bound, int n_heads, int rows, int groups, int max_splits) {
   int s = (keys_bound + kChunk - 1) / kChunk;
   if (s > max_splits) s = max_splits;
   // clusters of 8 measured 3-6 us per launch slower than clusters of 7 at every context from 1k to 8k tokens (they are
   // harder to place beside the resident projection CTAs), so a head is cut into at most 7 splits
   if (s > 7) s = 7;
+  // Several row blocks (a tree of more than 64 nodes, sequences side by side, prompt chunks): no more CTAs than run at a time
+  // (two per SM).  A second wave and the merge cost more than shorter ranges give; 32 heads, us per launch, 7 splits against
+  // this rule: 128 rows at 2.1k keys 30.1 / 22.7 (4 splits; 5, just over a wave, no better than 7), four sequences of 64 rows at
+  // 0.3k 21.9 / 16.7 (2), a prompt's first 512 tokens 40.5 / 23.8 and its fourth 512 73 / 44 (1).
+  const int units = n_heads * groups * ((rows + kRows - 1) / kRows), fit = 2 * a->sm_count / units;
+  if (units > n_heads && s > fit) s = fit;
   return s < 1 ? 1 : s;
 }
 
