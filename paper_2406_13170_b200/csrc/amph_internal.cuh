@@ -204,9 +204,10 @@ void launch_swiglu(PartialView P, void* act, int dtype, int rows, int f, cudaStr
                    int early = 0);
 
 struct GemmSeg { const void* w; };
-// P[row][seg*out + o] = sum_k X[row][k] * W_seg[o][k]; plain CUDA-core kernel, one split.
+// P[row][seg*out + o] = sum_k X[row][k] * W_seg[o][k]; plain CUDA-core kernel, one split.  wait_first: no weight is read before the
+// kernel ahead in the stream has finished.
 void launch_gemm_generic(const void* x, int ldx, const GemmSeg* segs, int n_seg, int out, int in,
-                         float* P, int ldp, int rows, int dtype, cudaStream_t st);
+                         float* P, int ldp, int rows, int dtype, cudaStream_t st, int wait_first = 0);
 
 // ---- draft-module specific
 // (one launch per batch; a void* with a stride is sequence 0's copy of a per-sequence buffer, the next `stride` bytes further on)
@@ -264,7 +265,8 @@ void launch_accept_compact(const AcceptArgs& a, int batch, int dtype, cudaStream
 void launch_sample_rows(const float* logits, int vocab, int row0, int n_rows, int rows_per, int batch, const TreeDev* tree, const int* tok,
                         const void* state, size_t state_stride, int seq0, int stream_id, float temperature, unsigned long long seed,
                         int* choice, float* uniforms_out, cudaStream_t st);
-void launch_reduce_partials(PartialView P, float* y, int rows, int cols, cudaStream_t st);
+// y[rows][cols] = sum over the splits.  err (may be NULL): device flag that is handed to *status (may be NULL) and cleared.
+void launch_reduce_partials(PartialView P, float* y, int rows, int cols, cudaStream_t st, int* err = nullptr, int* status = nullptr);
 void launch_kv_export(KvView kv, int which, int dtype, int row0, int rows, int n_heads, int head_dim, int max_ctx,
                       float* dst, cudaStream_t st);
 void launch_prefill_tail(DevState* s, const int* amax, int last_row, const float* hidden, float* pend_h,

@@ -51,6 +51,7 @@ struct TcParams {
   int n_heads, dh, max_ctx;
   int* err_flag;
   unsigned long long wait_limit_ns;   // a barrier wait gives up after this long
+  int wait_first;                      // wait for the kernel before this one ahead of the first weight (see tc_gemm_wait_first)
   uint32_t extra_tx;                   // self-test only: bytes the first stage's barrier expects beyond what is copied
 };
 
@@ -199,6 +200,7 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
     }
     // Weights do not depend on the previous kernel: fill the ring with weight tiles first, then wait for
     // the producer of the activations, then fetch the activation tiles of those stages.
+    if (prm.wait_first) pdl_wait();
     const int npre = nit < stages ? nit : stages;
     const int npf = nit < npre + prm.l2_prefetch ? nit : npre + prm.l2_prefetch;
     if (leader) {
@@ -542,6 +544,7 @@ bool tc_gemm_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   prm.l2_prefetch = 1;
   prm.err_flag = g->err_flag;
   prm.wait_limit_ns = g->wait_limit_ns;
+  prm.wait_first = g->wait_first;
   prm.extra_tx = g->extra_tx;
   const size_t smem = (size_t)stages * stage_bytes + 1024;
   launch_pdl(tc_gemm_kernel<EPI_PARTIAL>, dim3(tiles, splits), dim3(kThreads), smem, st, pack, prm);
@@ -678,6 +681,8 @@ void tc_gemm_rebind(TcGemm* g, int xb, void* ptr, int rows, int cols, int* err_f
   g->err_flag = err_flag;
   if (g->cache.size() > 512) g->cache.clear();          // a long-lived plan set must not grow without bound
 }
+
+void tc_gemm_wait_first(TcGemm* g) { g->wait_first = 1; }
 
 void tc_gemm_set_selftest(TcGemm* g, unsigned long long wait_limit_ns, unsigned extra_tx) {
   g->wait_limit_ns = wait_limit_ns;

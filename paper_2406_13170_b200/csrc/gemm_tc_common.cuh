@@ -107,6 +107,7 @@ struct TcGemm {
   int max_smem = 0;
   unsigned long long wait_limit_ns = tc::kWaitLimitNs;
   uint32_t extra_tx = 0;
+  int wait_first = 0;
   std::map<std::tuple<const void*, const void*, int, int, int>, CUtensorMap> pair_cache;   // (lower, upper matrix, rows, cols, K blocks)
 
   // Two [rows, cols] matrices as one 4-D tensor (column, row, K block, matrix): a box of 64 rows of both.

@@ -58,6 +58,7 @@ struct WideParams {
   __nv_bfloat16* q;         // ROPE
   RopeGroups gr;
   int n_heads, dh, max_ctx;
+  int wait_first;           // see tc_gemm_wait_first
   int* err_flag;
   unsigned long long wait_limit_ns;
 };
@@ -219,6 +220,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
       tma_pair_3d(smem + (size_t)st * stage_bytes + kUnitKb * a_tile, &maps.x, 0, rb * n + (int)rank * (n / 2), u * kUnitKb, bar);
     };
     // weights do not depend on the kernel before: fill the ring with them, then wait, then fetch those stages' activations
+    if (prm.wait_first) pdl_wait();
     SegIter it = first;
     Segment sg;
     bool have = it.next(sg);
@@ -503,6 +505,7 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
   prm->stages = (int)((kWideSmem - 1024 - out_bytes) / stage);
   if (prm->stages > kMaxStages) prm->stages = kMaxStages;
   prm->flags = g->wide_flags;
+  prm->wait_first = g->wait_first;
   prm->err_flag = g->err_flag;
   prm->wait_limit_ns = g->wait_limit_ns;
   return true;

@@ -677,7 +677,8 @@ constexpr int kPlainChunk = 1024;        // bytes of a row per step: two 16-byte
 
 template <typename T, int R, int O>
 __global__ void __launch_bounds__(kPlainThreads)
-gemm_generic_kernel(const T* __restrict__ X, int ldx, const __grid_constant__ GemmSegs segs, int out, int in, float* __restrict__ P, int ldp, int rows) {
+gemm_generic_kernel(const T* __restrict__ X, int ldx, const __grid_constant__ GemmSegs segs, int out, int in, float* __restrict__ P, int ldp, int rows,
+                    int wait_first) {
   pdl_launch_dependents();
   constexpr int V = Vec16<T>::N, KC = kPlainChunk / (int)sizeof(T);
   __shared__ __align__(16) uint4 xs[2][R][kPlainChunk / 16];
@@ -704,6 +705,7 @@ gemm_generic_kernel(const T* __restrict__ X, int ldx, const __grid_constant__ Ge
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  if (wait_first) pdl_wait();
   load_w(0);
   pdl_wait();
   load_x(0);
@@ -765,13 +767,13 @@ gemm_generic_kernel(const T* __restrict__ X, int ldx, const __grid_constant__ Ge
 // R = 4 for the drafting heads' few rows, else 16; two features a warp (half of the shared-memory reads) once one feature a warp
 // gives more than two blocks per SM.
 void launch_gemm_generic(const void* x, int ldx, const GemmSeg* segs, int n_seg, int out, int in, float* P,
-                         int ldp, int rows, int dtype, cudaStream_t st) {
+                         int ldp, int rows, int dtype, cudaStream_t st, int wait_first) {
   GemmSegs gs;
   for (int s = 0; s < kMaxK; ++s) gs.s[s].w = s < n_seg ? segs[s].w : nullptr;
   const int blocks = (out + 7) / 8;
   auto run = [&](auto kernel, int R, int O, auto* X) {
     launch_pdl(kernel, dim3((out + 8 * O - 1) / (8 * O), n_seg, (rows + R - 1) / R), dim3(kPlainThreads), 0, st, X, ldx, gs, out, in, P, ldp,
-               rows);
+               rows, wait_first);
   };
   AMPH_DISPATCH(dtype, const T* X = (const T*)x;
                 if (rows <= 4) run(gemm_generic_kernel<T, 4, 1>, 4, 1, X);
@@ -1441,21 +1443,26 @@ void launch_sample_rows(const float* logits, int vocab, int row0, int n_rows, in
              choice, uniforms_out);
 }
 
-__global__ void reduce_partials_kernel(PartialView P, float* __restrict__ y, int rows, int cols) {
+// Grid (512-column chunk, row).  Bound: L2 (the splits' sums were just written); the loads of all splits are in flight together.
+__global__ void __launch_bounds__(128)
+reduce_partials_kernel(PartialView P, float* __restrict__ y, int cols, int vec, int* err, int* status) {
   pdl_wait();
   pdl_launch_dependents();
-  const size_t n = (size_t)rows * cols;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int r = (int)(i / cols), c = (int)(i - (size_t)r * cols);
-    y[i] = sum_partials(P, r, c);
+  if (err != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    if (status != nullptr) *status = *err;
+    *err = 0;
+  }
+  const int r = blockIdx.y, c = (blockIdx.x * 128 + threadIdx.x) * 4;
+  if (vec) {
+    if (c < cols) store4(y + (size_t)r * cols + c, sum_partials4_wide(P, r, c));
+  } else {
+    for (int e = c; e < cols && e < c + 4; ++e) y[(size_t)r * cols + e] = sum_partials(P, r, e);
   }
 }
 
-void launch_reduce_partials(PartialView P, float* y, int rows, int cols, cudaStream_t st) {
-  const size_t n = (size_t)rows * cols;
-  int blocks = (int)((n + 255) / 256);
-  if (blocks > 148 * 8) blocks = 148 * 8;
-  launch_pdl(reduce_partials_kernel, dim3(blocks), dim3(256), 0, st, P, y, rows, cols);
+void launch_reduce_partials(PartialView P, float* y, int rows, int cols, cudaStream_t st, int* err, int* status) {
+  const int vec = cols % 4 == 0 && P.ld % 4 == 0 && P.split_stride % 4 == 0 && ((uintptr_t)y & 15) == 0;
+  launch_pdl(reduce_partials_kernel, dim3((cols + 511) / 512, rows), dim3(128), 0, st, P, y, cols, vec, err, status);
 }
 
 template <typename T>

@@ -89,15 +89,13 @@ amph_status amph_project_noalloc(const void* x_dev, int32_t x_rows_cap, const vo
   amph_status rc = scratch_for_current_device(&base, err_msg, err_len);
   if (rc != AMPH_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  int* err = status_dev ? status_dev : (int*)base;
+  int* err = (int*)base;
   float* P = (float*)((char*)base + 256);
   const size_t p_floats = (kStaticScratchBytes - 256) / sizeof(float);
-  // The array keeps whatever the previous call left.  Only the status word must start at zero; the partial
-  // sums are fully overwritten before anything reads them.
-  if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) {
-    say(err_msg, err_len, "clearing the status word failed: %s", cudaGetErrorString(cudaGetLastError()));
-    return AMPH_ERR_CUDA;
-  }
+  // The array keeps whatever the previous call left: the error flag in its header is zero (the reduction hands it to the
+  // caller's status word and clears it, so a call is two kernels and no memset between dependent launches), the partial sums
+  // are fully overwritten before anything reads them.  The kernels wait for their predecessor before they read a weight:
+  // it may be a kernel of the caller's that writes it and lets its successor start early.
   PartialView pv;
   pv.p = P;
   pv.ld = (int)ld;
@@ -113,6 +111,7 @@ amph_status amph_project_noalloc(const void* x_dev, int32_t x_rows_cap, const vo
     TcGemm*& g = g_plans[dev];
     if (!g) g = tc_gemm_create(xb, xr, xc, 1, err);
     if (!g) { say(err_msg, err_len, "tensor-map encoder unavailable or not an sm_100 device"); return AMPH_ERR_CUDA; }
+    tc_gemm_wait_first(g);
     tc_gemm_rebind(g, 0, xb[0], xr[0], xc[0], err);
     int splits = 0;
     size_t stride = 0;
@@ -123,11 +122,11 @@ amph_status amph_project_noalloc(const void* x_dev, int32_t x_rows_cap, const vo
   } else {
     GemmSeg segs[kMaxK];
     for (int s = 0; s < n_seg; ++s) segs[s].w = w[s];
-    launch_gemm_generic(x_dev, in, segs, n_seg, out, in, P, (int)ld, rows, dtype, st);
+    launch_gemm_generic(x_dev, in, segs, n_seg, out, in, P, (int)ld, rows, dtype, st, 1);
     pv.splits = 1;
     pv.split_stride = 0;
   }
-  launch_reduce_partials(pv, y_dev, rows, (int)ld, st);
+  launch_reduce_partials(pv, y_dev, rows, (int)ld, st, err, status_dev);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { say(err_msg, err_len, "launch failed: %s", cudaGetErrorString(e)); return AMPH_ERR_CUDA; }
   return AMPH_OK;
