@@ -8,11 +8,13 @@
 //   warp 1      MMA issuer: S = Q K^T (tcgen05.mma, M = 64 rows, N = 128 keys, accumulator in tensor memory), then
 //               O_c = P V (A = the probabilities written back to shared memory as a K-major operand, B = the V rows
 //               as they sit in the cache, i.e. an MN-major operand).
-//   warps 2-5   softmax: scores from tensor memory (tcgen05.ld), mask, running max / sum in fp32, probabilities to
-//               shared memory in bf16, running output in registers (the chunk outputs are added with the usual
-//               rescaling, so tensor memory never has to be rescaled).
-// The KV splits of one head form a thread-block cluster and merge their partial outputs through distributed shared
-// memory; with more than 8 splits the partials go to global scratch for attn_combine_kernel.
+//   warps 2-9   softmax, two warps per 16 rows, each with half of a chunk's keys and half of the head dimension: scores from
+//               tensor memory (tcgen05.ld), mask, running max / sum in fp32 (the maxima of the two halves meet in shared
+//               memory), probabilities to shared memory in bf16, running output in registers (the chunk outputs are added
+//               with the usual rescaling, so tensor memory never has to be rescaled).
+// The KV splits of one head form a thread-block cluster: every CTA sends its partial rows, one bulk copy per peer, to the CTAs
+// that merge them, into shared memory the owner no longer needs; with the separate merge the partials go to global scratch for
+// attn_combine_kernel.
 // Every barrier wait is bounded; a wait that gives up raises the error flag and the CTA leaves in order.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -34,7 +36,8 @@ namespace {
 
 constexpr int kRows = 64;            // query rows per CTA (UMMA M)
 constexpr int kChunk = 128;          // keys per pipeline stage (UMMA N of the score MMA)
-constexpr int kThreads = 192;
+constexpr int kSoftmaxThreads = 256;
+constexpr int kThreads = 64 + kSoftmaxThreads;
 constexpr int kTmemCols = 256;       // S in columns [0, 128), O in [128, 128 + DH): room is left for the projection CTAs that
                                      // become resident beside this kernel and allocate their accumulators
 constexpr unsigned long long kWaitLimitNs = 1000000000ull;
@@ -127,12 +130,12 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr) {
   d |= (uint64_t)2 << 61;
   return d;
 }
-// The same for the MN-major operand V ([key][64 head dims] rows of 128 bytes): an MMA of N = 64 spans exactly one swizzle
-// atom along MN, so the only stride in play is the one between groups of 8 keys (1024 bytes); both offset fields carry it.
-__device__ __forceinline__ uint64_t umma_desc_mn(uint32_t smem_addr) {
+// The same for the MN-major operand V ([key][64 head dims] rows of 128 bytes): swizzle atoms of 64 head dims x 8 keys, the next
+// 8 keys 1024 bytes on (second offset field), the next 64 head dims `block` bytes on (first one).
+__device__ __forceinline__ uint64_t umma_desc_mn(uint32_t smem_addr, uint32_t block) {
   uint64_t d = 0;
   d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)(1024 >> 4) << 16;
+  d |= (uint64_t)(block >> 4) << 16;
   d |= (uint64_t)(1024 >> 4) << 32;
   d |= (uint64_t)1 << 46;
   d |= (uint64_t)2 << 61;
@@ -161,6 +164,13 @@ __device__ __forceinline__ void tmem_ld_frag64(uint32_t taddr, uint32_t* v) {
                : "r"(taddr)
                : "memory");
 }
+// The same for 32 columns.
+__device__ __forceinline__ void tmem_ld_frag32(uint32_t taddr, uint32_t* v) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+               : "r"(taddr)
+               : "memory");
+}
 // 2^x on the special-function unit: ex2(-inf) = +0, so masked scores need no test of their own
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
@@ -171,23 +181,19 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
 }
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ uint32_t peer_smem(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ float4 ld_peer4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ float2 ld_peer2(uint32_t addr) {
-  float2 v;
-  asm volatile("ld.shared::cluster.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
-  return v;
+// Orders execution only: what it stands for (operands read, copies received) has been observed through mbarriers, and nothing
+// written before it is read by a peer after it.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
+// shared memory of this CTA -> shared memory of a CTA of the cluster; the bytes are counted by a barrier there
+__device__ __forceinline__ void bulk_to_peer(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "r"(smem_u32(src)), "r"(bytes), "r"(bar) : "memory");
 }
 
 // Bits [0, 128) of (ones below `nctx`, then the 128-bit mask m shifted up by nctx), shifted down by `sh` (< 8).
@@ -208,16 +214,19 @@ __device__ __forceinline__ void chunk_visibility(u64 m0, u64 m1, bool live, int 
 
 template <int DH, bool MERGE, int NG>
 __global__ void __launch_bounds__(kThreads, 2)
-tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const AttnParams<NG> prm) {
+tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_constant__ AttnParams<NG> prm) {
   constexpr int NB = DH / 64;                        // 64-wide blocks of the head dimension (one 128-byte swizzle row each)
   constexpr uint32_t kQBlock = kRows * 128;          // bytes of one Q / P block: 64 rows x 128 bytes
   constexpr uint32_t kKvBlock = kChunk * 128;        // bytes of one K / V block: 128 keys x 128 bytes
   constexpr uint32_t kStage = 2 * NB * kKvBlock;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t q_full, p_ready, o_full;
+  __shared__ __align__(8) uint64_t q_full, p_ready, o_full, recv_full;
   __shared__ __align__(8) uint64_t k_full[4], v_full[4], k_empty[4], v_empty[4], s_full;
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
+  __shared__ float max_s[2][2][kRows];               // [chunk parity][half][row]: maxima of the two halves of a chunk
+  __shared__ float sum_s[2][kRows];                  // [half][row]
+  __shared__ u64 mask_s[kRows][2];                   // ancestor masks (registers are short: two CTAs share an SM)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h = blockIdx.x, split = blockIdx.y;
@@ -233,10 +242,11 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const AttnParams<
   if (threadIdx.x == 0) {
     abort_flag = 0;
     mbar_init(&q_full, 1);
-    mbar_init(&p_ready, 128);
+    mbar_init(&p_ready, kSoftmaxThreads);
     mbar_init(&o_full, 1);
     for (int s = 0; s < 4; ++s) { mbar_init(&k_full[s], 1); mbar_init(&v_full[s], 1); mbar_init(&k_empty[s], 1); mbar_init(&v_empty[s], 1); }
     mbar_init(&s_full, 1);
+    mbar_init(&recv_full, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -252,21 +262,25 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const AttnParams<
   // predecessor before it lets its successor start), so it may be read before the dependency wait.
   const int base = meta->base, n_rows = meta->n_rows;
   const int total = base + n_rows;
-  int len = (total + (int)gridDim.y - 1) / (int)gridDim.y;
+  const int S = gridDim.y;                             // splits of the head
+  int len = (total + S - 1) / S;
   len = (len + kChunk - 1) / kChunk * kChunk;          // whole chunks: a chunk never straddles two splits
   const int s_lo = split * len;
   int s_hi = s_lo + len;
   if (s_hi > total) s_hi = total;
   if (s_hi > prm.max_ctx) s_hi = prm.max_ctx;
+  const int slots = (kRows + S - 1) / S;               // rows that one CTA of the cluster merges
+  const uint32_t block_bytes = (uint32_t)slots * (DH + 4) * 4;
+  constexpr uint32_t kRecvAt = DH == 128 ? 40 * 1024 : 20 * 1024;      // 71 rows of (DH + 4) floats lie below it
   const int n_chunks = s_hi > s_lo ? (s_hi - s_lo + kChunk - 1) / kChunk : 0;
 
   // softmax warps: running output of rows row_a and row_a + 8 as accumulator fragments
-  // (acc[4 * rep + 2 * hi + e] = row row_a + 8 * hi, head dim 8 * rep + 2 * qd + e), running max (base 2) and sum
-  float acc[DH / 2];
+  // (acc[4 * rep + 2 * hi + e] = row row_a + 8 * hi, head dim DH / 2 * half + 8 * rep + 2 * qd + e), running max (base 2) and sum
+  float acc[DH / 4];
   float m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;
 #pragma unroll
-  for (int i = 0; i < DH / 2; ++i) acc[i] = 0.f;
-  const int quarter = warp & 3;
+  for (int i = 0; i < DH / 4; ++i) acc[i] = 0.f;
+  const int quarter = warp & 3, half = warp >= 2 ? (warp - 2) >> 2 : 0;
   const int row_a = quarter * 16 + (lane >> 2), qd = lane & 3;
 
   if (warp == 0) {
@@ -334,7 +348,7 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const AttnParams<
     // ---------------- MMA issuer
     pdl_wait();
     const bool leader = elect_one();
-    const uint32_t idesc_s = umma_idesc(kChunk, 0), idesc_o = umma_idesc(64, 1);
+    const uint32_t idesc_s = umma_idesc(kChunk, 0), idesc_o = umma_idesc(DH, 1);
     const uint32_t q_addr = smem_u32(Qs), p_addr = smem_u32(Ps);
     auto issue_scores = [&](int c) {                   // S[c & 1] = Q K_c^T
       const uint32_t k_addr = smem_u32(St + (size_t)(c % stages) * kStage);
@@ -363,15 +377,13 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const AttnParams<
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (leader) {
-        // O_c = P_c V_c: 8 steps of 16 keys; V is the MN-major operand (128-byte rows of 64 head dims, one row per key:
-        // the next 8 keys are 1024 bytes on, a step of 16 keys 2048 bytes), one N = 64 MMA per 64-wide block of the head dim
+        // O_c = P_c V_c: 8 steps of 16 keys; V is the MN-major operand (128-byte rows of 64 head dims, one row per key: the next
+        // 8 keys are 1024 bytes on, a step of 16 keys 2048 bytes, the next 64 head dims a block of kKvBlock)
         const uint32_t v_addr = smem_u32(St + (size_t)st * kStage) + NB * kKvBlock;
 #pragma unroll
         for (int k = 0; k < kChunk / 16; ++k) {
           const uint64_t adesc = umma_desc(p_addr + (uint32_t)(k >> 2) * kQBlock) + (uint64_t)(2 * (k & 3));
-#pragma unroll
-          for (int j = 0; j < NB; ++j)
-            umma_f16(tmem + kChunk + 64 * j, adesc, umma_desc_mn(v_addr + j * kKvBlock + (uint32_t)k * 2048), idesc_o, k ? 1u : 0u);
+          umma_f16(tmem + kChunk, adesc, umma_desc_mn(v_addr + (uint32_t)k * 2048, kKvBlock), idesc_o, k ? 1u : 0u);
         }
         umma_commit(&o_full);
         umma_commit(&v_empty[st]);
@@ -388,62 +400,61 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const AttnParams<
     }
   } else {
     // ---------------- softmax.  Warp w may touch TMEM lanes 32 (w % 4) .. + 31; an M = 64 accumulator keeps row r in lane
-    // 32 (r / 16) + r % 16, so a warp owns 16 rows.  They are read as accumulator fragments (all 32 lanes busy): this
-    // thread holds rows row_a and row_a + 8, two adjacent columns of every group of 8.
+    // 32 (r / 16) + r % 16, so two warps share 16 rows.  They are read as accumulator fragments (all 32 lanes busy): this
+    // thread holds rows row_a and row_a + 8, two adjacent columns of every group of 8 of its half.
     pdl_wait();                                        // these warps write the output rows
     const int ga = rb * kRows + row_a, gb = ga + 8;
     const bool live_a = ga < n_rows, live_b = gb < n_rows;
-    u64 ma0 = 0, ma1 = 0, mb0 = 0, mb1 = 0;
-    if (live_a) { ma0 = meta->mask[ga][0]; ma1 = meta->mask[ga][1]; }
-    if (live_b) { mb0 = meta->mask[gb][0]; mb1 = meta->mask[gb][1]; }
+    if (qd < 2) {                                      // read back by the same warp (its own rows)
+      mask_s[row_a][qd] = live_a ? meta->mask[ga][qd] : 0ull;
+      mask_s[row_a + 8][qd] = live_b ? meta->mask[gb][qd] : 0ull;
+    }
+    __syncwarp();
     const float scale_log2 = 1.4426950408889634f / sqrtf((float)DH);
     const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
     auto add_output = [&]() {                          // acc += O of the chunk whose P V has completed
 #pragma unroll
       for (int hb = 0; hb < DH / 64; ++hb) {
-        uint32_t r[32];
-        tmem_ld_frag64(lane_addr + kChunk + 64 * hb, r);
+        uint32_t r[16];
+        tmem_ld_frag32(lane_addr + kChunk + DH / 2 * half + 32 * hb, r);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int i = 0; i < 32; ++i) acc[hb * 32 + i] += __uint_as_float(r[i]);
+        for (int i = 0; i < 16; ++i) acc[hb * 16 + i] += __uint_as_float(r[i]);
       }
     };
+    // a wait that gives up leaves the loop running (the later ones give up at once): the two warps of a row group meet at a
+    // barrier in every chunk
     bool ok = true;
     for (int c = 0; c < n_chunks; ++c) {
-      ok = __all_sync(0xffffffffu, mbar_wait(&s_full, c & 1, &abort_flag));
-      if (!ok) break;
+      ok = __all_sync(0xffffffffu, mbar_wait(&s_full, c & 1, &abort_flag)) && ok;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (c > 0) {             // the previous chunk's output (its P V was issued before these scores, so it is complete):
-                               // added while the running output is still at the previous chunk's scale
-        ok = __all_sync(0xffffffffu, mbar_wait(&o_full, (c - 1) & 1, &abort_flag));
-        if (!ok) break;
-        add_output();
-      }
-      uint32_t sr[kChunk / 2];
-      tmem_ld_frag64(lane_addr, sr);
-      tmem_ld_frag64(lane_addr + 64, sr + 32);
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      float s[kChunk / 2];
+      float s[kChunk / 4];
       const int key0 = s_lo + c * kChunk;
-      float tmax_a = -INFINITY, tmax_b = -INFINITY;
-      // visibility of the chunk's 128 keys for the two rows, as bit vectors already shifted to this thread's first column
-      // (key0 + 2 qd): committed slots are visible to every live row, slot base + m iff bit m of the row's ancestor mask
-      u64 va0, va1, vb0, vb1;
-      chunk_visibility(ma0, ma1, live_a, base - key0, 2 * qd, va0, va1);
-      chunk_visibility(mb0, mb1, live_b, base - key0, 2 * qd, vb0, vb1);
-      if (base - key0 >= kChunk && live_a && live_b) {                       // committed context: nothing is masked
+      {
+        uint32_t sr[kChunk / 4];
+        tmem_ld_frag64(lane_addr + kChunk / 2 * half, sr);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (base - key0 >= kChunk && live_a && live_b) {                     // committed context: nothing is masked
 #pragma unroll
-        for (int i = 0; i < kChunk / 2; ++i) s[i] = __uint_as_float(sr[i]);
-      } else {
+          for (int i = 0; i < kChunk / 4; ++i) s[i] = __uint_as_float(sr[i]);
+        } else {
+          // visibility of the chunk's 128 keys for the two rows, as bit vectors already shifted to this thread's first column
+          // (key0 + 2 qd): committed slots are visible to every live row, slot base + m iff bit m of the row's ancestor mask
+          u64 va0, va1, vb0, vb1;
+          chunk_visibility(mask_s[row_a][0], mask_s[row_a][1], live_a, base - key0, 2 * qd, va0, va1);
+          chunk_visibility(mask_s[row_a + 8][0], mask_s[row_a + 8][1], live_b, base - key0, 2 * qd, vb0, vb1);
+          const u64 wa = half ? va1 : va0, wb = half ? vb1 : vb0;
 #pragma unroll
-        for (int i = 0; i < kChunk / 2; ++i) {
-          const int bit = 8 * (i >> 2) + (i & 1);                            // column of this register minus 2 qd
-          const u64 w = ((i >> 1) & 1) ? (bit < 64 ? vb0 : vb1) : (bit < 64 ? va0 : va1);
-          s[i] = ((w >> (bit & 63)) & 1ull) ? __uint_as_float(sr[i]) : -INFINITY;       // raw scores; the scale joins the exponent below
+          for (int i = 0; i < kChunk / 4; ++i) {
+            const int bit = 8 * (i >> 2) + (i & 1);                          // column of this register minus 64 half + 2 qd
+            const u64 w = ((i >> 1) & 1) ? wb : wa;
+            s[i] = ((w >> bit) & 1ull) ? __uint_as_float(sr[i]) : -INFINITY;       // raw scores; the scale joins the exponent below
+          }
         }
       }
+      float tmax_a = -INFINITY, tmax_b = -INFINITY;
 #pragma unroll
-      for (int i = 0; i < kChunk / 2; ++i) {
+      for (int i = 0; i < kChunk / 4; ++i) {
         if ((i >> 1) & 1) tmax_b = fmaxf(tmax_b, s[i]);
         else tmax_a = fmaxf(tmax_a, s[i]);
       }
@@ -451,18 +462,32 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const AttnParams<
       tmax_a = fmaxf(tmax_a, __shfl_xor_sync(0xffffffffu, tmax_a, 2));
       tmax_b = fmaxf(tmax_b, __shfl_xor_sync(0xffffffffu, tmax_b, 1));
       tmax_b = fmaxf(tmax_b, __shfl_xor_sync(0xffffffffu, tmax_b, 2));
+      if (qd == 0) { max_s[c & 1][half][row_a] = tmax_a; max_s[c & 1][half][row_a + 8] = tmax_b; }
+      if (c > 0) {             // the previous chunk's output (its P V was issued before these scores, so it is complete):
+                               // added while the running output is still at the previous chunk's scale
+        ok = __all_sync(0xffffffffu, mbar_wait(&o_full, (c - 1) & 1, &abort_flag)) && ok;
+        add_output();
+      }
+      switch (quarter) {                               // barrier 1 + quarter: the two warps of these rows
+        case 0: asm volatile("bar.sync 1, 64;" ::: "memory"); break;
+        case 1: asm volatile("bar.sync 2, 64;" ::: "memory"); break;
+        case 2: asm volatile("bar.sync 3, 64;" ::: "memory"); break;
+        default: asm volatile("bar.sync 4, 64;" ::: "memory");
+      }
+      tmax_a = fmaxf(tmax_a, max_s[c & 1][half ^ 1][row_a]);
+      tmax_b = fmaxf(tmax_b, max_s[c & 1][half ^ 1][row_a + 8]);
       const float mn_a = fmaxf(m_a, tmax_a * scale_log2), mn_b = fmaxf(m_b, tmax_b * scale_log2);     // base-2 logits
       // a row that has seen no visible key yet (m = -inf) holds zeros: any finite factor will do
       const float ca = m_a == -INFINITY ? 1.f : ex2_approx(m_a - mn_a);
       const float cb = m_b == -INFINITY ? 1.f : ex2_approx(m_b - mn_b);
       if (ca != 1.f || cb != 1.f) {                    // the running maximum moved: bring the running output to the new scale
 #pragma unroll
-        for (int i = 0; i < DH / 2; ++i) acc[i] *= ((i >> 1) & 1) ? cb : ca;
+        for (int i = 0; i < DH / 4; ++i) acc[i] *= ((i >> 1) & 1) ? cb : ca;
       }
       const float sub_a = mn_a == -INFINITY ? 0.f : mn_a, sub_b = mn_b == -INFINITY ? 0.f : mn_b;
       float ps_a = 0.f, ps_b = 0.f;
 #pragma unroll
-      for (int rep = 0; rep < kChunk / 8; ++rep) {
+      for (int rep = 0; rep < kChunk / 16; ++rep) {
         float p[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -470,8 +495,8 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const AttnParams<
         }
         ps_a += p[0] + p[1];
         ps_b += p[2] + p[3];
-        // P block rep / 8 (64 keys each): row r, 16-byte chunk (rep % 8) of its 128-byte row sits at chunk ^ (r % 8)
-        uint8_t* blk = Ps + (rep >> 3) * kQBlock + ((((rep & 7) ^ (row_a & 7)) << 4) + qd * 4);
+        // P block of this half (64 keys): row r, 16-byte chunk rep of its 128-byte row sits at chunk ^ (r % 8)
+        uint8_t* blk = Ps + half * kQBlock + (((rep ^ (row_a & 7)) << 4) + qd * 4);
         *reinterpret_cast<uint32_t*>(blk + row_a * 128) = pack_bf16(p[0], p[1]);
         *reinterpret_cast<uint32_t*>(blk + (row_a + 8) * 128) = pack_bf16(p[2], p[3]);
       }
@@ -483,24 +508,39 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const AttnParams<
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       mbar_arrive(&p_ready);
     }
-    if (ok && n_chunks > 0) {
-      ok = __all_sync(0xffffffffu, mbar_wait(&o_full, (n_chunks - 1) & 1, &abort_flag));
-      if (ok) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        add_output();
-      }
-    }
+    if (n_chunks > 0) ok = __all_sync(0xffffffffu, mbar_wait(&o_full, (n_chunks - 1) & 1, &abort_flag)) && ok;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (MERGE && S > 1) cluster_arrive();              // the last MMA has read its operands: peers may write to this shared memory
+    if (n_chunks > 0) add_output();
     l_a += __shfl_xor_sync(0xffffffffu, l_a, 1);
     l_a += __shfl_xor_sync(0xffffffffu, l_a, 2);
     l_b += __shfl_xor_sync(0xffffffffu, l_b, 1);
     l_b += __shfl_xor_sync(0xffffffffu, l_b, 2);
     if (!ok) {                                         // a wait gave up: contribute nothing
 #pragma unroll
-      for (int i = 0; i < DH / 2; ++i) acc[i] = 0.f;
+      for (int i = 0; i < DH / 4; ++i) acc[i] = 0.f;
       m_a = m_b = -INFINITY;
       l_a = l_b = 0.f;
     }
+    if (qd == 0) { sum_s[half][row_a] = l_a; sum_s[half][row_a + 8] = l_b; }
+    if constexpr (MERGE) {                             // park the partial rows, in blocks of the rows that one CTA merges
+#pragma unroll
+      for (int hi = 0; hi < 2; ++hi) {
+        const int r = row_a + 8 * hi, owner = r / slots;
+        float* dst = reinterpret_cast<float*>(smem + (size_t)owner * block_bytes) + (r - owner * slots) * DH + DH / 2 * half + 2 * qd;
+#pragma unroll
+        for (int k = 0; k < DH / 16; ++k) *reinterpret_cast<float2*>(dst + 8 * k) = make_float2(acc[4 * k + 2 * hi], acc[4 * k + 2 * hi + 1]);
+        if (qd == 0) {                                 // (max, sum of the first half, sum of the second half, -)
+          float* ml = reinterpret_cast<float*>(smem + (size_t)owner * block_bytes + slots * DH * 4) + (r - owner * slots) * 4;
+          if (half == 0) *reinterpret_cast<float2*>(ml) = make_float2(hi ? m_b : m_a, hi ? l_b : l_a);
+          else ml[2] = hi ? l_b : l_a;
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the copies to the peers read through the async proxy
+    }
   }
+  __syncwarp();
+  if (MERGE && S > 1 && warp < 2) cluster_arrive();
 
   // ---------------- all tensor-core work of this CTA is complete (or abandoned): free tensor memory, then merge
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -509,73 +549,63 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const AttnParams<
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
-  if (threadIdx.x == 0 && abort_flag && prm.err_flag) *prm.err_flag = AMPH_ERR_TIMEOUT;
-  constexpr float kLn2 = 0.6931471805599453f;          // the running maximum is kept in base-2 units
   if constexpr (MERGE) {
-    // park the partial output and (max, sum); the K / V ring is free now
-    float* Os = reinterpret_cast<float*>(St);                       // [64][DH]
-    float* MLs = Os + kRows * DH;                                   // [64][2]
-    if (warp >= 2) {
-#pragma unroll
-      for (int rep = 0; rep < DH / 8; ++rep) {
-        *reinterpret_cast<float2*>(Os + row_a * DH + 8 * rep + 2 * qd) = make_float2(acc[4 * rep], acc[4 * rep + 1]);
-        *reinterpret_cast<float2*>(Os + (row_a + 8) * DH + 8 * rep + 2 * qd) = make_float2(acc[4 * rep + 2], acc[4 * rep + 3]);
+    // Rows [slots * j, slots * (j + 1)) are merged by CTA j of the cluster: everybody's block j goes there in one bulk copy.
+    const uint8_t* parts = smem;                       // S blocks, one per split
+    if (S > 1) {
+      uint8_t* recv = smem + kRecvAt;
+      __syncwarp();
+      cluster_wait();                                  // every CTA of the cluster is done with its operands
+      if (warp == 0) {
+        if (lane == 0) mbar_expect_tx(&recv_full, (uint32_t)S * block_bytes);
+        __syncwarp();
+        if (lane < S)
+          bulk_to_peer(peer_smem(smem_u32(recv + (size_t)split * block_bytes), (uint32_t)lane), smem + (size_t)lane * block_bytes, block_bytes,
+                       peer_smem(smem_u32(&recv_full), (uint32_t)lane));
       }
-      if (qd == 0) {
-        *reinterpret_cast<float2*>(MLs + row_a * 2) = make_float2(m_a * kLn2, l_a);
-        *reinterpret_cast<float2*>(MLs + (row_a + 8) * 2) = make_float2(m_b * kLn2, l_b);
-      }
+      mbar_wait(&recv_full, 0, &abort_flag);
+      __syncwarp();
+      cluster_arrive();                                // this CTA has received everything
+      parts = recv;
     }
-    cluster_sync_all();
-    // CTA `split` of the S in the cluster merges rows split, split + S, ...; one warp per row, a lane per 4 columns
-    const int S = gridDim.y;
-    const uint32_t os0 = smem_u32(Os), ml0 = smem_u32(MLs);
-    for (int r = split + S * warp; r < kRows; r += S * (kThreads / 32)) {
-      const int gr = rb * kRows + r;
-      if (gr >= prm.rows_cap) continue;
-      // every remote load of the row is issued before the first use: one round trip through the cluster
-      float2 ml = make_float2(-INFINITY, 0.f);
-      if (lane < S) ml = ld_peer2(peer_smem(ml0 + (uint32_t)r * 8, (uint32_t)lane));
-      float4 v[8];
-#pragma unroll
-      for (int s = 0; s < 8; ++s)
-        v[s] = (s < S && lane * 4 < DH) ? ld_peer4(peer_smem(os0 + (uint32_t)(r * DH + lane * 4) * 4, (uint32_t)s))
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
-      float M = ml.x;
-      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-      const float wgt = ml.x == -INFINITY ? 0.f : expf(ml.x - M);
-      float den = ml.y * wgt;
-      for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
+    for (int i = threadIdx.x; i < slots * (DH / 4); i += kThreads) {
+      const int slot = i / (DH / 4), col = (i - slot * (DH / 4)) * 4, r = split * slots + slot, gr = rb * kRows + r;
+      if (r >= kRows || gr >= prm.rows_cap) continue;
+      float M = -INFINITY;
+      for (int s = 0; s < S; ++s) M = fmaxf(M, *reinterpret_cast<const float*>(parts + (size_t)s * block_bytes + (slots * DH + slot * 4) * 4));
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int s = 0; s < 8; ++s) {
-        const float ws = __shfl_sync(0xffffffffu, wgt, s);
-        if (s < S && ws != 0.f) { a.x += v[s].x * ws; a.y += v[s].y * ws; a.z += v[s].z * ws; a.w += v[s].w * ws; }
+      float den = 0.f;
+      for (int s = 0; s < S; ++s) {
+        const float* blk = reinterpret_cast<const float*>(parts + (size_t)s * block_bytes);
+        const float4 ml = *reinterpret_cast<const float4*>(blk + slots * DH + slot * 4), v = *reinterpret_cast<const float4*>(blk + slot * DH + col);
+        const float w = ml.x == -INFINITY ? 0.f : exp2f(ml.x - M);             // the running maximum is kept in base-2 units
+        den += (ml.y + ml.z) * w;
+        a.x += v.x * w; a.y += v.y * w; a.z += v.z * w; a.w += v.w * w;
       }
-      if (lane * 4 < DH) {
-        const float inv = den > 0.f ? 1.0f / den : 0.f;
-        uint2 u;
-        u.x = pack_bf16(a.x * inv, a.y * inv);
-        u.y = pack_bf16(a.z * inv, a.w * inv);
-        *reinterpret_cast<uint2*>(prm.out + (size_t)(row_base + gr) * prm.n_heads * DH + h * DH + lane * 4) = u;
-      }
+      const float inv = den > 0.f ? 1.0f / den : 0.f;
+      *reinterpret_cast<uint2*>(prm.out + (size_t)(row_base + gr) * prm.n_heads * DH + h * DH + col) =
+          make_uint2(pack_bf16(a.x * inv, a.y * inv), pack_bf16(a.z * inv, a.w * inv));
     }
-    cluster_sync_all();                                // nobody leaves while a peer may still read its shared memory
+    __syncwarp();
+    if (S > 1) cluster_wait();                         // nobody leaves while a copy may still read its shared memory
   } else {
+    constexpr float kLn2 = 0.6931471805599453f;        // the separate merge works in natural units
     if (warp >= 2) {
-      const int ga = rb * kRows + row_a;
+      l_a = sum_s[0][row_a] + sum_s[1][row_a];
+      l_b = sum_s[0][row_a + 8] + sum_s[1][row_a + 8];
 #pragma unroll
       for (int hi = 0; hi < 2; ++hi) {
-        const int gr = ga + 8 * hi;
+        const int gr = rb * kRows + row_a + 8 * hi;
         if (gr >= prm.rows_cap) continue;
         const size_t o = ((size_t)split * prm.n_heads + h) * prm.rows_cap + gr;
 #pragma unroll
-        for (int rep = 0; rep < DH / 8; ++rep)
-          *reinterpret_cast<float2*>(prm.po + o * DH + 8 * rep + 2 * qd) = make_float2(acc[4 * rep + 2 * hi], acc[4 * rep + 2 * hi + 1]);
-        if (qd == 0) { prm.pml[o * 2] = (hi ? m_b : m_a) * kLn2; prm.pml[o * 2 + 1] = hi ? l_b : l_a; }
+        for (int k = 0; k < DH / 16; ++k)
+          *reinterpret_cast<float2*>(prm.po + o * DH + DH / 2 * half + 8 * k + 2 * qd) = make_float2(acc[4 * k + 2 * hi], acc[4 * k + 2 * hi + 1]);
+        if (half == 0 && qd == 0) { prm.pml[o * 2] = (hi ? m_b : m_a) * kLn2; prm.pml[o * 2 + 1] = hi ? l_b : l_a; }
       }
     }
   }
+  if (threadIdx.x == 0 && abort_flag && prm.err_flag) *prm.err_flag = AMPH_ERR_TIMEOUT;
 }
 
 typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
