@@ -1024,7 +1024,8 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
     const int cnt = n - start < Gmax * M ? n - start : Gmax * M;
     const bool last = start + cnt == n;
     const int G = (cnt + M - 1) / M;
-    const int rpg = G == 1 ? round_up(cnt, 16) : M;          // rows the kernels carry per group
+    // rows the kernels carry per group: the chunks of a pass are of equal height (130 tokens: 2 x 80 rows, not 2 x 128)
+    const int rpg = round_up((cnt + G - 1) / G, 16);
     rc = cuda_check(ctx, cudaMemcpyAsync(ctx->at<int>(l.tok), prompt_ids + start, sizeof(int) * cnt, cudaMemcpyHostToDevice, st), "prompt upload");
     if (rc != AMPH_OK) return rc;
     Pass ps;
@@ -1032,11 +1033,11 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
     ps.rpg = rpg;
     bind_tables(ctx, &ps, false, PassRows::kChain);
     for (int g = 0; g < G; ++g) {
-      const int nr = cnt - g * M < M ? cnt - g * M : M;
-      ps.src.base[g] = start + g * M;
+      const int nr = cnt - g * rpg < rpg ? cnt - g * rpg : rpg;
+      ps.src.base[g] = start + g * rpg;
       ps.src.n[g] = nr;
       ps.seq[g] = seq;
-      ps.keys[g] = start + g * M + nr;
+      ps.keys[g] = start + g * rpg + nr;
     }
     target_forward(ctx, ps);
     if (last) target_head(ctx, ps.rows());
@@ -1045,15 +1046,15 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
       rc = cuda_check(ctx, cudaMemcpyAsync(ctx->at<int>(l.next_tok), prompt_ids + start + 1, sizeof(int) * nrs, cudaMemcpyHostToDevice, st), "prompt upload");
       if (rc != AMPH_OK) return rc;
       Pass pss;
-      pss.G = (nrs + M - 1) / M;
+      pss.G = (nrs + rpg - 1) / rpg;
       pss.rpg = rpg;
       bind_tables(ctx, &pss, true, PassRows::kChain);
       for (int g = 0; g < pss.G; ++g) {
-        const int nr = nrs - g * M < M ? nrs - g * M : M;
-        pss.src.base[g] = start + g * M;
+        const int nr = nrs - g * rpg < rpg ? nrs - g * rpg : rpg;
+        pss.src.base[g] = start + g * rpg;
         pss.src.n[g] = nr;
         pss.seq[g] = seq;
-        pss.keys[g] = start + g * M + nr;
+        pss.keys[g] = start + g * rpg + nr;
       }
       run_sals(ctx, ctx->at<float>(l.hidden), ctx->at<int>(l.next_tok), sizeof(int) * rpg, pss);
     }
