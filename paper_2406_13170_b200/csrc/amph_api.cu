@@ -106,7 +106,14 @@ struct amph_ctx {
   cudaEvent_t join_ev = nullptr;
   bool side_dirty = false;                // helpers were launched since the last join
   // captured draft -> verify -> accept schedules of amph_step, by the attention grids they were sized for
-  struct StepGraph { long long key; cudaGraphExec_t exec; unsigned long long used; };
+  struct StepGraph {
+    long long key;
+    cudaGraphExec_t exec;
+    unsigned long long used;
+    cudaGraph_t graph;                    // owns the nodes; accept: the one that writes a step's results (NULL: not found)
+    cudaGraphNode_t accept;
+    int *out_tokens, *out_n;              // where it writes them now
+  };
   std::vector<StepGraph> graphs;          // at most kMaxGraphs
   unsigned long long graph_tick = 0;
   bool graph_off = false;   // capture is not possible (legacy stream, flag) or failed once
@@ -123,7 +130,12 @@ struct amph_ctx {
   DevState* state(int b) const { return grp<DevState>(lay.state, lay.state_s, b); }
   RowMeta* meta_v(int g) const { return grp<RowMeta>(lay.meta_v, lay.meta_s_, g); }
   RowMeta* meta_s(int g) const { return grp<RowMeta>(lay.meta_s, lay.meta_s_, g); }
-  void drop_graphs() { for (auto& g : graphs) cudaGraphExecDestroy(g.exec); graphs.clear(); }
+  void drop_graph(size_t i) {
+    cudaGraphExecDestroy(graphs[i].exec);
+    cudaGraphDestroy(graphs[i].graph);
+    graphs.erase(graphs.begin() + i);
+  }
+  void drop_graphs() { while (!graphs.empty()) drop_graph(graphs.size() - 1); }
   int max_ctx_hi() const { int m = 0; for (int b = 0; b < B; ++b) m = ctx_hi[b] > m ? ctx_hi[b] : m; return m; }
 };
 
@@ -804,13 +816,9 @@ void join_side(amph_ctx* ctx) {
   ctx->fork_used = 0;
 }
 
-// out_tokens, out_path: [B][K+1]; out_n, out_next_root: [B]
-amph_status do_accept(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n, int32_t* out_path, int32_t* out_next_root) {
+AcceptArgs accept_args(const amph_ctx* ctx) {
   const amph_config& c = ctx->cfg;
   const Layout& l = ctx->lay;
-  cudaStream_t st = ctx->stream;
-  join_side(ctx);
-  { ProfScope p(ctx, AMPH_PROF_ACCEPT);
   AcceptArgs a;
   a.tree = ctx->at<TreeDev>(l.tree);
   a.state = ctx->ws + l.state;    a.state_stride = l.state_s;
@@ -823,14 +831,68 @@ amph_status do_accept(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n, int32_
   a.hidden = ctx->at<float>(l.hidden);
   a.pend_h = ctx->at<float>(l.pend_h);
   a.pend_rows = kSmallRows;
-  launch_accept_compact(a, ctx->B, ctx->dtype, st);
+  a.out_tokens = a.out_n = nullptr;
+  a.out_k = c.K + 1;
+  return a;
+}
+
+// out_tokens, out_path: [B][K+1]; out_n, out_next_root: [B]
+amph_status do_accept(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n, int32_t* out_path, int32_t* out_next_root) {
+  join_side(ctx);
+  { ProfScope p(ctx, AMPH_PROF_ACCEPT);
+  launch_accept_compact(accept_args(ctx), ctx->B, ctx->dtype, ctx->stream);
   }
   const DevState* ds = ctx->state(0);
-  amph_status rc = copy_out_seq(ctx, out_tokens, ds->out_tok, c.K + 1);
+  amph_status rc = copy_out_seq(ctx, out_tokens, ds->out_tok, ctx->cfg.K + 1);
   if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_n, &ds->L, 1);
-  if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_path, ds->path, c.K + 1);
+  if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_path, ds->path, ctx->cfg.K + 1);
   if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_next_root, &ds->next_root, 1);
   return rc;
+}
+
+// Whether a kernel of this context may write to p.
+bool device_memory(const void* p) {
+  if (!p) return true;
+  cudaPointerAttributes at;
+  int dev = 0;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
+  return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
+// Points a captured step's results at the caller's arrays (*written), or at none: the caller copies them.  False: the schedule
+// could not be changed and may hold an earlier call's arrays, so it must not run again.
+bool redirect_results(amph_ctx* ctx, amph_ctx::StepGraph* g, int32_t* out_tokens, int32_t* out_n, bool* written) {
+  *written = g->accept && device_memory(out_tokens) && device_memory(out_n);
+  if (!*written) out_tokens = out_n = nullptr;
+  if (g->out_tokens == out_tokens && g->out_n == out_n) return true;
+  cudaKernelNodeParams np;
+  AcceptArgs a = accept_args(ctx);
+  a.out_tokens = out_tokens;
+  a.out_n = out_n;
+  void* args[1] = {&a};
+  if (cudaGraphKernelNodeGetParams(g->accept, &np) != cudaSuccess) return false;
+  np.kernelParams = args;
+  np.extra = nullptr;
+  if (cudaGraphExecKernelNodeSetParams(g->exec, g->accept, &np) != cudaSuccess) return false;
+  g->out_tokens = out_tokens;
+  g->out_n = out_n;
+  return true;
+}
+
+// The node of the kernel that ends a captured step.
+cudaGraphNode_t find_accept_node(const amph_ctx* ctx, cudaGraph_t graph) {
+  size_t n = 0;
+  if (cudaGraphGetNodes(graph, nullptr, &n) != cudaSuccess) return nullptr;
+  std::vector<cudaGraphNode_t> nodes(n);
+  if (cudaGraphGetNodes(graph, nodes.data(), &n) != cudaSuccess) return nullptr;
+  for (size_t i = n; i-- > 0;) {
+    cudaGraphNodeType t;
+    cudaKernelNodeParams np;
+    if (cudaGraphNodeGetType(nodes[i], &t) == cudaSuccess && t == cudaGraphNodeTypeKernel &&
+        cudaGraphKernelNodeGetParams(nodes[i], &np) == cudaSuccess && np.func == accept_compact_function(ctx->dtype))
+      return nodes[i];
+  }
+  return nullptr;
 }
 
 int attn_splits_for(const amph_ctx* ctx, int ctx_hi, int rows, int groups) {
@@ -1125,15 +1187,16 @@ amph_status amph_step(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n) {
   if (rc != AMPH_OK) return rc;
   const amph_config& c = ctx->cfg;
   const bool use_graph = !ctx->graph_off && !ctx->prof_on && !(c.flags & AMPH_FLAG_NO_GRAPH) && ctx->stream != nullptr;
-  cudaGraphExec_t exec = nullptr;
+  amph_ctx::StepGraph* sg = nullptr;
   if (use_graph) {
     // The kernels read every length from device state; only the attention grids depend on the host's
     // bound of the context length, so a captured schedule serves every step with the same grids.
     const long long key = graph_key_of(ctx);
     for (auto& g : ctx->graphs)
-      if (g.key == key) { exec = g.exec; g.used = ++ctx->graph_tick; }
-    if (!exec) {
+      if (g.key == key) sg = &g;
+    if (!sg) {
       cudaGraph_t graph = nullptr;
+      cudaGraphExec_t exec = nullptr;
       if (cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
         rc = do_draft(ctx, nullptr, nullptr);
         if (rc == AMPH_OK) rc = do_verify(ctx, nullptr, nullptr);
@@ -1144,31 +1207,43 @@ amph_status amph_step(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n) {
             size_t old = 0;                                // CUDA keeps a launched executable until it has finished)
             for (size_t i = 1; i < ctx->graphs.size(); ++i)
               if (ctx->graphs[i].used < ctx->graphs[old].used) old = i;
-            cudaGraphExecDestroy(ctx->graphs[old].exec);
-            ctx->graphs.erase(ctx->graphs.begin() + old);
+            ctx->drop_graph(old);
           }
-          ctx->graphs.push_back({key, exec, ++ctx->graph_tick});
+          ctx->graphs.push_back({key, exec, 0, graph, find_accept_node(ctx, graph), nullptr, nullptr});
+          sg = &ctx->graphs.back();
         } else {
-          exec = nullptr;
           ctx->graph_off = true;
+          if (graph) cudaGraphDestroy(graph);
         }
-        if (graph) cudaGraphDestroy(graph);
       } else {
         ctx->graph_off = true;
       }
       cudaGetLastError();
     }
   }
-  if (exec) {
-    rc = cuda_check(ctx, cudaGraphLaunch(exec, ctx->stream), "graph launch");
-  } else {
+  bool written = false;
+  if (sg) {
+    sg->used = ++ctx->graph_tick;
+    // The results go straight to the caller's arrays where the step's last kernel can write them (device memory): two copies
+    // behind every step cost 6 us of a small model's 160.
+    if (redirect_results(ctx, sg, out_tokens, out_n, &written)) {
+      rc = cuda_check(ctx, cudaGraphLaunch(sg->exec, ctx->stream), "graph launch");
+    } else {
+      cudaGetLastError();
+      ctx->drop_graphs();
+      ctx->graph_off = true;
+      written = false;
+      sg = nullptr;
+    }
+  }
+  if (!sg) {
     rc = do_draft(ctx, nullptr, nullptr);
     if (rc == AMPH_OK) rc = do_verify(ctx, nullptr, nullptr);
     if (rc == AMPH_OK) rc = do_accept(ctx, nullptr, nullptr, nullptr, nullptr);
   }
   const DevState* ds = ctx->state(0);
-  if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_tokens, ds->out_tok, c.K + 1);
-  if (rc == AMPH_OK) rc = copy_out_seq(ctx, out_n, &ds->L, 1);
+  if (rc == AMPH_OK && !written) rc = copy_out_seq(ctx, out_tokens, ds->out_tok, c.K + 1);
+  if (rc == AMPH_OK && !written) rc = copy_out_seq(ctx, out_n, &ds->L, 1);
   if (rc == AMPH_OK) rc = finish(ctx, "step");
   if (rc == AMPH_OK)
     for (int b = 0; b < ctx->B; ++b) ctx->ctx_hi[b] += c.K + 1;

@@ -255,7 +255,11 @@ struct AcceptArgs {
   const float* hidden;                         // [B][rows][d]
   float* pend_h;                               // [B][pend_rows][d]
   int pend_rows;
+  int* out_tokens;                             // [B][out_k] accepted tokens (-1 behind them), or NULL
+  int* out_n;                                  // [B] accepted counts, or NULL
+  int out_k;
 };
+const void* accept_compact_function(int dtype);      // the kernel, to find its node in a captured graph
 void launch_accept_compact(const AcceptArgs& a, int batch, int dtype, cudaStream_t st);
 // Sampling at temperature T > 0 (Table 2): choice[row] for rows row0 + b * rows_per + r, r < n_rows, of every sequence b = the
 // token the target draws after that row from softmax(logits / T) with the row's own uniform (Philox4x32-10 keyed by seed; counter

@@ -1260,7 +1260,13 @@ accept_compact_kernel(const AcceptArgs a) {
     s->root = nr;
     s->n_pending = L;
     s->step += 1;
+    for (int i = 0; a.out_tokens != nullptr && i < a.out_k; ++i) a.out_tokens[b * a.out_k + i] = i < L ? tok[path_s[i]] : -1;
+    if (a.out_n != nullptr) a.out_n[b] = L;
   }
+}
+
+const void* accept_compact_function(int dtype) {
+  return dtype == AMPH_DTYPE_F32 ? (const void*)accept_compact_kernel<float> : (const void*)accept_compact_kernel<bf16>;
 }
 
 void launch_accept_compact(const AcceptArgs& a, int batch, int dtype, cudaStream_t st) {

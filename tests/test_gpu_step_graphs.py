@@ -37,3 +37,36 @@ def test_lengths_that_come_back(name, lengths):
         assert _decode(graphs, prompts, 2) == _decode(plain, prompts, 2), (a, b)
     graphs.close()
     plain.close()
+
+
+@pytest.mark.parametrize("batch", [1, 3])
+def test_results_reach_whatever_arrays_a_step_is_given(batch):
+    """Device arrays, other device arrays, pinned and pageable host arrays, one of the two, none: each call's results arrive where
+    that call asked for them, and nowhere else."""
+    from paper_2406_13170_b200 import Amphista
+    shape = inputs.get_shape("small_bf16")
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    prompts = [inputs.make_prompt(shape.with_(prompt_len=n), seed=n).tolist() for n in (40, 130, 17)[:batch]]
+    K = shape.K
+    make = {"device": lambda s: torch.full(s, -7, dtype=torch.int32, device="cuda:0"),
+            "pinned": lambda s: torch.full(s, -7, dtype=torch.int32).pin_memory(), "pageable": lambda s: torch.full(s, -7, dtype=torch.int32),
+            "none": lambda s: None}
+    kinds = [("device", "device"), ("device", "device"), ("pinned", "pinned"), ("device", "pinned"), ("none", "none"), ("device", "none"),
+             ("pageable", "device"), ("none", "device"), ("device", "device")]
+
+    def run(flags):
+        m = Amphista(shape, topo, w, max_batch=batch, max_ctx=512, flags=flags)
+        for b, p in enumerate(prompts):
+            m.prefill(p, seq=b)
+        outs = []
+        for kt, kn in kinds:
+            t, n = make[kt]((batch, K + 1)), make[kn]((batch,))
+            m.step(t, n)
+            m.synchronize()
+            outs.append((t, n))
+        torch.cuda.synchronize()
+        m.close()
+        return [(None if t is None else t.tolist(), None if n is None else n.tolist()) for t, n in outs]
+
+    assert run(0) == run(2)                       # 2: kernels launched one by one, results copied
