@@ -293,8 +293,8 @@ void make_layout(const amph_config& c, int n_nodes, Layout* L, int* Mcap_out, si
   l.att_o = l.per_group(4 * (size_t)splits * c.n_heads * Mcap * c.head_dim, &l.att_o_s);
   l.att_ml = l.per_group(4 * (size_t)splits * c.n_heads * Mcap * 2, &l.att_ml_s);
   l.logits = l.take(4 * (size_t)Rcap * V);
-  l.ss_a = l.take(4 * (size_t)Rcap * 32);
-  l.ss_b = l.take(4 * (size_t)Rcap * 32);
+  l.ss_a = l.take(4 * (size_t)Rcap * (c.d_model / kWideScaleCols + 32));
+  l.ss_b = l.take(4 * (size_t)Rcap * (c.d_model / kWideScaleCols + 32));
   l.wide_flags = l.take(sizeof(int) * kWideFlags);
   *L = l;
   *Mcap_out = Mcap;
@@ -413,10 +413,11 @@ PartialView project_impl(amph_ctx* ctx, int xb, const void* const* w, int n_seg,
   return pv;
 }
 
-RowScale row_scale_of(const amph_ctx* ctx, size_t off) {
+// cols: columns per entry of the sums of squares
+RowScale row_scale_of(const amph_ctx* ctx, size_t off, int cols) {
   RowScale rs;
   rs.ss = ctx->at<float>(off);
-  rs.chunks = (ctx->cfg.d_model + kScaleChunkCols - 1) / kScaleChunkCols;
+  rs.chunks = (ctx->cfg.d_model + cols - 1) / cols;
   rs.d = ctx->cfg.d_model;
   rs.eps = ctx->cfg.rms_eps;
   return rs;
@@ -492,18 +493,18 @@ void fork_prefetch(amph_ctx* ctx, const LayerW& w, int rows) {
 // One decoder layer over the rows of the pass; cache_of(seq) gives the layer's cache of a sequence.
 // Entry: xn holds the input of the q/k/v projections: attn_norm * x / rms(x) if !entry_deferred, else
 // attn_norm * x with the row sums of squares in ss_a (the division is applied after the projection).
-// Exit: x is updated.  With next_gain and no hid: xn = next_gain * x, sums of squares in ss_a (deferred form
-// for the next layer; returns true).  With hid: xn and hid hold the normalised rows (returns false).
+// Exit: x is updated.  With next_gain and no hid: xn = next_gain * x, sums of squares in ss_a (deferred form for the next layer;
+// returns the columns per entry).  With hid: xn and hid hold the normalised rows (returns 0).
 template <typename CacheOf>
-bool layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, const Pass& ps, const void* next_gain,
-                   float* hid, bool entry_deferred) {
+int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, const Pass& ps, const void* next_gain,
+                  float* hid, int entry_deferred) {
   const amph_config& c = ctx->cfg;
   const Layout& l = ctx->lay;
   cudaStream_t st = ctx->stream;
   const int rows = ps.rows();
   const size_t d = c.d_model;
   const void* qkv[3] = {w.wq, w.wk, w.wv};
-  const RowScale rs = entry_deferred ? row_scale_of(ctx, l.ss_a) : RowScale();
+  const RowScale rs = entry_deferred ? row_scale_of(ctx, l.ss_a, entry_deferred) : RowScale();
   PartialView P = {nullptr, 0, 0, 0};
   bool fused_rope = false;
   RopeGroups gr;
@@ -572,21 +573,34 @@ bool layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, c
       launch_tree_attention(qg, kv, ps.meta[g], sc, og, ctx->dtype, ps.rpg, c.n_heads, c.head_dim, c.max_ctx, ps.keys[g],
                             l.attn_splits, st, last_g && ctx->tc != nullptr, (c.flags & AMPH_FLAG_SEPARATE_MERGE) != 0);
   }
-  const void* wo[1] = {w.wo};
-  P = project(ctx, XB_ATT, wo, 1, c.d_model, c.d_model, rows);
-  { ProfScope p(ctx, AMPH_PROF_NORM);
-  launch_resid_scale(x, P, 0, 1, w.ffn_norm, ctx->dtype, ctx->ws + l.xn, ctx->at<float>(l.ss_b), rows, c.d_model, st,
-                     ctx->last_proj_one_wave);
+  // output projection and residual update: one kernel for many rows
+  auto resid_fused = [&](int xb, const void* wt, int in, const void* gain, size_t ss) {
+    if (!ctx->tc || rows <= kWideFrom) return false;
+    ProfScope p(ctx, AMPH_PROF_PROJECTION);
+    const bool done = tc_wide_launch_resid(ctx->tc, xb, wt, c.d_model, in, rows, x, gain, ctx->ws + l.xn, ctx->at<float>(ss), st);
+    if (!done) cudaGetLastError();
+    if (done && p.rec) ctx->prof_bytes += (int64_t)c.d_model * in * (int64_t)ctx->esz;
+    if (done) ctx->last_proj_one_wave = false;
+    return done;
+  };
+  const bool fused_o = resid_fused(XB_ATT, w.wo, c.d_model, w.ffn_norm, l.ss_b);
+  if (!fused_o) {
+    const void* wo[1] = {w.wo};
+    P = project(ctx, XB_ATT, wo, 1, c.d_model, c.d_model, rows);
+    ProfScope p(ctx, AMPH_PROF_NORM);
+    launch_resid_scale(x, P, 0, 1, w.ffn_norm, ctx->dtype, ctx->ws + l.xn, ctx->at<float>(l.ss_b), rows, c.d_model, st,
+                       ctx->last_proj_one_wave);
   }
+  const RowScale rs_b = row_scale_of(ctx, l.ss_b, fused_o ? kWideScaleCols : kScaleChunkCols);
   bool fused_gu = false;
   if (ctx->tc && !(c.flags & AMPH_FLAG_SEPARATE_SWIGLU)) {         // gate / up projection with SwiGLU in its epilogue
     ProfScope p(ctx, AMPH_PROF_PROJECTION);
     if (rows > kWideFrom)
       fused_gu = tc_wide_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act,
-                                       row_scale_of(ctx, l.ss_b), st);
+                                       rs_b, st);
     else
       fused_gu = tc_gemm_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act,
-                                       row_scale_of(ctx, l.ss_b), st);
+                                       rs_b, st);
     if (fused_gu && p.rec) ctx->prof_bytes += 2LL * c.d_ffn * c.d_model * (int64_t)ctx->esz;
     if (fused_gu) ctx->last_proj_one_wave = false;
   }
@@ -594,18 +608,19 @@ bool layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, c
     const void* gu[2] = {w.w_gate, w.w_up};
     P = project(ctx, XB_XN, gu, 2, c.d_ffn, c.d_model, rows);
     ProfScope p(ctx, AMPH_PROF_SWIGLU);
-    launch_swiglu(P, ctx->ws + l.act, ctx->dtype, rows, c.d_ffn, st, row_scale_of(ctx, l.ss_b), ctx->last_proj_one_wave);
+    launch_swiglu(P, ctx->ws + l.act, ctx->dtype, rows, c.d_ffn, st, rs_b, ctx->last_proj_one_wave);
   }
+  if (hid == nullptr && resid_fused(XB_ACT, w.w_down, c.d_ffn, next_gain, l.ss_a)) return next_gain ? kWideScaleCols : 0;
   const void* wd[1] = {w.w_down};
   P = project(ctx, XB_ACT, wd, 1, c.d_model, c.d_ffn, rows);
   ProfScope p(ctx, AMPH_PROF_NORM);
   if (hid != nullptr) {
     launch_resid_norm(x, P, 0, 1, next_gain, ctx->dtype, ctx->ws + l.xn, hid, c.rms_eps, rows, c.d_model, st);
-    return false;
+    return 0;
   }
   launch_resid_scale(x, P, 0, 1, next_gain, ctx->dtype, ctx->ws + l.xn, ctx->at<float>(l.ss_a), rows, c.d_model, st,
                      ctx->last_proj_one_wave && next_gain != nullptr);
-  return next_gain != nullptr;
+  return next_gain ? kScaleChunkCols : 0;
 }
 
 // Target forward of the tokens in `tok` (one per row of the pass); leaves post-final-norm rows in hidden and xn.
@@ -618,7 +633,7 @@ void target_forward(amph_ctx* ctx, const Pass& ps) {
   launch_target_rows(ps.src, ps.G, ctx->tok_emb, ctx->dtype, ctx->at<int>(l.tok), c.vocab, c.d_model, ctx->layers[0].attn_norm, c.rms_eps, x,
                      ctx->ws + l.xn, st);
   }
-  bool deferred = false;
+  int deferred = 0;
   for (int i = 0; i < c.n_layers; ++i) {
     const bool last = i + 1 == c.n_layers;
     deferred = layer_forward(ctx, ctx->layers[i], [&](int b) { return ctx->kv_target[b][i]; }, x, ps,
@@ -658,7 +673,7 @@ void run_sals(amph_ctx* ctx, const float* feat, const int* next_tok, size_t next
     launch_resid_norm(hbuf, P, 0, 2, ctx->sal[s].attn_norm, ctx->dtype, ctx->ws + l.xn, nullptr, c.rms_eps, rows,
                       c.d_model, st);
     }
-    layer_forward(ctx, ctx->sal[s], [&](int b) { return ctx->kv_sal[b][s]; }, hbuf, ps, nullptr, nullptr, false);
+    layer_forward(ctx, ctx->sal[s], [&](int b) { return ctx->kv_sal[b][s]; }, hbuf, ps, nullptr, nullptr, 0);
     in_feat = hbuf;
   }
 }

@@ -117,8 +117,16 @@ __device__ __forceinline__ float4 sum_partials4(const PartialView& P, int row, i
 __device__ __forceinline__ float row_scale(const RowScale& rs, int row) {
   if (rs.ss == nullptr) return 1.0f;
   float tot = 0.f;
+  if (rs.chunks % 4 == 0) {
 #pragma unroll 8
-  for (int c = 0; c < rs.chunks; ++c) tot += rs.ss[row * rs.chunks + c];       // fixed order
+    for (int c = 0; c < rs.chunks; c += 4) {                                    // fixed order
+      const float4 v = *reinterpret_cast<const float4*>(rs.ss + row * rs.chunks + c);
+      tot += v.x; tot += v.y; tot += v.z; tot += v.w;
+    }
+  } else {
+#pragma unroll 8
+    for (int c = 0; c < rs.chunks; ++c) tot += rs.ss[row * rs.chunks + c];
+  }
   return 1.0f / sqrtf(tot / (float)rs.d + rs.eps);
 }
 #endif

@@ -44,6 +44,10 @@ void tc_wide_init(TcGemm* g);
 void tc_wide_bind(TcGemm* g, float* scratch, size_t scratch_floats, int* flags);
 bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out, int in, int rows, float* P, size_t p_floats,
                     int* splits, size_t* split_stride, cudaStream_t st);
+// Residual update in the epilogue: x += X . W^T and, with gain, xn <- gain * x (bf16) and ss[row][out / 128] <- sums of squares.
+constexpr int kWideScaleCols = 128;      // columns per entry of ss
+bool tc_wide_launch_resid(TcGemm* g, int xb, const void* w, int out, int in, int rows, float* x, const void* gain, void* xn, float* ss,
+                          cudaStream_t st);
 bool tc_wide_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_up, int f, int in, int rows, void* act, const RowScale& rs,
                            cudaStream_t st);
 bool tc_wide_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, const void* wv, int n_heads, int dh, int in, int rows, void* q,

@@ -173,6 +173,7 @@ struct TcGemm {
   float* wide_scratch = nullptr;
   size_t wide_scratch_floats = 0;
   int* wide_flags = nullptr;
+  int resid_clusters[5] = {0, 0, 0, 0, 0};     // clusters of that many pairs that run at a time (residual form)
 
   const CUtensorMap* get(const void* ptr, int rows, int cols, int box_rows, int box_kb = tc::kStageKb) {
     auto key = std::make_tuple(ptr, rows, cols, box_rows, box_kb);

@@ -14,7 +14,14 @@
 // flag) and may end inside one (the pair that holds a tile's first K columns waits for the flags of the groups after it, adds
 // their sums in order and runs the epilogue).  A flag is raised before its pair waits for anybody, and pairs are numbered
 // against the launch order, so a pair only ever waits for pairs that became resident before it; the wait is bounded all the
-// same.  Where the consumer adds split-K sums anyway (output and down projections) the K ranges are cut evenly per tile.
+// same.  Where the consumer adds split-K sums anyway the K ranges are cut evenly per tile.
+//
+// Output and down projection (WIDE_RESID) have few tiles (16 at d = 4096), so several pairs share one along K and all of them
+// finish it: the pairs of a tile form a cluster, each gets a share of the tile's rows from the others by bulk copies through
+// distributed shared memory, adds them in K order and applies the residual update.  Through global memory instead (sums
+// written, a second kernel that adds them) d = 4096 / d_ffn = 11008 took, mean of the two: 128 rows 15.2 + 2.9 us, now 18.1; 256
+// rows 20.9 + 5.6, now 27.0; 512 rows 28.0 + 8.8, now 31.8.  The projection behind it, whose ring fills while this one drains,
+// starts 1-2 us earlier as well: a prefill of 512 rows took 8.80 ms, now 8.43, a batch of 8 x 40 nodes 90.2 ms, now 87.5.
 //
 // Warp roles: 0 = TMA producer, 1 = MMA issuer (of the even CTA), 2-17 = epilogue.
 #include "gemm_tc_common.cuh"
@@ -36,7 +43,7 @@ struct WideMaps {
   CUtensorMap x;
 };
 
-enum { WIDE_PLAIN = 0, WIDE_SWIGLU = 1, WIDE_ROPE = 2 };
+enum { WIDE_PLAIN = 0, WIDE_SWIGLU = 1, WIDE_ROPE = 2, WIDE_RESID = 3 };
 
 struct WideParams {
   int tiles_per_seg, tiles;
@@ -52,6 +59,11 @@ struct WideParams {
   int ld;
   float* scratch;           // [pair][cta][quad of rows][128 features] float4: partial sums of a pair's first segment
   int* flags;               // [pair][cta]; zero between launches (whoever consumes a flag lowers it)
+  float* x;                 // RESID: residual rows, updated in place
+  const __nv_bfloat16* gain;      // the next norm's gain, or NULL: x only
+  __nv_bfloat16* xn;        // gain * x
+  float* ss;                // [row][out / 128] sums of squares
+  int out;
   __nv_bfloat16* act;       // SWIGLU
   int f, up_first;
   RowScale rs;
@@ -107,6 +119,18 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// Execution order only (see the uses).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
+// shared memory of this CTA -> shared memory of a CTA of the cluster; the bytes are counted by a barrier there
+__device__ __forceinline__ void bulk_to_peer(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "r"(smem_u32(src)), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ float4 bf16x4(const __nv_bfloat16* p) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+}
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
@@ -138,9 +162,9 @@ __device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t adesc, uint6
       : "memory");
 }
 // Arrives at the same barrier of both CTAs once the MMAs issued so far are complete.
-__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
+__device__ __forceinline__ void umma_commit_pair(uint64_t* bar, uint32_t lead) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+               ::"r"(smem_u32(bar)), "h"((uint16_t)(3u << lead)) : "memory");
 }
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
   uint32_t r[8];
@@ -167,18 +191,24 @@ template <int EPI>
 __global__ void __launch_bounds__(kWideThreads, 1)
 tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ float inv_s[EPI == WIDE_PLAIN ? 1 : 256];             // 1 / rms of this pair's activation rows
+  constexpr bool SCALED = EPI == WIDE_SWIGLU || EPI == WIDE_ROPE;   // the activation rows' RMS division is still to be done
+  __shared__ float inv_s[SCALED ? 256 : 1];                        // 1 / rms of this pair's activation rows
   __shared__ int slot_s[EPI == WIDE_ROPE ? 256 : 1];               // cache slot of a row, -1: not stored
   __shared__ const float2* table_s[EPI == WIDE_ROPE ? 256 : 1];    // its rotary table row
-  __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], accum_full[2], accum_empty[2];
+  __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], accum_full[2], accum_empty[2], recv_full;
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_rank();
-  const int pair = prm.groups * prm.nrb - 1 - (int)(blockIdx.x >> 1);        // against the launch order (see above)
-  const int group = pair / prm.nrb, rb = pair - group * prm.nrb;
+  const uint32_t crank = cluster_rank(), rank = crank & 1u, lead = crank & ~1u;     // in the cluster, in the pair; the pair's even CTA
+  int pair = prm.groups * prm.nrb - 1 - (int)(blockIdx.x >> 1);              // against the launch order (see above)
+  int group = pair / prm.nrb, rb = pair - group * prm.nrb;
+  if constexpr (EPI == WIDE_RESID) {                                         // a cluster holds the splits of one tile and row block
+    const int item = (int)blockIdx.x / (2 * prm.splits);
+    rb = item % prm.nrb;
+    group = item / prm.nrb * prm.splits + (int)(crank >> 1);
+  }
   const int stages = prm.stages, n = prm.n;
   const uint32_t b_tile = (uint32_t)n / 2 * 128, a_tile = kTileM * 128;         // one K block of each operand
   const uint32_t stage_bytes = kUnitKb * (a_tile + b_tile);
@@ -191,6 +221,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     abort_flag = 0;
     for (int s = 0; s < stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
     for (int s = 0; s < 2; ++s) { mbar_init(&accum_full[s], 1); mbar_init(&accum_empty[s], 2 * kEpiThreads / 32); }
+    mbar_init(&recv_full, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -209,14 +240,14 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     const uint64_t wpol = l2_evict_first_policy();
     auto load_w = [&](int st, const Segment& s, int u) {
       const int seg = s.tile / prm.tiles_per_seg, lt = s.tile - seg * prm.tiles_per_seg;
-      const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), 0);
+      const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), lead);
       uint8_t* dst = smem + (size_t)st * stage_bytes;
       if (rank == 0) mbar_expect_tx(&full_bar[st], 2 * stage_bytes);
       if (EPI == WIDE_SWIGLU) tma_pair_4d(dst, &maps.w[0], 0, (lt * 2 + (int)rank) * (kTileM / 2), 0, u * kUnitKb, bar, wpol);
       else tma_pair_3d(dst, &maps.w[seg], 0, (lt * 2 + (int)rank) * kTileM, u * kUnitKb, bar, wpol);
     };
     auto load_x = [&](int st, int u) {
-      const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), 0);
+      const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), lead);
       tma_pair_3d(smem + (size_t)st * stage_bytes + kUnitKb * a_tile, &maps.x, 0, rb * n + (int)rank * (n / 2), u * kUnitKb, bar);
     };
     // weights do not depend on the kernel before: fill the ring with them, then wait, then fetch those stages' activations
@@ -282,11 +313,11 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
               for (int k = 0; k < kTileK / kUmmaK; ++k)
                 umma_pair(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, u > sg.u0 || kk > 0 || k > 0 ? 1u : 0u);
             }
-            umma_commit_pair(&empty_bar[st]);
+            umma_commit_pair(&empty_bar[st], lead);
           }
           __syncwarp();
         }
-        if (ok && leader) umma_commit_pair(&accum_full[as]);
+        if (ok && leader) umma_commit_pair(&accum_full[as], lead);
         __syncwarp();
       }
     }
@@ -295,7 +326,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     const int quarter = warp & 3, sub = (warp - 2) >> 2, et = threadIdx.x - 64;
     const int row0 = rb * n, my_rows = prm.rows - row0 < n ? prm.rows - row0 : n;
     pdl_wait();
-    if constexpr (EPI != WIDE_PLAIN) {
+    if constexpr (SCALED) {
       if (et < my_rows) inv_s[et] = row_scale(prm.rs, row0 + et);
     }
     if constexpr (EPI == WIDE_ROPE) {
@@ -321,8 +352,79 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
       auto release = [&]() {                             // this warp has read the accumulator
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&accum_empty[as]), 0));
+        if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&accum_empty[as]), lead));
       };
+      if constexpr (EPI == WIDE_RESID) {
+        const int S = prm.splits, split = (int)(crank >> 1), per = ((n + S - 1) / S + 7) / 8 * 8;       // rows of a share
+        const int lo = split * per, hi = lo + per < my_rows ? lo + per : my_rows;
+        float* const park = reinterpret_cast<float*>(smem);                    // [n][128]: the ring is free
+        uint8_t* const recv = smem + (size_t)n * kTileM * 4;                   // the other splits' sums of this CTA's share
+        if (S > 1) {
+          __syncwarp();
+          cluster_arrive();                               // this CTA's MMAs have read their operands: peers may write here
+        }
+        for (int r = sub * kChunk; r < my_rows; r += kBatch) {
+          float v[kChunk];
+          tmem_ld8(t0 + (uint32_t)r, v);
+#pragma unroll
+          for (int e = 0; e < kChunk; ++e) park[(r + e) * kTileM + frow] = ok ? v[e] : 0.f;
+        }
+        const uint32_t share = (uint32_t)per * kTileM * 4;
+        if (S > 1) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");         // the copies read through the async proxy
+          epi_sync();
+          __syncwarp();
+          cluster_wait();
+          if (warp == 2) {
+            const uint32_t mine = hi > lo ? (uint32_t)(hi - lo) * kTileM * 4 : 0u;
+            if (lane == 0) mbar_expect_tx(&recv_full, (uint32_t)(S - 1) * mine);
+            __syncwarp();
+            if (lane < S && lane != split) {
+              const int olo = lane * per, ohi = olo + per < my_rows ? olo + per : my_rows;
+              const uint32_t to = (uint32_t)lane * 2 + rank;
+              if (ohi > olo)
+                bulk_to_peer(map_to_rank(smem_u32(recv + (size_t)(split < lane ? split : split - 1) * share), to), park + (size_t)olo * kTileM,
+                             (uint32_t)(ohi - olo) * kTileM * 4, map_to_rank(smem_u32(&recv_full), to));
+            }
+          }
+        } else {
+          epi_sync();
+        }
+        // a warp finishes whole rows of the tile's 128 features, four features a lane; the old values are on their way while
+        // the other splits' sums arrive
+        const int f0 = sg.tile * 256 + (int)rank * kTileM + lane * 4;
+        const float4 gn = prm.gain != nullptr ? bf16x4(prm.gain + f0) : make_float4(0.f, 0.f, 0.f, 0.f);
+        constexpr int kAhead = 4, kStep = kEpiThreads / 32;
+        bool arrived = S == 1;
+        for (int rl = lo + (et >> 5); rl < hi || !arrived; rl += kAhead * kStep) {
+          float4 v[kAhead];
+#pragma unroll
+          for (int q = 0; q < kAhead; ++q)
+            if (rl + q * kStep < hi) v[q] = *reinterpret_cast<const float4*>(prm.x + (size_t)(row0 + rl + q * kStep) * prm.out + f0);
+          if (!arrived) { __all_sync(0xffffffffu, mbar_wait(&recv_full, 0, &abort_flag, limit_ns)); arrived = true; }
+#pragma unroll
+          for (int q = 0; q < kAhead; ++q) {
+            const int r = rl + q * kStep;
+            if (r >= hi) continue;                        // uniform over the warp
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int s = 0; s < S; ++s) {                 // in K order
+              const float4 p = s == split ? *reinterpret_cast<const float4*>(park + (size_t)r * kTileM + lane * 4)
+                                          : *reinterpret_cast<const float4*>(recv + (size_t)(s < split ? s : s - 1) * share + ((size_t)(r - lo) * kTileM + lane * 4) * 4);
+              a.x += p.x; a.y += p.y; a.z += p.z; a.w += p.w;
+            }
+            v[q].x += a.x; v[q].y += a.y; v[q].z += a.z; v[q].w += a.w;
+            *reinterpret_cast<float4*>(prm.x + (size_t)(row0 + r) * prm.out + f0) = v[q];
+            if (prm.gain == nullptr) continue;
+            const __nv_bfloat162 y0 = __floats2bfloat162_rn(gn.x * v[q].x, gn.y * v[q].y), y1 = __floats2bfloat162_rn(gn.z * v[q].z, gn.w * v[q].w);
+            *reinterpret_cast<uint2*>(prm.xn + (size_t)(row0 + r) * prm.out + f0) =
+                make_uint2(*reinterpret_cast<const uint32_t*>(&y0), *reinterpret_cast<const uint32_t*>(&y1));
+            float sq = v[q].x * v[q].x + v[q].y * v[q].y + v[q].z * v[q].z + v[q].w * v[q].w;
+            for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+            if (lane == 0) prm.ss[(size_t)(row0 + r) * (prm.out / kTileM) + sg.tile * 2 + rank] = sq;
+          }
+        }
+        continue;
+      }
       if (prm.splits == 0 && sg.u0 > 0) {                // not the tile's first K columns: leave the sums to the pair that has them
         float4* dst = scratch + ((size_t)pair * 2 + rank) * slot_quads;
         for (int r = sub * kChunk; ok && r < my_rows; r += kBatch) {
@@ -452,6 +554,11 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
       }
     }
   }
+  if (EPI == WIDE_RESID && prm.splits > 1 && warp < 2) {  // the epilogue's barrier of the cluster
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   cluster_sync_all();                                     // no CTA leaves while its partner may still signal or read its shared memory
@@ -463,12 +570,13 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
 }
 
 constexpr size_t kWideSmem = 221 * 1024;                  // ring + alignment; the static part needs up to 5 KB of the 227
+constexpr size_t kResidSmem = 225 * 1024;                 // 256 parked rows and three quarters of them received; 1 KB static
 
 // Everything of a launch that does not depend on the epilogue; false: the shape is not covered.
 template <int EPI>
 bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int rows, int splits, float* scratch_end, size_t scratch_floats,
                  WideMaps* maps, WideParams* prm) {
-  constexpr size_t out_bytes = EPI == WIDE_PLAIN ? 0 : kPark;
+  constexpr size_t out_bytes = EPI == WIDE_SWIGLU || EPI == WIDE_ROPE ? kPark : 0;
   if (!g || g->wide_pairs < 2 || xb < 0 || xb >= g->n_x || g->xcols[xb] != in) return false;
   if (in % kTileK || rows < 32 || rows > kMaxWideRows || rows > g->xrows[xb] || n_seg < 1 || n_seg > kMaxSeg) return false;
   memset(maps, 0, sizeof *maps);
@@ -516,13 +624,13 @@ bool wide_run(const WideMaps& maps, const WideParams& prm, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * prm.groups * prm.nrb);
   cfg.blockDim = dim3(kWideThreads);
-  cfg.dynamicSmemBytes = kWideSmem;
+  cfg.dynamicSmemBytes = EPI == WIDE_RESID ? kResidSmem : kWideSmem;
   cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = 2;
+  at[1].val.clusterDim.x = EPI == WIDE_RESID ? 2 * prm.splits : 2;
   at[1].val.clusterDim.y = 1;
   at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
@@ -555,6 +663,20 @@ void tc_wide_init(TcGemm* g) {
     return;
   }
   g->wide_pairs = clusters < g->sm_count / 2 ? clusters : g->sm_count / 2;
+  // clusters of 1 .. 4 pairs that run at a time
+  cfg.dynamicSmemBytes = kResidSmem;
+  if (cudaFuncSetAttribute(tc_wide_kernel<WIDE_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidSmem) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  for (int s = 1; s <= 4; ++s) {
+    cfg.gridDim = dim3(g->sm_count / (2 * s) * (2 * s));
+    at[0].val.clusterDim.x = 2 * s;
+    if (cudaOccupancyMaxActiveClusters(&g->resid_clusters[s], tc_wide_kernel<WIDE_RESID>, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      g->resid_clusters[s] = 0;
+    }
+  }
 }
 
 void tc_wide_bind(TcGemm* g, float* scratch, size_t scratch_floats, int* flags) {
@@ -597,6 +719,28 @@ bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   *splits_out = splits > 0 ? splits : 1;
   *split_stride = stride;
   return true;
+}
+
+bool tc_wide_launch_resid(TcGemm* g, int xb, const void* w, int out, int in, int rows, float* x, const void* gain, void* xn, float* ss,
+                          cudaStream_t st) {
+  if (!g || !w || !x || out % 256 || in % kTileK || ((uintptr_t)w & 15) || (gain && (!xn || !ss))) return false;
+  // as many K ranges per tile as run at a time, at least four K blocks each
+  const int items = out / 256 * (rows > 256 ? 2 : 1), units = (in / kTileK + kUnitKb - 1) / kUnitKb;
+  int splits = 4;
+  while (splits > 1 && (g->resid_clusters[splits] < items || splits > units / 2)) --splits;
+  if (g->resid_clusters[splits] < 1) return false;
+  WideMaps maps;
+  WideParams prm;
+  if (!wide_params<WIDE_RESID>(g, xb, 1, out / 256, in, rows, splits, nullptr, 0, &maps, &prm)) return false;
+  const CUtensorMap* m = g->get(w, out, in, kTileM, kUnitKb);
+  if (!m) return false;
+  maps.w[0] = *m;
+  prm.x = x;
+  prm.gain = (const __nv_bfloat16*)gain;
+  prm.xn = (__nv_bfloat16*)xn;
+  prm.ss = ss;
+  prm.out = out;
+  return wide_run<WIDE_RESID>(maps, prm, st);
 }
 
 bool tc_wide_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_up, int f, int in, int rows, void* act, const RowScale& rs,

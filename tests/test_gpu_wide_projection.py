@@ -36,7 +36,7 @@ def test_fused_forms_against_the_separate_kernels(heads, dh, ffn, n):
     w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
     prompt = inputs.make_prompt(shape, seed=2).tolist()
     outs = []
-    for flags in (0, 4 | 16):
+    for flags in (0, 4 | 16, 1):                  # 1: the plain kernels, the residual update apart
         m = Amphista(shape, topo, w, max_ctx=1024, flags=flags)
         m.prefill(prompt)
         m.prefill(prompt)                         # the flags of cut tiles are lowered again after every launch
@@ -44,7 +44,7 @@ def test_fused_forms_against_the_separate_kernels(heads, dh, ffn, n):
         outs.append([m.get_tensor("hidden", ((n - 1) % 512 + 1, shape.d_model))] +
                     [m.get_tensor(f"kv.{c}.{i}", (n, shape.d_model)) for c in "kv" for i in (0, last)])
         m.close()
-    for a, b in zip(*outs):
+    for a, b in list(zip(outs[0], outs[1])) + list(zip(outs[0], outs[2])):
         assert bool(torch.isfinite(a).all())
         # the two forms round the same fp32 sums to bf16 at the same places; a last-bit difference (2^-8) propagates through
         # three layers of unit gain, as in the parity tests' bound
