@@ -37,6 +37,7 @@ constexpr int kWideThreads = 64 + kEpiThreads;
 constexpr int kUnitKb = 2;            // K blocks per pipeline stage = unit of work: ranges are cut at multiples of 128 columns
 constexpr int kMaxWideRows = 512;
 constexpr int kMaxStages = 8;
+constexpr int kMaxGroups = kWideFlags / 2;
 
 struct WideMaps {
   CUtensorMap w[kMaxSeg];
@@ -50,7 +51,7 @@ struct WideParams {
   int kblocks, units_per_tile;
   int splits;               // 0: equal ranges of all work (fix-up through scratch); > 0: K ranges per tile, one per group
   int groups, nrb;          // groups of nrb pairs (row blocks)
-  int snap;                 // see range_begin
+  int range[kMaxGroups + 1];   // splits == 0: first work unit of every group, and the end
   int n;                    // activation rows per MMA (a multiple of 32)
   int tmem_cols;
   int rows, stages;
@@ -93,17 +94,9 @@ struct SegIter {
 
 // First work unit of a group; range_begin(group + 1) is its end.
 __device__ __forceinline__ int range_begin(const WideParams& prm, int group) {
-  if (prm.splits > 0) {
-    const int t = group / prm.splits, s = group - t * prm.splits;
-    return t * prm.units_per_tile + s * prm.units_per_tile / prm.splits;
-  }
-  // a cut within prm.snap units of a tile's edge moves to the edge: the piece it would leave costs a whole epilogue (5-10 us
-  // when nothing runs above it) for a few units of 0.6 us
-  int u = (int)((long long)group * prm.tiles * prm.units_per_tile / prm.groups);
-  const int rem = u % prm.units_per_tile;
-  if (rem <= prm.snap) u -= rem;
-  else if (rem >= prm.units_per_tile - prm.snap) u += prm.units_per_tile - rem;
-  return u;
+  if (prm.splits == 0) return prm.range[group];
+  const int t = group / prm.splits, s = group - t * prm.splits;
+  return t * prm.units_per_tile + s * prm.units_per_tile / prm.splits;
 }
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -116,6 +109,13 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
+__device__ __forceinline__ uint32_t cluster_id() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -199,27 +199,15 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
+  // The way to the first MMA is a chain of latencies of about a microsecond each, so they run side by side: every warp arrives
+  // at the cluster's barrier as soon as its own part is done (barriers initialised, tensor memory allocated) and waits for it
+  // only where it needs the others; warp 0 issues the weights while warp 1 waits for the kernel before this one and then fetches
+  // the ring's first activations.  One after the other, it took 4.9 us from the CTA's start to the first full stage.
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t crank = cluster_rank(), rank = crank & 1u, lead = crank & ~1u;     // in the cluster, in the pair; the pair's even CTA
-  int pair = prm.groups * prm.nrb - 1 - (int)(blockIdx.x >> 1);              // against the launch order (see above)
-  int group = pair / prm.nrb, rb = pair - group * prm.nrb;
-  if constexpr (EPI == WIDE_RESID) {                                         // a cluster holds the splits of one tile and row block
-    const int item = (int)blockIdx.x / (2 * prm.splits);
-    rb = item % prm.nrb;
-    group = item / prm.nrb * prm.splits + (int)(crank >> 1);
-  }
-  const int stages = prm.stages, n = prm.n;
-  const uint32_t b_tile = (uint32_t)n / 2 * 128, a_tile = kTileM * 128;         // one K block of each operand
-  const uint32_t stage_bytes = kUnitKb * (a_tile + b_tile);
-  const unsigned long long limit_ns = prm.wait_limit_ns;
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  float* const small_park = reinterpret_cast<float*>(smem + (size_t)stages * stage_bytes); // fused forms: [kBatch][128]
-  const SegIter first = {range_begin(prm, group), range_begin(prm, group + 1), prm.units_per_tile};
-
   if (threadIdx.x == 0) {
     abort_flag = 0;
-    for (int s = 0; s < stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+    for (int s = 0; s < prm.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
     for (int s = 0; s < 2; ++s) { mbar_init(&accum_full[s], 1); mbar_init(&accum_empty[s], 2 * kEpiThreads / 32); }
     mbar_init(&recv_full, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -229,10 +217,32 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  cluster_sync_all();                                                // both CTAs' barriers exist before any copy or MMA signals them
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_d = tmem_base_slot;
+  __syncwarp();
+  cluster_arrive_release();
+  const uint32_t crank = cluster_rank(), rank = crank & 1u, lead = crank & ~1u;     // in the cluster, in the pair; the pair's even CTA
+  int pair = prm.groups * prm.nrb - 1 - (int)(blockIdx.x >> 1);              // against the launch order (see above)
+  int group = prm.nrb == 2 ? pair >> 1 : pair, rb = prm.nrb == 2 ? pair & 1 : 0;
+  if constexpr (EPI == WIDE_RESID) {                                         // a cluster holds the splits of one tile and row block
+    const int item = (int)cluster_id();
+    rb = prm.nrb == 2 ? item & 1 : 0;
+    group = (prm.nrb == 2 ? item >> 1 : item) * prm.splits + (int)(crank >> 1);
+  }
+  const int stages = prm.stages, n = prm.n;
+  const uint32_t b_tile = (uint32_t)n / 2 * 128, a_tile = kTileM * 128;         // one K block of each operand
+  const uint32_t stage_bytes = kUnitKb * (a_tile + b_tile);
+  const unsigned long long limit_ns = prm.wait_limit_ns;
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  float* const small_park = reinterpret_cast<float*>(smem + (size_t)stages * stage_bytes); // fused forms: [kBatch][128]
+  const SegIter first = {range_begin(prm, group), range_begin(prm, group + 1), prm.units_per_tile};
+  auto load_x = [&](int st, int u) {
+    const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), lead);
+    tma_pair_3d(smem + (size_t)st * stage_bytes + kUnitKb * a_tile, &maps.x, 0, rb * n + (int)rank * (n / 2), u * kUnitKb, bar);
+  };
+  // both CTAs' barriers and tensor memory exist behind this
+  auto cluster_ready = [&]() {
+    cluster_wait_acquire();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  };
 
   if (warp == 0) {
     // ---------------- TMA producer of this CTA's half of the operands
@@ -246,12 +256,9 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
       if (EPI == WIDE_SWIGLU) tma_pair_4d(dst, &maps.w[0], 0, (lt * 2 + (int)rank) * (kTileM / 2), 0, u * kUnitKb, bar, wpol);
       else tma_pair_3d(dst, &maps.w[seg], 0, (lt * 2 + (int)rank) * kTileM, u * kUnitKb, bar, wpol);
     };
-    auto load_x = [&](int st, int u) {
-      const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), lead);
-      tma_pair_3d(smem + (size_t)st * stage_bytes + kUnitKb * a_tile, &maps.x, 0, rb * n + (int)rank * (n / 2), u * kUnitKb, bar);
-    };
-    // weights do not depend on the kernel before: fill the ring with them, then wait, then fetch those stages' activations
+    // weights do not depend on the kernel before: fill the ring with them; warp 1 fetches those stages' activations
     if (prm.wait_first) pdl_wait();
+    cluster_ready();
     SegIter it = first;
     Segment sg;
     bool have = it.next(sg);
@@ -262,17 +269,6 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     }
     __syncwarp();
     pdl_wait();
-    {
-      SegIter bt = first;
-      Segment bs;
-      bt.next(bs);
-      int bu = bs.u0;
-      for (int j = 0; j < i; ++j) {
-        if (leader) load_x(j, bu);
-        if (++bu == bs.u1) { bt.next(bs); bu = bs.u0; }
-      }
-    }
-    __syncwarp();
     for (; have; ++i) {
       const int st = i % stages, round = i / stages;
       if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[st], (round & 1) ^ 1, &abort_flag, limit_ns))) break;
@@ -286,9 +282,23 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
         while (!mbar_try(&full_bar[j % stages], (j / stages) & 1) && now_ns() - t0 < limit_ns) {}
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer (even CTA)
+    // ---------------- the ring's first activations, then MMA issuer (even CTA)
+    const bool leader = elect_one();
+    pdl_wait();
+    cluster_ready();
+    {
+      SegIter it = first;
+      Segment sg;
+      bool have = it.next(sg);
+      int u = have ? sg.u0 : 0;
+      for (int i = 0; i < stages && have; ++i) {
+        if (leader) load_x(i, u);
+        if (++u == sg.u1) { have = it.next(sg); u = sg.u0; }
+      }
+      __syncwarp();
+    }
     if (rank == 0) {
-      const bool leader = elect_one();
+      const uint32_t tmem_d = tmem_base_slot;
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
       SegIter it = first;
       Segment sg;
@@ -325,6 +335,8 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     // ---------------- epilogue
     const int quarter = warp & 3, sub = (warp - 2) >> 2, et = threadIdx.x - 64;
     const int row0 = rb * n, my_rows = prm.rows - row0 < n ? prm.rows - row0 : n;
+    cluster_ready();
+    const uint32_t tmem_d = tmem_base_slot;
     pdl_wait();
     if constexpr (SCALED) {
       if (et < my_rows) inv_s[et] = row_scale(prm.rs, row0 + et);
@@ -564,7 +576,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   cluster_sync_all();                                     // no CTA leaves while its partner may still signal or read its shared memory
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(prm.tmem_cols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_slot), "r"(prm.tmem_cols) : "memory");
   }
   if (threadIdx.x == 0 && abort_flag && prm.err_flag) *prm.err_flag = AMPH_ERR_TIMEOUT;
 }
@@ -605,7 +617,16 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
     const size_t per_group = (size_t)prm->nrb * 2 * prm->n * kTileM;
     if ((size_t)prm->groups > scratch_floats / per_group) prm->groups = (int)(scratch_floats / per_group);
     if (prm->groups < 1 || !scratch_end || !g->wide_flags || 2 * prm->groups * prm->nrb > kWideFlags) return false;
-    prm->snap = units / prm->groups / 4 < prm->units_per_tile / 8 ? units / prm->groups / 4 : prm->units_per_tile / 8;
+    // a cut within `snap` units of a tile's edge moves to the edge: the piece it would leave costs a whole epilogue (5-10 us
+    // when nothing runs above it) for a few units of 0.6 us
+    const int upt = prm->units_per_tile, share = units / prm->groups / 4, snap = share < upt / 8 ? share : upt / 8;
+    for (int i = 0; i <= prm->groups; ++i) {
+      int u = (int)((long long)i * units / prm->groups);
+      const int rem = u % upt;
+      if (rem <= snap) u -= rem;
+      else if (rem >= upt - snap) u += upt - rem;
+      prm->range[i] = u;
+    }
     prm->scratch = scratch_end - (size_t)prm->groups * per_group;    // the buffer's end: its beginning may hold the result
   }
   prm->rows = rows;
