@@ -180,14 +180,18 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
     mbar_init(&accum_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // Barrier 2 tells warp 1 that the mbarriers exist, barrier 3 the epilogue that the accumulator does: warp 0 waits for nobody
+  // before its first weights, warp 1 only for the kernel before this one.
+  if (warp == 0) asm volatile("bar.arrive 2, 64;" ::: "memory");
   if (warp == 1) {                                   // TMEM allocation belongs to the MMA warp
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(tmem_cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
+  __syncwarp();
+  if (warp < 2) asm volatile("bar.arrive 3, 192;" ::: "memory");
+  else asm volatile("bar.sync 3, 192;" ::: "memory");
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_d = tmem_base_slot;
 
   if (warp == 0) {
     // ---------------- TMA producer (the warp stays converged, its elected lane issues)
@@ -198,8 +202,8 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(wmap) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.x) : "memory");
     }
-    // Weights do not depend on the previous kernel: fill the ring with weight tiles first, then wait for
-    // the producer of the activations, then fetch the activation tiles of those stages.
+    // Weights do not depend on the previous kernel: fill the ring with weight tiles first; warp 1 waits for the producer of
+    // the activations meanwhile and fetches the activation tiles of those stages.
     if (prm.wait_first) pdl_wait();
     const int npre = nit < stages ? nit : stages;
     const int npf = nit < npre + prm.l2_prefetch ? nit : npre + prm.l2_prefetch;
@@ -220,11 +224,6 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
     }
     __syncwarp();
     pdl_wait();
-    if (leader)
-      for (int i = 0; i < npre; ++i)
-        for (int z = 0; z < nblk; ++z)
-          tma_load_3d(smem + (size_t)i * stage_bytes + a_bytes + (size_t)z * b_slot, &maps.x, z * nt, kb_lo + i * ks, &full_bar[i]);
-    __syncwarp();
     int issued = npre;
     for (int i = npre; i < nit; ++i) {
       const int s = i % stages, round = i / stages;
@@ -251,6 +250,14 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
   } else if (warp == 1) {
     // ---------------- MMA issuer (the warp stays converged, its elected lane issues)
     const bool leader = elect_one();
+    pdl_wait();                                      // returns about 1.1 us after it is asked, also behind a finished kernel
+    asm volatile("bar.sync 2, 64;" ::: "memory");
+    if (leader)
+      for (int i = 0; i < nit && i < stages; ++i)
+        for (int z = 0; z < nblk; ++z)
+          tma_load_3d(smem + (size_t)i * stage_bytes + a_bytes + (size_t)z * b_slot, &maps.x, z * nt, kb_lo + i * ks, &full_bar[i]);
+    __syncwarp();
+    const uint32_t tmem_d = tmem_base_slot;
     const uint32_t idesc = umma_idesc(nt, EPI != EPI_PARTIAL ? kTileM / 2 : kTileM);
     bool ok = true;
     for (int i = 0; i < nit; ++i) {
@@ -293,6 +300,7 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
   } else {
     // ---------------- epilogue: warp w may touch TMEM lanes 32*(w%4) .. +31
     const int quarter = warp & 3;
+    const uint32_t tmem_d = tmem_base_slot;
     pdl_wait();                                      // P may still be read by the kernel before this one
     if constexpr (EPI != EPI_PARTIAL) {              // 1 / rms of the rows, while the main loop runs
       const int et = threadIdx.x - 64;
@@ -451,7 +459,7 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
   __syncthreads();
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(tmem_cols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_slot), "r"(tmem_cols) : "memory");
   }
   if (threadIdx.x == 0 && abort_flag && prm.err_flag) *prm.err_flag = AMPH_ERR_TIMEOUT;
 }
