@@ -258,8 +258,8 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base_slot;
 
-  // The row table was written several kernels ago (every kernel between it and this one waits for its own
-  // predecessor before it lets its successor start), so it may be read before the dependency wait.
+  // The kernel that wrote the row table has ended: it lets its successor start only by ending, or one between it and this one
+  // waits for its own predecessor before it lets its successor start.  So the table may be read before the dependency wait.
   const int base = meta->base, n_rows = meta->n_rows;
   const int total = base + n_rows;
   const int S = gridDim.y;                             // splits of the head

@@ -358,6 +358,21 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     Segment sg;
     for (int j = 0; it.next(sg); ++j) {
       const int as = j & 1;
+      // RESID: rows [lo, hi) are this CTA's share, a warp finishes whole rows of the tile's 128 features, four features a lane;
+      // the old values are fetched while the main loop runs
+      constexpr int kAhead = 8, kRowWarps = kEpiThreads / 32;
+      const int S = prm.splits, split = (int)(crank >> 1), per = EPI == WIDE_RESID ? ((n + S - 1) / S + 7) / 8 * 8 : 0;
+      const int lo = split * per, hi = lo + per < my_rows ? lo + per : my_rows, f0 = sg.tile * 256 + (int)rank * kTileM + lane * 4;
+      float4 old[kAhead], gn;
+      auto fetch_old = [&](int r) {
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q)
+          if (r + q * kRowWarps < hi) old[q] = *reinterpret_cast<const float4*>(prm.x + (size_t)(row0 + r + q * kRowWarps) * prm.out + f0);
+      };
+      if constexpr (EPI == WIDE_RESID) {
+        if (prm.gain != nullptr) gn = bf16x4(prm.gain + f0);
+        fetch_old(lo + (et >> 5));
+      }
       bool ok = __all_sync(0xffffffffu, mbar_wait(&accum_full[as], (j >> 1) & 1, &abort_flag, limit_ns));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t t0 = tmem_d + (uint32_t)(as * n) + ((uint32_t)(quarter * 32) << 16);
@@ -367,56 +382,38 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
         if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&accum_empty[as]), lead));
       };
       if constexpr (EPI == WIDE_RESID) {
-        const int S = prm.splits, split = (int)(crank >> 1), per = ((n + S - 1) / S + 7) / 8 * 8;       // rows of a share
-        const int lo = split * per, hi = lo + per < my_rows ? lo + per : my_rows;
         float* const park = reinterpret_cast<float*>(smem);                    // [n][128]: the ring is free
         uint8_t* const recv = smem + (size_t)n * kTileM * 4;                   // the other splits' sums of this CTA's share
-        if (S > 1) {
-          __syncwarp();
-          cluster_arrive();                               // this CTA's MMAs have read their operands: peers may write here
-        }
-        for (int r = sub * kChunk; r < my_rows; r += kBatch) {
-          float v[kChunk];
-          tmem_ld8(t0 + (uint32_t)r, v);
-#pragma unroll
-          for (int e = 0; e < kChunk; ++e) park[(r + e) * kTileM + frow] = ok ? v[e] : 0.f;
-        }
         const uint32_t share = (uint32_t)per * kTileM * 4;
-        if (S > 1) {
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");         // the copies read through the async proxy
-          epi_sync();
-          __syncwarp();
-          cluster_wait();
-          if (warp == 2) {
-            const uint32_t mine = hi > lo ? (uint32_t)(hi - lo) * kTileM * 4 : 0u;
-            if (lane == 0) mbar_expect_tx(&recv_full, (uint32_t)(S - 1) * mine);
-            __syncwarp();
-            if (lane < S && lane != split) {
-              const int olo = lane * per, ohi = olo + per < my_rows ? olo + per : my_rows;
-              const uint32_t to = (uint32_t)lane * 2 + rank;
-              if (ohi > olo)
-                bulk_to_peer(map_to_rank(smem_u32(recv + (size_t)(split < lane ? split : split - 1) * share), to), park + (size_t)olo * kTileM,
-                             (uint32_t)(ohi - olo) * kTileM * 4, map_to_rank(smem_u32(&recv_full), to));
-            }
-          }
-        } else {
-          epi_sync();
-        }
-        // a warp finishes whole rows of the tile's 128 features, four features a lane; the old values are on their way while
-        // the other splits' sums arrive
-        const int f0 = sg.tile * 256 + (int)rank * kTileM + lane * 4;
-        const float4 gn = prm.gain != nullptr ? bf16x4(prm.gain + f0) : make_float4(0.f, 0.f, 0.f, 0.f);
-        constexpr int kAhead = 4, kStep = kEpiThreads / 32;
-        bool arrived = S == 1;
-        for (int rl = lo + (et >> 5); rl < hi || !arrived; rl += kAhead * kStep) {
-          float4 v[kAhead];
+        __syncwarp();
+        cluster_arrive();                                 // this CTA's MMAs have read their operands: peers may write here
+        // The shares go out one by one while the next is read from tensor memory, this CTA's own comes last.  A warp reads
+        // pieces of 8 rows; a share begins where a piece does.
+        for (int i = 1; i <= S; ++i) {
+          const int o = split + i < S ? split + i : split + i - S, olo = o * per, ohi = olo + per < my_rows ? olo + per : my_rows;
+          for (int r = olo + sub * kChunk; r < ohi; r += kBatch) {
+            float v[kChunk];
+            tmem_ld8(t0 + (uint32_t)r, v);
 #pragma unroll
-          for (int q = 0; q < kAhead; ++q)
-            if (rl + q * kStep < hi) v[q] = *reinterpret_cast<const float4*>(prm.x + (size_t)(row0 + rl + q * kStep) * prm.out + f0);
-          if (!arrived) { __all_sync(0xffffffffu, mbar_wait(&recv_full, 0, &abort_flag, limit_ns)); arrived = true; }
+            for (int e = 0; e < kChunk; ++e) park[(r + e) * kTileM + frow] = ok ? v[e] : 0.f;
+          }
+          if (i < S) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the copies read through the async proxy
+          epi_sync();
+          if (i == 1) { __syncwarp(); cluster_wait(); }
+          if (i < S && et == 0 && ohi > olo) {
+            const uint32_t to = (uint32_t)o * 2 + rank;
+            bulk_to_peer(map_to_rank(smem_u32(recv + (size_t)(split < o ? split : split - 1) * share), to), park + (size_t)olo * kTileM,
+                         (uint32_t)(ohi - olo) * kTileM * 4, map_to_rank(smem_u32(&recv_full), to));
+          }
+          __syncwarp();
+        }
+        if (et == 0) mbar_expect_tx(&recv_full, hi > lo ? (uint32_t)(S - 1) * (uint32_t)(hi - lo) * kTileM * 4 : 0u);
+        __all_sync(0xffffffffu, mbar_wait(&recv_full, 0, &abort_flag, limit_ns));
+        for (int rl = lo + (et >> 5); rl < hi; rl += kAhead * kRowWarps) {
+          if (rl != lo + (et >> 5)) fetch_old(rl);
 #pragma unroll
           for (int q = 0; q < kAhead; ++q) {
-            const int r = rl + q * kStep;
+            const int r = rl + q * kRowWarps;
             if (r >= hi) continue;                        // uniform over the warp
             float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
             for (int s = 0; s < S; ++s) {                 // in K order
@@ -424,13 +421,14 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
                                           : *reinterpret_cast<const float4*>(recv + (size_t)(s < split ? s : s - 1) * share + ((size_t)(r - lo) * kTileM + lane * 4) * 4);
               a.x += p.x; a.y += p.y; a.z += p.z; a.w += p.w;
             }
-            v[q].x += a.x; v[q].y += a.y; v[q].z += a.z; v[q].w += a.w;
-            *reinterpret_cast<float4*>(prm.x + (size_t)(row0 + r) * prm.out + f0) = v[q];
+            float4 v = old[q];
+            v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
+            *reinterpret_cast<float4*>(prm.x + (size_t)(row0 + r) * prm.out + f0) = v;
             if (prm.gain == nullptr) continue;
-            const __nv_bfloat162 y0 = __floats2bfloat162_rn(gn.x * v[q].x, gn.y * v[q].y), y1 = __floats2bfloat162_rn(gn.z * v[q].z, gn.w * v[q].w);
+            const __nv_bfloat162 y0 = __floats2bfloat162_rn(gn.x * v.x, gn.y * v.y), y1 = __floats2bfloat162_rn(gn.z * v.z, gn.w * v.w);
             *reinterpret_cast<uint2*>(prm.xn + (size_t)(row0 + r) * prm.out + f0) =
                 make_uint2(*reinterpret_cast<const uint32_t*>(&y0), *reinterpret_cast<const uint32_t*>(&y1));
-            float sq = v[q].x * v[q].x + v[q].y * v[q].y + v[q].z * v[q].z + v[q].w * v[q].w;
+            float sq = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
             for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
             if (lane == 0) prm.ss[(size_t)(row0 + r) * (prm.out / kTileM) + sg.tile * 2 + rank] = sq;
           }
@@ -566,7 +564,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
       }
     }
   }
-  if (EPI == WIDE_RESID && prm.splits > 1 && warp < 2) {  // the epilogue's barrier of the cluster
+  if (EPI == WIDE_RESID && warp < 2) {  // the epilogue's barrier of the cluster
     __syncwarp();
     cluster_arrive();
     cluster_wait();
