@@ -431,19 +431,25 @@ def main():
     # kernels launched per step: projections + the fixed schedule around them (counted from the schedule)
     # per layer: q/k/v projection, rotary + cache write, attention (its KV splits merge in-launch on bf16 unless the
     # separate-merge flag is set), output projection, residual, gate/up projection, SwiGLU, down projection, residual
-    per_layer = 9 if (shape.dtype == "bf16" and not (args.flags & 8)) else 10
-    if uses_tc and not (args.flags & 16) and N <= 64:
-        per_layer -= 1                                           # SwiGLU in the gate / up projection's epilogue
-    if uses_tc and not (args.flags & 4) and N <= 64:
-        per_layer -= 1                                           # rotary + cache write in the q/k/v projection's epilogue
-    if uses_tc and not (args.flags & (4 | 256)) and N <= 64 and shape.d_ffn // 64 <= 148 * 2 * 13 // 16:
-        per_layer += 1                                           # the gate / up prefetch helper on the forked stream
-    sal = shape.n_sal * (3 + per_layer)
-    draft = 2 + sal + 1 + 2 + shape.aeb_layers * 4 + 3 + 1      # ... + (vocabulary projection, top-k slices, merge) + tree
+    def layer_launches(rows):
+        n = 10 if (shape.dtype == "bf16" and args.flags & 8) else 9
+        if not uses_tc:
+            return n
+        n -= (not args.flags & 16) + (not args.flags & 4)        # SwiGLU; rotary + cache write: in the projections' epilogues
+        if rows > 64:
+            n -= 2                                               # residual updates in the projections' epilogues
+        elif not (args.flags & (4 | 256)) and shape.d_ffn // 64 <= 148 * 2 * 13 // 16:
+            n += 1                                               # the gate / up prefetch helper on the forked stream
+        return n
+
+    sal = shape.n_sal * (3 + layer_launches(1))
+    draft = sal + 1 + 2 + shape.aeb_layers * 4 + 3              # ... + (vocabulary projection, top-k slices, merge and tree)
     if getattr(shape, "lm_rank", 0):
         draft += 2                                               # low-rank heads: one more projection + a gather
-    verify = 3 + shape.n_layers * per_layer + 3                  # ... + head projection, argmax slices, merge
-    line["gpu_launches"] = (draft + verify + 2) * steps
+    verify = 1 + shape.n_layers * layer_launches(N) + 3          # row set-up, ..., head projection, argmax slices, merge
+    if uses_tc and N > 64:
+        verify += 1                                              # the last layer's update also takes the final norm: a kernel of its own
+    line["gpu_launches"] = (draft + verify + 1) * steps
     if not args.no_cpu_baseline:
         v, cores, desc = cpu_baseline(shape, topo, gen_device=dev)
         line["cpu_baseline"] = {"value": v, "unit": UNIT, "cores": cores, "kind": "oracle", "sample": desc,
