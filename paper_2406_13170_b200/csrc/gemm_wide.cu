@@ -190,7 +190,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   constexpr bool SCALED = EPI == WIDE_SWIGLU || EPI == WIDE_ROPE;   // the activation rows' RMS division is still to be done
   __shared__ float inv_s[SCALED ? 256 : 1];                        // 1 / rms of this pair's activation rows
-  __shared__ int slot_s[EPI == WIDE_ROPE ? 256 : 1];               // cache slot of a row, -1: not stored
+  __shared__ __nv_bfloat16* dst_s[EPI == WIDE_ROPE ? 256 : 1];     // where the segment's matrix (q, k or v) of a row goes, NULL: nowhere
   __shared__ const float2* table_s[EPI == WIDE_ROPE ? 256 : 1];    // its rotary table row
   __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], accum_full[2], accum_empty[2], recv_full;
   __shared__ uint32_t tmem_base_slot;
@@ -340,13 +340,15 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     if constexpr (SCALED) {
       if (et < my_rows) inv_s[et] = row_scale(prm.rs, row0 + et);
     }
+    int my_group = 0, my_slot = -1;                      // ROPE: of row et
     if constexpr (EPI == WIDE_ROPE) {
       if (et < my_rows) {
-        const int g = (row0 + et) / prm.gr.rpg, rl = row0 + et - g * prm.gr.rpg;
-        const RowMeta* meta = prm.gr.meta[g];
+        my_group = (row0 + et) / prm.gr.rpg;
+        const int rl = row0 + et - my_group * prm.gr.rpg;
+        const RowMeta* meta = prm.gr.meta[my_group];
         const int slot = meta->slot[rl];
-        slot_s[et] = rl < meta->n_rows && slot >= 0 && slot < prm.max_ctx ? slot : -1;
-        table_s[et] = prm.gr.rope[g] + (size_t)rl * (prm.dh >> 1);
+        my_slot = rl < meta->n_rows && slot >= 0 && slot < prm.max_ctx ? slot : -1;
+        table_s[et] = prm.gr.rope[my_group] + (size_t)rl * (prm.dh >> 1);
       }
     }
     epi_sync();
@@ -512,9 +514,18 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
         // item i of a batch: row i / 16, outputs 4 (i % 16) .. + 3 (SwiGLU) or as many rotation pairs
         const int p4 = (et & 15) * 4;
         const int hdim = prm.dh >> 1;
-        const int lo_at = EPI == WIDE_ROPE ? p4 / hdim * prm.dh + p4 % hdim : p4;
-        const int hi_at = EPI == WIDE_ROPE ? lo_at + hdim : p4 + kTileM / 2;
+        // SwiGLU: lo = gate, hi = up, in the order they have in the tile
+        const int lo_at = EPI == WIDE_ROPE ? p4 / hdim * prm.dh + p4 % hdim : prm.up_first ? p4 + kTileM / 2 : p4;
+        const int hi_at = EPI == WIDE_ROPE ? lo_at + hdim : prm.up_first ? p4 : p4 + kTileM / 2;
         const int head = EPI == WIDE_ROPE ? (lt * 2 + (int)rank) * kTileM / prm.dh + p4 / hdim : 0;
+        // what a row's address needs is worked out once per segment and row, not per row and thread
+        const size_t col = EPI == WIDE_ROPE ? (size_t)head * (seg == 0 ? prm.dh : prm.max_ctx * prm.dh) + p4 % hdim
+                                            : (size_t)(lt * 2 + (int)rank) * (kTileM / 2) + p4;
+        if constexpr (EPI == WIDE_ROPE) {
+          if (et < my_rows)
+            dst_s[et] = seg == 0 ? prm.q + (size_t)(row0 + et) * prm.n_heads * prm.dh
+                                 : my_slot < 0 ? nullptr : (__nv_bfloat16*)(seg == 1 ? prm.gr.kc[my_group] : prm.gr.vc[my_group]) + (size_t)my_slot * prm.dh;
+        }
         float* const park = last ? reinterpret_cast<float*>(smem) : small_park;
         const int batch = last ? my_rows : kBatch;
         for (int b0 = 0; b0 < my_rows; b0 += batch) {
@@ -544,20 +555,14 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
             float4 a = *reinterpret_cast<const float4*>(row + lo_at), b = *reinterpret_cast<const float4*>(row + hi_at);
             a.x *= sc; a.y *= sc; a.z *= sc; a.w *= sc; b.x *= sc; b.y *= sc; b.z *= sc; b.w *= sc;
             if constexpr (EPI == WIDE_SWIGLU) {
-              if (prm.up_first) { const float4 t = a; a = b; b = t; }
               const __nv_bfloat162 y0 = __floats2bfloat162_rn(__fdividef(a.x, 1.0f + __expf(-a.x)) * b.x, __fdividef(a.y, 1.0f + __expf(-a.y)) * b.y);
               const __nv_bfloat162 y1 = __floats2bfloat162_rn(__fdividef(a.z, 1.0f + __expf(-a.z)) * b.z, __fdividef(a.w, 1.0f + __expf(-a.w)) * b.w);
-              *reinterpret_cast<uint2*>(prm.act + (size_t)(row0 + rl) * prm.f + (lt * 2 + (int)rank) * (kTileM / 2) + p4) =
+              *reinterpret_cast<uint2*>(prm.act + (size_t)(row0 + rl) * prm.f + col) =
                   make_uint2(*reinterpret_cast<const uint32_t*>(&y0), *reinterpret_cast<const uint32_t*>(&y1));
             } else {
-              __nv_bfloat16* dst = nullptr;
-              if (seg == 0) {
-                dst = prm.q + (size_t)(row0 + rl) * prm.n_heads * prm.dh + head * prm.dh + p4 % hdim;
-              } else if (slot_s[rl] >= 0) {
-                const int g = (row0 + rl) / prm.gr.rpg;
-                dst = (__nv_bfloat16*)(seg == 1 ? prm.gr.kc[g] : prm.gr.vc[g]) + ((size_t)head * prm.max_ctx + slot_s[rl]) * prm.dh + p4 % hdim;
-              }
-              if (dst != nullptr) {
+              __nv_bfloat16* const row_dst = dst_s[rl];
+              if (row_dst != nullptr) {
+                __nv_bfloat16* const dst = row_dst + col;
                 const __nv_bfloat162 l0 = __floats2bfloat162_rn(a.x * cs0.x - b.x * cs0.y, a.y * cs0.z - b.y * cs0.w);
                 const __nv_bfloat162 l1 = __floats2bfloat162_rn(a.z * cs1.x - b.z * cs1.y, a.w * cs1.z - b.w * cs1.w);
                 const __nv_bfloat162 h0 = __floats2bfloat162_rn(b.x * cs0.x + a.x * cs0.y, b.y * cs0.z + a.y * cs0.w);
@@ -597,7 +602,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   if (threadIdx.x == 0 && abort_flag && prm.err_flag) *prm.err_flag = AMPH_ERR_TIMEOUT;
 }
 
-constexpr size_t kWideSmem = 221 * 1024;                  // ring + alignment; the static part needs up to 5 KB of the 227
+constexpr size_t kWideSmem = 220 * 1024;                  // ring + alignment; the static part needs up to 6 KB of the 227
 constexpr size_t kResidSmem = 225 * 1024;                 // 256 parked rows and three quarters of them received; 1 KB static
 
 // Everything of a launch that does not depend on the epilogue; false: the shape is not covered.
@@ -647,7 +652,7 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
   }
   prm->rows = rows;
   const size_t stage = kUnitKb * ((size_t)kTileM * 128 + (size_t)prm->n / 2 * 128);
-  prm->stages = (int)((kWideSmem - 1024 - out_bytes) / stage);
+  prm->stages = (int)(((EPI == WIDE_RESID ? kResidSmem : kWideSmem) - 1024 - out_bytes) / stage);
   if (prm->stages > kMaxStages) prm->stages = kMaxStages;
   prm->flags = g->wide_flags;
   prm->wait_first = g->wait_first;
@@ -679,7 +684,7 @@ bool wide_run(const WideMaps& maps, const WideParams& prm, cudaStream_t st) {
 
 void tc_wide_init(TcGemm* g) {
   g->wide_pairs = 0;
-  if ((size_t)g->max_smem < kWideSmem + 6 * 1024) return;
+  if ((size_t)g->max_smem < kWideSmem + 7 * 1024) return;
   int clusters = 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(g->sm_count / 2 * 2);
