@@ -472,9 +472,22 @@ RowScale rows_from(RowScale rs, int row0) {
 // Forked right after the q / k / v projection is launched: measured -1.5 % per step; forked after the attention or the output
 // projection it costs 2-5 % (an event between two programmatically dependent launches), as does a larger budget.
 constexpr size_t kGateUpPrefetchBytes = 56u << 20;
+// The window closes as the context grows: attention then streams keys and values itself, and its first chunks wait behind the
+// helper's.  us per step with / without the helper, d = 4096 x 16 layers: 520 keys 2016 / 2056, 1000 2092 / 2093, 1500 2113 / 2103,
+// 2000 2188 / 2147, 3000 2221 / 2175, 4500 2382 / 2300; d = 5120 x 12 layers: 500 keys 2201 / 2220, from 1024 on equal.  Equal on
+// both sides between 16 and 25 MB of keys and values per layer.
+constexpr size_t kPrefetchKvBytes = 20u << 20;
 
-void fork_prefetch(amph_ctx* ctx, const LayerW& w, int rows) {
-  if (!(ctx->side && ctx->tc && rows <= 64)) return;
+// keys: cache slots that the pass's attention may read, all groups (the host's bound)
+bool prefetch_pays(const amph_ctx* ctx, long long keys) {
+  return (size_t)keys * 2 * ctx->cfg.d_model * ctx->esz <= kPrefetchKvBytes;
+}
+
+void fork_prefetch(amph_ctx* ctx, const LayerW& w, const Pass& ps) {
+  if (!(ctx->side && ctx->tc && ps.rows() <= 64)) return;
+  long long keys = 0;
+  for (int g = 0; g < ps.G; ++g) keys += ps.keys[g];
+  if (!prefetch_pays(ctx, keys)) return;
   const amph_config& c = ctx->cfg;
   // a gate / up launch of about a full wave (two CTAs per SM) gains nothing: measured +0.3 % at d_ffn = 17920 (280 tiles)
   if (c.d_ffn / 64 > ctx->sm_count * 2 * 13 / 16) return;
@@ -529,7 +542,7 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
     if (!fused_rope) cudaGetLastError();
   }
   if (!fused_rope) P = project(ctx, XB_XN, qkv, 3, c.d_model, c.d_model, rows);
-  if (fused_rope) fork_prefetch(ctx, w, rows);
+  if (fused_rope) fork_prefetch(ctx, w, ps);
   bool grouped_rope = false;
   if (!fused_rope && ps.G > 1) {                      // every group's rotary embedding + cache write in one launch
     ProfScope p(ctx, AMPH_PROF_ROPE_KV);
@@ -941,12 +954,15 @@ amph_status check_capacity(amph_ctx* ctx) {
 // drafting one runs at most one split behind) are 13 combinations.
 constexpr size_t kMaxGraphs = 16;
 
-// The captured schedule depends on the host's bounds only through the attention launches: one per sequence, or, where the
-// sequences of a batch share a launch (layer_forward), one sized for the longest of them.
+// The captured schedule depends on the host's bounds only through the prefetch helper and the attention launches: one per
+// sequence, or, where the sequences of a batch share a launch (layer_forward), one sized for the longest of them.
 long long graph_key_of(const amph_ctx* ctx) {
-  long long key = 0;
+  long long keys = 0;
+  for (int b = 0; b < ctx->B; ++b) keys += ctx->ctx_hi[b];
+  const int helper = (prefetch_pays(ctx, keys) ? 2 : 0) + (prefetch_pays(ctx, keys + (long long)ctx->B * ctx->tree_host.n_nodes) ? 1 : 0);
+  long long key = helper;
   if (ctx->attn_tc && ctx->B > 1 && !(ctx->cfg.flags & AMPH_FLAG_SEPARATE_MERGE))
-    return attn_splits_for(ctx, ctx->max_ctx_hi(), ctx->rows_small, ctx->B) * 128 +
+    return helper * 128 * 128 + attn_splits_for(ctx, ctx->max_ctx_hi(), ctx->rows_small, ctx->B) * 128 +
            attn_splits_for(ctx, ctx->max_ctx_hi() + ctx->tree_host.n_nodes, ctx->Mver, ctx->B);
   for (int b = 0; b < ctx->B; ++b)
     key = key * 4099 + attn_splits_for(ctx, ctx->ctx_hi[b], ctx->rows_small, 1) * 128 +
@@ -1202,8 +1218,8 @@ amph_status amph_step(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n) {
   const bool use_graph = !ctx->graph_off && !ctx->prof_on && !(c.flags & AMPH_FLAG_NO_GRAPH) && ctx->stream != nullptr;
   amph_ctx::StepGraph* sg = nullptr;
   if (use_graph) {
-    // The kernels read every length from device state; only the attention grids depend on the host's
-    // bound of the context length, so a captured schedule serves every step with the same grids.
+    // The kernels read every length from device state; only the attention grids and the
+    // prefetch helper depend on the host's bound of the context length, so a captured schedule serves every step that has the same.
     const long long key = graph_key_of(ctx);
     for (auto& g : ctx->graphs)
       if (g.key == key) sg = &g;

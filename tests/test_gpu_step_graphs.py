@@ -39,6 +39,23 @@ def test_lengths_that_come_back(name, lengths):
     plain.close()
 
 
+def test_context_grows_past_the_prefetch_helper():
+    """20 MB of keys and values per layer: below, a step's schedule has a prefetch helper per layer, above, none; first the
+    verification pass crosses the line, then the draft."""
+    from paper_2406_13170_b200 import Amphista
+    shape = inputs.get_shape("small_bf16")
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    n = (20 << 20) // (4 * shape.d_model) - shape.n_nodes - 12
+    prompt = inputs.make_prompt(shape.with_(prompt_len=n), seed=1).tolist()
+    outs = []
+    for flags in (0, 2):                              # 2: kernels launched one by one
+        m = Amphista(shape, topo, w, max_ctx=n + 256, flags=flags)
+        outs.append(_decode(m, [prompt], 14))
+        m.close()
+    assert outs[0] == outs[1]
+
+
 @pytest.mark.parametrize("batch", [1, 3])
 def test_results_reach_whatever_arrays_a_step_is_given(batch):
     """Device arrays, other device arrays, pinned and pageable host arrays, one of the two, none: each call's results arrive where
