@@ -431,25 +431,27 @@ def main():
     # kernels launched per step: projections + the fixed schedule around them (counted from the schedule)
     # per layer: q/k/v projection, rotary + cache write, attention (its KV splits merge in-launch on bf16 unless the
     # separate-merge flag is set), output projection, residual, gate/up projection, SwiGLU, down projection, residual
-    def layer_launches(rows):
+    def layer_launches(rows, keys):
         n = 10 if (shape.dtype == "bf16" and args.flags & 8) else 9
         if not uses_tc:
             return n
         n -= (not args.flags & 16) + (not args.flags & 4)        # SwiGLU; rotary + cache write: in the projections' epilogues
         if rows > 64:
             n -= 2                                               # residual updates in the projections' epilogues
-        elif not (args.flags & (4 | 256)) and shape.d_ffn // 64 <= 148 * 2 * 13 // 16:
+        elif not (args.flags & (4 | 256)) and shape.d_ffn // 64 <= 148 * 2 * 13 // 16 and 4 * keys * shape.d_model <= 20 << 20:
             n += 1                                               # the gate / up prefetch helper on the forked stream
         return n
 
-    sal = shape.n_sal * (3 + layer_launches(1))
-    draft = sal + 1 + 2 + shape.aeb_layers * 4 + 3              # ... + (vocabulary projection, top-k slices, merge and tree)
-    if getattr(shape, "lm_rank", 0):
-        draft += 2                                               # low-rank heads: one more projection + a gather
-    verify = 1 + shape.n_layers * layer_launches(N) + 3          # row set-up, ..., head projection, argmax slices, merge
-    if uses_tc and N > 64:
-        verify += 1                                              # the last layer's update also takes the final norm: a kernel of its own
-    line["gpu_launches"] = (draft + verify + 1) * steps
+    def step_launches(keys):                                     # keys: the library's bound of the committed context
+        draft = shape.n_sal * (3 + layer_launches(1, keys)) + 1 + 2 + shape.aeb_layers * 4 + 3   # ... + (vocabulary projection, top-k slices, merge and tree)
+        if getattr(shape, "lm_rank", 0):
+            draft += 2                                           # low-rank heads: one more projection + a gather
+        verify = 1 + shape.n_layers * layer_launches(N, keys + N) + 3        # row set-up, ..., head projection, argmax slices, merge
+        if uses_tc and N > 64:
+            verify += 1                                          # the last layer's update also takes the final norm: a kernel of its own
+        return draft + verify + 1                                # ... + acceptance
+
+    line["gpu_launches"] = sum(step_launches(C_start + i * (K + 1)) for i in range(steps))
     if not args.no_cpu_baseline:
         v, cores, desc = cpu_baseline(shape, topo, gen_device=dev)
         line["cpu_baseline"] = {"value": v, "unit": UNIT, "cores": cores, "kind": "oracle", "sample": desc,
