@@ -60,6 +60,10 @@ enum {
                                     * hidden state alone; draft.fc{s} is then [d, d] instead of [d, 2d]            */
   AMPH_FLAG_CHUNKED_PREFILL = 128, /* prefill one chunk of 128 prompt tokens per weight pass instead of four */
   AMPH_FLAG_MMA_SYNC_ATTENTION = 32, /* bf16 tree attention on the warp-level mma.sync kernel instead of the tcgen05 / TMA one */
+  AMPH_FLAG_NO_PAIR_PROJECTION = 512, /* passes of more than 64 rows on the projection kernel of smaller ones, with rotary embedding,
+                                       * SwiGLU and residual update as kernels of their own, prompts in chunks of 128 rows, and key
+                                       * ranges that do not depend on what else a launch carries: every sum in one order, whatever the
+                                       * height of a pass.  Always so with lm_rank > 0 (see amph_config)                           */
   AMPH_FLAG_NO_SIDE_PREFETCH = 256  /* no helper stream: by default (bf16, a stream of the caller's own) every layer of the captured schedule of amph_step forks a small
                                      * kernel onto a second stream, created by amph_init, that pulls the head of the gate / up
                                      * weights into L2 while attention runs; it joins the caller's stream before amph_accept /
@@ -98,7 +102,8 @@ typedef struct {
   int32_t flags;          /* AMPH_FLAG_*                                                    */
   int32_t lm_rank;        /* 0: each drafting head owns a [vocab, d] matrix (Eq. 6); r > 0: it owns two
                            * low-rank factors a [r, d] and b [vocab, r], logits = b (a x) (Appendix A.2.4);
-                           * r a multiple of 8, r <= d_model                                  */
+                           * r a multiple of 8, r <= d_model.  Candidates of such heads lie within the rounding of bf16
+                           * activations of one another, so a context with r > 0 works as with AMPH_FLAG_NO_PAIR_PROJECTION  */
   float temperature;      /* 0: greedy decoding (Table 1).  T > 0: random sampling (Table 2): the target draws every
                            * token from softmax(logits / T), and a drafted token is accepted by the rejection-sampling
                            * test of Section 2 for a point-mass proposal (see amph_accept)                        */

@@ -97,6 +97,13 @@ struct amph_ctx {
   int ctx_hi[kMaxSeq] = {0};   // host-side upper bound of each sequence's committed length
   std::string err;
   TcGemm* tc;               // tensor-core projection plans (NULL when disabled / unsupported)
+  // Low-rank drafting heads have no margin between their candidates: at rank 256 and 32000 ids, neighbours in a head's order lie
+  // closer than the rounding of the bf16 passes before (gaps of 0.002-0.15 where two orders of summation differ by 0.04-0.2, of
+  // a standard deviation of 11), so which of them enter the tree, and with that how a text is cut into steps, hangs on the order of
+  // every sum.  Such a context keeps one order for passes of any height: no pair projection (its ranges of K follow from the
+  // number of rows), prompt chunks of 128 rows, key ranges that do not depend on what else a launch carries.  A step of 128 nodes
+  // at d = 4096 takes 1158 us in place of 1001 (4 layers, 2048 tokens).
+  bool one_order = false;
   AttnTc* attn_tc = nullptr; // tcgen05 tree attention (NULL: fp32 caches, disabled or unsupported)
   int sm_count = 148;
   bool last_proj_one_wave = false;   // the last projection ran on the tensor-core kernel with a fully resident grid
@@ -503,6 +510,11 @@ void fork_prefetch(amph_ctx* ctx, const LayerW& w, const Pass& ps) {
   ctx->side_dirty = true;
 }
 
+// KV splits per head of a launch of `groups` groups of `rows` rows (tcgen05 attention).
+int key_splits(const amph_ctx* ctx, int keys, int rows, int groups) {
+  return attn_tc_splits(ctx->attn_tc, keys, ctx->cfg.n_heads, ctx->one_order ? 1 : rows, ctx->one_order ? 1 : groups, ctx->lay.attn_splits);
+}
+
 // One decoder layer over the rows of the pass; cache_of(seq) gives the layer's cache of a sequence.
 // Entry: xn holds the input of the q/k/v projections: attn_norm * x / rms(x) if !entry_deferred, else
 // attn_norm * x with the row sums of squares in ss_a (the division is applied after the projection).
@@ -560,7 +572,7 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
     KvView kvs[kMaxSeq];
     int keys = 0;
     for (int g = 0; g < ps.G; ++g) { kvs[g] = cache_of(ps.seq[g]); keys = ps.keys[g] > keys ? ps.keys[g] : keys; }
-    const int splits = attn_tc_splits(ctx->attn_tc, keys, c.n_heads, ps.rpg, ps.G, l.attn_splits);
+    const int splits = key_splits(ctx, keys, ps.rpg, ps.G);
     grouped_attn = launch_tree_attention_tc_groups(ctx->attn_tc, ctx->ws + l.q, ctx->Rcap, ps.G, kvs, ps.meta, ps.rpg, c.n_heads,
                                                    c.head_dim, c.max_ctx, splits, keys, st, ctx->ws + l.att, &ctx->state(0)->err);
     if (!grouped_attn) cudaGetLastError();
@@ -574,7 +586,7 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
     const bool last_g = g + 1 == ps.G;
     bool done = false;
     if (ctx->attn_tc) {
-      const int splits = attn_tc_splits(ctx->attn_tc, ps.keys[g], c.n_heads, ps.rpg, 1, l.attn_splits);
+      const int splits = key_splits(ctx, ps.keys[g], ps.rpg, 1);
       const bool merged = !(c.flags & AMPH_FLAG_SEPARATE_MERGE);
       done = launch_tree_attention_tc(ctx->attn_tc, qg, ctx->Rcap - g * ps.rpg, kv, ps.meta[g], sc, ps.rpg, c.n_heads, c.head_dim,
                                       c.max_ctx, splits, ps.keys[g], st, merged ? og : nullptr, &ctx->state(0)->err);
@@ -928,7 +940,7 @@ cudaGraphNode_t find_accept_node(const amph_ctx* ctx, cudaGraph_t graph) {
 
 int attn_splits_for(const amph_ctx* ctx, int ctx_hi, int rows, int groups) {
   if (ctx->attn_tc) {         // split count and ring depth both shape the captured launch
-    const int sp = attn_tc_splits(ctx->attn_tc, ctx_hi, ctx->cfg.n_heads, rows, groups, ctx->lay.attn_splits);
+    const int sp = key_splits(ctx, ctx_hi, rows, groups);
     return sp * 8 + attn_tc_stages(ctx_hi, sp, ctx->cfg.head_dim);
   }
   int s = (ctx_hi + 127) / 128;
@@ -1026,6 +1038,7 @@ amph_status amph_init(const amph_config* cfg, const amph_tree* tree, void* kv_de
   ctx->resolved = false;
   ctx->phase = PH_CREATED;
   ctx->tc = nullptr;
+  ctx->one_order = cfg->weight_dtype == AMPH_DTYPE_BF16 && (cfg->lm_rank > 0 || (cfg->flags & AMPH_FLAG_NO_PAIR_PROJECTION));
   { int dv = 0; cudaGetDevice(&dv); cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, dv); }
   if (ctx->stream != nullptr && cfg->weight_dtype == AMPH_DTYPE_BF16 && !(cfg->flags & (AMPH_FLAG_NO_SIDE_PREFETCH | AMPH_FLAG_NO_TENSOR_CORE))) {
     if (cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1103,6 +1116,7 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
                                  c.d_model, c.d_model, c.d_model,
                                  c.lm_rank > 0 ? c.lm_rank : 8};
     ctx->tc = tc_gemm_create(xb, xrows, xcols, XB_COUNT, &ctx->state(0)->err);
+    if (ctx->tc && ctx->one_order) tc_wide_off(ctx->tc);
     if (ctx->tc) tc_wide_bind(ctx->tc, ctx->at<float>(ctx->lay.partial), ctx->lay.partial_floats, ctx->at<int>(ctx->lay.wide_flags));
   }
   if (!ctx->attn_tc && c.kv_dtype == AMPH_DTYPE_BF16 && !(c.flags & AMPH_FLAG_MMA_SYNC_ATTENTION))
@@ -1121,7 +1135,7 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
     const bool last = start + cnt == n;
     const int G = (cnt + M - 1) / M;
     // rows the kernels carry per group: the chunks of a pass are of equal height (130 tokens: 2 x 80 rows, not 2 x 128)
-    const int rpg = round_up((cnt + G - 1) / G, 16);
+    const int rpg = ctx->one_order && G > 1 ? M : round_up((cnt + G - 1) / G, 16);
     rc = cuda_check(ctx, cudaMemcpyAsync(ctx->at<int>(l.tok), prompt_ids + start, sizeof(int) * cnt, cudaMemcpyHostToDevice, st), "prompt upload");
     if (rc != AMPH_OK) return rc;
     Pass ps;

@@ -12,6 +12,11 @@
 //               tensor memory (tcgen05.ld), mask, running max / sum in fp32 (the maxima of the two halves meet in shared
 //               memory), probabilities to shared memory in bf16, running output in registers (the chunk outputs are added
 //               with the usual rescaling, so tensor memory never has to be rescaled).
+//
+// Every sum has one order, whichever warp holds the terms: a row's sum runs through a chunk's columns from the first to the last
+// (the second half's warp goes on from what the first half's hands it, behind the arrival that starts P V), splits are merged in
+// pairs (s, s + 4), (s, s + 2), (s, s + 1).  Sums that depended on how many warps share a row would move the bf16 rounding of the
+// output, and with it drafted candidates that lie within a rounding of one another.
 // The KV splits of one head form a thread-block cluster: every CTA sends its partial rows, one bulk copy per peer, to the CTAs
 // that merge them, into shared memory the owner no longer needs; with the separate merge the partials go to global scratch for
 // attn_combine_kernel.
@@ -225,7 +230,8 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
   __shared__ float max_s[2][2][kRows];               // [chunk parity][half][row]: maxima of the two halves of a chunk
-  __shared__ float sum_s[2][kRows];                  // [half][row]
+  __shared__ float2 part_s[kSoftmaxThreads / 2];     // [thread of a half]: sums over the first half of a chunk, handed to the second
+  __shared__ float sum_s[kRows];
   __shared__ u64 mask_s[kRows][2];                   // ancestor masks (registers are short: two CTAs share an SM)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -271,6 +277,7 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
   if (s_hi > prm.max_ctx) s_hi = prm.max_ctx;
   const int slots = (kRows + S - 1) / S;               // rows that one CTA of the cluster merges
   const uint32_t block_bytes = (uint32_t)slots * (DH + 4) * 4;
+  constexpr float kLn2 = 0.6931471805599453f;          // the running maximum is kept in base-2 units, merges work in natural ones
   constexpr uint32_t kRecvAt = DH == 128 ? 40 * 1024 : 20 * 1024;      // 71 rows of (DH + 4) floats lie below it
   const int n_chunks = s_hi > s_lo ? (s_hi - s_lo + kChunk - 1) / kChunk : 0;
 
@@ -350,7 +357,7 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
     const bool leader = elect_one();
     const uint32_t idesc_s = umma_idesc(kChunk, 0), idesc_o = umma_idesc(DH, 1);
     const uint32_t q_addr = smem_u32(Qs), p_addr = smem_u32(Ps);
-    auto issue_scores = [&](int c) {                   // S[c & 1] = Q K_c^T
+    auto issue_scores = [&](int c) {                   // S = Q K_c^T
       const uint32_t k_addr = smem_u32(St + (size_t)(c % stages) * kStage);
       const uint32_t d = tmem;
 #pragma unroll
@@ -485,7 +492,7 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
         for (int i = 0; i < DH / 4; ++i) acc[i] *= ((i >> 1) & 1) ? cb : ca;
       }
       const float sub_a = mn_a == -INFINITY ? 0.f : mn_a, sub_b = mn_b == -INFINITY ? 0.f : mn_b;
-      float ps_a = 0.f, ps_b = 0.f;
+      float2 ps = make_float2(0.f, 0.f), pair[kChunk / 16];       // sums of the thread's two columns of every group of 8, both rows
 #pragma unroll
       for (int rep = 0; rep < kChunk / 16; ++rep) {
         float p[4];
@@ -493,20 +500,31 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
         for (int e = 0; e < 4; ++e) {
           p[e] = ex2_approx(fmaf(s[rep * 4 + e], scale_log2, -(e < 2 ? sub_a : sub_b)));
         }
-        ps_a += p[0] + p[1];
-        ps_b += p[2] + p[3];
+        pair[rep] = make_float2(p[0] + p[1], p[2] + p[3]);
+        ps.x += pair[rep].x;
+        ps.y += pair[rep].y;
         // P block of this half (64 keys): row r, 16-byte chunk rep of its 128-byte row sits at chunk ^ (r % 8)
         uint8_t* blk = Ps + half * kQBlock + (((rep ^ (row_a & 7)) << 4) + qd * 4);
         *reinterpret_cast<uint32_t*>(blk + row_a * 128) = pack_bf16(p[0], p[1]);
         *reinterpret_cast<uint32_t*>(blk + (row_a + 8) * 128) = pack_bf16(p[2], p[3]);
       }
-      l_a = l_a * ca + ps_a;                           // this thread's share of the row sums (added up at the end)
-      l_b = l_b * cb + ps_b;
       m_a = mn_a;
       m_b = mn_b;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // P is read by the tensor core's async proxy
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       mbar_arrive(&p_ready);
+      // row sums, kept by the second half (barrier 5 + quarter; the next chunk's barrier above keeps part_s until it is read)
+      if (half == 0) {
+        part_s[quarter * 32 + lane] = ps;
+        asm volatile("bar.arrive %0, 64;" ::"r"(5 + quarter) : "memory");
+      } else {
+        asm volatile("bar.sync %0, 64;" ::"r"(5 + quarter) : "memory");
+        ps = part_s[quarter * 32 + lane];
+#pragma unroll
+        for (int rep = 0; rep < kChunk / 16; ++rep) { ps.x += pair[rep].x; ps.y += pair[rep].y; }
+        l_a = l_a * ca + ps.x;                         // this thread's columns (added up over the four threads of a row at the end)
+        l_b = l_b * cb + ps.y;
+      }
     }
     if (n_chunks > 0) ok = __all_sync(0xffffffffu, mbar_wait(&o_full, (n_chunks - 1) & 1, &abort_flag)) && ok;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -522,7 +540,7 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
       m_a = m_b = -INFINITY;
       l_a = l_b = 0.f;
     }
-    if (qd == 0) { sum_s[half][row_a] = l_a; sum_s[half][row_a + 8] = l_b; }
+    if (half == 1 && qd == 0) { sum_s[row_a] = l_a; sum_s[row_a + 8] = l_b; }
     if constexpr (MERGE) {                             // park the partial rows, in blocks of the rows that one CTA merges
 #pragma unroll
       for (int hi = 0; hi < 2; ++hi) {
@@ -530,10 +548,9 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
         float* dst = reinterpret_cast<float*>(smem + (size_t)owner * block_bytes) + (r - owner * slots) * DH + DH / 2 * half + 2 * qd;
 #pragma unroll
         for (int k = 0; k < DH / 16; ++k) *reinterpret_cast<float2*>(dst + 8 * k) = make_float2(acc[4 * k + 2 * hi], acc[4 * k + 2 * hi + 1]);
-        if (qd == 0) {                                 // (max, sum of the first half, sum of the second half, -)
+        if (qd == 0) {                                 // (max in natural units, sum, -, -)
           float* ml = reinterpret_cast<float*>(smem + (size_t)owner * block_bytes + slots * DH * 4) + (r - owner * slots) * 4;
-          if (half == 0) *reinterpret_cast<float2*>(ml) = make_float2(hi ? m_b : m_a, hi ? l_b : l_a);
-          else ml[2] = hi ? l_b : l_a;
+          ml[half] = half == 0 ? (hi ? m_b : m_a) * kLn2 : hi ? l_b : l_a;
         }
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the copies to the peers read through the async proxy
@@ -574,14 +591,19 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
       float M = -INFINITY;
       for (int s = 0; s < S; ++s) M = fmaxf(M, *reinterpret_cast<const float*>(parts + (size_t)s * block_bytes + (slots * DH + slot * 4) * 4));
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      float den = 0.f;
-      for (int s = 0; s < S; ++s) {
+      float d[8];                                      // at most eight splits
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        d[s] = 0.f;
+        if (s >= S) continue;
         const float* blk = reinterpret_cast<const float*>(parts + (size_t)s * block_bytes);
-        const float4 ml = *reinterpret_cast<const float4*>(blk + slots * DH + slot * 4), v = *reinterpret_cast<const float4*>(blk + slot * DH + col);
-        const float w = ml.x == -INFINITY ? 0.f : exp2f(ml.x - M);             // the running maximum is kept in base-2 units
-        den += (ml.y + ml.z) * w;
+        const float2 ml = *reinterpret_cast<const float2*>(blk + slots * DH + slot * 4);
+        const float4 v = *reinterpret_cast<const float4*>(blk + slot * DH + col);
+        const float w = ml.x == -INFINITY ? 0.f : expf(ml.x - M);
+        d[s] = __fmul_rn(ml.y, w);
         a.x += v.x * w; a.y += v.y * w; a.z += v.z * w; a.w += v.w * w;
       }
+      const float den = ((d[0] + d[4]) + (d[2] + d[6])) + ((d[1] + d[5]) + (d[3] + d[7]));
       const float inv = den > 0.f ? 1.0f / den : 0.f;
       *reinterpret_cast<uint2*>(prm.out + (size_t)(row_base + gr) * prm.n_heads * DH + h * DH + col) =
           make_uint2(pack_bf16(a.x * inv, a.y * inv), pack_bf16(a.z * inv, a.w * inv));
@@ -589,10 +611,9 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
     __syncwarp();
     if (S > 1) cluster_wait();                         // nobody leaves while a copy may still read its shared memory
   } else {
-    constexpr float kLn2 = 0.6931471805599453f;        // the separate merge works in natural units
     if (warp >= 2) {
-      l_a = sum_s[0][row_a] + sum_s[1][row_a];
-      l_b = sum_s[0][row_a + 8] + sum_s[1][row_a + 8];
+      l_a = sum_s[row_a];
+      l_b = sum_s[row_a + 8];
 #pragma unroll
       for (int hi = 0; hi < 2; ++hi) {
         const int gr = rb * kRows + row_a + 8 * hi;

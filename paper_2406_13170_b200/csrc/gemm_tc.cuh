@@ -41,6 +41,7 @@ bool tc_gemm_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
 constexpr int kWideFrom = 64;            // rows above this take it
 constexpr int kWideFlags = 256;
 void tc_wide_init(TcGemm* g);
+void tc_wide_off(TcGemm* g);             // later launches of the plan set never take it
 void tc_wide_bind(TcGemm* g, float* scratch, size_t scratch_floats, int* flags);
 bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out, int in, int rows, float* P, size_t p_floats,
                     int* splits, size_t* split_stride, cudaStream_t st);

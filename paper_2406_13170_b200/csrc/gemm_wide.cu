@@ -721,6 +721,11 @@ void tc_wide_init(TcGemm* g) {
   }
 }
 
+void tc_wide_off(TcGemm* g) {
+  g->wide_pairs = 0;
+  for (int& c : g->resid_clusters) c = 0;
+}
+
 void tc_wide_bind(TcGemm* g, float* scratch, size_t scratch_floats, int* flags) {
   g->wide_scratch = scratch;
   g->wide_scratch_floats = scratch_floats / 64 * 64;
