@@ -457,6 +457,8 @@ void bind_tables(const amph_ctx* ctx, Pass* ps, bool sal, int source) {
   p.inv_freq = ctx->at<double>(l.inv_freq);
   p.state = ctx->ws + l.state;
   p.state_stride = l.state_s;
+  p.clear = nullptr;
+  p.n_clear = 0;
   for (int g = 0; g < kMaxSeq; ++g) p.base[g] = p.n[g] = 0;
   for (int g = 0; g < ps->G; ++g) {
     ps->meta[g] = reinterpret_cast<const RowMeta*>(p.meta + p.meta_stride * g);
@@ -1142,6 +1144,10 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
     ps.G = G;
     ps.rpg = rpg;
     bind_tables(ctx, &ps, false, PassRows::kChain);
+    if (start == 0 && ctx->tc) {                  // a timeout before may have left a flag of the pair projection raised
+      ps.src.clear = ctx->at<int>(l.wide_flags);
+      ps.src.n_clear = kWideFlags;
+    }
     for (int g = 0; g < G; ++g) {
       const int nr = cnt - g * rpg < rpg ? cnt - g * rpg : rpg;
       ps.src.base[g] = start + g * rpg;
@@ -1525,6 +1531,8 @@ amph_status amph_set_state(amph_ctx* ctx, int32_t ctx_len, int32_t root, int32_t
   s.next_root = root;
   for (int j = 0; j < 16; ++j) { s.path[j] = -1; s.out_tok[j] = -1; }
   amph_status rc = cuda_check(ctx, cudaMemcpyAsync(ctx->state(0), &s, sizeof s, cudaMemcpyHostToDevice, ctx->stream), "set_state");
+  if (rc == AMPH_OK)                                               // with the error word (see amph_prefill_seq)
+    rc = cuda_check(ctx, cudaMemsetAsync(ctx->at<int>(ctx->lay.wide_flags), 0, sizeof(int) * kWideFlags, ctx->stream), "set_state");
   if (rc == AMPH_OK) rc = cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "set_state");       // s lives on this stack frame
   if (rc == AMPH_OK)
     rc = cuda_check(ctx, cudaMemcpyAsync(ctx->at<float>(ctx->lay.pend_h), pend_hidden, sizeof(float) * (size_t)n_pending * c.d_model,
@@ -1545,6 +1553,7 @@ amph_status amph_profile_breakdown(amph_ctx* ctx, double* ms, int64_t* launches)
 amph_status amph_reset(amph_ctx* ctx) {
   if (!ctx) return fail(nullptr, AMPH_ERR_INVALID_ARG, "ctx must not be NULL");
   cudaError_t e = cudaMemsetAsync(ctx->ws + ctx->lay.state, 0, ctx->lay.state_s * kMaxSeq, ctx->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->at<int>(ctx->lay.wide_flags), 0, sizeof(int) * kWideFlags, ctx->stream);
   ctx->phase = PH_CREATED;
   for (int b = 0; b < kMaxSeq; ++b) { ctx->ctx_hi[b] = 0; ctx->prefilled[b] = false; }
   return cuda_check(ctx, e, "reset");

@@ -142,6 +142,7 @@ struct PassRows {
   const double* inv_freq;
   const char* state; size_t state_stride;    // DevState (kPending)
   int base[AMPH_MAX_BATCH], n[AMPH_MAX_BATCH];
+  int* clear; int n_clear;                   // ints that the first kernel of a target pass sets to zero, or NULL
 };
 void launch_target_rows(const PassRows& p, int G, const void* tok_emb, int dtype, const int* toks, int vocab, int d, const void* gain,
                         float eps, float* x, void* xn, cudaStream_t st);

@@ -244,7 +244,7 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
       for (int i = first; i < issued; ++i) {
         const int s = i % stages, round = i / stages;
         const unsigned long long t0 = now_ns();
-        while (!mbar_try(&full_bar[s], round & 1) && now_ns() - t0 < limit_ns) {}
+        while (!mbar_try(&full_bar[s], round & 1) && now_ns() - t0 < kDrainNs) {}
       }
     }
   } else if (warp == 1) {
@@ -498,7 +498,7 @@ bool tc_gemm_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   if (!g || xb < 0 || xb >= g->n_x) return false;
   if (out % kTileM || in % kTileK || n_seg < 1 || n_seg > kMaxSeg || rows < 1) return false;
   if (g->xcols[xb] != in) return false;
-  if (rows > kWideFrom && g->extra_tx == 0 && tc_wide_launch(g, xb, w, n_seg, out, in, rows, P, p_floats, splits_out, split_stride, st)) return true;
+  if (rows > kWideFrom && tc_wide_launch(g, xb, w, n_seg, out, in, rows, P, p_floats, splits_out, split_stride, st)) return true;
   // up to 128 rows: one MMA of N = rows rounded up to 16; more: 2..4 row blocks of 128 rows that share every weight tile
   // (the tile is streamed from HBM once and multiplied with each block: batched verification, dense prefill)
   const int nt_all = rows <= 16 ? 16 : (rows <= 128 ? (rows + 15) / 16 * 16 : (rows + 127) / 128 * 128);

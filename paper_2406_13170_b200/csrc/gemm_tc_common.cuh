@@ -22,6 +22,7 @@ constexpr int kUmmaK = 16;            // K per tcgen05.mma for 16-bit inputs
 constexpr int kStageKb = 2;           // 64-wide K blocks fetched by one TMA copy (one pipeline stage) when both operands' stage fits twice per CTA
 constexpr int kMaxSeg = 8;
 constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // a barrier wait gives up after one second
+constexpr unsigned long long kDrainNs = 10000000ull;         // what a CTA that gave up allows each of its copies to land (they take microseconds)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 

@@ -59,7 +59,8 @@ struct WideParams {
   size_t split_stride;
   int ld;
   float* scratch;           // [pair][cta][quad of rows][128 features] float4: partial sums of a pair's first segment
-  int* flags;               // [pair][cta]; zero between launches (whoever consumes a flag lowers it)
+  int* flags;               // [pair][cta]; zero between launches (whoever consumes a flag lowers it; a launch in which a wait gave up
+                            // may leave one raised: whoever clears the error word clears them too)
   float* x;                 // RESID: residual rows, updated in place
   const __nv_bfloat16* gain;      // the next norm's gain, or NULL: x only
   __nv_bfloat16* xn;        // gain * x
@@ -74,6 +75,7 @@ struct WideParams {
   int wait_first;           // see tc_gemm_wait_first
   int* err_flag;
   unsigned long long wait_limit_ns;
+  uint32_t extra_tx;        // self-test only: bytes that a pair's first stage expects beyond what is copied
 };
 
 struct Segment { int tile, u0, u1; };     // units [u0, u1) of a tile's K range
@@ -245,11 +247,11 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     // ---------------- TMA producer of this CTA's half of the operands
     const bool leader = elect_one();
     const uint64_t wpol = l2_evict_first_policy();
-    auto load_w = [&](int st, const Segment& s, int u) {
+    auto load_w = [&](int st, const Segment& s, int u, uint32_t more) {
       const int seg = s.tile / prm.tiles_per_seg, lt = s.tile - seg * prm.tiles_per_seg;
       const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), lead);
       uint8_t* dst = smem + (size_t)st * stage_bytes;
-      if (rank == 0) mbar_expect_tx(&full_bar[st], 2 * stage_bytes);
+      if (rank == 0) mbar_expect_tx(&full_bar[st], 2 * stage_bytes + more);
       if (EPI == WIDE_SWIGLU) tma_pair_4d(dst, &maps.w[0], 0, (lt * 2 + (int)rank) * (kTileM / 2), 0, u * kUnitKb, bar, wpol);
       else tma_pair_3d(dst, &maps.w[seg], 0, (lt * 2 + (int)rank) * kTileM, u * kUnitKb, bar, wpol);
     };
@@ -261,7 +263,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     bool have = it.next(sg);
     int u = have ? sg.u0 : 0, i = 0;
     for (; i < stages && have; ++i) {
-      if (leader) load_w(i, sg, u);
+      if (leader) load_w(i, sg, u, i == 0 ? prm.extra_tx : 0u);
       if (++u == sg.u1) { have = it.next(sg); u = sg.u0; }
     }
     __syncwarp();
@@ -269,16 +271,17 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     for (; have; ++i) {
       const int st = i % stages, round = i / stages;
       if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[st], (round & 1) ^ 1, &abort_flag, limit_ns))) break;
-      if (leader) { load_w(st, sg, u); load_x(st, u); }
+      if (leader) { load_w(st, sg, u, 0u); load_x(st, u); }
       __syncwarp();
       if (++u == sg.u1) { have = it.next(sg); u = sg.u0; }
     }
     for (int j = i > stages ? i - stages : 0; j < i; ++j)  // every commit to this CTA's barriers has arrived
       if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[j % stages], (j / stages) & 1, &abort_flag, limit_ns))) break;
     if (abort_flag && rank == 0 && lane == 0) {          // drain: both CTAs' copies signal the even CTA's barriers
-      const unsigned long long t0 = now_ns();
-      for (int j = i > stages ? i - stages : 0; j < i; ++j)
-        while (!mbar_try(&full_bar[j % stages], (j / stages) & 1) && now_ns() - t0 < limit_ns) {}
+      for (int j = i > stages ? i - stages : 0; j < i; ++j) {
+        const unsigned long long t0 = now_ns();
+        while (!mbar_try(&full_bar[j % stages], (j / stages) & 1) && now_ns() - t0 < kDrainNs) {}
+      }
     }
   } else if (warp == 1) {
     // ---------------- the ring's first activations, then MMA issuer (even CTA)
@@ -476,10 +479,10 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
           }
         }
         epi_sync();
-        ok = ok && *(volatile int*)&abort_flag == 0;
+        ok = __all_sync(0xffffffffu, ok && *(volatile int*)&abort_flag == 0);
       }
-      // a wait that gave up (the error flag is raised): this piece is not written.  Uniform over the epilogue warps only behind
-      // a barrier, so the fused forms, which need barriers of their own, run through with whatever the accumulator holds.
+      // a wait that gave up: the plain form writes nothing.  Uniform over the epilogue warps only behind a barrier, so the fused forms,
+      // which need barriers of their own, run through with whatever the accumulator holds; the end of the kernel replaces both.
       const int seg = sg.tile / prm.tiles_per_seg, lt = sg.tile - seg * prm.tiles_per_seg;
       const float4* src = scratch + ((size_t)(pair + prm.nrb) * 2 + rank) * slot_quads;
       const size_t next_helper = (size_t)prm.nrb * 2 * slot_quads;
@@ -599,7 +602,42 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_slot), "r"(prm.tmem_cols) : "memory");
   }
   __syncthreads();
-  if (threadIdx.x == 0 && abort_flag && prm.err_flag) *prm.err_flag = AMPH_ERR_TIMEOUT;
+  if (abort_flag) {
+    // A wait gave up.  Zeros in place of whatever this CTA has written: the caches must hold finite values whatever happens, because
+    // attention fetches whole tiles of them and masks by a probability of zero.  Out of the way of the main path: a test per batch
+    // of the epilogue cost a prefill of 128 tokens 0.4 %.
+    SegIter it = {range_begin(prm, group), range_begin(prm, group + 1), prm.units_per_tile};
+    Segment sg;
+    const int row0 = rb * n, my_rows = prm.rows - row0 < n ? prm.rows - row0 : n;
+    const __nv_bfloat16 zero = __float2bfloat16(0.f);
+    while (it.next(sg)) {
+      if (prm.splits == 0 && sg.u0 > 0) continue;          // the pair that has the tile's first K columns writes it
+      const int seg = sg.tile / prm.tiles_per_seg, lt = sg.tile - seg * prm.tiles_per_seg;
+      for (int i = threadIdx.x; i < my_rows * kTileM; i += kWideThreads) {
+        const int r = i / kTileM, c = i - r * kTileM, row = row0 + r;
+        if constexpr (EPI == WIDE_PLAIN) {
+          prm.P[(size_t)(prm.splits > 0 ? group % prm.splits : 0) * prm.split_stride + (size_t)row * prm.ld + (size_t)sg.tile * 256 + rank * kTileM + c] = 0.f;
+        } else if constexpr (EPI == WIDE_SWIGLU) {
+          if (c < kTileM / 2) prm.act[(size_t)row * prm.f + (size_t)(lt * 2 + (int)rank) * (kTileM / 2) + c] = zero;
+        } else if constexpr (EPI == WIDE_ROPE) {
+          const int g = row / prm.gr.rpg, rl = row - g * prm.gr.rpg, feat = (lt * 2 + (int)rank) * kTileM + c, head = feat / prm.dh;
+          const RowMeta* meta = prm.gr.meta[g];
+          const int slot = meta->slot[rl];
+          if (seg == 0) prm.q[(size_t)row * prm.n_heads * prm.dh + feat] = zero;
+          else if (rl < meta->n_rows && slot >= 0 && slot < prm.max_ctx)
+            ((__nv_bfloat16*)(seg == 1 ? prm.gr.kc[g] : prm.gr.vc[g]))[((size_t)head * prm.max_ctx + slot) * prm.dh + feat - head * prm.dh] = zero;
+        } else {
+          const int per = ((n + prm.splits - 1) / prm.splits + 7) / 8 * 8, lo = (int)(crank >> 1) * per;      // this CTA's share of the rows
+          if (r < lo || r >= lo + per) continue;
+          const size_t at = (size_t)row * prm.out + (size_t)sg.tile * 256 + rank * kTileM + c;
+          prm.x[at] = 0.f;
+          if (prm.gain != nullptr) prm.xn[at] = zero;
+          if (prm.gain != nullptr && c == 0) prm.ss[(size_t)row * (prm.out / kTileM) + sg.tile * 2 + rank] = 0.f;
+        }
+      }
+    }
+    if (threadIdx.x == 0 && prm.err_flag) *prm.err_flag = AMPH_ERR_TIMEOUT;
+  }
 }
 
 constexpr size_t kWideSmem = 220 * 1024;                  // ring + alignment; the static part needs up to 6 KB of the 227
@@ -658,6 +696,7 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
   prm->wait_first = g->wait_first;
   prm->err_flag = g->err_flag;
   prm->wait_limit_ns = g->wait_limit_ns;
+  prm->extra_tx = g->extra_tx;
   return true;
 }
 

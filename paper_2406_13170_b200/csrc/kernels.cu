@@ -221,6 +221,8 @@ target_rows_kernel(const PassRows p, const T* __restrict__ emb, const int* __res
   extern __shared__ __align__(16) float rowbuf[];
   __shared__ float red[32];
   const int r = blockIdx.x, g = r / p.rpg;
+  if (r == 0 && p.clear != nullptr)
+    for (int i = threadIdx.x; i < p.n_clear; i += blockDim.x) p.clear[i] = 0;
   int t = toks[r];
   t = t < 0 ? 0 : (t >= vocab ? vocab - 1 : t);
   const T* e = emb + (size_t)t * d;

@@ -144,3 +144,53 @@ def test_set_state_teacher_forces_the_draft():
         assert ids[k, :shape.topk[k]].tolist() == o_ids[k]
     assert m.get_tensor("tree_tokens", (topo.n_nodes,), torch.int32)[0].item() == forced_root
     m.close()
+
+
+@pytest.mark.parametrize("rows", [100, 300])
+def test_a_bounded_wait_of_the_pair_projection_runs_out(rows):
+    """The same for passes of more than 64 rows (two CTAs share a tile: the first stage of every pair can never fill)."""
+    from paper_2406_13170_b200 import binding
+    x = inputs.normal_tensor((384, 512), 1.0, 3, "x", dtype=torch.bfloat16).cuda()
+    w = inputs.normal_tensor((768, 512), 0.05, 3, "w", dtype=torch.bfloat16).cuda()
+    status, y = binding.selftest_wait_timeout(x, [w, w], rows=rows, limit_us=1000)
+    assert status == 8
+    assert torch.equal(y, torch.zeros_like(y))
+    y2 = binding.project(x, [w, w], rows=rows, use_tensor_core=True)
+    ref = x[:rows].double() @ torch.cat([w, w]).double().T
+    assert float((y2.double() - ref).abs().max()) < 1e-3 * float(ref.abs().max()) + 1e-4
+
+
+def test_nothing_of_a_timeout_outlives_a_reset_or_a_prefill():
+    """A wait that gave up may leave hand-over flags of the pair projection raised (the last 256 ints of the workspace): with one
+    raised, the next launch would add sums that are not written yet.  What clears the error word clears them."""
+    from paper_2406_13170_b200 import Amphista
+    shape = inputs.get_shape("small_bf16").with_(d_model=1024, n_heads=8, d_ffn=2816)
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    prompt = inputs.make_prompt(shape.with_(prompt_len=300), seed=4).tolist()
+    m = Amphista(shape, topo, w, max_ctx=512)
+
+    def result():
+        root = m.prefill(prompt)
+        return root, m.get_tensor("hidden", (300, shape.d_model)).clone()
+
+    want = result()
+    flags = m.ws[-1024:].view(torch.int32)
+
+    def raise_all():
+        m.synchronize()
+        assert int(flags.abs().sum()) == 0                       # zero between launches
+        flags.fill_(1)
+        torch.cuda.synchronize()
+
+    raise_all()
+    got = result()
+    assert got[0] == want[0] and torch.equal(got[1], want[1])
+    for clear in (m.reset, lambda: m.set_state(300, want[0], want[1][-1:], [want[0]])):
+        raise_all()
+        clear()
+        m.synchronize()
+        assert int(flags.abs().sum()) == 0
+        got = result()
+        assert got[0] == want[0] and torch.equal(got[1], want[1])
+    m.close()
