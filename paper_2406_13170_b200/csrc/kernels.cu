@@ -937,9 +937,10 @@ __device__ void block_best(float& v, int& i, float* sv, int* si) {
 
 struct TopkCounts { int c[kMaxK]; };
 
-// Selection keys: a larger key is a better candidate in the order above.  The high word orders the values (-0 counts as +0),
-// 0 is below every value and marks "nothing left".
+// Selection keys: a larger key is a better candidate in the order above (-0 counts as +0); 0 is below every value and marks
+// "nothing left", which is also what a NaN is: it compares with nothing, so it is nobody's candidate.
 __device__ __forceinline__ uint32_t order_key(float v) {
+  if (v != v) return 0u;
   const uint32_t u = __float_as_uint(v == 0.f ? 0.f : v);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }

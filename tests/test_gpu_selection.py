@@ -47,6 +47,31 @@ def test_candidates_are_the_exact_top_k(name, vocab, topk, batch):
 
 
 @pytest.mark.parametrize("name", ["tiny", "small_bf16"])
+def test_a_nan_logit_is_nobodys_candidate(name):
+    """Ids whose logit is not a number (either sign) are passed over; a head without any number has no candidates (id 2^31 - 1)."""
+    from paper_2406_13170_b200 import Amphista
+    shape = inputs.get_shape(name).with_(topk=(16, 5, 2, 3))
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    bad = torch.arange(0, shape.vocab, 3, device="cuda:0")
+    w["draft.lm_head.0"][bad] = float("nan")
+    w["draft.lm_head.1"][bad] = -float("nan")
+    w["draft.lm_head.3"][:] = float("nan")
+    m = Amphista(shape, topo, w)
+    m.prefill(inputs.make_prompt(shape).tolist())
+    ids = torch.zeros(shape.K, 16, dtype=torch.int32, device="cuda:0")
+    m.draft(ids)
+    m.synchronize()
+    logits = m.get_tensor("d_logits", (shape.K, shape.vocab)).cpu()
+    for k in range(3):
+        assert bool(torch.isnan(logits[k]).any()) == (k < 2)
+        want = torch.sort(logits[k].nan_to_num(nan=-float("inf")), descending=True, stable=True).indices
+        assert ids[k, :shape.topk[k]].tolist() == want[:shape.topk[k]].tolist()
+    assert ids[3, :3].tolist() == [2 ** 31 - 1] * 3
+    m.close()
+
+
+@pytest.mark.parametrize("name", ["tiny", "small_bf16"])
 def test_accepted_rows_move_in_every_layer(name):
     shape = inputs.get_shape(name)
     B = 3
