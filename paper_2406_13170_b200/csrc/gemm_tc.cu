@@ -498,15 +498,15 @@ bool tc_gemm_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   if (!g || xb < 0 || xb >= g->n_x) return false;
   if (out % kTileM || in % kTileK || n_seg < 1 || n_seg > kMaxSeg || rows < 1) return false;
   if (g->xcols[xb] != in) return false;
-  if (rows > kWideFrom && tc_wide_launch(g, xb, w, n_seg, out, in, rows, P, p_floats, splits_out, split_stride, st)) return true;
   // up to 128 rows: one MMA of N = rows rounded up to 16; more: 2..4 row blocks of 128 rows that share every weight tile
   // (the tile is streamed from HBM once and multiplied with each block: batched verification, dense prefill)
   const int nt_all = rows <= 16 ? 16 : (rows <= 128 ? (rows + 15) / 16 * 16 : (rows + 127) / 128 * 128);
   const int nblk = nt_all <= 128 ? 1 : nt_all / 128;
   const int nt = nblk == 1 ? nt_all : 128;
-  if (nblk > 4 || nt_all > g->xrows[xb]) return false;
-  const int tiles = n_seg * (out / kTileM), kblocks = in / kTileK;
   const size_t ld = (size_t)n_seg * out;
+  if (nblk > 4 || nt_all > g->xrows[xb] || (size_t)nt_all * ld > p_floats) return false;      // whichever kernel takes it
+  if (rows > kWideFrom && tc_wide_launch(g, xb, w, n_seg, out, in, rows, P, p_floats, splits_out, split_stride, st)) return true;
+  const int tiles = n_seg * (out / kTileM), kblocks = in / kTileK;
   // K-splits: nearly two CTAs per SM (7/8 of the slots measured best: one split fewer costs no bandwidth and
   // saves partial sums), keep at least four 64-wide K blocks per CTA.  With several row blocks a CTA needs most of an
   // SM's shared and tensor memory: one CTA per SM.
@@ -518,7 +518,6 @@ bool tc_gemm_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   if (splits > 16) splits = 16;
   while (splits > 1 && (size_t)splits * nt_all * ld > p_floats) --splits;
   if (splits < 1) splits = 1;
-  if ((size_t)nt_all * ld > p_floats) return false;
   TmapPack pack;
   memset(&pack, 0, sizeof pack);
   for (int s = 0; s < n_seg; ++s) {

@@ -59,3 +59,21 @@ def test_tensor_core_rejects_uncovered_shapes():
     x = torch.zeros(16, 688, dtype=torch.bfloat16, device=dev)
     with pytest.raises(AmphError):
         project(x, [w], 4, True)
+
+
+@pytest.mark.parametrize("rows,cap", [(9, 9), (33, 47), (70, 79), (100, 100), (128, 127), (129, 255), (300, 383), (512, 511)])
+def test_activation_buffers_shorter_than_the_kernels_blocks_are_refused(rows, cap):
+    """x must hold rows rounded up to 16, or to 128 beyond 128 rows, on every tensor-core route."""
+    from paper_2406_13170_b200 import project, project_noalloc
+    from paper_2406_13170_b200.binding import AmphError
+    w = torch.zeros(256, 128, dtype=torch.bfloat16, device="cuda:0")
+    need = (rows + 15) // 16 * 16 if rows <= 128 else (rows + 127) // 128 * 128
+    project(torch.zeros(need, 128, dtype=torch.bfloat16, device="cuda:0"), [w], rows, True)
+    x = torch.zeros(cap, 128, dtype=torch.bfloat16, device="cuda:0")
+    with pytest.raises(AmphError) as e:
+        project(x, [w], rows, True)
+    assert e.value.status == 2                                       # AMPH_ERR_SHAPE
+    if rows <= 128:
+        with pytest.raises(AmphError) as e:
+            project_noalloc(x, [w], rows, True, torch.zeros(rows, 256, device="cuda:0"))
+        assert e.value.status == 2
