@@ -1,5 +1,6 @@
 // Host side of the Amphista step library: argument validation, workspace layout, weight
 // registry and the kernel schedule of prefill / draft / verify / accept (declared in amph.h).
+#include <cuda.h>
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -106,6 +107,8 @@ struct amph_ctx {
   bool one_order = false;
   AttnTc* attn_tc = nullptr; // tcgen05 tree attention (NULL: fp32 caches, disabled or unsupported)
   int sm_count = 148;
+  int device = 0;
+  CUresult (*address_range)(CUdeviceptr*, size_t*, CUdeviceptr) = nullptr;   // cuMemGetAddressRange
   bool last_proj_one_wave = false;   // the last projection ran on the tensor-core kernel with a fully resident grid
   cudaStream_t side = nullptr;            // forked stream of the gate / up prefetch helpers (NULL: disabled)
   std::vector<cudaEvent_t> fork_ev;       // one event per fork of a step, reused from step to step
@@ -895,19 +898,25 @@ amph_status do_accept(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n, int32_
   return rc;
 }
 
-// Whether a kernel of this context may write to p.
-bool device_memory(const void* p) {
+// Whether a kernel of this context may write `bytes` to p: whole ints inside one allocation of its own, current device.  Anything
+// else is left to a copy, which takes any address and alignment and refuses what it cannot reach.
+bool kernel_may_write(const amph_ctx* ctx, const void* p, size_t bytes) {
   if (!p) return true;
   cudaPointerAttributes at;
   int dev = 0;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (((uintptr_t)p & 3) || !ctx->address_range) return false;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
-  return at.type == cudaMemoryTypeDevice && at.device == dev;
+  if (at.type != cudaMemoryTypeDevice || at.device != ctx->device || dev != ctx->device) return false;
+  return ctx->address_range(&base, &size, (CUdeviceptr)(uintptr_t)p) == CUDA_SUCCESS && (uintptr_t)p - base + bytes <= size;
 }
 
 // Points a captured step's results at the caller's arrays (*written), or at none: the caller copies them.  False: the schedule
 // could not be changed and may hold an earlier call's arrays, so it must not run again.
 bool redirect_results(amph_ctx* ctx, amph_ctx::StepGraph* g, int32_t* out_tokens, int32_t* out_n, bool* written) {
-  *written = g->accept && device_memory(out_tokens) && device_memory(out_n);
+  *written = g->accept && kernel_may_write(ctx, out_tokens, sizeof(int32_t) * ctx->B * (ctx->cfg.K + 1)) &&
+             kernel_may_write(ctx, out_n, sizeof(int32_t) * ctx->B);
   if (!*written) out_tokens = out_n = nullptr;
   if (g->out_tokens == out_tokens && g->out_n == out_n) return true;
   cudaKernelNodeParams np;
@@ -1041,7 +1050,14 @@ amph_status amph_init(const amph_config* cfg, const amph_tree* tree, void* kv_de
   ctx->phase = PH_CREATED;
   ctx->tc = nullptr;
   ctx->one_order = cfg->weight_dtype == AMPH_DTYPE_BF16 && (cfg->lm_rank > 0 || (cfg->flags & AMPH_FLAG_NO_PAIR_PROJECTION));
-  { int dv = 0; cudaGetDevice(&dv); cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, dv); }
+  cudaGetDevice(&ctx->device);
+  cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device);
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult found;
+  if (cudaGetDriverEntryPoint("cuMemGetAddressRange", &fn, cudaEnableDefault, &found) == cudaSuccess && found == cudaDriverEntryPointSuccess)
+    ctx->address_range = (CUresult(*)(CUdeviceptr*, size_t*, CUdeviceptr))fn;
+  else
+    cudaGetLastError();
   if (ctx->stream != nullptr && cfg->weight_dtype == AMPH_DTYPE_BF16 && !(cfg->flags & (AMPH_FLAG_NO_SIDE_PREFETCH | AMPH_FLAG_NO_TENSOR_CORE))) {
     if (cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->join_ev, cudaEventDisableTiming) != cudaSuccess) {

@@ -87,3 +87,29 @@ def test_results_reach_whatever_arrays_a_step_is_given(batch):
         return [(None if t is None else t.tolist(), None if n is None else n.tolist()) for t, n in outs]
 
     assert run(0) == run(2)                       # 2: kernels launched one by one, results copied
+
+
+@pytest.mark.parametrize("batch", [1, 3])
+def test_results_reach_arrays_at_any_byte(batch):
+    """Device arrays that do not start at a multiple of four bytes: results arrive by copy."""
+    from paper_2406_13170_b200 import Amphista
+    shape = inputs.get_shape("small_bf16")
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    K = shape.K
+    outs = []
+    for shifts in (((0, 0), (0, 0), (0, 0), (0, 0)), ((1, 0), (0, 2), (3, 1), (0, 0))):
+        m = Amphista(shape, topo, w, max_batch=batch, max_ctx=512)
+        for b in range(batch):
+            m.prefill(inputs.make_prompt(shape, seed=b).tolist(), seq=b)
+        got = []
+        for st, sn in shifts:
+            t = torch.zeros(4 * batch * (K + 1) + 4, dtype=torch.uint8, device="cuda:0")
+            n = torch.zeros(4 * batch + 4, dtype=torch.uint8, device="cuda:0")
+            m.step(t[st:], n[sn:])
+            m.synchronize()
+            got.append((t[st:].cpu()[:4 * batch * (K + 1)].clone().view(torch.int32).tolist(), n[sn:].cpu()[:4 * batch].clone().view(torch.int32).tolist()))
+        m.close()
+        outs.append(got)
+    assert outs[0] == outs[1]
+    assert all(1 <= c <= K + 1 for _, n in outs[0] for c in n)
