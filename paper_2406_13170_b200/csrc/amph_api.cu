@@ -6,6 +6,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <array>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -115,9 +116,11 @@ struct amph_ctx {
   size_t fork_used = 0;
   cudaEvent_t join_ev = nullptr;
   bool side_dirty = false;                // helpers were launched since the last join
-  // captured draft -> verify -> accept schedules of amph_step, by the attention grids they were sized for
+  // captured draft -> verify -> accept schedules of amph_step, by what they were sized for: the prefetch helper and the attention
+  // grids of the draft's and the verification's passes, per sequence (or one for all, see step_key)
+  typedef std::array<int, 2 + 2 * kMaxSeq> StepKey;
   struct StepGraph {
-    long long key;
+    StepKey key;
     cudaGraphExec_t exec;
     unsigned long long used;
     cudaGraph_t graph;                    // owns the nodes; accept: the one that writes a step's results (NULL: not found)
@@ -979,17 +982,19 @@ constexpr size_t kMaxGraphs = 16;
 
 // The captured schedule depends on the host's bounds only through the prefetch helper and the attention launches: one per
 // sequence, or, where the sequences of a batch share a launch (layer_forward), one sized for the longest of them.
-long long graph_key_of(const amph_ctx* ctx) {
+amph_ctx::StepKey step_key(const amph_ctx* ctx) {
+  const int N = ctx->tree_host.n_nodes, B = ctx->B;
+  amph_ctx::StepKey key = {};
   long long keys = 0;
-  for (int b = 0; b < ctx->B; ++b) keys += ctx->ctx_hi[b];
-  const int helper = (prefetch_pays(ctx, keys) ? 2 : 0) + (prefetch_pays(ctx, keys + (long long)ctx->B * ctx->tree_host.n_nodes) ? 1 : 0);
-  long long key = helper;
-  if (ctx->attn_tc && ctx->B > 1 && !(ctx->cfg.flags & AMPH_FLAG_SEPARATE_MERGE))
-    return helper * 128 * 128 + attn_splits_for(ctx, ctx->max_ctx_hi(), ctx->rows_small, ctx->B) * 128 +
-           attn_splits_for(ctx, ctx->max_ctx_hi() + ctx->tree_host.n_nodes, ctx->Mver, ctx->B);
-  for (int b = 0; b < ctx->B; ++b)
-    key = key * 4099 + attn_splits_for(ctx, ctx->ctx_hi[b], ctx->rows_small, 1) * 128 +
-          attn_splits_for(ctx, ctx->ctx_hi[b] + ctx->tree_host.n_nodes, ctx->Mver, 1);
+  for (int b = 0; b < B; ++b) keys += ctx->ctx_hi[b];
+  key[0] = prefetch_pays(ctx, keys);
+  key[1] = prefetch_pays(ctx, keys + (long long)B * N);
+  const bool shared = ctx->attn_tc && B > 1 && !(ctx->cfg.flags & AMPH_FLAG_SEPARATE_MERGE);
+  for (int b = 0; b < (shared ? 1 : B); ++b) {
+    const int hi = shared ? ctx->max_ctx_hi() : ctx->ctx_hi[b], groups = shared ? B : 1;
+    key[2 + 2 * b] = attn_splits_for(ctx, hi, ctx->rows_small, groups);
+    key[3 + 2 * b] = attn_splits_for(ctx, hi + N, ctx->Mver, groups);
+  }
   return key;
 }
 
@@ -1256,7 +1261,7 @@ amph_status amph_step(amph_ctx* ctx, int32_t* out_tokens, int32_t* out_n) {
   if (use_graph) {
     // The kernels read every length from device state; only the attention grids and the
     // prefetch helper depend on the host's bound of the context length, so a captured schedule serves every step that has the same.
-    const long long key = graph_key_of(ctx);
+    const amph_ctx::StepKey key = step_key(ctx);
     for (auto& g : ctx->graphs)
       if (g.key == key) sg = &g;
     if (!sg) {

@@ -39,6 +39,22 @@ def test_lengths_that_come_back(name, lengths):
     plain.close()
 
 
+def test_eight_sequences_of_different_lengths():
+    """Eight sequences with a split count each: combinations that differ in one of them only are different schedules."""
+    from paper_2406_13170_b200 import Amphista
+    shape = inputs.get_shape("tiny")
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    texts = {n: inputs.make_prompt(shape.with_(prompt_len=n), seed=n).tolist() for n in (20, 150, 280)}
+    graphs = Amphista(shape, topo, w, max_batch=8, max_ctx=512)
+    plain = Amphista(shape, topo, w, max_batch=8, max_ctx=512, flags=2)
+    for longer in (None, 0, 7, 3, 0, None):
+        prompts = [texts[280 if b == longer else 150 if b % 2 else 20] for b in range(8)]
+        assert _decode(graphs, prompts, 2) == _decode(plain, prompts, 2), longer
+    graphs.close()
+    plain.close()
+
+
 def test_context_grows_past_the_prefetch_helper():
     """20 MB of keys and values per layer: below, a step's schedule has a prefetch helper per layer, above, none; first the
     verification pass crosses the line, then the draft."""
