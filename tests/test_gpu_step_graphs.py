@@ -129,3 +129,31 @@ def test_results_reach_arrays_at_any_byte(batch):
         outs.append(got)
     assert outs[0] == outs[1]
     assert all(1 <= c <= K + 1 for _, n in outs[0] for c in n)
+
+
+def test_helper_launches_follow_the_context():
+    """The schedule that a step replays has a helper for every layer of a pass that may read at most 20 MB of keys and values per
+    layer, and none for the others: counted from the kernels that ran, with lengths that come back."""
+    from paper_2406_13170_b200 import Amphista
+    from torch.profiler import ProfilerActivity, profile
+    shape = inputs.get_shape("small_bf16")
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    limit, N = (20 << 20) // (4 * shape.d_model), shape.n_nodes
+    m = Amphista(shape, topo, w, max_ctx=limit + N + 64)
+    root = m.prefill(inputs.make_prompt(shape.with_(prompt_len=limit + 1), seed=1).tolist())
+    pending = torch.ones(1, shape.d_model)
+    both, draft, none = shape.n_sal + shape.n_layers, shape.n_sal, 0
+    for n, want in ((limit - N, both), (limit - N + 1, draft), (limit, draft), (limit + 1, none), (limit - N, both), (limit, draft)):
+        m.set_state(n, root, pending, [root])
+        m.step()                                  # captures the schedule, or finds it
+        m.set_state(n, root, pending, [root])
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            m.step()
+            torch.cuda.synchronize()
+        names = [e.key for e in prof.key_averages() for _ in range(e.count)]
+        if not any("accept_compact_kernel" in k for k in names):
+            pytest.skip("the profiler records no kernels here")
+        assert sum("tc_prefetch_pair_kernel" in k for k in names) == want, n
+    m.close()
