@@ -245,6 +245,8 @@ class Amphista:
 
     def get_tensor(self, name: str, shape, dtype=torch.float32) -> torch.Tensor:
         out = torch.empty(shape, dtype=dtype, device=self.device)
+        if not torch.cuda.current_stream(self.device).query():
+            self._after_torch()               # kernels torch has queued may still use the block that `out` was given
         with torch.cuda.device(self.device):
             self._check(self.L.amph_get_tensor(self.ctx, name.encode(), _ptr(out), out.numel() * out.element_size()),
                         self.ctx)

@@ -53,3 +53,27 @@ def test_reuse_and_bitwise_determinism(name):
     assert e[0] == a[0] and e[1:3] == a[1:3]
     assert torch.equal(e[3], a[3]) and torch.equal(e[4], a[4])
     m2.close()
+
+
+def test_a_tap_is_not_overwritten_by_what_torch_has_queued():
+    """get_tensor's result may sit in a block of torch's pool that kernels queued on torch's stream still write."""
+    from paper_2406_13170_b200 import Amphista
+    shape = inputs.get_shape("small_bf16")
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    m = Amphista(shape, topo, inputs.make_weights(shape, seed=0, device="cuda:0"))
+    n = 48
+    m.prefill(inputs.make_prompt(shape.with_(prompt_len=n)).tolist())
+    want = m.get_tensor("logits", (n, shape.vocab)).clone()
+    for cycles in (1, 100_000_000):                    # the second time about 50 ms (the first one loads the kernels)
+        torch.cuda.synchronize()
+        busy = torch.empty(n, shape.vocab, device="cuda:0")
+        torch.cuda._sleep(cycles)
+        busy.fill_(7.0)
+        block = busy.data_ptr()
+        del busy
+        got = m.get_tensor("logits", (n, shape.vocab))
+        assert got.data_ptr() == block
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
+        del got
+    m.close()
