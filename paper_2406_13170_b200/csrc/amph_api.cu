@@ -1139,7 +1139,7 @@ amph_status amph_prefill_seq(amph_ctx* ctx, int32_t seq, const int32_t* prompt_i
                                  c.d_model, c.d_model, c.d_model,
                                  c.lm_rank > 0 ? c.lm_rank : 8};
     ctx->tc = tc_gemm_create(xb, xrows, xcols, XB_COUNT, &ctx->state(0)->err);
-    if (ctx->tc && ctx->one_order) tc_wide_off(ctx->tc);
+    if (ctx->tc) ctx->one_order ? tc_wide_off(ctx->tc) : tc_wide_init(ctx->tc);
     if (ctx->tc) tc_wide_bind(ctx->tc, ctx->at<float>(ctx->lay.partial), ctx->lay.partial_floats, ctx->at<int>(ctx->lay.wide_flags));
   }
   if (!ctx->attn_tc && c.kv_dtype == AMPH_DTYPE_BF16 && !(c.flags & AMPH_FLAG_MMA_SYNC_ATTENTION))

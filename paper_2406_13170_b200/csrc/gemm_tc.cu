@@ -489,7 +489,6 @@ TcGemm* tc_gemm_create(void* const* xbufs, const int* xrows, const int* xcols, i
   cudaFuncSetAttribute(tc_gemm_kernel<EPI_PARTIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, g->max_smem - 2048);
   cudaFuncSetAttribute(tc_gemm_kernel<EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, g->max_smem - 2048);
   cudaFuncSetAttribute(tc_gemm_kernel<EPI_ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, g->max_smem - 2048);
-  tc_wide_init(g);
   return g;
 }
 

@@ -40,7 +40,7 @@ bool tc_gemm_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
 // kWideFlags ints) that cut tiles go through; the fused forms need them.  tc_gemm_launch takes the plain form by itself.
 constexpr int kWideFrom = 64;            // rows above this take it
 constexpr int kWideFlags = 256;
-void tc_wide_init(TcGemm* g);
+void tc_wide_init(TcGemm* g);            // optional: asks the device about it now (a plan set that is kept may meet it inside a capture)
 void tc_wide_off(TcGemm* g);             // later launches of the plan set never take it
 void tc_wide_bind(TcGemm* g, float* scratch, size_t scratch_floats, int* flags);
 bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out, int in, int rows, float* P, size_t p_floats,

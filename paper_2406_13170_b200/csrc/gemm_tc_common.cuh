@@ -169,12 +169,12 @@ struct TcGemm {
     return &(pair_cache[key] = m);
   }
 
-  // pair kernel: CTA pairs that run at a time (0: not available), scratch and flags of cut tiles
-  int wide_pairs = 0;
+  // pair kernel: CTA pairs that run at a time (0: not available, -1: not asked yet), scratch and flags of cut tiles
+  int wide_pairs = -1;
   float* wide_scratch = nullptr;
   size_t wide_scratch_floats = 0;
   int* wide_flags = nullptr;
-  int resid_clusters[5] = {0, 0, 0, 0, 0};     // clusters of that many pairs that run at a time (residual form)
+  int resid_clusters[5] = {0, 0, 0, 0, 0};     // clusters of that many pairs that run at a time (residual form); [0]: asked
 
   const CUtensorMap* get(const void* ptr, int rows, int cols, int box_rows, int box_kb = tc::kStageKb) {
     auto key = std::make_tuple(ptr, rows, cols, box_rows, box_kb);

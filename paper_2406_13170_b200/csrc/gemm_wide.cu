@@ -643,12 +643,61 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
 constexpr size_t kWideSmem = 220 * 1024;                  // ring + alignment; the static part needs up to 6 KB of the 227
 constexpr size_t kResidSmem = 225 * 1024;                 // 256 parked rows and three quarters of them received; 1 KB static
 
+// Clusters of `ctas` that run at a time (0: none, or the question failed).
+int active_clusters(const TcGemm* g, const void* kernel, int ctas, size_t smem) {
+  int n = 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(g->sm_count / ctas * ctas);
+  cfg.blockDim = dim3(kWideThreads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+  return n;
+}
+bool allow_smem(const void* kernel, size_t bytes) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
+}
+
+// What runs at a time, asked for by the first launch that may take the kernel (or by tc_wide_init): amph_project makes a plan set
+// per call, mostly for fewer rows, and needs the plain form only (16 rows: 14.7 us of host time per call when every plan set asked for
+// everything, 13.5 now; 100 rows 10.8, now 9.7).
+bool wide_available(TcGemm* g) {
+  if (!g) return false;
+  if (g->wide_pairs < 0) {
+    g->wide_pairs = 0;
+    if ((size_t)g->max_smem >= kWideSmem + 7 * 1024 && allow_smem((const void*)tc_wide_kernel<WIDE_PLAIN>, kWideSmem) &&
+        allow_smem((const void*)tc_wide_kernel<WIDE_SWIGLU>, kWideSmem) && allow_smem((const void*)tc_wide_kernel<WIDE_ROPE>, kWideSmem)) {
+      const int clusters = active_clusters(g, (const void*)tc_wide_kernel<WIDE_ROPE>, 2, kWideSmem);
+      g->wide_pairs = clusters < g->sm_count / 2 ? clusters : g->sm_count / 2;
+    }
+  }
+  return g->wide_pairs > 1;
+}
+// clusters of 1 .. 4 pairs of the residual form
+bool resid_available(TcGemm* g) {
+  if (!wide_available(g)) return false;
+  if (g->resid_clusters[0] == 0) {
+    g->resid_clusters[0] = 1;
+    if (allow_smem((const void*)tc_wide_kernel<WIDE_RESID>, kResidSmem))
+      for (int s = 1; s <= 4; ++s) g->resid_clusters[s] = active_clusters(g, (const void*)tc_wide_kernel<WIDE_RESID>, 2 * s, kResidSmem);
+  }
+  return true;
+}
+
 // Everything of a launch that does not depend on the epilogue; false: the shape is not covered.
 template <int EPI>
 bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int rows, int splits, float* scratch_end, size_t scratch_floats,
                  WideMaps* maps, WideParams* prm) {
   constexpr size_t out_bytes = EPI == WIDE_SWIGLU || EPI == WIDE_ROPE ? kPark : 0;
-  if (!g || g->wide_pairs < 2 || xb < 0 || xb >= g->n_x || g->xcols[xb] != in) return false;
+  if (!wide_available(g) || xb < 0 || xb >= g->n_x || g->xcols[xb] != in) return false;
   if (in % kTileK || rows < 32 || rows > kMaxWideRows || rows > g->xrows[xb] || n_seg < 1 || n_seg > kMaxSeg) return false;
   memset(maps, 0, sizeof *maps);
   memset(prm, 0, sizeof *prm);
@@ -721,48 +770,10 @@ bool wide_run(const WideMaps& maps, const WideParams& prm, cudaStream_t st) {
 
 }  // namespace
 
-void tc_wide_init(TcGemm* g) {
-  g->wide_pairs = 0;
-  if ((size_t)g->max_smem < kWideSmem + 7 * 1024) return;
-  int clusters = 0;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(g->sm_count / 2 * 2);
-  cfg.blockDim = dim3(kWideThreads);
-  cfg.dynamicSmemBytes = kWideSmem;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  if (cudaFuncSetAttribute(tc_wide_kernel<WIDE_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_wide_kernel<WIDE_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem) != cudaSuccess ||
-      cudaFuncSetAttribute(tc_wide_kernel<WIDE_ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem) != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&clusters, tc_wide_kernel<WIDE_ROPE>, &cfg) != cudaSuccess || clusters < 1) {
-    cudaGetLastError();
-    return;
-  }
-  g->wide_pairs = clusters < g->sm_count / 2 ? clusters : g->sm_count / 2;
-  // clusters of 1 .. 4 pairs that run at a time
-  cfg.dynamicSmemBytes = kResidSmem;
-  if (cudaFuncSetAttribute(tc_wide_kernel<WIDE_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidSmem) != cudaSuccess) {
-    cudaGetLastError();
-    return;
-  }
-  for (int s = 1; s <= 4; ++s) {
-    cfg.gridDim = dim3(g->sm_count / (2 * s) * (2 * s));
-    at[0].val.clusterDim.x = 2 * s;
-    if (cudaOccupancyMaxActiveClusters(&g->resid_clusters[s], tc_wide_kernel<WIDE_RESID>, &cfg) != cudaSuccess) {
-      cudaGetLastError();
-      g->resid_clusters[s] = 0;
-    }
-  }
-}
+void tc_wide_init(TcGemm* g) { resid_available(g); }
 
 void tc_wide_off(TcGemm* g) {
   g->wide_pairs = 0;
-  for (int& c : g->resid_clusters) c = 0;
 }
 
 void tc_wide_bind(TcGemm* g, float* scratch, size_t scratch_floats, int* flags) {
@@ -773,7 +784,7 @@ void tc_wide_bind(TcGemm* g, float* scratch, size_t scratch_floats, int* flags) 
 
 bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out, int in, int rows, float* P, size_t p_floats,
                     int* splits_out, size_t* split_stride, cudaStream_t st) {
-  if (!g || g->wide_pairs < 2 || out % 256 || in % kTileK) return false;
+  if (out % 256 || in % kTileK || !wide_available(g)) return false;
   const int tiles = n_seg * (out / 256), units = (in / kTileK + kUnitKb - 1) / kUnitKb;
   const size_t ld = (size_t)n_seg * out, stride = (size_t)rows * ld;
   if (stride > p_floats) return false;
@@ -809,7 +820,7 @@ bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
 
 bool tc_wide_launch_resid(TcGemm* g, int xb, const void* w, int out, int in, int rows, float* x, const void* gain, void* xn, float* ss,
                           cudaStream_t st) {
-  if (!g || !w || !x || out % 256 || in % kTileK || ((uintptr_t)w & 15) || (gain && (!xn || !ss))) return false;
+  if (!g || !w || !x || out % 256 || in % kTileK || ((uintptr_t)w & 15) || (gain && (!xn || !ss)) || !resid_available(g)) return false;
   // as many K ranges per tile as run at a time, at least four K blocks each
   const int items = out / 256 * (rows > 256 ? 2 : 1), units = (in / kTileK + kUnitKb - 1) / kUnitKb;
   int splits = 4;

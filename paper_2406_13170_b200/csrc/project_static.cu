@@ -109,7 +109,10 @@ amph_status amph_project_noalloc(const void* x_dev, int32_t x_rows_cap, const vo
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lock(g_setup_mutex);
     TcGemm*& g = g_plans[dev];
-    if (!g) g = tc_gemm_create(xb, xr, xc, 1, err);
+    if (!g) {
+      g = tc_gemm_create(xb, xr, xc, 1, err);
+      if (g) tc_wide_init(g);
+    }
     if (!g) { say(err_msg, err_len, "tensor-map encoder unavailable or not an sm_100 device"); return AMPH_ERR_CUDA; }
     tc_gemm_wait_first(g);
     tc_gemm_rebind(g, 0, xb[0], xr[0], xc[0], err);
