@@ -766,8 +766,10 @@ gemm_generic_kernel(const T* __restrict__ X, int ldx, const __grid_constant__ Ge
   }
 }
 
-// R = 4 for the drafting heads' few rows, else 16; two features a warp (half of the shared-memory reads) once one feature a warp
-// gives more than two blocks per SM.
+// R = 4 for the drafting heads' few rows, 8 for theirs in a batch of two, else 16 (the rows a block does not have cost it as much
+// as those it has: 5 to 8 rows in blocks of 16 took 70 us at 11008 x 4096 in bf16, now 41; 102 at 3 x 4096 x 4096 in fp32, now 73); two
+// features a warp (half of the shared-memory reads) once one feature a warp gives more than two blocks per SM (8 rows: 51 us and
+// 82 us with one).
 void launch_gemm_generic(const void* x, int ldx, const GemmSeg* segs, int n_seg, int out, int in, float* P,
                          int ldp, int rows, int dtype, cudaStream_t st, int wait_first) {
   GemmSegs gs;
@@ -779,6 +781,8 @@ void launch_gemm_generic(const void* x, int ldx, const GemmSeg* segs, int n_seg,
   };
   AMPH_DISPATCH(dtype, const T* X = (const T*)x;
                 if (rows <= 4) run(gemm_generic_kernel<T, 4, 1>, 4, 1, X);
+                else if (rows <= 8 && blocks * n_seg <= 296) run(gemm_generic_kernel<T, 8, 1>, 8, 1, X);
+                else if (rows <= 8) run(gemm_generic_kernel<T, 8, 2>, 8, 2, X);
                 else if ((long long)blocks * n_seg * ((rows + 15) / 16) <= 296) run(gemm_generic_kernel<T, 16, 1>, 16, 1, X);
                 else run(gemm_generic_kernel<T, 16, 2>, 16, 2, X));
 }

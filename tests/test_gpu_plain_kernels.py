@@ -25,6 +25,14 @@ def test_projection_against_double(dtype, rows, n_seg, out, inner):
     assert bool(((y - want).abs() <= bound).all())
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("rows", [6, 8, 9])
+@pytest.mark.parametrize("n_seg,out,inner", [(3, 9, 256), (8, 296, 264), (8, 297, 520), (1, 2369, 128)])
+def test_blocks_of_eight_rows(dtype, rows, n_seg, out, inner):
+    """Five to eight rows; 296 and 297 blocks of one feature per warp are the two sides of two features per warp."""
+    test_projection_against_double(dtype, rows, n_seg, out, inner)
+
+
 @pytest.mark.parametrize("heads,dh", [(4, 64), (2, 128)])
 @pytest.mark.parametrize("n", [1, 15, 48, 63, 64, 65, 111, 113, 200, 400])
 def test_tree_attention_inside_a_step(heads, dh, n):
