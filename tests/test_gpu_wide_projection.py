@@ -50,3 +50,48 @@ def test_fused_forms_against_the_separate_kernels(heads, dh, ffn, n):
         # three layers of unit gain, as in the parity tests' bound
         assert float((a - b).abs().max()) <= 2e-2 * max(1.0, float(b.abs().max()))
         assert float((a - b).norm() / b.norm()) <= 1e-2
+
+
+# 384 = 3 * 128: the q / k / v and the residual form decline (they own 256 columns at a time), gate / up does not
+@pytest.mark.parametrize("heads,dh,ffn", [(8, 64, 1408), (4, 128, 1408), (3, 128, 1408), (10, 128, 3456)])
+@pytest.mark.parametrize("n", [70, 128, 300, 513])
+def test_pair_projections_against_the_kernels_of_fewer_rows(heads, dh, ffn, n):
+    from paper_2406_13170_b200 import Amphista
+    shape = inputs.get_shape("small_bf16").with_(d_model=heads * dh, n_heads=heads, head_dim=dh, d_ffn=ffn, prompt_len=n, n_nodes=100,
+                                                 topk=(16, 16, 16, 16))
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    prompt = inputs.make_prompt(shape, seed=2).tolist()
+    toks = torch.randint(0, shape.vocab, (shape.n_nodes,), dtype=torch.int32, generator=torch.Generator().manual_seed(n)).cuda()
+    outs = []
+    for flags in (0, 512):                        # 512: no pair projection, and with it no residual update in an epilogue
+        m = Amphista(shape, topo, w, max_ctx=1024, flags=flags)
+        m.prefill(prompt)
+        m.set_tensor("root", toks[:1])
+        m.draft()
+        m.verify_tree(toks)
+        m.synchronize()
+        outs.append([m.get_tensor("hidden", (shape.n_nodes, shape.d_model)), m.get_tensor("logits", (shape.n_nodes, shape.vocab))] +
+                    [m.get_tensor(f"kv.{c}.{shape.n_layers - 1}", (n + shape.n_nodes, shape.d_model)) for c in "kv"])
+        m.close()
+    for a, b in zip(*outs):
+        assert bool(torch.isfinite(a).all())
+        assert float((a - b).norm() / b.norm()) <= 1e-2       # sums in another order, roundings to bf16 in the same places (see above)
+
+
+@pytest.mark.parametrize("n", [70, 97, 128])
+def test_residual_update_behind_the_same_sums(n):
+    """At widths of 256 nothing is split along K, so both routes have the same sums, and with SwiGLU and the rotary embedding as
+    kernels of their own on both sides what differs is the residual update: in the output and down projections' epilogues, or as a
+    kernel of its own.  Both add 128 columns' squares in a warp, then the two parts: bit for bit the same."""
+    shape = inputs.get_shape("small_bf16").with_(d_model=256, n_heads=4, head_dim=64, d_ffn=256, n_layers=4, prompt_len=n)
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    prompt = inputs.make_prompt(shape, seed=2).tolist()
+    outs = []
+    for flags in (4 | 16, 4 | 16 | 512):
+        m = Amphista(shape, topo, w, max_ctx=512, flags=flags)
+        m.prefill(prompt)
+        outs.append(m.get_tensor("hidden", (n, shape.d_model)))
+        m.close()
+    assert torch.equal(outs[0], outs[1])
