@@ -84,6 +84,7 @@ def test_residual_update_behind_the_same_sums(n):
     """At widths of 256 nothing is split along K, so both routes have the same sums, and with SwiGLU and the rotary embedding as
     kernels of their own on both sides what differs is the residual update: in the output and down projections' epilogues, or as a
     kernel of its own.  Both add 128 columns' squares in a warp, then the two parts: bit for bit the same."""
+    from paper_2406_13170_b200 import Amphista
     shape = inputs.get_shape("small_bf16").with_(d_model=256, n_heads=4, head_dim=64, d_ffn=256, n_layers=4, prompt_len=n)
     topo = inputs.make_tree(shape.n_nodes, shape.topk)
     w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
