@@ -48,7 +48,7 @@ def algorithmic_bytes(shape, ctx_len: int) -> int:
 # bytes of a launch, so the step's average launch is scaled by this ratio.  The counters belong to one version of the
 # kernel: the digest below is that of the kernel source they were taken with, and the field is null for any other source.
 NCU_TRAFFIC_PER_WEIGHT_BYTE = 1.03
-NCU_KERNEL_SOURCE_SHA256_16 = "ccf1f32d5acbd32d"
+NCU_KERNEL_SOURCE_SHA256_16 = "919be553d09979f8"
 
 
 def kernel_source_digest() -> str:
@@ -431,13 +431,17 @@ def main():
     # kernels launched per step: projections + the fixed schedule around them (counted from the schedule)
     # per layer: q/k/v projection, rotary + cache write, attention (its KV splits merge in-launch on bf16 unless the
     # separate-merge flag is set), output projection, residual, gate/up projection, SwiGLU, down projection, residual
+    # passes of more than 64 rows: the pair projection, unless the context keeps one order of sums
+    pairs = uses_tc and not args.flags & 512 and not getattr(shape, "lm_rank", 0)
+
     def layer_launches(rows, keys):
         n = 10 if (shape.dtype == "bf16" and args.flags & 8) else 9
         if not uses_tc:
             return n
-        n -= (not args.flags & 16) + (not args.flags & 4)        # SwiGLU; rotary + cache write: in the projections' epilogues
+        if rows <= 64 or pairs:
+            n -= (not args.flags & 16) + (not args.flags & 4)    # SwiGLU; rotary + cache write: in the projections' epilogues
         if rows > 64:
-            n -= 2                                               # residual updates in the projections' epilogues
+            n -= 2 * pairs                                       # residual updates in the projections' epilogues
         elif not (args.flags & (4 | 256)) and shape.d_ffn // 64 <= 148 * 2 * 13 // 16 and 4 * keys * shape.d_model <= 20 << 20:
             n += 1                                               # the gate / up prefetch helper on the forked stream
         return n
@@ -447,8 +451,8 @@ def main():
         if getattr(shape, "lm_rank", 0):
             draft += 2                                           # low-rank heads: one more projection + a gather
         verify = 1 + shape.n_layers * layer_launches(N, keys + N) + 3        # row set-up, ..., head projection, argmax slices, merge
-        if uses_tc and N > 64:
-            verify += 1                                          # the last layer's update also takes the final norm: a kernel of its own
+        if N > 64:
+            verify += pairs                                      # the last layer's update also takes the final norm: a kernel of its own
         return draft + verify + 1                                # ... + acceptance
 
     line["gpu_launches"] = sum(step_launches(C_start + i * (K + 1)) for i in range(steps))
