@@ -442,7 +442,7 @@ def main():
             n -= (not args.flags & 16) + (not args.flags & 4)    # SwiGLU; rotary + cache write: in the projections' epilogues
         if rows > 64:
             n -= 2 * pairs                                       # residual updates in the projections' epilogues
-        elif not (args.flags & (4 | 256)) and shape.d_ffn // 64 <= 148 * 2 * 13 // 16 and 4 * keys * shape.d_model <= 20 << 20:
+        elif not (args.flags & (4 | 256)) and 4 * keys * shape.d_model <= 20 << 20:
             n += 1                                               # the gate / up prefetch helper on the forked stream
         return n
 

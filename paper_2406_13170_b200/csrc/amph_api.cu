@@ -306,8 +306,10 @@ void make_layout(const amph_config& c, int n_nodes, Layout* L, int* Mcap_out, si
   l.att_o = l.per_group(4 * (size_t)splits * c.n_heads * Mcap * c.head_dim, &l.att_o_s);
   l.att_ml = l.per_group(4 * (size_t)splits * c.n_heads * Mcap * 2, &l.att_ml_s);
   l.logits = l.take(4 * (size_t)Rcap * V);
-  l.ss_a = l.take(4 * (size_t)Rcap * (c.d_model / kWideScaleCols + 32));
-  l.ss_b = l.take(4 * (size_t)Rcap * (c.d_model / kWideScaleCols + 32));
+  // one entry per tile of the kernel that updates the residual: 128 columns, 16 in a small model
+  const size_t ss_cols = c.d_model / (c.d_model <= kRowsResidMax ? 16 : kWideScaleCols) + 32;
+  l.ss_a = l.take(4 * (size_t)Rcap * ss_cols);
+  l.ss_b = l.take(4 * (size_t)Rcap * ss_cols);
   l.wide_flags = l.take(sizeof(int) * kWideFlags);
   *L = l;
   *Mcap_out = Mcap;
@@ -482,11 +484,14 @@ RowScale rows_from(RowScale rs, int row0) {
 }
 
 // While attention, the output projection and the residual kernel of a layer run, HBM is nearly idle (they are latency
-// chains over L2-resident data).  A helper on a forked stream uses that window to pull the head of the layer's gate / up
-// weights (kGateUpPrefetchBytes, about a third of them at 7B) into L2, so that the gate / up projection starts on L2 hits.
-// Forked right after the q / k / v projection is launched: measured -1.5 % per step; forked after the attention or the output
-// projection it costs 2-5 % (an event between two programmatically dependent launches), as does a larger budget.
-constexpr size_t kGateUpPrefetchBytes = 56u << 20;
+// chains over L2-resident data).  A helper on a forked stream uses that window to pull kGateUpPrefetchBytes of the layer's gate / up
+// weights into L2, spread evenly over the K range, so that the gate / up projection mixes L2 hits with its stream from HBM.
+// Us per step with 0 / 28 / 56 / 75 / 92 / 110 MB: d = 4096 x 8 layers, 64 rows 1288 / 1261 / 1243 / 1242 / 1244 / 1250, 16 rows
+// 1190 / 1178 / 1163 / 1162 / 1174 / 1190; d = 5120 x 8 layers 1693 / 1681 / 1657 / 1639 / 1660 / 1651; d = 6656 x 6 layers
+// 2273 / 2189 / 2180 / 2160 / 2175 / 2168.  (The first 56 MB of the K range instead: 1271 at d = 4096, and a loss at 6656.)
+// Forked right after the q / k / v projection is launched; forked after the attention or the output projection it costs 2-5 %
+// (an event between two programmatically dependent launches).
+constexpr size_t kGateUpPrefetchBytes = 75u << 20;
 // The window closes as the context grows: attention then streams keys and values itself, and its first chunks wait behind the
 // helper's.  us per step with / without the helper, d = 4096 x 16 layers: 520 keys 2016 / 2056, 1000 2092 / 2093, 1500 2113 / 2103,
 // 2000 2188 / 2147, 3000 2221 / 2175, 4500 2382 / 2300; d = 5120 x 12 layers: 500 keys 2201 / 2220, from 1024 on equal.  Equal on
@@ -504,8 +509,6 @@ void fork_prefetch(amph_ctx* ctx, const LayerW& w, const Pass& ps) {
   for (int g = 0; g < ps.G; ++g) keys += ps.keys[g];
   if (!prefetch_pays(ctx, keys)) return;
   const amph_config& c = ctx->cfg;
-  // a gate / up launch of about a full wave (two CTAs per SM) gains nothing: measured +0.3 % at d_ffn = 17920 (280 tiles)
-  if (c.d_ffn / 64 > ctx->sm_count * 2 * 13 / 16) return;
   // only inside the captured schedule of amph_step: launched call by call, the host-side fork and join cost more than the
   // prefetch gains (measured +95 us per step on the draft / verify / accept path)
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -556,7 +559,10 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
   }
   if (!fused_rope && ctx->tc && ps.G == 1 && !(c.flags & AMPH_FLAG_SEPARATE_ROPE)) {   // q / k / v projection that rotates and writes the cache itself
     ProfScope p(ctx, AMPH_PROF_PROJECTION);
-    fused_rope = tc_gemm_launch_qkv_rope(ctx->tc, XB_XN, w.wq, w.wk, w.wv, c.n_heads, c.head_dim, c.d_model, rows, ctx->ws + l.q,
+    fused_rope = tc_rows_launch_qkv_rope(ctx->tc, XB_XN, w.wq, w.wk, w.wv, c.n_heads, c.head_dim, c.d_model, rows, ctx->ws + l.q,
+                                         cache_of(ps.seq[0]), ps.meta[0], ps.rope[0], c.max_ctx, rs, st);
+    if (!fused_rope) cudaGetLastError();
+    if (!fused_rope) fused_rope = tc_gemm_launch_qkv_rope(ctx->tc, XB_XN, w.wq, w.wk, w.wv, c.n_heads, c.head_dim, c.d_model, rows, ctx->ws + l.q,
                                          cache_of(ps.seq[0]), ps.meta[0], ps.rope[0], c.max_ctx, rs, st);
     if (fused_rope && p.rec) ctx->prof_bytes += 3LL * c.d_model * c.d_model * (int64_t)ctx->esz;
     if (!fused_rope) cudaGetLastError();
@@ -606,11 +612,15 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
       launch_tree_attention(qg, kv, ps.meta[g], sc, og, ctx->dtype, ps.rpg, c.n_heads, c.head_dim, c.max_ctx, ps.keys[g],
                             l.attn_splits, st, last_g && ctx->tc != nullptr, (c.flags & AMPH_FLAG_SEPARATE_MERGE) != 0);
   }
-  // output projection and residual update: one kernel for many rows
+  // output projection and residual update: one kernel for many rows, and in a small model
+  int resid_cols = kWideScaleCols;
   auto resid_fused = [&](int xb, const void* wt, int in, const void* gain, size_t ss) {
-    if (!ctx->tc || rows <= kWideFrom) return false;
+    if (!ctx->tc) return false;
+    if (rows <= kWideFrom && (ctx->one_order || c.d_model > kRowsResidMax || in > kRowsResidMax)) return false;
     ProfScope p(ctx, AMPH_PROF_PROJECTION);
-    const bool done = tc_wide_launch_resid(ctx->tc, xb, wt, c.d_model, in, rows, x, gain, ctx->ws + l.xn, ctx->at<float>(ss), st);
+    const bool done = rows > kWideFrom
+                          ? tc_wide_launch_resid(ctx->tc, xb, wt, c.d_model, in, rows, x, gain, ctx->ws + l.xn, ctx->at<float>(ss), st)
+                          : tc_rows_launch_resid(ctx->tc, xb, wt, c.d_model, in, rows, x, gain, ctx->ws + l.xn, ctx->at<float>(ss), &resid_cols, st);
     if (!done) cudaGetLastError();
     if (done && p.rec) ctx->prof_bytes += (int64_t)c.d_model * in * (int64_t)ctx->esz;
     if (done) ctx->last_proj_one_wave = false;
@@ -624,16 +634,18 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
     launch_resid_scale(x, P, 0, 1, w.ffn_norm, ctx->dtype, ctx->ws + l.xn, ctx->at<float>(l.ss_b), rows, c.d_model, st,
                        ctx->last_proj_one_wave);
   }
-  const RowScale rs_b = row_scale_of(ctx, l.ss_b, fused_o ? kWideScaleCols : kScaleChunkCols);
+  const RowScale rs_b = row_scale_of(ctx, l.ss_b, fused_o ? resid_cols : kScaleChunkCols);
   bool fused_gu = false;
   if (ctx->tc && !(c.flags & AMPH_FLAG_SEPARATE_SWIGLU)) {         // gate / up projection with SwiGLU in its epilogue
     ProfScope p(ctx, AMPH_PROF_PROJECTION);
     if (rows > kWideFrom)
       fused_gu = tc_wide_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act,
                                        rs_b, st);
-    else
-      fused_gu = tc_gemm_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act,
-                                       rs_b, st);
+    else {
+      fused_gu = tc_rows_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act, rs_b, st);
+      if (!fused_gu)
+        fused_gu = tc_gemm_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act, rs_b, st);
+    }
     if (fused_gu && p.rec) ctx->prof_bytes += 2LL * c.d_ffn * c.d_model * (int64_t)ctx->esz;
     if (fused_gu) ctx->last_proj_one_wave = false;
   }
@@ -643,7 +655,7 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
     ProfScope p(ctx, AMPH_PROF_SWIGLU);
     launch_swiglu(P, ctx->ws + l.act, ctx->dtype, rows, c.d_ffn, st, rs_b, ctx->last_proj_one_wave);
   }
-  if (hid == nullptr && resid_fused(XB_ACT, w.w_down, c.d_ffn, next_gain, l.ss_a)) return next_gain ? kWideScaleCols : 0;
+  if (hid == nullptr && resid_fused(XB_ACT, w.w_down, c.d_ffn, next_gain, l.ss_a)) return next_gain ? resid_cols : 0;
   const void* wd[1] = {w.w_down};
   P = project(ctx, XB_ACT, wd, 1, c.d_model, c.d_ffn, rows);
   ProfScope p(ctx, AMPH_PROF_NORM);

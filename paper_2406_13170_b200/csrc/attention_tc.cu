@@ -96,13 +96,14 @@ __device__ __forceinline__ unsigned long long now_ns() {
 }
 // Bounded wait: false (and the CTA-wide abort flag raised) if the phase never completes or another role gave up.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = now_ns();
+  unsigned long long t0 = 0;
   for (uint32_t i = 1;; ++i) {
     if (mbar_try(bar, parity)) return true;
     if ((i & 63u) == 0u) {
       if (*abort_flag) return false;
-      if (now_ns() - t0 > kWaitLimitNs) break;
+      const unsigned long long t = now_ns();
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > kWaitLimitNs) break;
     }
   }
   *abort_flag = 1;

@@ -225,9 +225,8 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
     __syncwarp();
     pdl_wait();
     int issued = npre;
-    for (int i = npre; i < nit; ++i) {
-      const int s = i % stages, round = i / stages;
-      if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], (round & 1) ^ 1, &abort_flag, limit_ns))) break;
+    for (int i = npre, s = 0, ph = 0; i < nit; ++i) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], ph, &abort_flag, limit_ns))) break;
       if (leader) {
         uint8_t* a = smem + (size_t)s * stage_bytes;
         mbar_expect_tx(&full_bar[s], a_bytes + (uint32_t)nblk * b_bytes);
@@ -238,6 +237,7 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
       }
       __syncwarp();
       issued = i + 1;
+      if (++s == stages) { s = 0; ph ^= 1; }
     }
     if (abort_flag && lane == 0) {                     // drain: let every copy that was issued land
       const int first = issued > stages ? issued - stages : 0;
@@ -260,9 +260,8 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
     const uint32_t tmem_d = tmem_base_slot;
     const uint32_t idesc = umma_idesc(nt, EPI != EPI_PARTIAL ? kTileM / 2 : kTileM);
     bool ok = true;
-    for (int i = 0; i < nit; ++i) {
-      const int s = i % stages, round = i / stages;
-      ok = __all_sync(0xffffffffu, mbar_wait(&full_bar[s], round & 1, &abort_flag, limit_ns));
+    for (int i = 0, s = 0, ph = 0; i < nit; ++i) {
+      ok = __all_sync(0xffffffffu, mbar_wait(&full_bar[s], ph, &abort_flag, limit_ns));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (leader) {
@@ -294,6 +293,7 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
         umma_commit(&empty_bar[s]);                    // frees the stage once these MMAs have read it
       }
       __syncwarp();
+      if (++s == stages) { s = 0; ph ^= 1; }
     }
     if (ok && leader) umma_commit(&accum_bar);
     __syncwarp();
@@ -652,28 +652,32 @@ bool tc_gemm_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
 }
 
 namespace {
-// One thread per CTA asks the TMA unit to bring the first `stages` pipeline stages of every gate / up tile into L2 (stage by
-// stage over all tiles, the order in which the projection's CTAs will ask for them), with the same evict-first policy as the
-// copies themselves: prefetched at normal priority, the weights push the step's L2-resident working set out.
-__global__ void tc_prefetch_pair_kernel(const __grid_constant__ CUtensorMap map, int tiles, int stages, int ks) {
+// One thread per CTA asks the TMA unit to bring `picks` of the `stages` pipeline stages of every gate / up tile into L2, evenly
+// spread over the K range, with the same evict-first policy as the copies themselves: prefetched at normal priority, the weights
+// push the step's L2-resident working set out.  Spread, because a tile's stages are consumed in order: with the first third of
+// them in L2 HBM stands still while that third is consumed.
+__global__ void tc_prefetch_pair_kernel(const __grid_constant__ CUtensorMap map, int tiles, int stages, int picks, int ks) {
   if (threadIdx.x != 0) return;
   const uint64_t pol = l2_evict_first_policy();
-  for (int i = 0; i < stages; ++i)
+  for (int i = 0; i < picks; ++i) {
+    const int stage = (2 * i + 1) * stages / (2 * picks);
     for (int t = blockIdx.x; t < tiles; t += gridDim.x)
       asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile.L2::cache_hint [%0, {%1, %2, %3, %4}], %5;"
-                   ::"l"(&map), "r"(0), "r"(t * (kTileM / 2)), "r"(i * ks), "r"(0), "l"(pol) : "memory");
+                   ::"l"(&map), "r"(0), "r"(t * (kTileM / 2)), "r"(stage * ks), "r"(0), "l"(pol) : "memory");
+  }
 }
 }  // namespace
 
 bool tc_gemm_prefetch_swiglu(TcGemm* g, const void* w_gate, const void* w_up, int f, int in, size_t budget_bytes, cudaStream_t st) {
   if (!g || f % (kTileM / 2) || in % (kTileK * kStageKb)) return false;
-  const int stages = (int)(budget_bytes / ((size_t)(f / (kTileM / 2)) * kStageKb * kTileM * kTileK * 2));
-  if (stages <= 0) return false;
+  const int stages = in / kTileK / kStageKb;
+  int picks = (int)(budget_bytes / ((size_t)(f / (kTileM / 2)) * kStageKb * kTileM * kTileK * 2));
+  if (picks > stages) picks = stages;
+  if (picks <= 0) return false;
   const bool up_first = (const char*)w_up < (const char*)w_gate;
   const CUtensorMap* mw = g->get_pair(up_first ? w_up : w_gate, up_first ? w_gate : w_up, f, in, kStageKb);
   if (!mw) return false;
-  const int max_stages = in / kTileK / kStageKb;
-  tc_prefetch_pair_kernel<<<g->sm_count, 32, 0, st>>>(*mw, f / (kTileM / 2), stages < max_stages ? stages : max_stages, kStageKb);
+  tc_prefetch_pair_kernel<<<g->sm_count, 32, 0, st>>>(*mw, f / (kTileM / 2), stages, picks, kStageKb);
   return true;
 }
 

@@ -36,6 +36,17 @@ bool tc_gemm_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
                              int rows, void* q, KvView kv, const RowMeta* meta, const float2* rope, int max_ctx,
                              const RowScale& rs, cudaStream_t st);
 
+// The same two, and the residual update, with the activation rows as the MMA's M operand (gemm_rows.cu): at most 64 rows.  Each
+// returns false, nothing launched, where the form is not available or another kernel is the faster one.
+bool tc_rows_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_up, int f, int in, int rows, void* act, const RowScale& rs,
+                           cudaStream_t st);
+bool tc_rows_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, const void* wv, int n_heads, int dh, int in, int rows, void* q,
+                             KvView kv, const RowMeta* meta, const float2* rope, int max_ctx, const RowScale& rs, cudaStream_t st);
+// x += X . W^T and, with gain, xn <- gain * x (bf16) and ss[row][out / *cols] <- sums of squares.
+constexpr int kRowsResidMax = 2048;      // longest side it takes
+bool tc_rows_launch_resid(TcGemm* g, int xb, const void* w, int out, int in, int rows, float* x, const void* gain, void* xn, float* ss,
+                          int* cols, cudaStream_t st);
+
 // The pair kernel (gemm_wide.cu) for many activation rows.  tc_wide_bind names the scratch (fp32) and the flags (zeroed,
 // kWideFlags ints) that cut tiles go through; the fused forms need them.  tc_gemm_launch takes the plain form by itself.
 constexpr int kWideFrom = 64;            // rows above this take it

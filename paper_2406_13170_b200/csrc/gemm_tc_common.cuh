@@ -52,13 +52,14 @@ __device__ __forceinline__ unsigned long long now_ns() {
 }
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                           unsigned long long limit_ns) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = now_ns();
+  unsigned long long t0 = 0;
   for (uint32_t i = 1;; ++i) {
     if (mbar_try(bar, parity)) return true;
     if ((i & 63u) == 0u) {
       if (*abort_flag) return false;
-      if (now_ns() - t0 > limit_ns) break;
+      const unsigned long long t = now_ns();
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > limit_ns) break;
     }
   }
   *abort_flag = 1;
@@ -168,6 +169,27 @@ struct TcGemm {
     if (r != CUDA_SUCCESS) return nullptr;
     return &(pair_cache[key] = m);
   }
+
+  // Rows [0, rows) of a matrix and the rows `gap` bytes behind them, as (column, row, half, K block): a box is box_rows rows of
+  // both halves per K block, one after the other.  The halves are two matrices, or the two halves of a head's rotation pairs.
+  std::map<std::tuple<const void*, uint64_t, int, int, int, int>, CUtensorMap> halves_cache;
+  const CUtensorMap* get_halves(const void* ptr, uint64_t gap, int rows, int cols, int box_rows, int box_kb) {
+    auto key = std::make_tuple(ptr, gap, rows, cols, box_rows, box_kb);
+    auto it = halves_cache.find(key);
+    if (it != halves_cache.end()) return &it->second;
+    if (gap == 0 || (gap & 15) || gap >= (1ull << 40)) return nullptr;
+    CUtensorMap m;
+    const cuuint64_t dims[4] = {(cuuint64_t)tc::kTileK, (cuuint64_t)rows, 2, (cuuint64_t)cols / tc::kTileK};
+    const cuuint64_t strides[3] = {(cuuint64_t)cols * 2, (cuuint64_t)gap, (cuuint64_t)tc::kTileK * 2};
+    const cuuint32_t box[4] = {(cuuint32_t)tc::kTileK, (cuuint32_t)box_rows, 2, (cuuint32_t)box_kb};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    const CUresult r = encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return nullptr;
+    return &(halves_cache[key] = m);
+  }
+  bool rows_ready[3] = {false, false, false};  // tc_rows_kernel's forms: shared memory limit raised
 
   // pair kernel: CTA pairs that run at a time (0: not available, -1: not asked yet), scratch and flags of cut tiles
   int wide_pairs = -1;

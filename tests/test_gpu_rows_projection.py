@@ -1,0 +1,51 @@
+"""The projections that finish their rows themselves in passes of up to 64 rows (gate / up with SwiGLU, q / k / v with rotary embedding
+and cache write, output and down projection with the residual update) against the separate kernels, at the edges of their tiles:
+rows around multiples of 16, a last tile that is not whole, one tile height per head dimension."""
+import pytest
+import torch
+
+import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _outputs(shape, w, prompts, flags):
+    from paper_2406_13170_b200 import Amphista
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    m = Amphista(shape, topo, w, max_ctx=256, max_batch=len(prompts), flags=flags)
+    toks = torch.randint(0, shape.vocab, (len(prompts), shape.n_nodes), dtype=torch.int32, generator=torch.Generator().manual_seed(3)).cuda()
+    out = []
+    for b, p in enumerate(prompts):
+        m.prefill(p, seq=b)
+        out.append(m.get_tensor("hidden", (len(p), shape.d_model)))
+    for b in range(len(prompts)):
+        m.set_tensor("root" if b == 0 else f"root#{b}", toks[b, :1].contiguous())
+    m.draft()
+    m.verify_tree(toks if len(prompts) > 1 else toks[0])
+    m.synchronize()
+    last = shape.n_layers - 1
+    for b, p in enumerate(prompts):
+        out.append(m.get_tensor(f"hidden#{b}", (shape.n_nodes, shape.d_model)))
+        out.append(m.get_tensor(f"sal_h#{b}", (2, shape.d_model)))
+        out += [m.get_tensor(f"kv.{c}.{i}#{b}", (len(p) + shape.n_nodes, shape.d_model)) for c in "kv" for i in (0, last)]
+    m.close()
+    return out
+
+
+def _compare(a, b, rel):
+    for x, y in zip(a, b):
+        assert bool(torch.isfinite(x).all())
+        assert float((x - y).norm() / y.norm()) <= rel
+
+
+# 11008 = 137 tiles of 80 and one of 48 (rows above 16), 2432 = 101 of 24 and one of 8; width 2176: no residual form
+@pytest.mark.parametrize("heads,dh,ffn", [(8, 64, 1408), (4, 128, 2432), (10, 128, 3456), (4, 128, 11008), (17, 128, 1408)])
+@pytest.mark.parametrize("n,nodes", [(1, 5), (16, 16), (17, 33), (48, 43), (63, 50), (64, 64)])
+def test_bf16_forms_against_the_separate_kernels(heads, dh, ffn, n, nodes):
+    shape = inputs.get_shape("small_bf16").with_(d_model=heads * dh, n_heads=heads, head_dim=dh, d_ffn=ffn, n_nodes=nodes, topk=(16, 16, 16, 16))
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    prompts = [inputs.make_prompt(shape.with_(prompt_len=n), seed=2).tolist()]
+    # 512: no residual update in an epilogue.  Sums in another order, roundings to bf16 (2^-8) in the same places; three layers of
+    # unit gain, as in the tests of the projection of many rows
+    _compare(_outputs(shape, w, prompts, 0), _outputs(shape, w, prompts, 4 | 16 | 512), 1e-2)
+
