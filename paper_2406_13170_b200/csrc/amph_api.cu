@@ -306,8 +306,9 @@ void make_layout(const amph_config& c, int n_nodes, Layout* L, int* Mcap_out, si
   l.att_o = l.per_group(4 * (size_t)splits * c.n_heads * Mcap * c.head_dim, &l.att_o_s);
   l.att_ml = l.per_group(4 * (size_t)splits * c.n_heads * Mcap * 2, &l.att_ml_s);
   l.logits = l.take(4 * (size_t)Rcap * V);
-  // one entry per tile of the kernel that updates the residual: 128 columns, 16 in a small model
-  const size_t ss_cols = c.d_model / (c.d_model <= kRowsResidMax ? 16 : kWideScaleCols) + 32;
+  // one entry per tile of the kernel that updates the residual: 128 columns, 16 or 8 in a small model
+  static_assert(kRowsResidMax == kPlainResidMax, "one bound for both");
+  const size_t ss_cols = c.d_model / (c.d_model <= kPlainResidMax ? kPlainScaleCols : kWideScaleCols) + 32;
   l.ss_a = l.take(4 * (size_t)Rcap * ss_cols);
   l.ss_b = l.take(4 * (size_t)Rcap * ss_cols);
   l.wide_flags = l.take(sizeof(int) * kWideFlags);
@@ -567,6 +568,13 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
     if (fused_rope && p.rec) ctx->prof_bytes += 3LL * c.d_model * c.d_model * (int64_t)ctx->esz;
     if (!fused_rope) cudaGetLastError();
   }
+  const bool f32 = ctx->dtype == AMPH_DTYPE_F32;
+  if (f32 && !(c.flags & AMPH_FLAG_SEPARATE_ROPE)) {
+    ProfScope p(ctx, AMPH_PROF_PROJECTION);
+    launch_plain_qkv_rope(ctx->ws + l.xn, qkv, c.d_model, c.head_dim, c.d_model, rows, ctx->ws + l.q, gr, c.max_ctx, rs, st);
+    if (p.rec) ctx->prof_bytes += 3LL * c.d_model * c.d_model * (int64_t)ctx->esz;
+    fused_rope = true;
+  }
   if (!fused_rope) P = project(ctx, XB_XN, qkv, 3, c.d_model, c.d_model, rows);
   if (fused_rope) fork_prefetch(ctx, w, ps);
   bool grouped_rope = false;
@@ -615,6 +623,14 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
   // output projection and residual update: one kernel for many rows, and in a small model
   int resid_cols = kWideScaleCols;
   auto resid_fused = [&](int xb, const void* wt, int in, const void* gain, size_t ss) {
+    if (f32 && c.d_model <= kPlainResidMax) {
+      ProfScope p(ctx, AMPH_PROF_PROJECTION);
+      launch_plain_resid(xbuf_ptr(ctx, xb), wt, c.d_model, in, rows, x, gain, ctx->ws + l.xn, ctx->at<float>(ss), st);
+      if (p.rec) ctx->prof_bytes += (int64_t)c.d_model * in * (int64_t)ctx->esz;
+      ctx->last_proj_one_wave = false;
+      resid_cols = kPlainScaleCols;
+      return true;
+    }
     if (!ctx->tc) return false;
     if (rows <= kWideFrom && (ctx->one_order || c.d_model > kRowsResidMax || in > kRowsResidMax)) return false;
     ProfScope p(ctx, AMPH_PROF_PROJECTION);
@@ -648,6 +664,13 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
     }
     if (fused_gu && p.rec) ctx->prof_bytes += 2LL * c.d_ffn * c.d_model * (int64_t)ctx->esz;
     if (fused_gu) ctx->last_proj_one_wave = false;
+  }
+  if (f32 && !(c.flags & AMPH_FLAG_SEPARATE_SWIGLU)) {
+    ProfScope p(ctx, AMPH_PROF_PROJECTION);
+    launch_plain_swiglu(ctx->ws + l.xn, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act, rs_b, st);
+    if (p.rec) ctx->prof_bytes += 2LL * c.d_ffn * c.d_model * (int64_t)ctx->esz;
+    ctx->last_proj_one_wave = false;
+    fused_gu = true;
   }
   if (!fused_gu) {
     const void* gu[2] = {w.w_gate, w.w_up};

@@ -218,6 +218,17 @@ struct GemmSeg { const void* w; };
 void launch_gemm_generic(const void* x, int ldx, const GemmSeg* segs, int n_seg, int out, int in,
                          float* P, int ldp, int rows, int dtype, cudaStream_t st, int wait_first = 0);
 
+// fp32 projections whose kernel finishes the job: SwiGLU; rotary embedding and cache write; x += X . W^T with, if gain, xn <- gain * x
+// and ss[row][out / kPlainScaleCols] <- sums of squares (see RowScale).
+constexpr int kPlainScaleCols = 8;
+constexpr int kPlainResidMax = 2048;     // longest residual row it takes: ss has an entry per eight columns
+void launch_plain_swiglu(const void* x, const void* w_gate, const void* w_up, int f, int in, int rows, void* act, const RowScale& rs,
+                         cudaStream_t st);
+void launch_plain_qkv_rope(const void* x, const void* const* w, int d, int dh, int in, int rows, void* q, const RopeGroups& gr, int max_ctx,
+                           const RowScale& rs, cudaStream_t st);
+void launch_plain_resid(const void* x_in, const void* w, int out, int in, int rows, float* x, const void* gain, void* xn, float* ss,
+                        cudaStream_t st);
+
 // ---- draft-module specific
 // (one launch per batch; a void* with a stride is sequence 0's copy of a per-sequence buffer, the next `stride` bytes further on)
 void launch_gather_last(const float* h1, const float* h2, int rows_per, const void* state, size_t state_stride, void* last /*[2][d]*/,

@@ -1,6 +1,6 @@
 """The projections that finish their rows themselves in passes of up to 64 rows (gate / up with SwiGLU, q / k / v with rotary embedding
 and cache write, output and down projection with the residual update) against the separate kernels, at the edges of their tiles:
-rows around multiples of 16, a last tile that is not whole, one tile height per head dimension."""
+rows around multiples of 16, a last tile that is not whole, one tile height per head dimension; bf16 and fp32."""
 import pytest
 import torch
 
@@ -49,3 +49,12 @@ def test_bf16_forms_against_the_separate_kernels(heads, dh, ffn, n, nodes):
     # unit gain, as in the tests of the projection of many rows
     _compare(_outputs(shape, w, prompts, 0), _outputs(shape, w, prompts, 4 | 16 | 512), 1e-2)
 
+
+@pytest.mark.parametrize("heads,dh,ffn", [(4, 64, 688), (3, 128, 1000), (1, 64, 8)])
+@pytest.mark.parametrize("lens,nodes", [((1,), 5), ((17,), 16), ((33,), 24), ((40, 7, 21), 19)])
+def test_fp32_forms_against_the_separate_kernels(heads, dh, ffn, lens, nodes):
+    shape = inputs.get_shape("tiny").with_(d_model=heads * dh, n_heads=heads, head_dim=dh, d_ffn=ffn, n_nodes=nodes, topk=(8, 8, 8, 8))
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    prompts = [inputs.make_prompt(shape.with_(prompt_len=n), seed=b).tolist() for b, n in enumerate(lens)]
+    # the same fp32 sums; the last operations may be contracted differently (a few ulps of 2^-24 per layer)
+    _compare(_outputs(shape, w, prompts, 0), _outputs(shape, w, prompts, 4 | 16), 4e-6)
