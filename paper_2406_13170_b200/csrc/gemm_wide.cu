@@ -3,8 +3,9 @@
 // A cluster of two CTAs owns 256 weight rows and a block of up to 256 activation rows: one tcgen05.mma.cta_group::2 (M = 256,
 // N <= 256) per 16 columns of K.  Each CTA stages its own 128 weight rows and HALF of the activation rows: 32 KB per 64
 // columns of K at N = 256, i.e. 64 bytes of L2 -> SM traffic per clock of MMA, against 80 with one CTA per 128 weight rows and
-// 512 activation rows (which made L2 the bound).  Stages hold two K blocks, one copy of up to 32 KB per operand: an SM retires
-// about one copy per 400 clocks, so with 16 KB copies the main loop ran at 790 clocks per K block instead of the MMA's 512.
+// 512 activation rows (which made L2 the bound).  A stage holds one K block (512 clocks of MMA at N = 256), so that six are in
+// flight; with two K blocks per stage and three stages a batch of 4 x 64 rows (8 layers, 12 steps) took 28.4 ms, now 27.5, a
+// prefill of 1900 tokens 32.1, now 32.0.  (The producers' and the issuer's loops must not divide for that: see below.)
 // With 257..512 rows two neighbouring pairs take the two row blocks of the same weights at the same time, so weights still
 // cross HBM once.  Tensor memory holds two accumulators: the epilogue of one piece of work runs under the next main loop.
 //
@@ -34,7 +35,7 @@ namespace {
 
 constexpr int kEpiThreads = 512;      // four warps per TMEM lane quarter
 constexpr int kWideThreads = 64 + kEpiThreads;
-constexpr int kUnitKb = 2;            // K blocks per pipeline stage = unit of work: ranges are cut at multiples of 128 columns
+constexpr int kUnitKb = 1;            // K blocks per pipeline stage = unit of work: ranges are cut at multiples of 64 columns
 constexpr int kMaxWideRows = 512;
 constexpr int kMaxStages = 8;
 constexpr int kMaxGroups = kWideFlags / 2;
@@ -247,8 +248,15 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     // ---------------- TMA producer of this CTA's half of the operands
     const bool leader = elect_one();
     const uint64_t wpol = l2_evict_first_policy();
-    auto load_w = [&](int st, const Segment& s, int u, uint32_t more) {
-      const int seg = s.tile / prm.tiles_per_seg, lt = s.tile - seg * prm.tiles_per_seg;
+    // a division by a run-time value is about 170 clocks, so a segment's matrix and tile are worked out once, and ring position and
+    // parity are counted
+    int seg = 0, lt = 0;
+    auto next_segment = [&](SegIter& it, Segment& s) {
+      const bool more = it.next(s);
+      if (more) { seg = s.tile / prm.tiles_per_seg; lt = s.tile - seg * prm.tiles_per_seg; }
+      return more;
+    };
+    auto load_w = [&](int st, int u, uint32_t more) {
       const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), lead);
       uint8_t* dst = smem + (size_t)st * stage_bytes;
       if (rank == 0) mbar_expect_tx(&full_bar[st], 2 * stage_bytes + more);
@@ -260,20 +268,20 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
     cluster_ready();
     SegIter it = first;
     Segment sg;
-    bool have = it.next(sg);
+    bool have = next_segment(it, sg);
     int u = have ? sg.u0 : 0, i = 0;
     for (; i < stages && have; ++i) {
-      if (leader) load_w(i, sg, u, i == 0 ? prm.extra_tx : 0u);
-      if (++u == sg.u1) { have = it.next(sg); u = sg.u0; }
+      if (leader) load_w(i, u, i == 0 ? prm.extra_tx : 0u);
+      if (++u == sg.u1) { have = next_segment(it, sg); u = sg.u0; }
     }
     __syncwarp();
     pdl_wait();
-    for (; have; ++i) {
-      const int st = i % stages, round = i / stages;
-      if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[st], (round & 1) ^ 1, &abort_flag, limit_ns))) break;
-      if (leader) { load_w(st, sg, u, 0u); load_x(st, u); }
+    for (int st = 0, ph = 0; have; ++i) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[st], ph, &abort_flag, limit_ns))) break;
+      if (leader) { load_w(st, u, 0u); load_x(st, u); }
       __syncwarp();
-      if (++u == sg.u1) { have = it.next(sg); u = sg.u0; }
+      if (++u == sg.u1) { have = next_segment(it, sg); u = sg.u0; }
+      if (++st == stages) { st = 0; ph ^= 1; }
     }
     for (int j = i > stages ? i - stages : 0; j < i; ++j)  // every commit to this CTA's barriers has arrived
       if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[j % stages], (j / stages) & 1, &abort_flag, limit_ns))) break;
@@ -305,15 +313,14 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
       SegIter it = first;
       Segment sg;
       bool ok = true;
-      int i = 0;
+      int st = 0, ph = 0;
       for (int j = 0; ok && it.next(sg); ++j) {
         const int as = j & 1, around = j >> 1;
         if (around > 0) ok = __all_sync(0xffffffffu, mbar_wait(&accum_empty[as], (around & 1) ^ 1, &abort_flag, limit_ns));
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t d = tmem_d + (uint32_t)(as * n);
-        for (int u = sg.u0; ok && u < sg.u1; ++u, ++i) {
-          const int st = i % stages;
-          ok = __all_sync(0xffffffffu, mbar_wait(&full_bar[st], (i / stages) & 1, &abort_flag, limit_ns));
+        for (int u = sg.u0; ok && u < sg.u1; ++u) {
+          ok = __all_sync(0xffffffffu, mbar_wait(&full_bar[st], ph, &abort_flag, limit_ns));
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           if (leader) {                                  // K blocks past the end of K have arrived as zeros
@@ -328,6 +335,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
             umma_commit_pair(&empty_bar[st], lead);
           }
           __syncwarp();
+          if (++st == stages) { st = 0; ph ^= 1; }
         }
         if (ok && leader) umma_commit_pair(&accum_full[as], lead);
         __syncwarp();
@@ -719,8 +727,8 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
     if (splits > prm->units_per_tile) return false;
     prm->groups = prm->tiles * splits;
   } else {
-    // at least four units (512 columns) a group, unless there are more tiles than that; no more pairs than scratch
-    const int most = units / 4 > prm->tiles ? units / 4 : prm->tiles;
+    // at least 512 columns a group, unless there are more tiles than that; no more pairs than scratch
+    const int most = units * kUnitKb / 8 > prm->tiles ? units * kUnitKb / 8 : prm->tiles;
     if (prm->groups > most) prm->groups = most;
     const size_t per_group = (size_t)prm->nrb * 2 * prm->n * kTileM;
     if ((size_t)prm->groups > scratch_floats / per_group) prm->groups = (int)(scratch_floats / per_group);
@@ -793,7 +801,7 @@ bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   const int groups = g->wide_pairs / (rows > 256 ? 2 : 1);
   if (tiles * 2 <= groups || !g->wide_flags) {
     splits = groups / tiles;
-    if (splits > units / 2) splits = units / 2;            // at least four K blocks per pair
+    if (splits > units * kUnitKb / 4) splits = units * kUnitKb / 4;            // at least four K blocks per pair
     if (splits > 16) splits = 16;
     while (splits > 1 && splits * stride > p_floats) --splits;
     if (splits < 1) splits = 1;
@@ -824,7 +832,7 @@ bool tc_wide_launch_resid(TcGemm* g, int xb, const void* w, int out, int in, int
   // as many K ranges per tile as run at a time, at least four K blocks each
   const int items = out / 256 * (rows > 256 ? 2 : 1), units = (in / kTileK + kUnitKb - 1) / kUnitKb;
   int splits = 4;
-  while (splits > 1 && (g->resid_clusters[splits] < items || splits > units / 2)) --splits;
+  while (splits > 1 && (g->resid_clusters[splits] < items || splits > units * kUnitKb / 4)) --splits;
   if (g->resid_clusters[splits] < 1) return false;
   WideMaps maps;
   WideParams prm;
