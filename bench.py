@@ -433,9 +433,15 @@ def main():
     # separate-merge flag is set), output projection, residual, gate/up projection, SwiGLU, down projection, residual
     # passes of more than 64 rows: the pair projection, unless the context keeps one order of sums
     pairs = uses_tc and not args.flags & 512 and not getattr(shape, "lm_rank", 0)
+    # small models: the residual updates are in the projections' epilogues whatever the rows
+    short = shape.d_model <= 2048 and (shape.dtype == "fp32" or (pairs and shape.d_ffn <= 2048))
 
     def layer_launches(rows, keys):
         n = 10 if (shape.dtype == "bf16" and args.flags & 8) else 9
+        if rows <= 64 or not uses_tc:
+            n -= 2 * short
+        if shape.dtype == "fp32":
+            return n - (not args.flags & 16) - (not args.flags & 4)
         if not uses_tc:
             return n
         if rows <= 64 or pairs:
@@ -451,8 +457,8 @@ def main():
         if getattr(shape, "lm_rank", 0):
             draft += 2                                           # low-rank heads: one more projection + a gather
         verify = 1 + shape.n_layers * layer_launches(N, keys + N) + 3        # row set-up, ..., head projection, argmax slices, merge
-        if N > 64:
-            verify += pairs                                      # the last layer's update also takes the final norm: a kernel of its own
+        if N > 64 or short:
+            verify += pairs or short                                     # the last layer's update also takes the final norm: a kernel of its own
         return draft + verify + 1                                # ... + acceptance
 
     line["gpu_launches"] = sum(step_launches(C_start + i * (K + 1)) for i in range(steps))

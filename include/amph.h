@@ -65,7 +65,7 @@ enum {
                                        * ranges that do not depend on what else a launch carries: every sum in one order, whatever the
                                        * height of a pass.  Always so with lm_rank > 0 (see amph_config)                           */
   AMPH_FLAG_NO_SIDE_PREFETCH = 256  /* no helper stream: by default (bf16, a stream of the caller's own) every layer of the captured schedule of amph_step forks a small
-                                     * kernel onto a second stream, created by amph_init, that pulls the head of the gate / up
+                                     * kernel onto a second stream, created by amph_init, that pulls a part of the gate / up
                                      * weights into L2 while attention runs; it joins the caller's stream before amph_accept /
                                      * amph_step / amph_prefill return their work to it */
 };
