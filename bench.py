@@ -448,6 +448,7 @@ def main():
             n -= (not args.flags & 16) + (not args.flags & 4)    # SwiGLU; rotary + cache write: in the projections' epilogues
         if rows > 64:
             n -= 2 * pairs                                       # residual updates in the projections' epilogues
+            n -= not pairs and rows <= 128 and not args.flags & 16   # one order of sums: SwiGLU in the projection's epilogue
         elif not (args.flags & (4 | 256)) and 4 * keys * shape.d_model <= 20 << 20:
             n += 1                                               # the gate / up prefetch helper on the forked stream
         return n

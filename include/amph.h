@@ -60,8 +60,8 @@ enum {
                                     * hidden state alone; draft.fc{s} is then [d, d] instead of [d, 2d]            */
   AMPH_FLAG_CHUNKED_PREFILL = 128, /* prefill one chunk of 128 prompt tokens per weight pass instead of four */
   AMPH_FLAG_MMA_SYNC_ATTENTION = 32, /* bf16 tree attention on the warp-level mma.sync kernel instead of the tcgen05 / TMA one */
-  AMPH_FLAG_NO_PAIR_PROJECTION = 512, /* passes of more than 64 rows on the projection kernel of smaller ones, with rotary embedding,
-                                       * SwiGLU and residual update as kernels of their own, prompts in chunks of 128 rows, and key
+  AMPH_FLAG_NO_PAIR_PROJECTION = 512, /* passes of more than 64 rows on the projection kernels of smaller ones, with rotary embedding
+                                       * and residual update (above 128 rows SwiGLU too) as kernels of their own, prompts in chunks of 128 rows, and key
                                        * ranges that do not depend on what else a launch carries: every sum in one order, whatever the
                                        * height of a pass.  Always so with lm_rank > 0 (see amph_config)                           */
   AMPH_FLAG_NO_SIDE_PREFETCH = 256  /* no helper stream: by default (bf16, a stream of the caller's own) every layer of the captured schedule of amph_step forks a small

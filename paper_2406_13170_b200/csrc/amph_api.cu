@@ -558,7 +558,7 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
     if (fused_rope && p.rec) ctx->prof_bytes += 3LL * c.d_model * c.d_model * (int64_t)ctx->esz;
     if (!fused_rope) cudaGetLastError();
   }
-  if (!fused_rope && ctx->tc && ps.G == 1 && !(c.flags & AMPH_FLAG_SEPARATE_ROPE)) {   // q / k / v projection that rotates and writes the cache itself
+  if (!fused_rope && ctx->tc && ps.G == 1 && rows <= 64 && !(c.flags & AMPH_FLAG_SEPARATE_ROPE)) {   // q / k / v projection that rotates and writes the cache itself
     ProfScope p(ctx, AMPH_PROF_PROJECTION);
     fused_rope = tc_rows_launch_qkv_rope(ctx->tc, XB_XN, w.wq, w.wk, w.wv, c.n_heads, c.head_dim, c.d_model, rows, ctx->ws + l.q,
                                          cache_of(ps.seq[0]), ps.meta[0], ps.rope[0], c.max_ctx, rs, st);
@@ -657,7 +657,7 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
     if (rows > kWideFrom)
       fused_gu = tc_wide_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act,
                                        rs_b, st);
-    else {
+    if (!fused_gu && (rows <= 64 || (ctx->one_order && rows <= 128))) {
       fused_gu = tc_rows_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act, rs_b, st);
       if (!fused_gu)
         fused_gu = tc_gemm_launch_swiglu(ctx->tc, XB_XN, w.w_gate, w.w_up, c.d_ffn, c.d_model, rows, ctx->ws + l.act, rs_b, st);

@@ -1,6 +1,6 @@
-// bf16 projections of up to 64 activation rows whose epilogue needs the whole sum:  Y[rows][out] = X . W^T.
+// bf16 projections of up to 64 activation rows (gate / up: 128) whose epilogue needs the whole sum:  Y[rows][out] = X . W^T.
 //
-// The activation rows are the MMA operand A (M = 64), the weight rows operand B (N = 8 .. 256 of them, a multiple of 8), so a
+// The activation rows are the MMA operand A (M = 64, or 128), the weight rows operand B (N = 8 .. 256 of them, a multiple of 8), so a
 // tile may have any height that spreads a matrix evenly over the SMs, and a thread of the epilogue holds neighbouring features
 // of a row: gate and up of a feature, or both members of a rotation pair, meet in one thread's registers.  A CTA owns the whole
 // K range of its tile.  Weights and activations have a ring each: weights come from HBM and need many bytes in flight,
@@ -21,7 +21,6 @@ using namespace tc;
 namespace {
 
 constexpr int kRowsThreads = 224;
-constexpr int kRowsM = 64;            // activation rows of the MMA
 constexpr int kMaxRing = 12;
 
 enum { ROWS_SWIGLU = 0, ROWS_ROPE = 1, ROWS_RESID = 2 };
@@ -36,7 +35,8 @@ struct RowsParams {
   int kblocks;
   int half;                 // weight rows of one half of a tile (SWIGLU: gate or up; ROPE: one half of the pairs); RESID: the tile
   int n;                    // weight rows of a tile: N of the MMA
-  int nt;                   // rows of an activation box (a multiple of 16, at most 64)
+  int nt;                   // rows of an activation box (a multiple of 16, at most M)
+  int kb_cut;               // M = 128: K blocks from here on go to an accumulator of their own (kblocks: there is one only)
   int rows;
   int w_stages, x_stages;
   int l2_prefetch;          // weight stages beyond the ring that are asked into L2 ahead of the dependency
@@ -107,12 +107,13 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-template <int EPI, int KS>
+template <int EPI, int KS, int M>
 __global__ void __launch_bounds__(kRowsThreads)
 tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
   constexpr bool PAIR = EPI != ROWS_RESID;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ float inv_s[PAIR ? kRowsM : 1];                       // 1 / rms of the activation rows
+  static_assert(M == 64 || (KS == 1 && EPI == ROWS_SWIGLU), "a cut between two accumulators falls between two stages");
+  __shared__ float inv_s[PAIR ? M : 1];                            // 1 / rms of the activation rows
   __shared__ __align__(8) uint64_t w_full[kMaxRing], w_empty[kMaxRing], x_full[kMaxRing], x_empty[kMaxRing], accum_bar;
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
@@ -130,7 +131,7 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
   const uint32_t w_tile = (uint32_t)prm.n * 128, x_tile = (uint32_t)prm.nt * 128;       // one K block of each operand
   const uint32_t w_bytes = w_tile * KS, x_bytes = x_tile * KS;
   uint8_t* const xs = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t* const ws = xs + (size_t)prm.x_stages * x_bytes;         // behind the activations: an MMA reads 64 rows whatever nt is
+  uint8_t* const ws = xs + (size_t)prm.x_stages * x_bytes;         // behind the activations: an MMA reads M rows whatever nt is
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -202,7 +203,7 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
     const bool leader = elect_one();
     asm volatile("bar.sync 2, 96;" ::: "memory");
     const uint32_t tmem_d = tmem_base_slot;
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(prm.n >> 3) << 17) | ((uint32_t)(kRowsM >> 4) << 24);
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(prm.n >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
     const uint32_t xa = smem_u32(xs), wa = smem_u32(ws);
     const uint64_t ad0 = umma_desc(xa), bd0 = umma_desc(wa);       // the address is the descriptor's lowest field, in 16 bytes
     bool ok = true;
@@ -216,7 +217,10 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
 #pragma unroll
         for (int kk = 0; kk < KS; ++kk, ad += x_tile >> 4, bd += w_tile >> 4) {      // K blocks past the end are zeros
 #pragma unroll
-          for (int k = 0; k < kTileK / kUmmaK; ++k) mma(tmem_d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (i | kk | k) ? 1u : 0u);
+          for (int k = 0; k < kTileK / kUmmaK; ++k) {
+            if constexpr (M == 64) mma(tmem_d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (i | kk | k) ? 1u : 0u);
+            else mma(tmem_d + (i >= prm.kb_cut ? (uint32_t)prm.n : 0u), ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (i != 0 && i != prm.kb_cut) || k ? 1u : 0u);
+          }
         }
         commit(&w_empty[wst]);
         commit(&x_empty[xst]);
@@ -228,11 +232,9 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
     if (ok && leader) commit(&accum_bar);
     __syncwarp();
   } else {
-    // ---------------- epilogue: row r of the accumulator sits in TMEM lane 32 (r / 16) + r % 16; the warp of quarter q has rows
-    // 16 q .. 16 q + 15, this thread ra and rb, columns 8 j + 2 (lane % 4) and the next one
-    const int quarter = warp & 3, ra = quarter * 16 + (lane >> 2), rb = ra + 8, cq = 2 * (lane & 3);
-    const bool la = ra < prm.rows, lb = rb < prm.rows;
-    const uint32_t taddr = tmem_base_slot + ((uint32_t)(quarter * 32) << 16);
+    // ---------------- epilogue: row r of the accumulator sits in TMEM lane 32 (r / 16) + r % 16 (M = 64), or r (M = 128); the warp of
+    // quarter q takes 16 rows at a time, this thread ra and rb of them, columns 8 j + 2 (lane % 4) and the next one
+    const int quarter = warp & 3, cq = 2 * (lane & 3);
     pdl_wait();
     if constexpr (PAIR) {
       const int et = threadIdx.x - 64;
@@ -240,6 +242,25 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
       asm volatile("bar.sync 1, 128;" ::: "memory");
     }
     constexpr int U = 4;                               // pieces of 8 columns in flight
+    const bool two = M == 128 && prm.kb_cut < prm.kblocks;
+    for (int part = 0; part < M / 64; ++part) {
+    const int ra = quarter * (M / 4) + part * 16 + (lane >> 2), rb = ra + 8;
+    const bool la = ra < prm.rows, lb = rb < prm.rows;
+    const uint32_t taddr = tmem_base_slot + ((uint32_t)(quarter * 32 + part * 16) << 16);
+    // the second accumulator's sums join the first one's, in the order in which split-K sums are added
+    auto join = [&](uint32_t at, float (*v)[4], int c0) {
+      if constexpr (M == 128) {
+        if (!two) return;
+        float w[U][4];
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+          if (c0 + 8 * j < prm.half) ld_frag8(at + (uint32_t)prm.n + c0 + 8 * j, w[j]);
+        ld_wait();
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+          if (c0 + 8 * j < prm.half) { v[j][0] += w[j][0]; v[j][1] += w[j][1]; v[j][2] += w[j][2]; v[j][3] += w[j][3]; }
+      }
+    };
     if constexpr (EPI == ROWS_SWIGLU) {
       const float sa = la ? inv_s[ra] : 0.f, sb = lb ? inv_s[rb] : 0.f;
       const bool ok = __all_sync(0xffffffffu, mbar_wait(&accum_bar, 0, &abort_flag, limit_ns));
@@ -247,13 +268,20 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
       const uint32_t tg = taddr + (prm.up_first ? (uint32_t)prm.half : 0u), tu = taddr + (prm.up_first ? 0u : (uint32_t)prm.half);
       __nv_bfloat16* const pa = prm.act + (size_t)ra * prm.f + row0 + cq;
       __nv_bfloat16* const pb = prm.act + (size_t)rb * prm.f + row0 + cq;
-      auto glu = [](float g, float u, float sc) { const float t = g * sc; return __fdividef(t, 1.0f + __expf(-t)) * (u * sc); };
+      // M = 128 stands for split-K sums and swiglu_kernel, whose exponential and division it keeps
+      auto glu = [](float g, float u, float sc) {
+        const float t = g * sc;
+        if constexpr (M == 128) return t / (1.0f + expf(-t)) * (u * sc);
+        else return __fdividef(t, 1.0f + __expf(-t)) * (u * sc);
+      };
       for (int c0 = 0; c0 < prm.half; c0 += 8 * U) {
         float g[U][4], u[U][4];
 #pragma unroll
         for (int j = 0; j < U; ++j)
           if (c0 + 8 * j < prm.half) { ld_frag8(tg + c0 + 8 * j, g[j]); ld_frag8(tu + c0 + 8 * j, u[j]); }
         ld_wait();
+        join(tg, g, c0);
+        join(tu, u, c0);
 #pragma unroll
         for (int j = 0; j < U; ++j) {
           const int c = c0 + 8 * j;
@@ -356,6 +384,7 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
         if ((lane & 3) == 0 && lb) prm.ss[(size_t)rb * prm.tiles_per_seg + lt] = qb;
       }
     }
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -373,17 +402,19 @@ constexpr int kGateUpKb = 2, kQkvKb = 2, kResidKb = 4;
 constexpr size_t kGateUpSmem = 215 * 1024, kTwoPerSm = 110 * 1024;
 
 // Rings, tensor memory and everything else that does not depend on the epilogue; false: not covered.
-bool rows_params(TcGemm* g, int xb, int n, int in, int rows, size_t smem_limit, int ks, RowsMaps* maps, RowsParams* prm, size_t* smem) {
-  if (!g || xb < 0 || xb >= g->n_x || g->xcols[xb] != in || in % kTileK || rows < 1 || rows > kRowsM || n < 8 || n > 256 || n % 8) return false;
+bool rows_params(TcGemm* g, int xb, int n, int in, int rows, size_t smem_limit, int ks, int m, int accs, RowsMaps* maps, RowsParams* prm,
+                 size_t* smem) {
+  if (!g || xb < 0 || xb >= g->n_x || g->xcols[xb] != in || in % kTileK || rows < 1 || rows > m || n < 8 || n > 256 || n % (m / 8) || n * accs > 256) return false;
   memset(maps, 0, sizeof *maps);
   memset(prm, 0, sizeof *prm);
   prm->nt = (rows + 15) / 16 * 16;
   if (prm->nt > g->xrows[xb]) return false;
   prm->n = n;
   prm->rows = rows;
-  prm->kblocks = in / kTileK;
+  prm->kblocks = prm->kb_cut = in / kTileK;
+  if (accs == 2) prm->kb_cut = prm->kblocks / 2;
   const size_t x_stage = (size_t)ks * prm->nt * 128, w_stage = (size_t)ks * n * 128;
-  int x_stages = 3;                                  // one less where it would leave fewer than four of weights
+  int x_stages = m == 128 ? 4 : 3;                                  // one less where it would leave fewer than four of weights
   while (x_stages > 2 && 1024 + x_stages * x_stage + 4 * w_stage > smem_limit) --x_stages;
   const size_t x_ring = x_stages * x_stage;
   prm->x_stages = x_stages;
@@ -395,9 +426,9 @@ bool rows_params(TcGemm* g, int xb, int n, int in, int rows, size_t smem_limit, 
   prm->w_stages = ws;
   prm->l2_prefetch = 1;                              // 0 and 2: the same, 4: +0.5 % on a step
   prm->tmem_cols = 32;
-  while (prm->tmem_cols < n) prm->tmem_cols *= 2;
+  while (prm->tmem_cols < n * accs) prm->tmem_cols *= 2;
   *smem = 1024 + x_ring + ws * w_stage;
-  const size_t floor = 1024 + x_ring + (size_t)kRowsM * 128;       // an MMA reads 64 rows from the last activation box on
+  const size_t floor = 1024 + x_ring + (size_t)m * 128;            // an MMA reads M rows from the last activation box on
   if (*smem < floor) *smem = floor;
   if (*smem > (size_t)g->max_smem - 2048) return false;
   const CUtensorMap* mx = g->get(g->xptr[xb], g->xrows[xb], in, prm->nt, ks);
@@ -408,13 +439,13 @@ bool rows_params(TcGemm* g, int xb, int n, int in, int rows, size_t smem_limit, 
   return true;
 }
 
-template <int EPI, int KS>
+template <int EPI, int KS, int M = 64>
 bool rows_run(TcGemm* g, const RowsMaps& maps, const RowsParams& prm, int tiles, size_t smem, cudaStream_t st) {
-  if (!g->rows_ready[EPI]) {
-    if (cudaFuncSetAttribute(tc_rows_kernel<EPI, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, g->max_smem - 2048) != cudaSuccess) return false;
-    g->rows_ready[EPI] = true;
+  if (!g->rows_ready[M == 128 ? 3 : EPI]) {
+    if (cudaFuncSetAttribute(tc_rows_kernel<EPI, KS, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, g->max_smem - 2048) != cudaSuccess) return false;
+    g->rows_ready[M == 128 ? 3 : EPI] = true;
   }
-  return launch_pdl(tc_rows_kernel<EPI, KS>, dim3(tiles), dim3(kRowsThreads), smem, st, maps, prm) == cudaSuccess;
+  return launch_pdl(tc_rows_kernel<EPI, KS, M>, dim3(tiles), dim3(kRowsThreads), smem, st, maps, prm) == cudaSuccess;
 }
 
 }  // namespace
@@ -426,17 +457,23 @@ bool tc_rows_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_
   // whose activations leave their ring deep enough, and from 1.5 tiles per SM on, when tiles of up to 128 rows here leave too few
   // stages.  Us a launch, back to back, at 4096 x 2 x 11008: 16 rows 29.7, here 31.5; 32 rows 32.7 / 31.6; 64 rows 35.0 / 30.9.
   // A step's layer at 6656 x 2 x 17920: 2 % slower here.  Small matrices come here whatever the rows: more and shorter tiles.
+  // More than 64 rows (contexts that keep one order of sums): in place of tc_gemm_launch's split-K sums and swiglu_kernel, where there
+  // are at most two of them, bit for bit.  128 rows, 4096 x 2 x 11008 (7B, 2048 tokens of context, six steps): 28.6 ms with the two
+  // kernels (37.9 + 4.5 us a layer), now 27.6.
+  const bool m128 = rows > 64;
+  const int accs = m128 ? tc_gemm_splits(g, 2 * (f / kTileM), in / kTileK, rows) : 1;
+  if (m128 && (accs > 2 || f % kTileM || in / kTileK % accs)) return false;
   const int tiles64 = f / 64;
   if (tiles64 * 2 > g->sm_count && (rows <= 16 || tiles64 * 2 > 3 * g->sm_count)) return false;
-  int half = ((f + g->sm_count - 1) / g->sm_count + 7) / 8 * 8;
+  int half = ((f + g->sm_count - 1) / g->sm_count + 7) / 8 * 8;      // (M = 128 takes N in steps of 16)
   if (half > 128) half = 128;
   RowsMaps maps;
   RowsParams prm;
   size_t smem;
-  if (!rows_params(g, xb, 2 * half, in, rows, kGateUpSmem, kGateUpKb, &maps, &prm, &smem)) return false;
+  if (!rows_params(g, xb, 2 * half, in, rows, kGateUpSmem, m128 ? 1 : kGateUpKb, m128 ? 128 : 64, accs, &maps, &prm, &smem)) return false;
   const bool up_first = (const char*)w_up < (const char*)w_gate;
   const uint64_t gap = up_first ? (const char*)w_gate - (const char*)w_up : (const char*)w_up - (const char*)w_gate;
-  const CUtensorMap* m = g->get_halves(up_first ? w_up : w_gate, gap, f, in, half, kGateUpKb);
+  const CUtensorMap* m = g->get_halves(up_first ? w_up : w_gate, gap, f, in, half, m128 ? 1 : kGateUpKb);
   if (!m) return false;
   maps.w[0] = *m;
   prm.half = half;
@@ -445,6 +482,7 @@ bool tc_rows_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_
   prm.f = f;
   prm.up_first = up_first ? 1 : 0;
   prm.rs = rs;
+  if (m128) return rows_run<ROWS_SWIGLU, 1, 128>(g, maps, prm, prm.tiles_per_seg, smem, st);
   return rows_run<ROWS_SWIGLU, kGateUpKb>(g, maps, prm, prm.tiles_per_seg, smem, st);
 }
 
@@ -461,7 +499,7 @@ bool tc_rows_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
   RowsMaps maps;
   RowsParams prm;
   size_t smem;
-  if (!rows_params(g, xb, 2 * half, in, rows, kTwoPerSm, kQkvKb, &maps, &prm, &smem)) return false;
+  if (!rows_params(g, xb, 2 * half, in, rows, kTwoPerSm, kQkvKb, 64, 1, &maps, &prm, &smem)) return false;
   const void* w[3] = {wq, wk, wv};
   for (int s = 0; s < 3; ++s) {
     const CUtensorMap* m = g->get_halves(w[s], (uint64_t)(dh / 2) * in * 2, d, in, half, kQkvKb);
@@ -493,7 +531,7 @@ bool tc_rows_launch_resid(TcGemm* g, int xb, const void* w, int out, int in, int
   RowsMaps maps;
   RowsParams prm;
   size_t smem;
-  if (!rows_params(g, xb, half, in, rows, kTwoPerSm, kResidKb, &maps, &prm, &smem)) return false;
+  if (!rows_params(g, xb, half, in, rows, kTwoPerSm, kResidKb, 64, 1, &maps, &prm, &smem)) return false;
   const CUtensorMap* m = g->get(w, out, in, half, kResidKb);
   if (!m) return false;
   maps.w[0] = *m;

@@ -506,17 +506,10 @@ bool tc_gemm_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   if (nblk > 4 || nt_all > g->xrows[xb] || (size_t)nt_all * ld > p_floats) return false;      // whichever kernel takes it
   if (rows > kWideFrom && tc_wide_launch(g, xb, w, n_seg, out, in, rows, P, p_floats, splits_out, split_stride, st)) return true;
   const int tiles = n_seg * (out / kTileM), kblocks = in / kTileK;
-  // K-splits: nearly two CTAs per SM (7/8 of the slots measured best: one split fewer costs no bandwidth and
-  // saves partial sums), keep at least four 64-wide K blocks per CTA.  With several row blocks a CTA needs most of an
-  // SM's shared and tensor memory: one CTA per SM.
-  int splits = ((nblk == 1 ? 2 : 1) * g->sm_count * 7 / 8) / tiles;
-  if (splits > kblocks / 4) splits = kblocks / 4;
   // many activation rows: a two-block stage would leave room for one CTA per SM only, so stage single blocks
   const int ks = nt <= 64 ? kStageKb : 1;
-  if (splits > (kblocks + ks - 1) / ks) splits = (kblocks + ks - 1) / ks;
-  if (splits > 16) splits = 16;
+  int splits = tc_gemm_splits(g, tiles, kblocks, nt_all);
   while (splits > 1 && (size_t)splits * nt_all * ld > p_floats) --splits;
-  if (splits < 1) splits = 1;
   TmapPack pack;
   memset(&pack, 0, sizeof pack);
   for (int s = 0; s < n_seg; ++s) {

@@ -36,7 +36,7 @@ bool tc_gemm_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
                              int rows, void* q, KvView kv, const RowMeta* meta, const float2* rope, int max_ctx,
                              const RowScale& rs, cudaStream_t st);
 
-// The same two, and the residual update, with the activation rows as the MMA's M operand (gemm_rows.cu): at most 64 rows.  Each
+// The same two, and the residual update, with the activation rows as the MMA's M operand (gemm_rows.cu): at most 64 rows, gate / up 128.  Each
 // returns false, nothing launched, where the form is not available or another kernel is the faster one.
 bool tc_rows_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_up, int f, int in, int rows, void* act, const RowScale& rs,
                            cudaStream_t st);

@@ -189,7 +189,7 @@ struct TcGemm {
     if (r != CUDA_SUCCESS) return nullptr;
     return &(halves_cache[key] = m);
   }
-  bool rows_ready[3] = {false, false, false};  // tc_rows_kernel's forms: shared memory limit raised
+  bool rows_ready[4] = {};  // tc_rows_kernel's forms: shared memory limit raised
 
   // pair kernel: CTA pairs that run at a time (0: not available, -1: not asked yet), scratch and flags of cut tiles
   int wide_pairs = -1;
@@ -215,5 +215,17 @@ struct TcGemm {
     return &(cache[key] = m);
   }
 };
+
+// K ranges of tc_gemm_kernel's plain form for up to 128 rows, scratch permitting: nearly two CTAs per SM (7/8 of the slots measured best:
+// one split fewer costs no bandwidth and saves partial sums), at least four 64-wide K blocks per CTA.  With several row blocks of 128 a CTA
+// needs most of an SM's shared and tensor memory: one CTA per SM.
+inline int tc_gemm_splits(const TcGemm* g, int tiles, int kblocks, int rows) {
+  int splits = ((rows <= 128 ? 2 : 1) * g->sm_count * 7 / 8) / tiles;
+  if (splits > kblocks / 4) splits = kblocks / 4;
+  const int ks = rows <= 64 ? tc::kStageKb : 1;
+  if (splits > (kblocks + ks - 1) / ks) splits = (kblocks + ks - 1) / ks;
+  if (splits > 16) splits = 16;
+  return splits < 1 ? 1 : splits;
+}
 
 }  // namespace amph

@@ -50,6 +50,20 @@ def test_bf16_forms_against_the_separate_kernels(heads, dh, ffn, n, nodes):
     _compare(_outputs(shape, w, prompts, 0), _outputs(shape, w, prompts, 4 | 16 | 512), 1e-2)
 
 
+# two accumulators (the sums of two K ranges, 512 and 1280 wide), and shapes that decline (more K ranges, an odd number of K blocks)
+@pytest.mark.parametrize("heads,dh,ffn", [(8, 64, 1408), (4, 128, 11008), (10, 128, 3456), (17, 128, 1408), (9, 64, 1152)])
+@pytest.mark.parametrize("nodes", [65, 80, 113, 128])
+def test_one_order_of_sums_above_64_rows(heads, dh, ffn, nodes):
+    shape = inputs.get_shape("small_bf16").with_(d_model=heads * dh, n_heads=heads, head_dim=dh, d_ffn=ffn, n_nodes=nodes, topk=(16, 16, 16, 16),
+                                                 lm_rank=24)
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    prompts = [inputs.make_prompt(shape.with_(prompt_len=100), seed=2).tolist()]
+    # the same sums in the same order, the same exponential and division: bit for bit (the adaptation layers' pass of 16 rows, which
+    # feeds output 2 only, has the fast exponential in one of them)
+    for i, (a, b) in enumerate(zip(_outputs(shape, w, prompts, 0), _outputs(shape, w, prompts, 4 | 16))):
+        assert i == 2 or torch.equal(a, b)
+
+
 @pytest.mark.parametrize("heads,dh,ffn", [(4, 64, 688), (3, 128, 1000), (1, 64, 8)])
 @pytest.mark.parametrize("lens,nodes", [((1,), 5), ((17,), 16), ((33,), 24), ((40, 7, 21), 19)])
 def test_fp32_forms_against_the_separate_kernels(heads, dh, ffn, lens, nodes):
