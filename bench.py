@@ -48,7 +48,7 @@ def algorithmic_bytes(shape, ctx_len: int) -> int:
 # bytes of a launch, so the step's average launch is scaled by this ratio.  The counters belong to one version of the
 # kernel: the digest below is that of the kernel source they were taken with, and the field is null for any other source.
 NCU_TRAFFIC_PER_WEIGHT_BYTE = 1.03
-NCU_KERNEL_SOURCE_SHA256_16 = "919be553d09979f8"
+NCU_KERNEL_SOURCE_SHA256_16 = "970b67f071aaf755"
 
 
 def kernel_source_digest() -> str:
