@@ -63,7 +63,8 @@ enum {
   AMPH_FLAG_NO_PAIR_PROJECTION = 512, /* passes of more than 64 rows on the projection kernels of smaller ones, with rotary embedding
                                        * and residual update (above 128 rows SwiGLU too) as kernels of their own, prompts in chunks of 128 rows, and key
                                        * ranges that do not depend on what else a launch carries: every sum in one order, whatever the
-                                       * height of a pass.  Always so with lm_rank > 0 (see amph_config)                           */
+                                       * height of a pass.  Always so with lm_rank > 0 (see amph_config).  fp32: the residual update
+                                       * as a kernel of its own                                                              */
   AMPH_FLAG_NO_SIDE_PREFETCH = 256  /* no helper stream: by default (bf16, a stream of the caller's own) every layer of the captured schedule of amph_step forks a small
                                      * kernel onto a second stream, created by amph_init, that pulls a part of the gate / up
                                      * weights into L2 while attention runs; it joins the caller's stream before amph_accept /

@@ -623,7 +623,9 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
   // output projection and residual update: one kernel for many rows, and in a small model
   int resid_cols = kWideScaleCols;
   auto resid_fused = [&](int xb, const void* wt, int in, const void* gain, size_t ss) {
-    if (f32 && c.d_model <= kPlainResidMax) {
+    if (f32) {
+      // low-rank heads: the squares of a row are added in one order whatever the height of a pass
+      if ((c.flags & AMPH_FLAG_NO_PAIR_PROJECTION) || c.lm_rank > 0 || !plain_resid_pays(c.d_model, rows)) return false;
       ProfScope p(ctx, AMPH_PROF_PROJECTION);
       launch_plain_resid(xbuf_ptr(ctx, xb), wt, c.d_model, in, rows, x, gain, ctx->ws + l.xn, ctx->at<float>(ss), st);
       if (p.rec) ctx->prof_bytes += (int64_t)c.d_model * in * (int64_t)ctx->esz;

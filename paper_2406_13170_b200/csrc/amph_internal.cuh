@@ -226,6 +226,7 @@ void launch_plain_swiglu(const void* x, const void* w_gate, const void* w_up, in
                          cudaStream_t st);
 void launch_plain_qkv_rope(const void* x, const void* const* w, int d, int dh, int in, int rows, void* q, const RopeGroups& gr, int max_ctx,
                            const RowScale& rs, cudaStream_t st);
+bool plain_resid_pays(int out, int rows);       // (it needs room for out / kPlainScaleCols entries a row in ss)
 void launch_plain_resid(const void* x_in, const void* w, int out, int in, int rows, float* x, const void* gain, void* xn, float* ss,
                         cudaStream_t st);
 

@@ -673,19 +673,36 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool live
                : "memory");
 }
 
+// row_scale shared by the 16 lanes of a half warp (all of them call; rows beyond `rows`: 1); t: the lane's first entry
+__device__ __forceinline__ float row_scale16(const RowScale& rs, int row, int rows, float t) {
+  if (rs.ss == nullptr) return 1.0f;
+  if (row < rows)
+    for (int c = 16 + (threadIdx.x & 15); c < rs.chunks; c += 16) t += rs.ss[(size_t)row * rs.chunks + c];
+#pragma unroll
+  for (int m = 8; m > 0; m >>= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
+  return row < rows ? 1.0f / sqrtf(t / (float)rs.d + rs.eps) : 1.0f;
+}
+
 struct GemmSegs { GemmSeg s[kMaxK]; };
 constexpr int kPlainThreads = 256;
 constexpr int kPlainChunk = 1024;        // bytes of a row per step: two 16-byte loads per lane
+constexpr int kPlainOneFeature = 296;    // blocks (two per SM) up to which a warp has one feature: see launch_gemm_generic
 
 // What becomes of the sums (16-row blocks of fp32 models; PLAIN: they go to P).  A launch per layer and step saved for each of the
 // others: in a 2-layer model of width 256 rotary embedding 2.1 us of the chain, SwiGLU 1.9, each residual update 1.4.
 //   SWIGLU: O = 2, a warp has a feature's gate and up row;  ROPE: O = 2, both members of a rotation pair, blockIdx.y = q, k, v;
 //   RESID: O = 1, x += sum, xn = gain * x, and the eight features' squares of a row meet in shared memory (ss[row][block]).
+// SWIGLU and ROPE let the next kernel start only by ending.  Its blocks would be placed beside theirs, on the few SMs with room, and
+// stay there: attention right behind ROPE took 24.8 us instead of 8.9 (width 256, 64 rows), the down projection behind SWIGLU lost
+// its spread too.  RESID triggers at once: what follows it starts with weights that wait for nothing.
+// Us a step of an 8-layer model with separate kernels / with these forms: width 256, 16 rows 252 / 212, 512 rows 1338 / 1174; width
+// 512 402 / 369 and 2451 / 2406; width 1024 692 / 621 and 6167 / 6035; width 2048 1499 / 1331 and 19000 / 18337.
 enum { PLAIN_P = 0, PLAIN_SWIGLU = 1, PLAIN_ROPE = 2, PLAIN_RESID = 3 };
 struct PlainEpi {
   RowScale rs;              // SWIGLU, ROPE: deferred division of the activation rows
   void* dst;                // SWIGLU: act [rows][out]; ROPE: q [rows][d]; RESID: xn [rows][out]
   RopeGroups gr;            // ROPE
+  float inv_rpg;            // ROPE: 1 / gr.rpg
   int dh, max_ctx;
   float* x;                 // RESID [rows][out]
   const void* gain;         // RESID: or NULL (x only)
@@ -696,14 +713,14 @@ template <typename T, int R, int O, int EPI>
 __global__ void __launch_bounds__(kPlainThreads)
 gemm_generic_kernel(const T* __restrict__ X, int ldx, const __grid_constant__ GemmSegs segs, int out, int in, float* __restrict__ P, int ldp, int rows,
                     int wait_first, const __grid_constant__ PlainEpi epi) {
-  pdl_launch_dependents();
+  if (EPI == PLAIN_P || EPI == PLAIN_RESID) pdl_launch_dependents();
   constexpr int V = Vec16<T>::N, KC = kPlainChunk / (int)sizeof(T);
   __shared__ __align__(16) uint4 xs[2][R][kPlainChunk / 16];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int item = blockIdx.x * (kPlainThreads / 32) + warp, r0 = blockIdx.z * R;
   // first feature of this warp, the distance of its others, and their matrix
-  const int half = EPI == PLAIN_ROPE ? epi.dh >> 1 : 0;
-  const int o0 = EPI == PLAIN_ROPE ? item / half * epi.dh + item % half : EPI == PLAIN_SWIGLU ? item : item * O;
+  const int half = EPI == PLAIN_ROPE ? epi.dh >> 1 : 0;          // a power of two
+  const int o0 = EPI == PLAIN_ROPE ? 2 * (item & -half) + (item & (half - 1)) : EPI == PLAIN_SWIGLU ? item : item * O;
   const int step = EPI == PLAIN_ROPE ? half : EPI == PLAIN_SWIGLU ? 0 : 1;
   auto weights = [&](int i) { return (const T*)segs.s[EPI == PLAIN_SWIGLU ? i : blockIdx.y].w; };
   const int chunks = (in + KC - 1) / KC;
@@ -729,33 +746,34 @@ gemm_generic_kernel(const T* __restrict__ X, int ldx, const __grid_constant__ Ge
   if (wait_first) pdl_wait();
   load_w(0);
   pdl_wait();
-  load_x(0);
-  // the row that this lane ends up with, and what its epilogue reads, ahead of the main loop
+  auto group_of = [&](int r) { return (int)(((float)r + 0.5f) * epi.inv_rpg); };       // r / rpg: both are below 2^10
+  // the row that this lane ends up with
   constexpr int same = R <= 32 ? 32 / R : 1;             // lanes that end up with the same row
-  int row = 0;
+  auto own_row = [&] {
+    int row = 0;
 #pragma unroll
-  for (int h = R / 2, m = 16; h > 0; h >>= 1, m >>= 1) row += (lane & m) ? h : 0;
-  const int rg = r0 + row;
-  const bool mine = lane % same == 0 && rg < rows && o0 < out;
-  float scale = 1.f, old = 0.f;
+    for (int h = R / 2, m = 16; h > 0; h >>= 1, m >>= 1) row += (lane & m) ? h : 0;
+    return row;
+  };
+  constexpr bool SCALED = EPI == PLAIN_SWIGLU || EPI == PLAIN_ROPE;
+  __shared__ float inv_s[SCALED ? R : 1];                // 1 / rms of the block's rows, from 16 lanes each
+  static_assert(!SCALED || R * 16 == kPlainThreads, "16 lanes a row");
+  // What the epilogue reads is asked for ahead of the activations and looked at behind the main loop's first loads, or its end: a
+  // stall ahead of them is added to every block (512 rows at width 512, gate / up 91 us, now 85; q / k / v 56 and 51).
+  float old = 0.f, ss0 = 0.f;
   float2 cs = make_float2(1.f, 0.f);
-  T* dst = nullptr;
-  if (EPI == PLAIN_SWIGLU || EPI == PLAIN_ROPE) { if (mine) scale = row_scale(epi.rs, rg); }
-  if constexpr (EPI == PLAIN_RESID) { if (mine) old = epi.x[(size_t)rg * out + o0]; }
-  if constexpr (EPI == PLAIN_ROPE) {
-    if (mine) {
-      const int g = rg / epi.gr.rpg, rl = rg - g * epi.gr.rpg, h = o0 / epi.dh, i = o0 - h * epi.dh;
-      const RowMeta* meta = epi.gr.meta[g];
-      if (blockIdx.y < 2) cs = epi.gr.rope[g][(size_t)rl * half + i];
-      if (blockIdx.y == 0) {
-        dst = (T*)epi.dst + (size_t)rg * out + o0;
-      } else {
-        const int slot = meta->slot[rl];
-        if (rl < meta->n_rows && slot >= 0 && slot < epi.max_ctx)
-          dst = (T*)(blockIdx.y == 1 ? epi.gr.kc[g] : epi.gr.vc[g]) + ((size_t)h * epi.max_ctx + slot) * epi.dh + i;
-      }
+  int slot = -1, live = 0;
+  if (EPI != PLAIN_P) {
+    const int rg = r0 + own_row(), rs = r0 + (int)(threadIdx.x >> 4);
+    if (SCALED && epi.rs.ss != nullptr && rs < rows && (threadIdx.x & 15) < epi.rs.chunks) ss0 = epi.rs.ss[rs * epi.rs.chunks + (threadIdx.x & 15)];
+    if (EPI == PLAIN_RESID && rg < rows && o0 < out) old = epi.x[(size_t)rg * out + o0];
+    if (EPI == PLAIN_ROPE && rg < rows && o0 < out) {
+      const int g = group_of(rg), rl = rg - g * epi.gr.rpg;
+      if (blockIdx.y < 2) cs = epi.gr.rope[g][(size_t)rl * half + (o0 & (half - 1))];
+      if (blockIdx.y > 0) { slot = epi.gr.meta[g]->slot[rl]; live = epi.gr.meta[g]->n_rows; }
     }
   }
+  load_x(0);
   float acc[O][R];
 #pragma unroll
   for (int i = 0; i < O; ++i)
@@ -770,10 +788,13 @@ gemm_generic_kernel(const T* __restrict__ X, int ldx, const __grid_constant__ Ge
     if (c + 1 < chunks) {
       load_x(c + 1);
       load_w(c + 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
+    if (SCALED && c == 0) {
+      const float inv = row_scale16(epi.rs, r0 + (int)(threadIdx.x >> 4), rows, ss0);
+      if ((threadIdx.x & 15) == 0) inv_s[threadIdx.x >> 4] = inv;
+    }
+    if (c + 1 < chunks) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < R; ++r)
@@ -804,17 +825,28 @@ gemm_generic_kernel(const T* __restrict__ X, int ldx, const __grid_constant__ Ge
         acc[i][0] += __shfl_xor_sync(0xffffffffu, acc[i][0], m);
       }
     }
-    if (EPI == PLAIN_P && lane % same == 0 && rg < rows && o0 + i < out) P[(size_t)rg * ldp + blockIdx.y * out + o0 + i] = acc[i][0];
+    if constexpr (EPI == PLAIN_P) {
+      const int rg = r0 + own_row();
+      if (lane % same == 0 && rg < rows && o0 + i < out) P[(size_t)rg * ldp + blockIdx.y * out + o0 + i] = acc[i][0];
+    }
   }
+  const int row = own_row(), rg = r0 + row;
+  const bool mine = lane % same == 0 && rg < rows && o0 < out;
   if constexpr (EPI == PLAIN_SWIGLU) {
-    const float t = acc[0][0] * scale;
+    const float scale = inv_s[row], t = acc[0][0] * scale;
     if (mine) ((T*)epi.dst)[(size_t)rg * out + o0] = from_f<T>(t / (1.0f + expf(-t)) * (acc[1][0] * scale));
   } else if constexpr (EPI == PLAIN_ROPE) {
-    const float a = acc[0][0] * scale, b = acc[1][0] * scale;
-    if (dst != nullptr) {
-      dst[0] = from_f<T>(blockIdx.y < 2 ? a * cs.x - b * cs.y : a);
-      dst[half] = from_f<T>(blockIdx.y < 2 ? b * cs.x + a * cs.y : b);
+    const float scale = inv_s[row], a = acc[0][0] * scale, b = acc[1][0] * scale;
+    if (!mine) return;
+    T* dst = (T*)epi.dst + (size_t)rg * out + o0;
+    if (blockIdx.y > 0) {
+      const int g = group_of(rg), i = o0 & (half - 1);
+      if (rg - g * epi.gr.rpg >= live || slot < 0 || slot >= epi.max_ctx) return;
+      // head o0 / dh
+      dst = (T*)(blockIdx.y == 1 ? epi.gr.kc[g] : epi.gr.vc[g]) + (size_t)(o0 - i) * epi.max_ctx + (size_t)slot * epi.dh + i;
     }
+    dst[0] = from_f<T>(blockIdx.y < 2 ? a * cs.x - b * cs.y : a);
+    dst[half] = from_f<T>(blockIdx.y < 2 ? b * cs.x + a * cs.y : b);
   } else if constexpr (EPI == PLAIN_RESID) {
     __shared__ float sq[kPlainThreads / 32][R];
     const float v = acc[0][0] + old;
@@ -849,13 +881,15 @@ void launch_gemm_generic(const void* x, int ldx, const GemmSeg* segs, int n_seg,
   };
   AMPH_DISPATCH(dtype, const T* X = (const T*)x;
                 if (rows <= 4) run(gemm_generic_kernel<T, 4, 1, PLAIN_P>, 4, 1, X);
-                else if (rows <= 8 && blocks * n_seg <= 296) run(gemm_generic_kernel<T, 8, 1, PLAIN_P>, 8, 1, X);
+                else if (rows <= 8 && blocks * n_seg <= kPlainOneFeature) run(gemm_generic_kernel<T, 8, 1, PLAIN_P>, 8, 1, X);
                 else if (rows <= 8) run(gemm_generic_kernel<T, 8, 2, PLAIN_P>, 8, 2, X);
-                else if ((long long)blocks * n_seg * ((rows + 15) / 16) <= 296) run(gemm_generic_kernel<T, 16, 1, PLAIN_P>, 16, 1, X);
+                else if ((long long)blocks * n_seg * ((rows + 15) / 16) <= kPlainOneFeature) run(gemm_generic_kernel<T, 16, 1, PLAIN_P>, 16, 1, X);
                 else run(gemm_generic_kernel<T, 16, 2, PLAIN_P>, 16, 2, X));
 }
 
-// The fused forms, fp32: 16-row blocks, eight features (pairs) a block.
+// The fused forms, fp32: 16-row blocks, eight features (pairs) a block.  RESID only where launch_gemm_generic would take one feature a
+// warp too: beyond that its blocks stage the activation rows twice as often as those of two features (256 rows at width 1024: 4716 us a
+// prefill with it everywhere, 3350 with this rule, 3521 with no fused form).
 static void plain_fused(void (*kernel)(const float*, int, GemmSegs, int, int, float*, int, int, int, PlainEpi), const void* x, const void* const* w,
                         int n_w, int items, int ny, int out, int in, int rows, const PlainEpi& epi, cudaStream_t st) {
   GemmSegs gs;
@@ -879,9 +913,14 @@ void launch_plain_qkv_rope(const void* x, const void* const* w, int d, int dh, i
   e.rs = rs;
   e.dst = q;
   e.gr = gr;
+  e.inv_rpg = 1.0f / (float)gr.rpg;
   e.dh = dh;
   e.max_ctx = max_ctx;
   plain_fused(gemm_generic_kernel<float, 16, 2, PLAIN_ROPE>, x, w, 3, d / 2, 3, d, in, rows, e, st);
+}
+
+bool plain_resid_pays(int out, int rows) {
+  return out <= kPlainResidMax && (long long)((out + 7) / 8) * ((rows + 15) / 16) <= kPlainOneFeature;
 }
 
 void launch_plain_resid(const void* x_in, const void* w, int out, int in, int rows, float* x, const void* gain, void* xn, float* ss,
