@@ -57,8 +57,12 @@ struct DevState {
 // Programmatic dependent launch.  Every kernel of the step is launched with the attribute below, so it
 // may become resident before its predecessor in the stream has finished; it must call pdl_wait() before
 // touching anything the predecessor writes.  pdl_launch_dependents() lets the successor start launching.
-// Rule used here: weight-streaming projections trigger at once, prefetch weights, then wait; every other
-// kernel waits first and triggers right after, so at most two consecutive kernels ever overlap.
+// Rule used here: weight-streaming projections trigger early, prefetch weights, then wait; every other kernel waits first and
+// triggers right after, or only by ending.  Results depend on nothing but the waits: a run of projections (the output, gate / up,
+// down and q / k / v projection of a small bf16 model, then attention) may be resident all at once.
+// A kernel that takes tensor memory triggers only behind the allocation, so a CTA that is still asking for columns never has a later
+// kernel of its stream beside it: who holds columns ends without it.  (Triggered ahead of the allocation, a CTA of a successor could
+// have taken the columns first, when another stream's kernel gives them back, and waited for its predecessor with them.)
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -118,7 +118,6 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
-  pdl_launch_dependents();
   const unsigned long long limit_ns = prm.wait_limit_ns;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile = blockIdx.x, seg = tile / prm.tiles_per_seg, lt = tile - seg * prm.tiles_per_seg;
@@ -145,6 +144,7 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(prm.tmem_cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    pdl_launch_dependents();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncwarp();

@@ -144,7 +144,6 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
-  pdl_launch_dependents();                          // the consumer kernel may get resident and wait
   const unsigned long long limit_ns = prm.wait_limit_ns;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile = blockIdx.x, split = blockIdx.y;
@@ -186,6 +185,7 @@ tc_gemm_kernel(const __grid_constant__ TmapPack maps, const TcParams prm) {
   if (warp == 1) {                                   // TMEM allocation belongs to the MMA warp
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(tmem_cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    pdl_launch_dependents();                         // the consumer kernel may get resident and wait
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncwarp();

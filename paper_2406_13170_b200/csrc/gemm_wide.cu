@@ -203,7 +203,6 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   // at the cluster's barrier as soon as its own part is done (barriers initialised, tensor memory allocated) and waits for it
   // only where it needs the others; warp 0 issues the weights while warp 1 waits for the kernel before this one and then fetches
   // the ring's first activations.  One after the other, it took 4.9 us from the CTA's start to the first full stage.
-  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -215,6 +214,7 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(prm.tmem_cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    pdl_launch_dependents();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncwarp();

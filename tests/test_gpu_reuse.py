@@ -77,3 +77,42 @@ def test_a_tap_is_not_overwritten_by_what_torch_has_queued():
         assert torch.equal(got, want)
         del got
     m.close()
+
+
+def test_two_contexts_on_two_streams_at_once():
+    """Every projection and attention CTA takes tensor memory, several kernels of a context are resident at a time, and two contexts
+    share the SMs: each gives what it gives alone.  (Passes of up to 64 rows, of more, and prompts of both.)"""
+    from paper_2406_13170_b200 import Amphista
+    steps = 12
+
+    def build(n_nodes, n, heads):
+        shape = inputs.get_shape("small_bf16").with_(d_model=heads * 128, n_heads=heads, n_nodes=n_nodes, topk=(16, 16, 16, 16), prompt_len=n)
+        w = inputs.make_weights(shape, seed=n, device="cuda:0", init="fan_in")
+        m = Amphista(shape, inputs.make_tree(n_nodes, shape.topk), w, max_ctx=n + steps * (shape.K + 1) + n_nodes + 8)
+        out = torch.zeros(steps, shape.K + 2, dtype=torch.int32, device="cuda:0")
+        return m, shape, inputs.make_prompt(shape).tolist(), out
+
+    def enqueue(c, i):
+        c[0].step(c[3][i, : c[1].K + 1], c[3][i, c[1].K + 1 :])
+
+    def results(c):
+        c[0].synchronize()
+        return [c[3].clone(), c[0].get_tensor("logits", (c[1].n_nodes, c[1].vocab)), c[0].get_tensor("kv.k.2", (c[0].get_state()[0], c[1].d_model))]
+
+    pair = [build(64, 300, 4), build(100, 50, 8)]
+    torch.cuda.synchronize()
+    alone = []
+    for c in pair:
+        c[0].prefill(c[2])
+        for i in range(steps):
+            enqueue(c, i)
+        alone.append(results(c))
+    for c in pair:
+        c[0].prefill(c[2])
+    for i in range(steps):
+        for c in pair:
+            enqueue(c, i)
+    for c, want in zip(pair, alone):
+        for a, b in zip(results(c), want):
+            assert torch.equal(a, b)
+        c[0].close()
