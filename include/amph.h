@@ -294,6 +294,13 @@ amph_status amph_selftest_wait_timeout(const void* x_dev, int32_t x_rows_cap, co
                                        int32_t out, int32_t in, int32_t rows, float* y_dev, void* ws_dev, size_t ws_bytes,
                                        void* stream, int32_t limit_us);
 
+/* The same for the projections inside a context's passes (those with SwiGLU, rotary embedding or residual update in their
+ * epilogues included): from this call on, every tensor-core projection that ctx launches gives up after limit_us microseconds as
+ * described above and stands for sums of zero, until a call with limit_us = 0.  Calls that report device-side errors return
+ * AMPH_ERR_TIMEOUT meanwhile; after limit_us = 0, amph_prefill starts afresh.  Synchronises the stream.  AMPH_ERR_STATE without
+ * tensor-core projections (fp32, AMPH_FLAG_NO_TENSOR_CORE, before the first amph_prefill). */
+amph_status amph_selftest_context_timeout(amph_ctx* ctx, int32_t limit_us);
+
 /* (No counterpart in the paper: a packaging variant of amph_project.)
  * The same projection for callers that cannot allocate device memory at the time of the call: for
  * example code running after a serving engine has taken all free GPU memory into its own pool, where

@@ -1566,6 +1566,17 @@ amph_status amph_selftest_wait_timeout(const void* x_dev, int32_t x_rows_cap, co
                             (unsigned long long)limit_us * 1000ull, 1024u);
 }
 
+amph_status amph_selftest_context_timeout(amph_ctx* ctx, int32_t limit_us) {
+  if (!ctx) return fail(nullptr, AMPH_ERR_INVALID_ARG, "ctx must not be NULL");
+  if (limit_us < 0 || limit_us > 1000000) return fail(ctx, AMPH_ERR_INVALID_ARG, "limit_us must be in 0..1000000");
+  if (!ctx->tc) return fail(ctx, AMPH_ERR_STATE, "no tensor-core projections yet (before the first amph_prefill), or none in this context");
+  const amph_status rc = cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "selftest");
+  if (rc != AMPH_OK) return rc;
+  ctx->drop_graphs();                                // captured schedules hold the launches' parameters
+  tc_gemm_set_selftest(ctx->tc, (unsigned long long)limit_us * 1000ull, limit_us ? 1024u : 0u);
+  return AMPH_OK;
+}
+
 amph_status amph_set_state(amph_ctx* ctx, int32_t ctx_len, int32_t root, int32_t n_pending, const float* pend_hidden,
                            const int32_t* pend_next) {
   if (!ctx) return fail(nullptr, AMPH_ERR_INVALID_ARG, "ctx must not be NULL");

@@ -10,8 +10,8 @@
 // them are 350 clocks, as much as ten MMAs of this size; a gate / up launch of 180 MB took 40.7 us with them, 30.9 without.
 //
 // Warp roles: 0 = TMA producer of the weights (waits for no other kernel), 1 = MMA issuer (owns the tensor memory), 2-5 =
-// epilogue, 6 = TMA producer of the activations.  Every barrier wait is bounded: if one gives up the CTA raises the error flag,
-// lets its copies land and leaves; its outputs are finite then (sums of zero).
+// epilogue, 6 = TMA producer of the activations.  Every barrier wait is bounded, counted from the end of the kernel ahead: if one gives
+// up the CTA raises the error flag, lets its copies land and its MMAs finish and leaves; its outputs are finite then (sums of zero).
 #include "gemm_tc_common.cuh"
 
 namespace amph {
@@ -58,6 +58,7 @@ struct RowsParams {
   int out;
   int* err_flag;
   unsigned long long wait_limit_ns;
+  uint32_t extra_tx;        // self-test only: bytes the first stage's barrier expects beyond what is copied
 };
 
 __device__ __forceinline__ void load_w(void* dst, const CUtensorMap* map, int row, int kb, uint64_t* bar, uint64_t pol, bool pair) {
@@ -114,7 +115,7 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   static_assert(M == 64 || (KS == 1 && EPI == ROWS_SWIGLU), "a cut between two accumulators falls between two stages");
   __shared__ float inv_s[PAIR ? M : 1];                            // 1 / rms of the activation rows
-  __shared__ __align__(8) uint64_t w_full[kMaxRing], w_empty[kMaxRing], x_full[kMaxRing], x_empty[kMaxRing], accum_bar;
+  __shared__ __align__(8) uint64_t w_full[kMaxRing], w_empty[kMaxRing], x_full[kMaxRing], x_empty[kMaxRing], accum_bar, drain_bar;
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
@@ -137,6 +138,7 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
     for (int s = 0; s < prm.w_stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
     for (int s = 0; s < prm.x_stages; ++s) { mbar_init(&x_full[s], 1); mbar_init(&x_empty[s], 1); }
     mbar_init(&accum_bar, 1);
+    mbar_init(&drain_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // Barrier 2 tells the warps that use the mbarriers that they exist, barrier 3 the epilogue that the accumulator does.
@@ -160,9 +162,10 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
     if (leader) asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
     int issued = 0;
     for (int i = 0, s = 0, ph = 1; i < its; ++i) {
+      if (i == prm.w_stages) pdl_wait();             // the time spent behind the kernel ahead does not count for the limit
       if (i >= prm.w_stages && !__all_sync(0xffffffffu, mbar_wait(&w_empty[s], ph, &abort_flag, limit_ns))) break;
       if (leader) {
-        mbar_expect_tx(&w_full[s], w_bytes);
+        mbar_expect_tx(&w_full[s], w_bytes + (i == 0 ? prm.extra_tx : 0u));
         load_w(ws + (size_t)s * w_bytes, map, row0, i * KS, &w_full[s], pol, PAIR);
         if (i == prm.w_stages - 1)
           for (int j = 1; j <= prm.l2_prefetch && i + j < its; ++j) prefetch_w(map, row0, (i + j) * KS, PAIR);
@@ -201,6 +204,7 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
   } else if (warp == 1) {
     // ---------------- MMA issuer (the warp stays converged, its elected lane issues)
     const bool leader = elect_one();
+    pdl_wait();
     asm volatile("bar.sync 2, 96;" ::: "memory");
     const uint32_t tmem_d = tmem_base_slot;
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(prm.n >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
@@ -230,6 +234,12 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
       if (++xst == prm.x_stages) { xst = 0; xph ^= 1; }
     }
     if (ok && leader) commit(&accum_bar);
+    if (!ok) {                                       // no tensor memory is given back under an MMA
+      if (leader) commit(&drain_bar);
+      __syncwarp();
+      const unsigned long long t0 = now_ns();
+      while (!mbar_try(&drain_bar, 0) && now_ns() - t0 < kDrainNs) {}
+    }
     __syncwarp();
   } else {
     // ---------------- epilogue: row r of the accumulator sits in TMEM lane 32 (r / 16) + r % 16 (M = 64), or r (M = 128); the warp of
@@ -242,6 +252,11 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
       asm volatile("bar.sync 1, 128;" ::: "memory");
     }
     constexpr int U = 4;                               // pieces of 8 columns in flight
+    auto sums_ready = [&] {
+      const bool ok = __all_sync(0xffffffffu, mbar_wait(&accum_bar, 0, &abort_flag, limit_ns));
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      return ok;
+    };
     const bool two = M == 128 && prm.kb_cut < prm.kblocks;
     for (int part = 0; part < M / 64; ++part) {
     const int ra = quarter * (M / 4) + part * 16 + (lane >> 2), rb = ra + 8;
@@ -263,8 +278,7 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
     };
     if constexpr (EPI == ROWS_SWIGLU) {
       const float sa = la ? inv_s[ra] : 0.f, sb = lb ? inv_s[rb] : 0.f;
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(&accum_bar, 0, &abort_flag, limit_ns));
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const bool ok = sums_ready();
       const uint32_t tg = taddr + (prm.up_first ? (uint32_t)prm.half : 0u), tu = taddr + (prm.up_first ? 0u : (uint32_t)prm.half);
       __nv_bfloat16* const pa = prm.act + (size_t)ra * prm.f + row0 + cq;
       __nv_bfloat16* const pb = prm.act + (size_t)rb * prm.f + row0 + cq;
@@ -312,8 +326,7 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
       const float2* const ta = prm.rope + (size_t)ra * hdim + i0;
       const float2* const tb = prm.rope + (size_t)rb * hdim + i0;
       const float4 unit = make_float4(1.f, 0.f, 1.f, 0.f);
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(&accum_bar, 0, &abort_flag, limit_ns));
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const bool ok = sums_ready();
       for (int c0 = 0; c0 < prm.half; c0 += 8 * U) {
         float lo[U][4], hi[U][4];
         float4 ca[U], cb[U];
@@ -356,8 +369,7 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
         if (lb) ob[j] = *reinterpret_cast<const float2*>(xb + 8 * j);
         if (prm.gain != nullptr) gn[j] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(prm.gain + f0 + 8 * j));
       }
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(&accum_bar, 0, &abort_flag, limit_ns));
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const bool ok = sums_ready();
       float v[U][4];
 #pragma unroll
       for (int j = 0; j < U; ++j)
@@ -436,6 +448,7 @@ bool rows_params(TcGemm* g, int xb, int n, int in, int rows, size_t smem_limit, 
   maps->x = *mx;
   prm->err_flag = g->err_flag;
   prm->wait_limit_ns = g->wait_limit_ns;
+  prm->extra_tx = g->extra_tx;
   return true;
 }
 

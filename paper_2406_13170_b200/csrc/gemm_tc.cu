@@ -588,6 +588,7 @@ bool tc_gemm_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_
   prm.rs = rs;
   prm.err_flag = g->err_flag;
   prm.wait_limit_ns = g->wait_limit_ns;
+  prm.extra_tx = g->extra_tx;
   const size_t smem = (size_t)stages * stage_bytes + 1024;
   return launch_pdl(tc_gemm_kernel<EPI_SWIGLU>, dim3(tiles, 1), dim3(kThreads), smem, st, pack, prm) == cudaSuccess;
 }
@@ -640,6 +641,7 @@ bool tc_gemm_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
   prm.max_ctx = max_ctx;
   prm.err_flag = g->err_flag;
   prm.wait_limit_ns = g->wait_limit_ns;
+  prm.extra_tx = g->extra_tx;
   const size_t smem = (size_t)stages * stage_bytes + 1024;
   return launch_pdl(tc_gemm_kernel<EPI_ROPE>, dim3(3 * tiles_per_seg, 1), dim3(kThreads), smem, st, pack, prm) == cudaSuccess;
 }
@@ -688,7 +690,7 @@ void tc_gemm_rebind(TcGemm* g, int xb, void* ptr, int rows, int cols, int* err_f
 void tc_gemm_wait_first(TcGemm* g) { g->wait_first = 1; }
 
 void tc_gemm_set_selftest(TcGemm* g, unsigned long long wait_limit_ns, unsigned extra_tx) {
-  g->wait_limit_ns = wait_limit_ns;
+  g->wait_limit_ns = wait_limit_ns ? wait_limit_ns : kWaitLimitNs;
   g->extra_tx = extra_tx;
 }
 

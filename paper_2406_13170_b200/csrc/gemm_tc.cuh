@@ -79,8 +79,8 @@ void tc_gemm_rebind(TcGemm* g, int xb, void* ptr, int rows, int cols, int* err_f
 // while it still runs): for callers whose weights that kernel may have written.
 void tc_gemm_wait_first(TcGemm* g);
 
-// Failure-path self-test: every barrier wait of later launches gives up after wait_limit_ns, and the first stage's
-// barrier of each CTA expects extra_tx bytes more than its copies deliver (so that wait can never complete).
+// Failure-path self-test: every barrier wait of later launches gives up after wait_limit_ns (0: the usual limit), and the first
+// stage's barrier of each CTA expects extra_tx bytes more than its copies deliver (so that wait can never complete).
 void tc_gemm_set_selftest(TcGemm* g, unsigned long long wait_limit_ns, unsigned extra_tx);
 
 }  // namespace amph

@@ -194,3 +194,52 @@ def test_nothing_of_a_timeout_outlives_a_reset_or_a_prefill():
         got = result()
         assert got[0] == want[0] and torch.equal(got[1], want[1])
     m.close()
+
+
+# passes of up to 64 rows (16 weight features a tile, whole tiles of both), of 65-128 rows in one order of sums (two accumulators), of
+# up to 16 rows at 7B widths, and the pair projection's forms
+@pytest.mark.parametrize("change,n", [(dict(n_nodes=43), 40), (dict(d_ffn=11008, n_nodes=100, lm_rank=24), 100),
+                                      (dict(d_model=4096, n_heads=32, d_ffn=11008, n_layers=1, n_nodes=16), 12),
+                                      (dict(n_nodes=100), 300)])
+def test_waits_of_the_projections_inside_a_pass_run_out(change, n):
+    """Every projection of a prefill, then of a draft and a verification, gives up after 1 ms: the calls say so, the caches hold zeros
+    (nothing else a projection gave up on may be in them, attention fetches whole tiles), and the next prefill is as it was."""
+    from paper_2406_13170_b200 import Amphista
+    from paper_2406_13170_b200.binding import AmphError
+    shape = inputs.get_shape("small_bf16").with_(topk=(16, 16, 16, 16), **change)
+    topo = inputs.make_tree(shape.n_nodes, shape.topk)
+    m = Amphista(shape, topo, inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in"), max_ctx=512)
+    prompt = inputs.make_prompt(shape.with_(prompt_len=n), seed=4).tolist()
+    with pytest.raises(AmphError):
+        m.selftest_timeout(1000)                                                       # no projections yet
+
+    def result():
+        root = m.prefill(prompt)
+        return [torch.tensor(root)] + [m.get_tensor(f"kv.{c}.{i}", (n, shape.d_model)) for c in "kv" for i in (0, shape.n_layers - 1)]
+
+    def timed_out(call):
+        with pytest.raises(AmphError) as e:
+            call()
+        assert e.value.status == 8
+
+    want = result()
+    m.selftest_timeout(1000)
+    timed_out(lambda: m.prefill(prompt))
+    for t in [m.get_tensor(f"kv.{c}.{i}", (n, shape.d_model)) for c in "kv" for i in (0, shape.n_layers - 1)]:
+        assert torch.equal(t, torch.zeros_like(t))
+    assert bool(torch.isfinite(m.get_tensor("hidden", (n, shape.d_model))).all())
+    m.selftest_timeout(0)
+    assert all(torch.equal(a, b) for a, b in zip(result(), want))
+    m.selftest_timeout(1000)
+    m.draft()
+    m.verify_tree()
+    m.synchronize()
+    timed_out(m.get_state)
+    for c in "kv":
+        t = m.get_tensor(f"kv.{c}.0", (n + shape.n_nodes, shape.d_model))
+        assert torch.equal(t[n:], torch.zeros_like(t[n:]))
+    assert bool(torch.isfinite(m.get_tensor("hidden", (shape.n_nodes, shape.d_model))).all())
+    m.selftest_timeout(0)
+    m.reset()
+    assert all(torch.equal(a, b) for a, b in zip(result(), want))
+    m.close()
