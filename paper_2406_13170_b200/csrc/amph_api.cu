@@ -307,7 +307,7 @@ void make_layout(const amph_config& c, int n_nodes, Layout* L, int* Mcap_out, si
   l.att_ml = l.per_group(4 * (size_t)splits * c.n_heads * Mcap * 2, &l.att_ml_s);
   l.logits = l.take(4 * (size_t)Rcap * V);
   // one entry per tile of the kernel that updates the residual: 128 columns, 16 or 8 in a small model
-  static_assert(kRowsResidMax == kPlainResidMax, "one bound for both");
+  static_assert(kRowsResidOut <= kPlainResidMax, "the lower bound decides");
   const size_t ss_cols = c.d_model / (c.d_model <= kPlainResidMax ? kPlainScaleCols : kWideScaleCols) + 32;
   l.ss_a = l.take(4 * (size_t)Rcap * ss_cols);
   l.ss_b = l.take(4 * (size_t)Rcap * ss_cols);
@@ -634,7 +634,7 @@ int layer_forward(amph_ctx* ctx, const LayerW& w, CacheOf cache_of, float* x, co
       return true;
     }
     if (!ctx->tc) return false;
-    if (rows <= kWideFrom && (ctx->one_order || c.d_model > kRowsResidMax || in > kRowsResidMax)) return false;
+    if (rows <= kWideFrom && (ctx->one_order || c.d_model > kRowsResidOut || in > kRowsResidMax)) return false;
     ProfScope p(ctx, AMPH_PROF_PROJECTION);
     const bool done = rows > kWideFrom
                           ? tc_wide_launch_resid(ctx->tc, xb, wt, c.d_model, in, rows, x, gain, ctx->ws + l.xn, ctx->at<float>(ss), st)

@@ -504,9 +504,11 @@ bool tc_rows_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
   if (!g || !wq || !wk || !wv || !q || !kv.k || !kv.v || !meta || !rope || (dh != 64 && dh != 128)) return false;
   if (((uintptr_t)wq | (uintptr_t)wk | (uintptr_t)wv) & 15) return false;
   const int d = n_heads * dh;
-  // up to 32 rows tc_gemm_kernel's tiles (the same ones, at d >= 2048) are as fast: 4096 x 3 x 4096, 16 rows 18.4 us, here 19.3;
-  // 32 rows 19.5 / 19.1; 48 rows 21.2 / 19.9; 64 rows 21.7 / 20.7; a step's layer at 32 rows 0.5 us slower here
-  if (3 * d / 64 > g->sm_count && rows <= 32) return false;
+  // Up to 32 rows tc_gemm_kernel's 64-row tiles, from 2/5 of a wave of them on: us a step of 8 layers there / here, 16 rows, width 512
+  // 258.5 / 253.4, 768 295 / 292, 1024 312 / 313, 1280 333 / 343, 1536 368 / 373, 2048 430 / 442; 32 rows, width 1280 340 / 350, 2048
+  // 447 / 457.  Above 32 rows here: 4096 x 3 x 4096 back to back, 48 rows 21.2 / 19.9, 64 rows 21.7 / 20.7; a pass of 8 steps x 8 layers,
+  // 48 rows 9780 / 9660, 64 rows 10097 / 9963, at 6656 (6 layers x 6 steps) 14036 / 13767.
+  if (rows <= 32 && 3 * d / 64 * 5 > 2 * g->sm_count) return false;
   int half = 8;                                      // the smallest tile that leaves all CTAs resident at once
   while (half < dh / 2 && 3 * d / 2 / half > 2 * g->sm_count) half *= 2;
   RowsMaps maps;
@@ -536,10 +538,11 @@ bool tc_rows_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
 bool tc_rows_launch_resid(TcGemm* g, int xb, const void* w, int out, int in, int rows, float* x, const void* gain, void* xn, float* ss,
                           int* cols, cudaStream_t st) {
   if (!g || !w || !x || ((uintptr_t)w & 15) || (gain && (!xn || !ss))) return false;
-  // Without split-K every CTA reads all activation rows for a tile of 16 features, so only where both sides are short.  Three
-  // layers of 512 x 512 and 512 x 1408, prefill and eight steps of 32 rows: 1909 us with split-K sums and a kernel that adds them,
-  // 1790 with this; a launch at 4096 x 4096 (16 rows) 11.6 us against 7.3 + 3.0.
-  if (out > kRowsResidMax || in > kRowsResidMax || out % 16) return false;
+  // Without split-K every CTA reads all activation rows for a tile of 16 features, so only where both sides are short.  Us a step of
+  // 8 layers, 16 / 32 / 64 rows, with split-K sums and a kernel that adds them | with this: width 1280 347 / 360 / 370 | 346 / 353 / 361,
+  // 1536 378 / 389 / 400 | 375 / 387 / 395, 2048 432 / 450 / 465 | 444 / 458 / 464; the down projection alone, 2048 -> 1024 303 / 320 / 318 |
+  // 307 / 309 / 310, 2048 -> 768 292 / 299 / 304 | 282 / 290 / 289; a launch at 4096 x 4096 (16 rows) 11.6 us against 7.3 + 3.0.
+  if (out > kRowsResidOut || in > kRowsResidMax || out % 16) return false;
   const int half = 16;
   RowsMaps maps;
   RowsParams prm;

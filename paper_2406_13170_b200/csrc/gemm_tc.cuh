@@ -43,7 +43,7 @@ bool tc_rows_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_
 bool tc_rows_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, const void* wv, int n_heads, int dh, int in, int rows, void* q,
                              KvView kv, const RowMeta* meta, const float2* rope, int max_ctx, const RowScale& rs, cudaStream_t st);
 // x += X . W^T and, with gain, xn <- gain * x (bf16) and ss[row][out / *cols] <- sums of squares.
-constexpr int kRowsResidMax = 2048;      // longest side it takes
+constexpr int kRowsResidMax = 2048, kRowsResidOut = 1536;      // longest K and most features it takes
 bool tc_rows_launch_resid(TcGemm* g, int xb, const void* w, int out, int in, int rows, float* x, const void* gain, void* xn, float* ss,
                           int* cols, cudaStream_t st);
 
