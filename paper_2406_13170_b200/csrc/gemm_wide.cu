@@ -3,9 +3,8 @@
 // A cluster of two CTAs owns 256 weight rows and a block of up to 256 activation rows: one tcgen05.mma.cta_group::2 (M = 256,
 // N <= 256) per 16 columns of K.  Each CTA stages its own 128 weight rows and HALF of the activation rows: 32 KB per 64
 // columns of K at N = 256, i.e. 64 bytes of L2 -> SM traffic per clock of MMA, against 80 with one CTA per 128 weight rows and
-// 512 activation rows (which made L2 the bound).  A stage holds one K block (512 clocks of MMA at N = 256), so that six are in
-// flight; with two K blocks per stage and three stages a batch of 4 x 64 rows (8 layers, 12 steps) took 28.4 ms, now 27.5, a
-// prefill of 1900 tokens 32.1, now 32.0.  (The producers' and the issuer's loops must not divide for that: see below.)
+// 512 activation rows (which made L2 the bound).  A stage holds one or two K blocks (see unit_kb; the producers' and the
+// issuer's loops must not divide for one block, 512 clocks of MMA at N = 256, to be enough: see below).
 // With 257..512 rows two neighbouring pairs take the two row blocks of the same weights at the same time, so weights still
 // cross HBM once.  Tensor memory holds two accumulators: the epilogue of one piece of work runs under the next main loop.
 //
@@ -35,7 +34,6 @@ namespace {
 
 constexpr int kEpiThreads = 512;      // four warps per TMEM lane quarter
 constexpr int kWideThreads = 64 + kEpiThreads;
-constexpr int kUnitKb = 1;            // K blocks per pipeline stage = unit of work: ranges are cut at multiples of 64 columns
 constexpr int kMaxWideRows = 512;
 constexpr int kMaxStages = 8;
 constexpr int kMaxGroups = kWideFlags / 2;
@@ -50,6 +48,7 @@ enum { WIDE_PLAIN = 0, WIDE_SWIGLU = 1, WIDE_ROPE = 2, WIDE_RESID = 3 };
 struct WideParams {
   int tiles_per_seg, tiles;
   int kblocks, units_per_tile;
+  int kb;                   // K blocks per pipeline stage = unit of work: ranges are cut at multiples of 64 kb columns
   int splits;               // 0: equal ranges of all work (fix-up through scratch); > 0: K ranges per tile, one per group
   int groups, nrb;          // groups of nrb pairs (row blocks)
   int range[kMaxGroups + 1];   // splits == 0: first work unit of every group, and the end
@@ -187,7 +186,7 @@ constexpr int kChunk = 8;                               // activation rows a war
 constexpr int kBatch = kEpiThreads / 128 * kChunk;      // rows of a batch
 constexpr int kPark = kBatch * kTileM * 4;              // bytes
 
-template <int EPI>
+template <int EPI, int KB>
 __global__ void __launch_bounds__(kWideThreads, 1)
 tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -229,14 +228,14 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
   }
   const int stages = prm.stages, n = prm.n;
   const uint32_t b_tile = (uint32_t)n / 2 * 128, a_tile = kTileM * 128;         // one K block of each operand
-  const uint32_t stage_bytes = kUnitKb * (a_tile + b_tile);
+  const uint32_t stage_bytes = KB * (a_tile + b_tile);
   const unsigned long long limit_ns = prm.wait_limit_ns;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   float* const small_park = reinterpret_cast<float*>(smem + (size_t)stages * stage_bytes); // fused forms: [kBatch][128]
   const SegIter first = {range_begin(prm, group), range_begin(prm, group + 1), prm.units_per_tile};
   auto load_x = [&](int st, int u) {
     const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), lead);
-    tma_pair_3d(smem + (size_t)st * stage_bytes + kUnitKb * a_tile, &maps.x, 0, rb * n + (int)rank * (n / 2), u * kUnitKb, bar);
+    tma_pair_3d(smem + (size_t)st * stage_bytes + KB * a_tile, &maps.x, 0, rb * n + (int)rank * (n / 2), u * KB, bar);
   };
   // both CTAs' barriers and tensor memory exist behind this
   auto cluster_ready = [&]() {
@@ -260,8 +259,8 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
       const uint32_t bar = map_to_rank(smem_u32(&full_bar[st]), lead);
       uint8_t* dst = smem + (size_t)st * stage_bytes;
       if (rank == 0) mbar_expect_tx(&full_bar[st], 2 * stage_bytes + more);
-      if (EPI == WIDE_SWIGLU) tma_pair_4d(dst, &maps.w[0], 0, (lt * 2 + (int)rank) * (kTileM / 2), 0, u * kUnitKb, bar, wpol);
-      else tma_pair_3d(dst, &maps.w[seg], 0, (lt * 2 + (int)rank) * kTileM, u * kUnitKb, bar, wpol);
+      if (EPI == WIDE_SWIGLU) tma_pair_4d(dst, &maps.w[0], 0, (lt * 2 + (int)rank) * (kTileM / 2), 0, u * KB, bar, wpol);
+      else tma_pair_3d(dst, &maps.w[seg], 0, (lt * 2 + (int)rank) * kTileM, u * KB, bar, wpol);
     };
     // weights do not depend on the kernel before: fill the ring with them; warp 1 fetches those stages' activations
     if (prm.wait_first) pdl_wait();
@@ -326,8 +325,8 @@ tc_wide_kernel(const __grid_constant__ WideMaps maps, const WideParams prm) {
           if (leader) {                                  // K blocks past the end of K have arrived as zeros
             const uint32_t a_addr = smem_u32(smem + (size_t)st * stage_bytes);
 #pragma unroll
-            for (int kk = 0; kk < kUnitKb; ++kk) {
-              const uint64_t ad = umma_desc(a_addr + kk * a_tile), bd = umma_desc(a_addr + kUnitKb * a_tile + kk * b_tile);
+            for (int kk = 0; kk < KB; ++kk) {
+              const uint64_t ad = umma_desc(a_addr + kk * a_tile), bd = umma_desc(a_addr + KB * a_tile + kk * b_tile);
 #pragma unroll
               for (int k = 0; k < kTileK / kUmmaK; ++k)
                 umma_pair(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, u > sg.u0 || kk > 0 || k > 0 ? 1u : 0u);
@@ -668,11 +667,20 @@ int active_clusters(const TcGemm* g, const void* kernel, int ctas, size_t smem) 
   if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
   return n;
 }
-bool allow_smem(const void* kernel, size_t bytes) {
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess) return true;
+template <int EPI>
+bool allow_smem(size_t bytes) {
+  if (cudaFuncSetAttribute(tc_wide_kernel<EPI, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess &&
+      cudaFuncSetAttribute(tc_wide_kernel<EPI, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess)
+    return true;
   cudaGetLastError();
   return false;
 }
+// K blocks of a stage.  One, so that six are in flight, where a block's MMAs take longer than the step from one stage to the next (two
+// barrier waits, a commit, two copies) and K is long: 4 x 64 rows at 4096, 8 layers, 12 steps 28.4 ms with two (three stages), 27.9 with
+// one, a prompt of 300 tokens 1970 / 1910 us.  Two otherwise: trees of 70 / 96 / 128 nodes at 4096 with one block 8150 / 8230 / 8500 us
+// (8 layers, 6 steps), with two 7990 / 8090 / 8370, a prompt of 100 tokens 1400 / 1375; 8 x 64 rows at width 512 495 / 487 us a step, at
+// 1024 607 / 597, at 2048 (K = 5632 in the down projection) 801 / 805.
+int unit_kb(int in, int rows) { return rows <= 128 || in <= 2816 ? 2 : 1; }
 
 // What runs at a time, asked for by the first launch that may take the kernel (or by tc_wide_init): amph_project makes a plan set
 // per call, mostly for fewer rows, and needs the plain form only (16 rows: 14.7 us of host time per call when every plan set asked for
@@ -681,9 +689,9 @@ bool wide_available(TcGemm* g) {
   if (!g) return false;
   if (g->wide_pairs < 0) {
     g->wide_pairs = 0;
-    if ((size_t)g->max_smem >= kWideSmem + 7 * 1024 && allow_smem((const void*)tc_wide_kernel<WIDE_PLAIN>, kWideSmem) &&
-        allow_smem((const void*)tc_wide_kernel<WIDE_SWIGLU>, kWideSmem) && allow_smem((const void*)tc_wide_kernel<WIDE_ROPE>, kWideSmem)) {
-      const int clusters = active_clusters(g, (const void*)tc_wide_kernel<WIDE_ROPE>, 2, kWideSmem);
+    if ((size_t)g->max_smem >= kWideSmem + 7 * 1024 && allow_smem<WIDE_PLAIN>(kWideSmem) && allow_smem<WIDE_SWIGLU>(kWideSmem) &&
+        allow_smem<WIDE_ROPE>(kWideSmem)) {
+      const int clusters = active_clusters(g, (const void*)tc_wide_kernel<WIDE_ROPE, 1>, 2, kWideSmem);
       g->wide_pairs = clusters < g->sm_count / 2 ? clusters : g->sm_count / 2;
     }
   }
@@ -694,8 +702,8 @@ bool resid_available(TcGemm* g) {
   if (!wide_available(g)) return false;
   if (g->resid_clusters[0] == 0) {
     g->resid_clusters[0] = 1;
-    if (allow_smem((const void*)tc_wide_kernel<WIDE_RESID>, kResidSmem))
-      for (int s = 1; s <= 4; ++s) g->resid_clusters[s] = active_clusters(g, (const void*)tc_wide_kernel<WIDE_RESID>, 2 * s, kResidSmem);
+    if (allow_smem<WIDE_RESID>(kResidSmem))
+      for (int s = 1; s <= 4; ++s) g->resid_clusters[s] = active_clusters(g, (const void*)tc_wide_kernel<WIDE_RESID, 1>, 2 * s, kResidSmem);
   }
   return true;
 }
@@ -711,7 +719,8 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
   memset(prm, 0, sizeof *prm);
   prm->nrb = rows > 256 ? 2 : 1;
   prm->n = ((rows + prm->nrb - 1) / prm->nrb + 31) / 32 * 32;        // an M = 256 pair MMA takes N in steps of 32
-  const CUtensorMap* mx = g->get(g->xptr[xb], g->xrows[xb], in, prm->n / 2, kUnitKb);
+  const int kb = prm->kb = unit_kb(in, rows);
+  const CUtensorMap* mx = g->get(g->xptr[xb], g->xrows[xb], in, prm->n / 2, kb);
   if (!mx) return false;
   maps->x = *mx;
   prm->tmem_cols = 64;
@@ -719,7 +728,7 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
   prm->tiles_per_seg = tiles_per_seg;
   prm->tiles = n_seg * tiles_per_seg;
   prm->kblocks = in / kTileK;
-  prm->units_per_tile = (prm->kblocks + kUnitKb - 1) / kUnitKb;
+  prm->units_per_tile = (prm->kblocks + kb - 1) / kb;
   prm->splits = splits;
   prm->groups = g->wide_pairs / prm->nrb;
   const int units = prm->tiles * prm->units_per_tile;
@@ -728,13 +737,13 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
     prm->groups = prm->tiles * splits;
   } else {
     // at least 512 columns a group, unless there are more tiles than that; no more pairs than scratch
-    const int most = units * kUnitKb / 8 > prm->tiles ? units * kUnitKb / 8 : prm->tiles;
+    const int most = units * kb / 8 > prm->tiles ? units * kb / 8 : prm->tiles;
     if (prm->groups > most) prm->groups = most;
     const size_t per_group = (size_t)prm->nrb * 2 * prm->n * kTileM;
     if ((size_t)prm->groups > scratch_floats / per_group) prm->groups = (int)(scratch_floats / per_group);
     if (prm->groups < 1 || !scratch_end || !g->wide_flags || 2 * prm->groups * prm->nrb > kWideFlags) return false;
     // a cut within `snap` units of a tile's edge moves to the edge: the piece it would leave costs a whole epilogue (5-10 us
-    // when nothing runs above it) for a few units of 0.6 us
+    // when nothing runs above it) for a few K blocks of 0.3 us
     const int upt = prm->units_per_tile, share = units / prm->groups / 4, snap = share < upt / 8 ? share : upt / 8;
     for (int i = 0; i <= prm->groups; ++i) {
       int u = (int)((long long)i * units / prm->groups);
@@ -746,7 +755,7 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
     prm->scratch = scratch_end - (size_t)prm->groups * per_group;    // the buffer's end: its beginning may hold the result
   }
   prm->rows = rows;
-  const size_t stage = kUnitKb * ((size_t)kTileM * 128 + (size_t)prm->n / 2 * 128);
+  const size_t stage = kb * ((size_t)kTileM * 128 + (size_t)prm->n / 2 * 128);
   prm->stages = (int)(((EPI == WIDE_RESID ? kResidSmem : kWideSmem) - 1024 - out_bytes) / stage);
   if (prm->stages > kMaxStages) prm->stages = kMaxStages;
   prm->flags = g->wide_flags;
@@ -773,7 +782,7 @@ bool wide_run(const WideMaps& maps, const WideParams& prm, cudaStream_t st) {
   at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, tc_wide_kernel<EPI>, maps, prm) == cudaSuccess;
+  return cudaLaunchKernelEx(&cfg, prm.kb == 2 ? tc_wide_kernel<EPI, 2> : tc_wide_kernel<EPI, 1>, maps, prm) == cudaSuccess;
 }
 
 }  // namespace
@@ -793,7 +802,7 @@ void tc_wide_bind(TcGemm* g, float* scratch, size_t scratch_floats, int* flags) 
 bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out, int in, int rows, float* P, size_t p_floats,
                     int* splits_out, size_t* split_stride, cudaStream_t st) {
   if (out % 256 || in % kTileK || !wide_available(g)) return false;
-  const int tiles = n_seg * (out / 256), units = (in / kTileK + kUnitKb - 1) / kUnitKb;
+  const int tiles = n_seg * (out / 256);
   const size_t ld = (size_t)n_seg * out, stride = (size_t)rows * ld;
   if (stride > p_floats) return false;
   // Few tiles: the consumer adds the K ranges' sums (one per group).  Many: equal ranges of all the work, one sum.
@@ -801,7 +810,7 @@ bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   const int groups = g->wide_pairs / (rows > 256 ? 2 : 1);
   if (tiles * 2 <= groups || !g->wide_flags) {
     splits = groups / tiles;
-    if (splits > units * kUnitKb / 4) splits = units * kUnitKb / 4;            // at least four K blocks per pair
+    if (splits > in / kTileK / 4) splits = in / kTileK / 4;            // at least four K blocks per pair
     if (splits > 16) splits = 16;
     while (splits > 1 && splits * stride > p_floats) --splits;
     if (splits < 1) splits = 1;
@@ -813,7 +822,7 @@ bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   if (!wide_params<WIDE_PLAIN>(g, xb, n_seg, out / 256, in, rows, splits, P + end, end > used ? end - used : 0, &maps, &prm)) return false;
   for (int s = 0; s < n_seg; ++s) {
     if ((uintptr_t)w[s] & 15) return false;
-    const CUtensorMap* m = g->get(w[s], out, in, kTileM, kUnitKb);
+    const CUtensorMap* m = g->get(w[s], out, in, kTileM, prm.kb);
     if (!m) return false;
     maps.w[s] = *m;
   }
@@ -830,14 +839,14 @@ bool tc_wide_launch_resid(TcGemm* g, int xb, const void* w, int out, int in, int
                           cudaStream_t st) {
   if (!g || !w || !x || out % 256 || in % kTileK || ((uintptr_t)w & 15) || (gain && (!xn || !ss)) || !resid_available(g)) return false;
   // as many K ranges per tile as run at a time, at least four K blocks each
-  const int items = out / 256 * (rows > 256 ? 2 : 1), units = (in / kTileK + kUnitKb - 1) / kUnitKb;
+  const int items = out / 256 * (rows > 256 ? 2 : 1);
   int splits = 4;
-  while (splits > 1 && (g->resid_clusters[splits] < items || splits > units * kUnitKb / 4)) --splits;
+  while (splits > 1 && (g->resid_clusters[splits] < items || splits > in / kTileK / 4)) --splits;
   if (g->resid_clusters[splits] < 1) return false;
   WideMaps maps;
   WideParams prm;
   if (!wide_params<WIDE_RESID>(g, xb, 1, out / 256, in, rows, splits, nullptr, 0, &maps, &prm)) return false;
-  const CUtensorMap* m = g->get(w, out, in, kTileM, kUnitKb);
+  const CUtensorMap* m = g->get(w, out, in, kTileM, prm.kb);
   if (!m) return false;
   maps.w[0] = *m;
   prm.x = x;
@@ -855,7 +864,7 @@ bool tc_wide_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_
   WideParams prm;
   if (!wide_params<WIDE_SWIGLU>(g, xb, 1, f / 128, in, rows, 0, g->wide_scratch + g->wide_scratch_floats, g->wide_scratch_floats, &maps, &prm)) return false;
   const bool up_first = (const char*)w_up < (const char*)w_gate;
-  const CUtensorMap* m = g->get_wide_pair(up_first ? w_up : w_gate, up_first ? w_gate : w_up, f, in, kUnitKb);
+  const CUtensorMap* m = g->get_wide_pair(up_first ? w_up : w_gate, up_first ? w_gate : w_up, f, in, prm.kb);
   if (!m) return false;
   maps.w[0] = *m;
   prm.act = (__nv_bfloat16*)act;
@@ -875,7 +884,7 @@ bool tc_wide_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
   if (!wide_params<WIDE_ROPE>(g, xb, 3, d / 256, in, rows, 0, g->wide_scratch + g->wide_scratch_floats, g->wide_scratch_floats, &maps, &prm)) return false;
   const void* w[3] = {wq, wk, wv};
   for (int s = 0; s < 3; ++s) {
-    const CUtensorMap* m = g->get(w[s], d, in, kTileM, kUnitKb);
+    const CUtensorMap* m = g->get(w[s], d, in, kTileM, prm.kb);
     if (!m) return false;
     maps.w[s] = *m;
   }
