@@ -36,10 +36,15 @@ def _compare(a, b, rel):
     for x, y in zip(a, b):
         assert bool(torch.isfinite(x).all())
         assert float((x - y).norm() / y.norm()) <= rel
+        # a tile that went wrong may be a fraction of a per cent of a tensor's norm: twice the bound for every element, in units of the
+        # largest one (the pair projection's tests)
+        assert float((x - y).abs().max()) <= 2 * rel * max(1.0, float(y.abs().max()))
 
 
-# 11008 = 137 tiles of 80 and one of 48 (rows above 16), 2432 = 101 of 24 and one of 8; width 2176: no residual form
-@pytest.mark.parametrize("heads,dh,ffn", [(8, 64, 1408), (4, 128, 2432), (10, 128, 3456), (4, 128, 11008), (17, 128, 1408)])
+# 11008 = 137 tiles of 80 and one of 48 (rows above 16), 2432 = 101 of 24 and one of 8; width 2176: no residual form; widths 576 and 320:
+# an odd number of K blocks, the last stage of two has one that does not exist
+@pytest.mark.parametrize("heads,dh,ffn", [(8, 64, 1408), (4, 128, 2432), (10, 128, 3456), (4, 128, 11008), (17, 128, 1408), (9, 64, 1152),
+                                          (5, 64, 1408)])
 @pytest.mark.parametrize("n,nodes", [(1, 5), (16, 16), (17, 33), (48, 43), (63, 50), (64, 64)])
 def test_bf16_forms_against_the_separate_kernels(heads, dh, ffn, n, nodes):
     shape = inputs.get_shape("small_bf16").with_(d_model=heads * dh, n_heads=heads, head_dim=dh, d_ffn=ffn, n_nodes=nodes, topk=(16, 16, 16, 16))
@@ -48,6 +53,25 @@ def test_bf16_forms_against_the_separate_kernels(heads, dh, ffn, n, nodes):
     # 512: no residual update in an epilogue.  Sums in another order, roundings to bf16 (2^-8) in the same places; three layers of
     # unit gain, as in the tests of the projection of many rows
     _compare(_outputs(shape, w, prompts, 0), _outputs(shape, w, prompts, 4 | 16 | 512), 1e-2)
+
+
+@pytest.mark.parametrize("n_nodes", [16, 43, 64, 100])
+def test_up_matrix_below_the_gate_matrix(n_nodes):
+    """Gate and up come through one tensor map that begins at the lower of the two: the same bits whichever that is."""
+    shape = inputs.get_shape("small_bf16").with_(n_nodes=n_nodes, topk=(16, 16, 16, 16))
+    w = inputs.make_weights(shape, seed=0, device="cuda:0", init="fan_in")
+    prompts = [inputs.make_prompt(shape, seed=2).tolist()]
+    outs = []
+    for first, second in (("w_gate", "w_up"), ("w_up", "w_gate")):
+        v = dict(w)
+        for name in [k for k in w if k.endswith("w_gate")]:
+            pre = name[: -len("w_gate")]
+            both = torch.empty(2, *w[name].shape, dtype=w[name].dtype, device="cuda:0")
+            both[0].copy_(w[pre + first])
+            both[1].copy_(w[pre + second])
+            v[pre + first], v[pre + second] = both[0], both[1]
+        outs.append(_outputs(shape, v, prompts, 0))
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
 
 
 # two accumulators (the sums of two K ranges, 512 and 1280 wide), and shapes that decline (more K ranges, an odd number of K blocks)
