@@ -46,15 +46,19 @@ def algorithmic_bytes(shape, ctx_len: int) -> int:
 # DRAM traffic of the projection kernel per weight byte, from its ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum of one launch over the weight bytes that launch streams).  Traffic is proportional to the weight
 # bytes of a launch, so the step's average launch is scaled by this ratio.  The counters belong to one version of the
-# kernel: the digest below is that of the kernel source they were taken with, and the field is null for any other source.
+# kernels: the digest below is that of the sources they were taken with (both projection kernels of up to 64 rows, and what they
+# share), and the field is null for any other source.
 NCU_TRAFFIC_PER_WEIGHT_BYTE = 1.03
 NCU_KERNEL_SOURCE_SHA256_16 = "970b67f071aaf755"
 
 
 def kernel_source_digest() -> str:
     import hashlib
-    with open(os.path.join(ROOT, "paper_2406_13170_b200", "csrc", "gemm_tc.cu"), "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for name in ("gemm_tc.cu", "gemm_rows.cu", "gemm_tc_common.cuh"):
+        with open(os.path.join(ROOT, "paper_2406_13170_b200", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def ncu_traffic(weight_bytes_per_launch: float):
@@ -431,35 +435,39 @@ def main():
     # kernels launched per step: projections + the fixed schedule around them (counted from the schedule)
     # per layer: q/k/v projection, rotary + cache write, attention (its KV splits merge in-launch on bf16 unless the
     # separate-merge flag is set), output projection, residual, gate/up projection, SwiGLU, down projection, residual
-    # passes of more than 64 rows: the pair projection, unless the context keeps one order of sums
-    pairs = uses_tc and not args.flags & 512 and not getattr(shape, "lm_rank", 0)
-    # small models: the residual updates are in the projections' epilogues whatever the rows
-    short = shape.d_model <= 2048 and (shape.dtype == "fp32" or (pairs and shape.d_ffn <= 2048))
+    # The forms' conditions are those of the library's dispatch (148 SMs), for widths that are multiples of 256.
+    d, F, flags, f32 = shape.d_model, shape.d_ffn, args.flags, shape.dtype == "fp32"
+    one_order = bool(flags & 512 or getattr(shape, "lm_rank", 0))    # bf16: no pair projection above 64 rows
+
+    def resid_fused(rows, k):                                    # in the epilogue of the output (k = d) or the down projection (k = F)
+        if f32:
+            return not one_order and d <= 2048 and -(-d // 8) * -(-rows // 16) <= 296
+        return uses_tc and not one_order and (rows > 64 or (d <= 1536 and k <= 2048))
+
+    def swiglu_fused(rows):
+        if flags & 16 or not (f32 or uses_tc):
+            return False
+        if f32 or rows <= 64 or not one_order:
+            return True
+        splits = max(1, min(259 // (2 * F // 128), d // 64 // 4, 16))     # at most two accumulators, 1.5 tiles of 64 rows per SM
+        return rows <= 128 and splits <= 2 and F % 128 == 0 and d // 64 % splits == 0 and 2 * (F // 64) <= 3 * 148
+
+    def rope_fused(rows):
+        return not flags & 4 and (f32 or (uses_tc and (rows <= 64 or not one_order)))
 
     def layer_launches(rows, keys):
-        n = 10 if (shape.dtype == "bf16" and args.flags & 8) else 9
-        if rows <= 64 or not uses_tc:
-            n -= 2 * short
-        if shape.dtype == "fp32":
-            return n - (not args.flags & 16) - (not args.flags & 4)
-        if not uses_tc:
-            return n
-        if rows <= 64 or pairs:
-            n -= (not args.flags & 16) + (not args.flags & 4)    # SwiGLU; rotary + cache write: in the projections' epilogues
-        if rows > 64:
-            n -= 2 * pairs                                       # residual updates in the projections' epilogues
-            n -= not pairs and rows <= 128 and not args.flags & 16   # one order of sums: SwiGLU in the projection's epilogue
-        elif not (args.flags & (4 | 256)) and 4 * keys * shape.d_model <= 20 << 20:
+        merge = keys > 128 if f32 else bool(flags & 8)
+        n = 9 + merge - rope_fused(rows) - swiglu_fused(rows) - resid_fused(rows, d) - resid_fused(rows, F)
+        if uses_tc and rows <= 64 and not flags & (4 | 256) and 4 * keys * d <= 20 << 20:
             n += 1                                               # the gate / up prefetch helper on the forked stream
         return n
 
     def step_launches(keys):                                     # keys: the library's bound of the committed context
-        draft = shape.n_sal * (3 + layer_launches(1, keys)) + 1 + 2 + shape.aeb_layers * 4 + 3   # ... + (vocabulary projection, top-k slices, merge and tree)
+        draft = shape.n_sal * (3 + layer_launches(16, keys)) + 1 + 2 + shape.aeb_layers * 4 + 3   # ... + (vocabulary projection, top-k slices, merge and tree)
         if getattr(shape, "lm_rank", 0):
             draft += 2                                           # low-rank heads: one more projection + a gather
         verify = 1 + shape.n_layers * layer_launches(N, keys + N) + 3        # row set-up, ..., head projection, argmax slices, merge
-        if N > 64 or short:
-            verify += pairs or short                                     # the last layer's update also takes the final norm: a kernel of its own
+        verify += resid_fused(N, F)                              # the last layer's update also takes the final norm: a kernel of its own
         return draft + verify + 1                                # ... + acceptance
 
     line["gpu_launches"] = sum(step_launches(C_start + i * (K + 1)) for i in range(steps))

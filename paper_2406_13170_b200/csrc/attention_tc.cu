@@ -582,51 +582,48 @@ tree_attn_tc_kernel(const __grid_constant__ AttnMaps<NG> maps, const __grid_cons
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
-  if (MERGE && S == 1) {
-  } else if constexpr (MERGE) {
-    // Rows [slots * j, slots * (j + 1)) are merged by CTA j of the cluster: everybody's block j goes there in one bulk copy.
-    const uint8_t* parts;                              // S blocks, one per split
-    {
-      uint8_t* recv = smem + kRecvAt;
+  if constexpr (MERGE) {
+    if (S > 1) {                                       // (of a single key range the rows are out)
+      // Rows [slots * j, slots * (j + 1)) are merged by CTA j of the cluster: everybody's block j goes there in one bulk copy.
+      uint8_t* const parts = smem + kRecvAt;           // S blocks, one per split
       __syncwarp();
       cluster_wait();                                  // every CTA of the cluster is done with its operands
       if (warp == 0) {
         if (lane == 0) mbar_expect_tx(&recv_full, (uint32_t)S * block_bytes);
         __syncwarp();
         if (lane < S)
-          bulk_to_peer(peer_smem(smem_u32(recv + (size_t)split * block_bytes), (uint32_t)lane), smem + (size_t)lane * block_bytes, block_bytes,
+          bulk_to_peer(peer_smem(smem_u32(parts + (size_t)split * block_bytes), (uint32_t)lane), smem + (size_t)lane * block_bytes, block_bytes,
                        peer_smem(smem_u32(&recv_full), (uint32_t)lane));
       }
       mbar_wait(&recv_full, 0, &abort_flag);
       __syncwarp();
       cluster_arrive();                                // this CTA has received everything
-      parts = recv;
-    }
-    for (int i = threadIdx.x; i < slots * (DH / 4); i += kThreads) {
-      const int slot = i / (DH / 4), col = (i - slot * (DH / 4)) * 4, r = split * slots + slot, gr = rb * kRows + r;
-      if (r >= kRows || gr >= prm.rows_cap) continue;
-      float M = -INFINITY;
-      for (int s = 0; s < S; ++s) M = fmaxf(M, *reinterpret_cast<const float*>(parts + (size_t)s * block_bytes + (slots * DH + slot * 4) * 4));
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      float d[8];                                      // at most eight splits
+      for (int i = threadIdx.x; i < slots * (DH / 4); i += kThreads) {
+        const int slot = i / (DH / 4), col = (i - slot * (DH / 4)) * 4, r = split * slots + slot, gr = rb * kRows + r;
+        if (r >= kRows || gr >= prm.rows_cap) continue;
+        float M = -INFINITY;
+        for (int s = 0; s < S; ++s) M = fmaxf(M, *reinterpret_cast<const float*>(parts + (size_t)s * block_bytes + (slots * DH + slot * 4) * 4));
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        float d[8];                                      // at most eight splits
 #pragma unroll
-      for (int s = 0; s < 8; ++s) {
-        d[s] = 0.f;
-        if (s >= S) continue;
-        const float* blk = reinterpret_cast<const float*>(parts + (size_t)s * block_bytes);
-        const float2 ml = *reinterpret_cast<const float2*>(blk + slots * DH + slot * 4);
-        const float4 v = *reinterpret_cast<const float4*>(blk + slot * DH + col);
-        const float w = ml.x == -INFINITY ? 0.f : expf(ml.x - M);
-        d[s] = __fmul_rn(ml.y, w);
-        a.x += v.x * w; a.y += v.y * w; a.z += v.z * w; a.w += v.w * w;
+        for (int s = 0; s < 8; ++s) {
+          d[s] = 0.f;
+          if (s >= S) continue;
+          const float* blk = reinterpret_cast<const float*>(parts + (size_t)s * block_bytes);
+          const float2 ml = *reinterpret_cast<const float2*>(blk + slots * DH + slot * 4);
+          const float4 v = *reinterpret_cast<const float4*>(blk + slot * DH + col);
+          const float w = ml.x == -INFINITY ? 0.f : expf(ml.x - M);
+          d[s] = __fmul_rn(ml.y, w);
+          a.x += v.x * w; a.y += v.y * w; a.z += v.z * w; a.w += v.w * w;
+        }
+        const float den = ((d[0] + d[4]) + (d[2] + d[6])) + ((d[1] + d[5]) + (d[3] + d[7]));
+        const float inv = den > 0.f ? 1.0f / den : 0.f;
+        *reinterpret_cast<uint2*>(prm.out + (size_t)(row_base + gr) * prm.n_heads * DH + h * DH + col) =
+            make_uint2(pack_bf16(a.x * inv, a.y * inv), pack_bf16(a.z * inv, a.w * inv));
       }
-      const float den = ((d[0] + d[4]) + (d[2] + d[6])) + ((d[1] + d[5]) + (d[3] + d[7]));
-      const float inv = den > 0.f ? 1.0f / den : 0.f;
-      *reinterpret_cast<uint2*>(prm.out + (size_t)(row_base + gr) * prm.n_heads * DH + h * DH + col) =
-          make_uint2(pack_bf16(a.x * inv, a.y * inv), pack_bf16(a.z * inv, a.w * inv));
+      __syncwarp();
+      cluster_wait();                                    // nobody leaves while a copy may still read its shared memory
     }
-    __syncwarp();
-    cluster_wait();                                    // nobody leaves while a copy may still read its shared memory
   } else {
     if (warp >= 2) {
       l_a = sum_s[row_a];

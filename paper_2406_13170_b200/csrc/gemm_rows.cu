@@ -259,143 +259,143 @@ tc_rows_kernel(const __grid_constant__ RowsMaps maps, const RowsParams prm) {
     };
     const bool two = M == 128 && prm.kb_cut < prm.kblocks;
     for (int part = 0; part < M / 64; ++part) {
-    const int ra = quarter * (M / 4) + part * 16 + (lane >> 2), rb = ra + 8;
-    const bool la = ra < prm.rows, lb = rb < prm.rows;
-    const uint32_t taddr = tmem_base_slot + ((uint32_t)(quarter * 32 + part * 16) << 16);
-    // the second accumulator's sums join the first one's, in the order in which split-K sums are added
-    auto join = [&](uint32_t at, float (*v)[4], int c0) {
-      if constexpr (M == 128) {
-        if (!two) return;
-        float w[U][4];
+      const int ra = quarter * (M / 4) + part * 16 + (lane >> 2), rb = ra + 8;
+      const bool la = ra < prm.rows, lb = rb < prm.rows;
+      const uint32_t taddr = tmem_base_slot + ((uint32_t)(quarter * 32 + part * 16) << 16);
+      // the second accumulator's sums join the first one's, in the order in which split-K sums are added
+      auto join = [&](uint32_t at, float (*v)[4], int c0) {
+        if constexpr (M == 128) {
+          if (!two) return;
+          float w[U][4];
 #pragma unroll
-        for (int j = 0; j < U; ++j)
-          if (c0 + 8 * j < prm.half) ld_frag8(at + (uint32_t)prm.n + c0 + 8 * j, w[j]);
-        ld_wait();
+          for (int j = 0; j < U; ++j)
+            if (c0 + 8 * j < prm.half) ld_frag8(at + (uint32_t)prm.n + c0 + 8 * j, w[j]);
+          ld_wait();
 #pragma unroll
-        for (int j = 0; j < U; ++j)
-          if (c0 + 8 * j < prm.half) { v[j][0] += w[j][0]; v[j][1] += w[j][1]; v[j][2] += w[j][2]; v[j][3] += w[j][3]; }
-      }
-    };
-    if constexpr (EPI == ROWS_SWIGLU) {
-      const float sa = la ? inv_s[ra] : 0.f, sb = lb ? inv_s[rb] : 0.f;
-      const bool ok = sums_ready();
-      const uint32_t tg = taddr + (prm.up_first ? (uint32_t)prm.half : 0u), tu = taddr + (prm.up_first ? 0u : (uint32_t)prm.half);
-      __nv_bfloat16* const pa = prm.act + (size_t)ra * prm.f + row0 + cq;
-      __nv_bfloat16* const pb = prm.act + (size_t)rb * prm.f + row0 + cq;
-      // M = 128 stands for split-K sums and swiglu_kernel, whose exponential and division it keeps
-      auto glu = [](float g, float u, float sc) {
-        const float t = g * sc;
-        if constexpr (M == 128) return t / (1.0f + expf(-t)) * (u * sc);
-        else return __fdividef(t, 1.0f + __expf(-t)) * (u * sc);
+          for (int j = 0; j < U; ++j)
+            if (c0 + 8 * j < prm.half) { v[j][0] += w[j][0]; v[j][1] += w[j][1]; v[j][2] += w[j][2]; v[j][3] += w[j][3]; }
+        }
       };
-      for (int c0 = 0; c0 < prm.half; c0 += 8 * U) {
-        float g[U][4], u[U][4];
+      if constexpr (EPI == ROWS_SWIGLU) {
+        const float sa = la ? inv_s[ra] : 0.f, sb = lb ? inv_s[rb] : 0.f;
+        const bool ok = sums_ready();
+        const uint32_t tg = taddr + (prm.up_first ? (uint32_t)prm.half : 0u), tu = taddr + (prm.up_first ? 0u : (uint32_t)prm.half);
+        __nv_bfloat16* const pa = prm.act + (size_t)ra * prm.f + row0 + cq;
+        __nv_bfloat16* const pb = prm.act + (size_t)rb * prm.f + row0 + cq;
+        // M = 128 stands for split-K sums and swiglu_kernel, whose exponential and division it keeps
+        auto glu = [](float g, float u, float sc) {
+          const float t = g * sc;
+          if constexpr (M == 128) return t / (1.0f + expf(-t)) * (u * sc);
+          else return __fdividef(t, 1.0f + __expf(-t)) * (u * sc);
+        };
+        for (int c0 = 0; c0 < prm.half; c0 += 8 * U) {
+          float g[U][4], u[U][4];
 #pragma unroll
-        for (int j = 0; j < U; ++j)
-          if (c0 + 8 * j < prm.half) { ld_frag8(tg + c0 + 8 * j, g[j]); ld_frag8(tu + c0 + 8 * j, u[j]); }
-        ld_wait();
-        join(tg, g, c0);
-        join(tu, u, c0);
+          for (int j = 0; j < U; ++j)
+            if (c0 + 8 * j < prm.half) { ld_frag8(tg + c0 + 8 * j, g[j]); ld_frag8(tu + c0 + 8 * j, u[j]); }
+          ld_wait();
+          join(tg, g, c0);
+          join(tu, u, c0);
 #pragma unroll
-        for (int j = 0; j < U; ++j) {
-          const int c = c0 + 8 * j;
-          if (c < prm.half && row0 + c < prm.f) {
-            const uint32_t ya = ok ? pack2(glu(g[j][0], u[j][0], sa), glu(g[j][1], u[j][1], sa)) : 0u;
-            const uint32_t yb = ok ? pack2(glu(g[j][2], u[j][2], sb), glu(g[j][3], u[j][3], sb)) : 0u;
-            if (la) *reinterpret_cast<uint32_t*>(pa + c) = ya;
-            if (lb) *reinterpret_cast<uint32_t*>(pb + c) = yb;
+          for (int j = 0; j < U; ++j) {
+            const int c = c0 + 8 * j;
+            if (c < prm.half && row0 + c < prm.f) {
+              const uint32_t ya = ok ? pack2(glu(g[j][0], u[j][0], sa), glu(g[j][1], u[j][1], sa)) : 0u;
+              const uint32_t yb = ok ? pack2(glu(g[j][2], u[j][2], sb), glu(g[j][3], u[j][3], sb)) : 0u;
+              if (la) *reinterpret_cast<uint32_t*>(pa + c) = ya;
+              if (lb) *reinterpret_cast<uint32_t*>(pb + c) = yb;
+            }
           }
         }
-      }
-    } else if constexpr (EPI == ROWS_ROPE) {
-      const float sa = la ? inv_s[ra] : 0.f, sb = lb ? inv_s[rb] : 0.f;
-      const int hdim = prm.dh >> 1, h = row0 / prm.dh, i0 = row0 - h * prm.dh + cq;      // head, this thread's first pair
-      __nv_bfloat16 *da = nullptr, *db = nullptr;
-      if (seg == 0) {
-        da = prm.q + (size_t)ra * prm.n_heads * prm.dh + h * prm.dh + i0;
-        db = prm.q + (size_t)rb * prm.n_heads * prm.dh + h * prm.dh + i0;
-        if (!la) da = nullptr;
-        if (!lb) db = nullptr;
+      } else if constexpr (EPI == ROWS_ROPE) {
+        const float sa = la ? inv_s[ra] : 0.f, sb = lb ? inv_s[rb] : 0.f;
+        const int hdim = prm.dh >> 1, h = row0 / prm.dh, i0 = row0 - h * prm.dh + cq;      // head, this thread's first pair
+        __nv_bfloat16 *da = nullptr, *db = nullptr;
+        if (seg == 0) {
+          da = prm.q + (size_t)ra * prm.n_heads * prm.dh + h * prm.dh + i0;
+          db = prm.q + (size_t)rb * prm.n_heads * prm.dh + h * prm.dh + i0;
+          if (!la) da = nullptr;
+          if (!lb) db = nullptr;
+        } else {
+          __nv_bfloat16* const cache = (seg == 1 ? prm.kc : prm.vc) + (size_t)h * prm.max_ctx * prm.dh + i0;
+          const int n_rows = prm.meta->n_rows;
+          const int pa = la && ra < n_rows ? prm.meta->slot[ra] : -1, pb = lb && rb < n_rows ? prm.meta->slot[rb] : -1;
+          if (pa >= 0 && pa < prm.max_ctx) da = cache + (size_t)pa * prm.dh;
+          if (pb >= 0 && pb < prm.max_ctx) db = cache + (size_t)pb * prm.dh;
+        }
+        const float2* const ta = prm.rope + (size_t)ra * hdim + i0;
+        const float2* const tb = prm.rope + (size_t)rb * hdim + i0;
+        const float4 unit = make_float4(1.f, 0.f, 1.f, 0.f);
+        const bool ok = sums_ready();
+        for (int c0 = 0; c0 < prm.half; c0 += 8 * U) {
+          float lo[U][4], hi[U][4];
+          float4 ca[U], cb[U];
+#pragma unroll
+          for (int j = 0; j < U; ++j) {
+            const int c = c0 + 8 * j;
+            if (c < prm.half) { ld_frag8(taddr + c, lo[j]); ld_frag8(taddr + prm.half + c, hi[j]); }
+            ca[j] = seg < 2 && la && c < prm.half ? *reinterpret_cast<const float4*>(ta + c) : unit;       // (cos, sin) of two pairs
+            cb[j] = seg < 2 && lb && c < prm.half ? *reinterpret_cast<const float4*>(tb + c) : unit;
+          }
+          ld_wait();
+#pragma unroll
+          for (int j = 0; j < U; ++j) {
+            const int c = c0 + 8 * j;
+            if (c >= prm.half) continue;
+            auto put = [&](__nv_bfloat16* dst, float a0, float a1, float b0, float b1, const float4& cs, float sc) {
+              if (dst == nullptr) return;
+              if (!ok) { a0 = a1 = b0 = b1 = 0.f; }
+              a0 *= sc; a1 *= sc; b0 *= sc; b1 *= sc;
+              const uint32_t l = seg < 2 ? pack2(a0 * cs.x - b0 * cs.y, a1 * cs.z - b1 * cs.w) : pack2(a0, a1);
+              const uint32_t u = seg < 2 ? pack2(b0 * cs.x + a0 * cs.y, b1 * cs.z + a1 * cs.w) : pack2(b0, b1);
+              *reinterpret_cast<uint32_t*>(dst + c) = l;
+              *reinterpret_cast<uint32_t*>(dst + hdim + c) = u;
+            };
+            put(da, lo[j][0], lo[j][1], hi[j][0], hi[j][1], ca[j], sa);
+            put(db, lo[j][2], lo[j][3], hi[j][2], hi[j][3], cb[j], sb);
+          }
+        }
       } else {
-        __nv_bfloat16* const cache = (seg == 1 ? prm.kc : prm.vc) + (size_t)h * prm.max_ctx * prm.dh + i0;
-        const int n_rows = prm.meta->n_rows;
-        const int pa = la && ra < n_rows ? prm.meta->slot[ra] : -1, pb = lb && rb < n_rows ? prm.meta->slot[rb] : -1;
-        if (pa >= 0 && pa < prm.max_ctx) da = cache + (size_t)pa * prm.dh;
-        if (pb >= 0 && pb < prm.max_ctx) db = cache + (size_t)pb * prm.dh;
-      }
-      const float2* const ta = prm.rope + (size_t)ra * hdim + i0;
-      const float2* const tb = prm.rope + (size_t)rb * hdim + i0;
-      const float4 unit = make_float4(1.f, 0.f, 1.f, 0.f);
-      const bool ok = sums_ready();
-      for (int c0 = 0; c0 < prm.half; c0 += 8 * U) {
-        float lo[U][4], hi[U][4];
-        float4 ca[U], cb[U];
+        // residual update; the tile has at most 8 U features, their old values are fetched under the main loop
+        const int f0 = row0 + cq;
+        float* const xa = prm.x + (size_t)ra * prm.out + f0;
+        float* const xb = prm.x + (size_t)rb * prm.out + f0;
+        float2 oa[U], ob[U], gn[U];
 #pragma unroll
         for (int j = 0; j < U; ++j) {
-          const int c = c0 + 8 * j;
-          if (c < prm.half) { ld_frag8(taddr + c, lo[j]); ld_frag8(taddr + prm.half + c, hi[j]); }
-          ca[j] = seg < 2 && la && c < prm.half ? *reinterpret_cast<const float4*>(ta + c) : unit;       // (cos, sin) of two pairs
-          cb[j] = seg < 2 && lb && c < prm.half ? *reinterpret_cast<const float4*>(tb + c) : unit;
+          oa[j] = ob[j] = gn[j] = make_float2(0.f, 0.f);
+          if (8 * j >= prm.half) continue;
+          if (la) oa[j] = *reinterpret_cast<const float2*>(xa + 8 * j);
+          if (lb) ob[j] = *reinterpret_cast<const float2*>(xb + 8 * j);
+          if (prm.gain != nullptr) gn[j] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(prm.gain + f0 + 8 * j));
         }
+        const bool ok = sums_ready();
+        float v[U][4];
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+          if (8 * j < prm.half) ld_frag8(taddr + 8 * j, v[j]);
         ld_wait();
+        float qa = 0.f, qb = 0.f;
 #pragma unroll
         for (int j = 0; j < U; ++j) {
-          const int c = c0 + 8 * j;
-          if (c >= prm.half) continue;
-          auto put = [&](__nv_bfloat16* dst, float a0, float a1, float b0, float b1, const float4& cs, float sc) {
-            if (dst == nullptr) return;
-            if (!ok) { a0 = a1 = b0 = b1 = 0.f; }
-            a0 *= sc; a1 *= sc; b0 *= sc; b1 *= sc;
-            const uint32_t l = seg < 2 ? pack2(a0 * cs.x - b0 * cs.y, a1 * cs.z - b1 * cs.w) : pack2(a0, a1);
-            const uint32_t u = seg < 2 ? pack2(b0 * cs.x + a0 * cs.y, b1 * cs.z + a1 * cs.w) : pack2(b0, b1);
-            *reinterpret_cast<uint32_t*>(dst + c) = l;
-            *reinterpret_cast<uint32_t*>(dst + hdim + c) = u;
-          };
-          put(da, lo[j][0], lo[j][1], hi[j][0], hi[j][1], ca[j], sa);
-          put(db, lo[j][2], lo[j][3], hi[j][2], hi[j][3], cb[j], sb);
+          if (8 * j >= prm.half) continue;
+          if (!ok) v[j][0] = v[j][1] = v[j][2] = v[j][3] = 0.f;
+          const float a0 = oa[j].x + v[j][0], a1 = oa[j].y + v[j][1], b0 = ob[j].x + v[j][2], b1 = ob[j].y + v[j][3];
+          if (la) *reinterpret_cast<float2*>(xa + 8 * j) = make_float2(a0, a1);
+          if (lb) *reinterpret_cast<float2*>(xb + 8 * j) = make_float2(b0, b1);
+          if (prm.gain == nullptr) continue;
+          if (la) *reinterpret_cast<uint32_t*>(prm.xn + (size_t)ra * prm.out + f0 + 8 * j) = pack2(gn[j].x * a0, gn[j].y * a1);
+          if (lb) *reinterpret_cast<uint32_t*>(prm.xn + (size_t)rb * prm.out + f0 + 8 * j) = pack2(gn[j].x * b0, gn[j].y * b1);
+          qa += a0 * a0 + a1 * a1;
+          qb += b0 * b0 + b1 * b1;
+        }
+        if (prm.gain != nullptr) {
+          qa += __shfl_xor_sync(0xffffffffu, qa, 1); qa += __shfl_xor_sync(0xffffffffu, qa, 2);
+          qb += __shfl_xor_sync(0xffffffffu, qb, 1); qb += __shfl_xor_sync(0xffffffffu, qb, 2);
+          if ((lane & 3) == 0 && la) prm.ss[(size_t)ra * prm.tiles_per_seg + lt] = qa;
+          if ((lane & 3) == 0 && lb) prm.ss[(size_t)rb * prm.tiles_per_seg + lt] = qb;
         }
       }
-    } else {
-      // residual update; the tile has at most 8 U features, their old values are fetched under the main loop
-      const int f0 = row0 + cq;
-      float* const xa = prm.x + (size_t)ra * prm.out + f0;
-      float* const xb = prm.x + (size_t)rb * prm.out + f0;
-      float2 oa[U], ob[U], gn[U];
-#pragma unroll
-      for (int j = 0; j < U; ++j) {
-        oa[j] = ob[j] = gn[j] = make_float2(0.f, 0.f);
-        if (8 * j >= prm.half) continue;
-        if (la) oa[j] = *reinterpret_cast<const float2*>(xa + 8 * j);
-        if (lb) ob[j] = *reinterpret_cast<const float2*>(xb + 8 * j);
-        if (prm.gain != nullptr) gn[j] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(prm.gain + f0 + 8 * j));
-      }
-      const bool ok = sums_ready();
-      float v[U][4];
-#pragma unroll
-      for (int j = 0; j < U; ++j)
-        if (8 * j < prm.half) ld_frag8(taddr + 8 * j, v[j]);
-      ld_wait();
-      float qa = 0.f, qb = 0.f;
-#pragma unroll
-      for (int j = 0; j < U; ++j) {
-        if (8 * j >= prm.half) continue;
-        if (!ok) v[j][0] = v[j][1] = v[j][2] = v[j][3] = 0.f;
-        const float a0 = oa[j].x + v[j][0], a1 = oa[j].y + v[j][1], b0 = ob[j].x + v[j][2], b1 = ob[j].y + v[j][3];
-        if (la) *reinterpret_cast<float2*>(xa + 8 * j) = make_float2(a0, a1);
-        if (lb) *reinterpret_cast<float2*>(xb + 8 * j) = make_float2(b0, b1);
-        if (prm.gain == nullptr) continue;
-        if (la) *reinterpret_cast<uint32_t*>(prm.xn + (size_t)ra * prm.out + f0 + 8 * j) = pack2(gn[j].x * a0, gn[j].y * a1);
-        if (lb) *reinterpret_cast<uint32_t*>(prm.xn + (size_t)rb * prm.out + f0 + 8 * j) = pack2(gn[j].x * b0, gn[j].y * b1);
-        qa += a0 * a0 + a1 * a1;
-        qb += b0 * b0 + b1 * b1;
-      }
-      if (prm.gain != nullptr) {
-        qa += __shfl_xor_sync(0xffffffffu, qa, 1); qa += __shfl_xor_sync(0xffffffffu, qa, 2);
-        qb += __shfl_xor_sync(0xffffffffu, qb, 1); qb += __shfl_xor_sync(0xffffffffu, qb, 2);
-        if ((lane & 3) == 0 && la) prm.ss[(size_t)ra * prm.tiles_per_seg + lt] = qa;
-        if ((lane & 3) == 0 && lb) prm.ss[(size_t)rb * prm.tiles_per_seg + lt] = qb;
-      }
-    }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

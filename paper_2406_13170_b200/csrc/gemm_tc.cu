@@ -607,7 +607,7 @@ bool tc_gemm_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
   memset(&pack, 0, sizeof pack);
   const void* w[3] = {wq, wk, wv};
   for (int s = 0; s < 3; ++s) {
-    const CUtensorMap* m = g->get_rope(w[s], d, in, dh / 2, ks);
+    const CUtensorMap* m = g->get_halves(w[s], (uint64_t)(dh / 2) * in * 2, d, in, 32, ks);
     if (!m) return false;
     pack.w[s] = *m;
   }

@@ -131,47 +131,9 @@ struct TcGemm {
     return &(pair_cache[key] = m);
   }
 
-  // A [rows, cols] matrix as (column, row, half, K block) with the half `half_rows` rows apart: a box is 32 rows of
-  // both halves, i.e. 32 rotation pairs of one head, over box_kb K blocks.
-  std::map<std::tuple<const void*, int, int, int, int>, CUtensorMap> rope_cache;
-  const CUtensorMap* get_rope(const void* ptr, int rows, int cols, int half_rows, int box_kb) {
-    auto key = std::make_tuple(ptr, rows, cols, half_rows, box_kb);
-    auto it = rope_cache.find(key);
-    if (it != rope_cache.end()) return &it->second;
-    CUtensorMap m;
-    const cuuint64_t dims[4] = {(cuuint64_t)tc::kTileK, (cuuint64_t)rows, 2, (cuuint64_t)cols / tc::kTileK};
-    const cuuint64_t strides[3] = {(cuuint64_t)cols * 2, (cuuint64_t)half_rows * cols * 2, (cuuint64_t)tc::kTileK * 2};
-    const cuuint32_t box[4] = {(cuuint32_t)tc::kTileK, 32, 2, (cuuint32_t)box_kb};
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
-    const CUresult r = encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return nullptr;
-    return &(rope_cache[key] = m);
-  }
-
-  // The same for the pair kernel (gemm_wide.cu), as (column, row, matrix, K block): per K block, 64 rows of the lower matrix
-  // are followed by 64 of the upper one.
-  const CUtensorMap* get_wide_pair(const void* lo, const void* hi, int rows, int cols, int box_kb) {
-    auto key = std::make_tuple(lo, hi, rows, cols, -box_kb);
-    auto it = pair_cache.find(key);
-    if (it != pair_cache.end()) return &it->second;
-    const uint64_t gap = (uint64_t)((const char*)hi - (const char*)lo);
-    if (gap == 0 || (gap & 15) || gap >= (1ull << 40)) return nullptr;
-    CUtensorMap m;
-    const cuuint64_t dims[4] = {(cuuint64_t)tc::kTileK, (cuuint64_t)rows, 2, (cuuint64_t)cols / tc::kTileK};
-    const cuuint64_t strides[3] = {(cuuint64_t)cols * 2, (cuuint64_t)gap, (cuuint64_t)tc::kTileK * 2};
-    const cuuint32_t box[4] = {(cuuint32_t)tc::kTileK, (cuuint32_t)(tc::kTileM / 2), 2, (cuuint32_t)box_kb};
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
-    const CUresult r = encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(lo), dims, strides, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return nullptr;
-    return &(pair_cache[key] = m);
-  }
-
   // Rows [0, rows) of a matrix and the rows `gap` bytes behind them, as (column, row, half, K block): a box is box_rows rows of
-  // both halves per K block, one after the other.  The halves are two matrices, or the two halves of a head's rotation pairs.
+  // both halves per K block, one after the other.  The halves are two matrices, or the two halves of a head's rotation pairs (which
+  // makes the tensor's last rows end behind the matrix: no box asks for those).
   std::map<std::tuple<const void*, uint64_t, int, int, int, int>, CUtensorMap> halves_cache;
   const CUtensorMap* get_halves(const void* ptr, uint64_t gap, int rows, int cols, int box_rows, int box_kb) {
     auto key = std::make_tuple(ptr, gap, rows, cols, box_rows, box_kb);

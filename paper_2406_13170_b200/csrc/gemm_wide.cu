@@ -864,7 +864,8 @@ bool tc_wide_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_
   WideParams prm;
   if (!wide_params<WIDE_SWIGLU>(g, xb, 1, f / 128, in, rows, 0, g->wide_scratch + g->wide_scratch_floats, g->wide_scratch_floats, &maps, &prm)) return false;
   const bool up_first = (const char*)w_up < (const char*)w_gate;
-  const CUtensorMap* m = g->get_wide_pair(up_first ? w_up : w_gate, up_first ? w_gate : w_up, f, in, prm.kb);
+  const uint64_t gap = up_first ? (const char*)w_gate - (const char*)w_up : (const char*)w_up - (const char*)w_gate;
+  const CUtensorMap* m = g->get_halves(up_first ? w_up : w_gate, gap, f, in, kTileM / 2, prm.kb);
   if (!m) return false;
   maps.w[0] = *m;
   prm.act = (__nv_bfloat16*)act;
