@@ -197,10 +197,10 @@ def test_nothing_of_a_timeout_outlives_a_reset_or_a_prefill():
 
 
 # passes of up to 64 rows (16 weight features a tile, whole tiles of both), of 65-128 rows in one order of sums (two accumulators), of
-# up to 16 rows at 7B widths, and the pair projection's forms
+# up to 16 rows at 7B widths, and the pair projection's forms, with two K blocks a stage and with one
 @pytest.mark.parametrize("change,n", [(dict(n_nodes=43), 40), (dict(d_ffn=11008, n_nodes=100, lm_rank=24), 100),
                                       (dict(d_model=4096, n_heads=32, d_ffn=11008, n_layers=1, n_nodes=16), 12),
-                                      (dict(n_nodes=100), 300)])
+                                      (dict(n_nodes=100), 300), (dict(d_model=3072, n_heads=24, d_ffn=3456, n_layers=1, n_nodes=100), 300)])
 def test_waits_of_the_projections_inside_a_pass_run_out(change, n):
     """Every projection of a prefill, then of a draft and a verification, gives up after 1 ms: the calls say so, the caches hold zeros
     (nothing else a projection gave up on may be in them, attention fetches whole tiles), and the next prefill is as it was."""

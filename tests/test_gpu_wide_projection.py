@@ -10,7 +10,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("rows", [65, 96, 97, 128, 200, 256, 257, 300, 511, 512])
-@pytest.mark.parametrize("n_seg,out,inner", [(1, 256, 64), (3, 512, 192), (2, 768, 1408), (1, 6656, 512)])
+# stages of two K blocks up to 128 rows or K = 2816 (64, 192, 2816 and 2880: whole and half last stages), of one beyond
+@pytest.mark.parametrize("n_seg,out,inner", [(1, 256, 64), (3, 512, 192), (2, 768, 1408), (1, 6656, 512), (1, 768, 2816), (1, 768, 2880),
+                                             (2, 512, 4096)])
 def test_plain_form_against_double(rows, n_seg, out, inner):
     from paper_2406_13170_b200 import project
     g = torch.Generator(device="cuda").manual_seed(rows * 7 + out)
@@ -27,7 +29,8 @@ def test_plain_form_against_double(rows, n_seg, out, inner):
 
 
 # head_dim 64 and 128; odd numbers of tiles; prompts whose passes carry one ragged group, several groups, and two passes
-@pytest.mark.parametrize("heads,dh,ffn", [(8, 64, 1408), (4, 128, 1408), (10, 128, 3456), (6, 128, 896)])
+# (24 x 128: K above 2816, stages of one K block from 129 rows on)
+@pytest.mark.parametrize("heads,dh,ffn", [(8, 64, 1408), (4, 128, 1408), (10, 128, 3456), (6, 128, 896), (24, 128, 3456)])
 @pytest.mark.parametrize("n", [70, 128, 300, 513])
 def test_fused_forms_against_the_separate_kernels(heads, dh, ffn, n):
     from paper_2406_13170_b200 import Amphista
@@ -53,7 +56,7 @@ def test_fused_forms_against_the_separate_kernels(heads, dh, ffn, n):
 
 
 # 384 = 3 * 128: the q / k / v and the residual form decline (they own 256 columns at a time), gate / up does not
-@pytest.mark.parametrize("heads,dh,ffn", [(8, 64, 1408), (4, 128, 1408), (3, 128, 1408), (10, 128, 3456)])
+@pytest.mark.parametrize("heads,dh,ffn", [(8, 64, 1408), (4, 128, 1408), (3, 128, 1408), (10, 128, 3456), (24, 128, 3456)])
 @pytest.mark.parametrize("n", [70, 128, 300, 513])
 def test_pair_projections_against_the_kernels_of_fewer_rows(heads, dh, ffn, n):
     from paper_2406_13170_b200 import Amphista
