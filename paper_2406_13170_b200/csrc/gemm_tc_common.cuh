@@ -155,6 +155,7 @@ struct TcGemm {
 
   // pair kernel: CTA pairs that run at a time (0: not available, -1: not asked yet), scratch and flags of cut tiles
   int wide_pairs = -1;
+  bool wide_ready[4][2] = {};                   // forms by K blocks of a stage: shared memory limit raised
   float* wide_scratch = nullptr;
   size_t wide_scratch_floats = 0;
   int* wide_flags = nullptr;

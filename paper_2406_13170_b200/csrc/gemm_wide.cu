@@ -668,12 +668,15 @@ int active_clusters(const TcGemm* g, const void* kernel, int ctas, size_t smem) 
   return n;
 }
 template <int EPI>
-bool allow_smem(size_t bytes) {
-  if (cudaFuncSetAttribute(tc_wide_kernel<EPI, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess &&
-      cudaFuncSetAttribute(tc_wide_kernel<EPI, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess)
-    return true;
-  cudaGetLastError();
-  return false;
+constexpr size_t ring_smem() { return EPI == WIDE_RESID ? kResidSmem : kWideSmem; }
+// Raises the shared memory limit of a form that is about to be launched, once per plan set: amph_project makes one per call, and three forms
+// more than it needs cost it 0.5 us (100 rows: 10.5 us of host time, now 9.9).
+template <int EPI, int KB>
+bool allow_smem(TcGemm* g) {
+  bool& ready = g->wide_ready[EPI][KB - 1];
+  if (!ready) ready = cudaFuncSetAttribute(tc_wide_kernel<EPI, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_smem<EPI>()) == cudaSuccess;
+  if (!ready) cudaGetLastError();
+  return ready;
 }
 // K blocks of a stage.  One, so that six are in flight, where a block's MMAs take longer than the step from one stage to the next (two
 // barrier waits, a commit, two copies) and K is long: 4 x 64 rows at 4096, 8 layers, 12 steps 28.4 ms with two (three stages), 27.9 with
@@ -689,8 +692,7 @@ bool wide_available(TcGemm* g) {
   if (!g) return false;
   if (g->wide_pairs < 0) {
     g->wide_pairs = 0;
-    if ((size_t)g->max_smem >= kWideSmem + 7 * 1024 && allow_smem<WIDE_PLAIN>(kWideSmem) && allow_smem<WIDE_SWIGLU>(kWideSmem) &&
-        allow_smem<WIDE_ROPE>(kWideSmem)) {
+    if ((size_t)g->max_smem >= kWideSmem + 7 * 1024 && allow_smem<WIDE_ROPE, 1>(g)) {
       const int clusters = active_clusters(g, (const void*)tc_wide_kernel<WIDE_ROPE, 1>, 2, kWideSmem);
       g->wide_pairs = clusters < g->sm_count / 2 ? clusters : g->sm_count / 2;
     }
@@ -702,7 +704,7 @@ bool resid_available(TcGemm* g) {
   if (!wide_available(g)) return false;
   if (g->resid_clusters[0] == 0) {
     g->resid_clusters[0] = 1;
-    if (allow_smem<WIDE_RESID>(kResidSmem))
+    if (allow_smem<WIDE_RESID, 1>(g))
       for (int s = 1; s <= 4; ++s) g->resid_clusters[s] = active_clusters(g, (const void*)tc_wide_kernel<WIDE_RESID, 1>, 2 * s, kResidSmem);
   }
   return true;
@@ -756,7 +758,7 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
   }
   prm->rows = rows;
   const size_t stage = kb * ((size_t)kTileM * 128 + (size_t)prm->n / 2 * 128);
-  prm->stages = (int)(((EPI == WIDE_RESID ? kResidSmem : kWideSmem) - 1024 - out_bytes) / stage);
+  prm->stages = (int)((ring_smem<EPI>() - 1024 - out_bytes) / stage);
   if (prm->stages > kMaxStages) prm->stages = kMaxStages;
   prm->flags = g->wide_flags;
   prm->wait_first = g->wait_first;
@@ -767,11 +769,12 @@ bool wide_params(TcGemm* g, int xb, int n_seg, int tiles_per_seg, int in, int ro
 }
 
 template <int EPI>
-bool wide_run(const WideMaps& maps, const WideParams& prm, cudaStream_t st) {
+bool wide_run(TcGemm* g, const WideMaps& maps, const WideParams& prm, cudaStream_t st) {
+  if (!(prm.kb == 2 ? allow_smem<EPI, 2>(g) : allow_smem<EPI, 1>(g))) return false;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * prm.groups * prm.nrb);
   cfg.blockDim = dim3(kWideThreads);
-  cfg.dynamicSmemBytes = EPI == WIDE_RESID ? kResidSmem : kWideSmem;
+  cfg.dynamicSmemBytes = ring_smem<EPI>();
   cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -829,7 +832,7 @@ bool tc_wide_launch(TcGemm* g, int xb, const void* const* w, int n_seg, int out,
   prm.P = P;
   prm.ld = (int)ld;
   prm.split_stride = stride;
-  if (!wide_run<WIDE_PLAIN>(maps, prm, st)) return false;
+  if (!wide_run<WIDE_PLAIN>(g, maps, prm, st)) return false;
   *splits_out = splits > 0 ? splits : 1;
   *split_stride = stride;
   return true;
@@ -854,7 +857,7 @@ bool tc_wide_launch_resid(TcGemm* g, int xb, const void* w, int out, int in, int
   prm.xn = (__nv_bfloat16*)xn;
   prm.ss = ss;
   prm.out = out;
-  return wide_run<WIDE_RESID>(maps, prm, st);
+  return wide_run<WIDE_RESID>(g, maps, prm, st);
 }
 
 bool tc_wide_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_up, int f, int in, int rows, void* act, const RowScale& rs,
@@ -872,7 +875,7 @@ bool tc_wide_launch_swiglu(TcGemm* g, int xb, const void* w_gate, const void* w_
   prm.f = f;
   prm.up_first = up_first ? 1 : 0;
   prm.rs = rs;
-  return wide_run<WIDE_SWIGLU>(maps, prm, st);
+  return wide_run<WIDE_SWIGLU>(g, maps, prm, st);
 }
 
 bool tc_wide_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, const void* wv, int n_heads, int dh, int in, int rows, void* q,
@@ -895,7 +898,7 @@ bool tc_wide_launch_qkv_rope(TcGemm* g, int xb, const void* wq, const void* wk, 
   prm.dh = dh;
   prm.max_ctx = max_ctx;
   prm.rs = rs;
-  return wide_run<WIDE_ROPE>(maps, prm, st);
+  return wide_run<WIDE_ROPE>(g, maps, prm, st);
 }
 
 }  // namespace amph
