@@ -49,7 +49,7 @@ def algorithmic_bytes(shape, ctx_len: int) -> int:
 # kernels: the digest below is that of the sources they were taken with (both projection kernels of up to 64 rows, and what they
 # share), and the field is null for any other source.
 NCU_TRAFFIC_PER_WEIGHT_BYTE = 1.03
-NCU_KERNEL_SOURCE_SHA256_16 = "11fb1dd4ce04a656"
+NCU_KERNEL_SOURCE_SHA256_16 = "129ee99b235e40c2"
 
 
 def kernel_source_digest() -> str:
